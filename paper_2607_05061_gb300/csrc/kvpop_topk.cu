@@ -1,33 +1,34 @@
 // Running top-k cutoffs over a prompt (App. C.1 mask, App. C.2 cutoff scan).
 //
-// Kernel 1 (one CTA per row) ranks the row's tokens by static priority, higher
-// first, equal priorities by position: a stable least-significant-digit radix
-// sort of the order-reversed fp32 bit pattern, 4 passes of 8 bits.  Within a
-// round of NT tokens the stable offset of each token inside its digit bucket
-// comes from a warp match on the digit plus per-warp bucket counts; one
-// histogram pass up front gives every pass its bucket bases.  The last pass
-// writes rank[position] directly.
+// Kernel 1 ranks a row's tokens by static priority, higher first, equal priorities by
+// position: a stable least-significant-digit radix sort of the order-reversed fp32 bit
+// pattern, 4 passes of 8 bits.  A cluster of up to 8 CTAs holds the row in registers and
+// shared memory (rank_cluster_kernel); rows too long for that take one CTA that sorts
+// through global memory (rank_kernel).  The last pass writes rank[position] directly.
 //
-// Kernel 2 (one CTA per row, the queries split into up to 16 chunks, one warp
-// each) computes tau_q for every query position.  The paper inserts each newly
-// eligible rank into a Fenwick tree and reads the k-th smallest by binary
-// lifting.  Here the same value comes from the observation
+// Kernel 2 computes tau_q for every query position, a row's queries split over CTAs and
+// their warps.  The paper inserts each newly eligible rank into a Fenwick tree and reads
+// the k-th smallest by binary lifting.  Here the same value comes from the observation
 // that tau_q never increases once k tokens are eligible: a bitset over ranks
 // (8 KB for 65536 tokens, in shared memory) marks the inserted ranks, and when a
 // newcomer ranks below the current cutoff the cutoff steps down to the next
-// marked rank below it -- the warp scans 32 bitset words per ballot.  Over a
-// whole row the cutoff moves down at most S ranks, so the scan is O(S) words
-// plus O(1) per query.  A chunk's warp starts from the state the scan would have
-// reached: it marks the ranks of the tokens already eligible and takes the
-// min(k, n)-th marked rank as the cutoff (a popcount prefix over the bitset).
+// marked rank below it -- the warp scans 32 bitset words per ballot.  A chunk's warp
+// starts from the state the scan would have reached: it marks the ranks of the tokens
+// already eligible and takes the min(k, n)-th marked rank as the cutoff (a popcount
+// prefix over the bitset).
 // While fewer than k tokens are eligible every one of them is kept, so tau_q is
 // the largest inserted rank (-1 while none is).
+#include <cooperative_groups.h>
+
 #include <algorithm>
+#include <climits>
 
 #include "kvpop_internal.cuh"
 
 namespace kvpop {
 namespace {
+
+namespace cg = cooperative_groups;
 
 constexpr int RK_NT = 512;
 constexpr int RK_NW = RK_NT / 32;
@@ -61,6 +62,122 @@ __device__ __forceinline__ int row_length(const int32_t* len, int rows_per_len, 
   return max(0, min(len[row / rows_per_len], S));
 }
 
+// A row's sort by a cluster: CTA c holds elements [c * SEG, (c + 1) * SEG), SEG = 512 * I,
+// each thread I of them in registers (warp-striped, so (warp, item, lane) is the element
+// order and the sort stays stable).  Per pass a warp ranks its elements inside their digit
+// (match + a running count per warp and digit), the CTAs exchange their 256 digit totals
+// through distributed shared memory, and every (key, position) goes to its place in the
+// owner's shared memory: no global traffic but the priorities in and the ranks out.
+// Latency-bound (two cluster barriers and I match rounds per pass), so a row is spread
+// over as many CTAs as leave the GPU about two CTAs per SM.  Device time, against one CTA
+// per row through global memory: 8 rows of 32768 tokens 35 us (458), 16 of 8192 21 us (117),
+// 48 of up to 2801 19 us (45), 8 of 2039 14 us (32).
+template <int I>
+__global__ void __launch_bounds__(RK_NT) rank_cluster_kernel(RankArgs a) {
+  constexpr int SEG = RK_NT * I;
+  extern __shared__ uint2 rk_buf[];              // [SEG] (key, position)
+  __shared__ uint32_t cnt[RK_NW][256];
+  __shared__ uint32_t tot[256], base[256], wsum[8];
+  cg::cluster_group cl = cg::this_cluster();
+  const int C = (int)cl.num_blocks(), c = (int)cl.block_rank();
+  const int row = blockIdx.x / C;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int S = a.S;
+  const int L = row_length(a.len, a.rows_per_len, row, S);
+  const int nsc = max(L - a.tail, 0);
+  const size_t ro = (size_t)row * S;
+  const uint32_t lt_mask = (1u << lane) - 1u;
+  const int e0 = warp * 32 * I + lane;           // element i of the thread: e0 + 32 i
+  uint32_t key[I];
+  int32_t pos[I];
+#pragma unroll
+  for (int i = 0; i < I; ++i) {
+    const int t = c * SEG + e0 + 32 * i;
+    pos[i] = t;
+    key[i] = t < nsc ? rank_key(a.prio[ro + t]) : rank_key(-INFINITY);
+  }
+  for (int p = 0; p < 4; ++p) {
+    for (int j = tid; j < RK_NW * 256; j += RK_NT) (&cnt[0][0])[j] = 0;
+    __syncthreads();
+    uint32_t rk[I];
+#pragma unroll
+    for (int i = 0; i < I; ++i) {
+      const bool ok = c * SEG + e0 + 32 * i < L;
+      const uint32_t dig = ok ? ((key[i] >> (8 * p)) & 255u) : 256u;
+      const uint32_t peers = __match_any_sync(0xffffffffu, dig);
+      const uint32_t within = __popc(peers & lt_mask);
+      const uint32_t old = ok ? cnt[warp][dig] : 0u;
+      __syncwarp();
+      if (ok && within == 0) cnt[warp][dig] = old + __popc(peers);
+      __syncwarp();
+      rk[i] = old + within;
+    }
+    __syncthreads();
+    if (tid < 256) {
+      uint32_t run = 0;
+#pragma unroll
+      for (int w = 0; w < RK_NW; ++w) {
+        const uint32_t n = cnt[w][tid];
+        cnt[w][tid] = run;
+        run += n;
+      }
+      tot[tid] = run;
+    }
+    cl.sync();                                   // every CTA's totals are written
+    uint32_t before = 0, all = 0, x = 0;
+    if (tid < 256) {
+      for (int r = 0; r < C; ++r) {
+        const uint32_t n = cl.map_shared_rank(tot, r)[tid];
+        if (r < c) before += n;
+        all += n;
+      }
+      x = all;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      if (lane == 31) wsum[warp] = x;
+    }
+    __syncthreads();
+    if (tid < 256) {
+      uint32_t off = 0;
+      for (int w = 0; w < warp; ++w) off += wsum[w];
+      base[tid] = off + x - all + before;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < I; ++i) {
+      if (c * SEG + e0 + 32 * i < L) {
+        const uint32_t dig = (key[i] >> (8 * p)) & 255u;
+        const uint32_t dst = base[dig] + cnt[warp][dig] + rk[i];
+        if (p < 3) {
+          cl.map_shared_rank(rk_buf, dst / SEG)[dst % SEG] = make_uint2(key[i], (uint32_t)pos[i]);
+        } else {
+          a.rank[ro + pos[i]] = (int32_t)dst;
+          a.order[ro + dst] = pos[i];
+        }
+      }
+    }
+    cl.sync();          // all elements placed; after the last pass: all totals read
+    if (p < 3) {
+#pragma unroll
+      for (int i = 0; i < I; ++i) {
+        if (c * SEG + e0 + 32 * i < L) {
+          const uint2 v = rk_buf[e0 + 32 * i];
+          key[i] = v.x;
+          pos[i] = (int32_t)v.y;
+        }
+      }
+    }
+  }
+  for (int i = L + c * RK_NT + tid; i < S; i += C * RK_NT) a.rank[ro + i] = -1;
+}
+
+// Rows longer than 8 * 512 * 32 tokens: one CTA per row, keys and positions in global memory.
+// Within a round of RK_NT tokens the stable offset of each token inside its digit bucket
+// comes from a warp match on the digit plus per-warp bucket counts; one histogram pass up
+// front gives every pass its bucket bases.
 __global__ void __launch_bounds__(RK_NT) rank_kernel(RankArgs a) {
   __shared__ uint32_t hist[4][256];
   __shared__ uint32_t base[256];
@@ -195,14 +312,14 @@ __device__ __forceinline__ int kth_marked(const uint32_t* bits, int words, int c
     const int wi = w0 + lane;
     const uint32_t v = wi < words ? bits[wi] : 0u;
     const int cnt = __popc(v);
-    int incl = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    const int total = __reduce_add_sync(0xffffffffu, cnt);
     if (base + total >= c) {
+      int incl = cnt;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
       const uint32_t hit = __ballot_sync(0xffffffffu, base + incl >= c);
       const int l = __ffs(hit) - 1;
       uint32_t word = __shfl_sync(0xffffffffu, v, l);
@@ -220,43 +337,62 @@ __device__ __forceinline__ int kth_marked(const uint32_t* bits, int words, int c
   return -1;
 }
 
-// One CTA per row; warp c takes the queries [c * chunk, (c + 1) * chunk).  It first
-// rebuilds the state the scan has just before its first query -- the bitset of
-// the ranks inserted so far and the cutoff, the min(k, n)-th smallest of them --
-// then runs the same per-query update, so every chunk's cutoffs equal those of
-// one scan over the whole row.
+// CTA (row, y) takes warps * chunk consecutive queries, warp c of it `chunk` of them.  The
+// CTA marks the ranks of the tokens already eligible at its first query once; each warp
+// copies that bitset, adds the tokens up to its own first query and so has the state the
+// scan has there -- the ranks inserted so far and the cutoff, the min(k, n)-th smallest of
+// them -- then runs the same per-query update, so every chunk's cutoffs equal those of
+// one scan over the whole row.  Bound by the serial chain of a warp's queries; with every
+// warp rebuilding its own state from the row's start a chunk had to be 512 queries long.
+// Device time before and now: 8 rows of 32768 tokens 489 -> 56 us, 16 of 8192 183 -> 22 us,
+// 48 of up to 2801 73 -> 17 us.
 __global__ void cutoff_kernel(CutArgs a, int chunk) {
-  extern __shared__ uint32_t bitsets[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  extern __shared__ uint32_t bitsets[];          // [words] of the CTA, then [warps][words]
+  __shared__ int n_base;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int row = blockIdx.x;
   const int S = a.S, words = (S + 31) >> 5;
   const int L = row_length(a.len, a.rows_per_len, row, S);
   const int32_t* rank = a.rank + (size_t)row * S;
   int32_t* tau_out = a.tau + (size_t)row * S;
-  if (warp == 0 && blockIdx.y == 0)
-    for (int i = L + lane; i < S; i += 32) tau_out[i] = -1;
-  // chunk blockIdx.y * warps + warp of the row: the row's chunks are spread over
-  // gridDim.y CTAs so that short batches still fill the GPU
-  const int qa = (blockIdx.y * (blockDim.x >> 5) + warp) * chunk;
+  const int qcta = blockIdx.y * (blockDim.x >> 5) * chunk;
+  for (int i = max(L, qcta) + tid; i < min(S, qcta + (int)(blockDim.x >> 5) * chunk); i += blockDim.x)
+    tau_out[i] = -1;
+  if (qcta >= L) return;
+  const int s = a.s, w = a.w, k = a.k;
+  for (int i = tid; i < words; i += blockDim.x) bitsets[i] = 0u;
+  if (tid == 0) n_base = 0;
+  __syncthreads();
+  // tokens inserted before query qcta: positions s .. qcta - 1 - w
+  int cnt = 0;
+#pragma unroll 8
+  for (int t = s + tid; t <= qcta - 1 - w; t += blockDim.x) {
+    const int r = rank[t];
+    if (r >= 0 && r < S) {
+      atomicOr(&bitsets[r >> 5], 1u << (r & 31));
+      ++cnt;
+    }
+  }
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
+  if (lane == 0 && cnt) atomicAdd(&n_base, cnt);
+  __syncthreads();
+  const int qa = qcta + warp * chunk;
   if (qa >= L) return;
   const int qb = min(qa + chunk, L);
-  uint32_t* bits = bitsets + (size_t)warp * words;
-  for (int i = lane; i < words; i += 32) bits[i] = 0u;
+  uint32_t* bits = bitsets + (size_t)(1 + warp) * words;
+  for (int i = lane; i < words; i += 32) bits[i] = bitsets[i];
   __syncwarp();
-  const int s = a.s, w = a.w, k = a.k;
-  // tokens inserted before query qa: positions s .. qa - 1 - w
-  int cnt = 0;
-  for (int t = s + lane; t <= qa - 1 - w; t += 32) {
+  cnt = 0;
+  for (int t = max(s, qcta - w) + lane; t <= qa - 1 - w; t += 32) {
     const int r = rank[t];
     if (r >= 0 && r < S) {
       atomicOr(&bits[r >> 5], 1u << (r & 31));
       ++cnt;
     }
   }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
   __syncwarp();
-  int n = cnt;
+  int n = n_base + cnt;
   int tau = n > 0 ? kth_marked(bits, words, min(k, n), lane) : -1;
   for (int q0 = qa; q0 < qb; q0 += 32) {
     const int tl = q0 + lane - w;
@@ -269,17 +405,57 @@ __global__ void cutoff_kernel(CutArgs a, int chunk) {
       if (t >= s) {
         const int r = __shfl_sync(0xffffffffu, r_l, j);
         if (r >= 0 && r < S) {
-          if (lane == 0) bits[r >> 5] |= 1u << (r & 31);
-          __syncwarp();
           ++n;
-          if (n <= k) tau = max(tau, r);
-          else if (r < tau) tau = marked_below(bits, tau, lane);
+          if (n <= k || r < tau) {               // ranks above a full cutoff never matter again
+            if (lane == 0) bits[r >> 5] |= 1u << (r & 31);
+            __syncwarp();
+            if (n <= k) tau = max(tau, r);
+            else tau = marked_below(bits, tau, lane);
+          }
         }
       }
       if (lane == j) mine = (k > 0) ? tau : -1;
     }
     if (lane < nq) tau_out[q0 + lane] = mine;
   }
+}
+
+template <int I>
+cudaError_t launch_rank_cluster(const RankArgs& ra, int C, cudaStream_t stream) {
+  const size_t smem = (size_t)RK_NT * I * sizeof(uint2);
+  cudaError_t e = raise_smem_limit(rank_cluster_kernel<I>, smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(ra.n_rows * C));
+  cfg.blockDim = dim3(RK_NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)C;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, rank_cluster_kernel<I>, ra);
+}
+
+// CTAs per row C (a power of two up to 8) and items per thread: the largest C that keeps the
+// grid within two CTAs per SM and gives every CTA at least 1024 elements, more where the row
+// does not fit otherwise.
+cudaError_t launch_rank(const RankArgs& ra, int sms, cudaStream_t stream) {
+  int C = 1;
+  while (C < 8 && (long long)ra.n_rows * (2 * C) <= 2 * sms && ra.S > 2 * RK_NT * C) C *= 2;
+  while (C < 8 && ra.S > 32 * RK_NT * C) C *= 2;
+  const int per = (ra.S + C - 1) / C;
+  if (per > 32 * RK_NT || (long long)ra.n_rows * C > INT_MAX) {
+    rank_kernel<<<ra.n_rows, RK_NT, 0, stream>>>(ra);
+    return cudaGetLastError();
+  }
+  if (per <= 2 * RK_NT) return launch_rank_cluster<2>(ra, C, stream);
+  if (per <= 4 * RK_NT) return launch_rank_cluster<4>(ra, C, stream);
+  if (per <= 8 * RK_NT) return launch_rank_cluster<8>(ra, C, stream);
+  if (per <= 16 * RK_NT) return launch_rank_cluster<16>(ra, C, stream);
+  return launch_rank_cluster<32>(ra, C, stream);
 }
 
 }  // namespace
@@ -306,19 +482,20 @@ cudaError_t launch_topk(const float* prio, const int32_t* len, int rows_per_len,
               reinterpret_cast<uint32_t*>(ws + 2 * al(n * 4)),
               reinterpret_cast<int32_t*>(ws + 3 * al(n * 4)), rank,
               order ? order : reinterpret_cast<int32_t*>(ws + 3 * al(n * 4))};
-  rank_kernel<<<n_rows, RK_NT, 0, stream>>>(ra);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  // chunks per row: up to 16 warps, each with its own bitset of S bits in shared memory
-  const size_t words_bytes = (size_t)((S + 31) / 32) * 4;
-  const int nch = (int)std::max<size_t>(1, std::min<size_t>(CUT_MAX_WARPS, (200 * 1024) / words_bytes));
-  // CTAs per row: enough for about two per SM, while every chunk keeps >= 512 queries
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaError_t e = launch_rank(ra, sms, stream);
+  if (e != cudaSuccess) return e;
+  // warps per CTA: up to 16, each with its own bitset of S bits beside the CTA's
+  const size_t words_bytes = (size_t)((S + 31) / 32) * 4;
+  const int nch = (int)std::max<size_t>(1, std::min<size_t>(CUT_MAX_WARPS, (200 * 1024) / words_bytes - 1));
+  // queries per warp: enough CTAs for about two per SM, at least 32 (a warp's reads of the
+  // newcomers' ranks) and at most 512 (the serial chain of one warp)
   const int want = std::max(1, (2 * sms + n_rows - 1) / n_rows);
-  const int split = std::max(1, std::min(want, S / (nch * 512)));
-  const int chunk = (S + nch * split - 1) / (nch * split);
-  const size_t smem = (size_t)nch * words_bytes;
+  const int per = (S + nch * want - 1) / (nch * want);
+  const int chunk = std::min(512, std::max(32, (per + 31) / 32 * 32));
+  const int split = (S + nch * chunk - 1) / (nch * chunk);
+  const size_t smem = (size_t)(nch + 1) * words_bytes;
   e = raise_smem_limit(cutoff_kernel, smem);
   if (e != cudaSuccess) return e;
   CutArgs ca{rank, len, rows_per_len, n_rows, S, s, w, k, tau};
