@@ -12,13 +12,17 @@
 // of the rest by (priority desc, position asc) -- an exact 4-pass radix select
 // on the order-preserving bit pattern of the fp32 priority, ties resolved by
 // position -- writes them to slots 0.. in ascending position, and loads the
-// window with the last min(P, D) tokens.
+// window with the last min(P, D) tokens.  A cluster of CTAs shares one pair.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "kvpop_argmin.cuh"
 
 namespace kvpop {
 namespace {
+
+namespace cg = cooperative_groups;
 
 constexpr int UT = 32;          // prompt tokens scored per CTA
 constexpr int NT1 = 256;
@@ -376,28 +380,44 @@ struct SelectArgs {
   int Pmax;
 };
 
-__device__ __forceinline__ int block_excl_scan_flag(bool f, int* wsum, int& total) {
+// Exclusive scan over the block of two 16-bit counts packed in a word; `total` gets the sums.
+__device__ __forceinline__ int block_excl_scan2(int v, int* wsum, int& total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned bal = __ballot_sync(0xffffffffu, f);
-  const int within = __popc(bal & ((1u << lane) - 1u));
-  if (lane == 0) wsum[warp] = __popc(bal);
+  int x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) wsum[warp] = x;
   __syncthreads();
   int before = 0, tot = 0;
+#pragma unroll
   for (int w = 0; w < NT2 / 32; ++w) {
-    const int x = wsum[w];
-    if (w < warp) before += x;
-    tot += x;
+    const int y = wsum[w];
+    if (w < warp) before += y;
+    tot += y;
   }
   __syncthreads();
   total = tot;
-  return before + within;
+  return before + x - v;
 }
 
+// A cluster of C CTAs per (sequence, KV head), each on a contiguous part of the eligible
+// tokens: digit counts and kept counts are exchanged through distributed shared memory, each
+// CTA compacts and copies the rows it keeps.  Bound by the chain of passes over the
+// priorities (L2) and by the copy of 2 B rows, both of which one CTA per pair leaves on too
+// few SMs when the batch is small.  Device time, against one CTA per pair with one atomic per
+// priority: 8 pairs of 32768 tokens (B = 4096) 39 us (352), 48 of up to 2801 (B = 1024)
+// 34 us (98), 64 of up to 4009 (all kept) 53 us (312).
 template <typename T>
 __global__ void __launch_bounds__(NT2) prefill_select_kernel(SelectArgs<T> a) {
+  constexpr int NW = NT2 / 32, EPT = 4;
+  cg::cluster_group cl = cg::this_cluster();
+  const int C = (int)cl.num_blocks(), c = (int)cl.block_rank();
   const Dims& dm = a.dm;
   const int d = dm.d, D = dm.D, G = dm.G, H = dm.H, B = dm.B, s = dm.s;
-  const int lp = blockIdx.x;
+  const int lp = blockIdx.x / C;
   const int bl = lp / H, h = lp - bl * H;
   const int pair = (a.first_seq + bl) * H + h;
   const int P = a.plen[bl];
@@ -408,11 +428,15 @@ __global__ void __launch_bounds__(NT2) prefill_select_kernel(SelectArgs<T> a) {
   const bool selecting = n_long > ksel;
   const size_t Pm = a.Pmax;
   const float* pr = a.prio + (size_t)lp * Pm;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // this CTA's part [lo, hi) of the eligible tokens
+  const int seg = (n_elig + C - 1) / C;
+  const int lo = min(c * seg, n_elig), hi = min(lo + seg, n_elig);
 
-  __shared__ unsigned hist[256];
-  __shared__ unsigned s_prefix, s_mask;
-  __shared__ int s_k;
-  __shared__ int wsum[NT2 / 32];
+  __shared__ unsigned hist[2][256];
+  __shared__ unsigned s_prefix;
+  __shared__ int s_k, n_gt, n_eq;
+  __shared__ int wsum[NW];
 
   uint32_t kth = 0;
   int need_eq = 0;
@@ -420,56 +444,121 @@ __global__ void __launch_bounds__(NT2) prefill_select_kernel(SelectArgs<T> a) {
     uint32_t prefix = 0, mask = 0;
     int k = ksel;
     for (int shift = 24; shift >= 0; shift -= 8) {
-      for (int i = threadIdx.x; i < 256; i += NT2) hist[i] = 0;
+      unsigned* hs = hist[(shift >> 3) & 1];
+      if (tid < 256) hs[tid] = 0;
       __syncthreads();
-      for (int u = s_eff + threadIdx.x; u < n_elig; u += NT2) {
-        const uint32_t key = order_key(pr[u]);
-        if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1u);
+      for (int u0 = max(lo, s_eff); u0 < hi; u0 += NT2) {
+        const int u = u0 + tid;
+        unsigned dig = 256u;
+        if (u < hi) {
+          const uint32_t key = order_key(pr[u]);
+          if ((key & mask) == prefix) dig = (key >> shift) & 255u;
+        }
+        // one addition per digit and warp: the top digits take few values
+        const unsigned peers = __match_any_sync(0xffffffffu, dig);
+        if (dig < 256u && (__ffs(peers) - 1) == lane) atomicAdd(&hs[dig], (unsigned)__popc(peers));
+      }
+      cl.sync();
+      // thread t holds digit 255 - t: the inclusive scan counts the keys at or above it
+      int all = 0, x = 0;
+      if (tid < 256) {
+        for (int r = 0; r < C; ++r) all += (int)cl.map_shared_rank(hs, r)[255 - tid];
+        x = all;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, x, o);
+          if (lane >= o) x += y;
+        }
+        if (lane == 31) wsum[warp] = x;
       }
       __syncthreads();
-      if (threadIdx.x == 0) {
-        int cum = 0;
-        for (int dg = 255; dg >= 0; --dg) {
-          const int c = (int)hist[dg];
-          if (cum + c >= k) { s_prefix = prefix | ((uint32_t)dg << shift); s_k = k - cum; break; }
-          cum += c;
+      if (tid < 256) {
+        for (int w = 0; w < warp; ++w) x += wsum[w];
+        if (x >= k && x - all < k) {
+          s_prefix = prefix | ((unsigned)(255 - tid) << shift);
+          s_k = k - (x - all);
         }
-        s_mask = mask | (255u << shift);
       }
       __syncthreads();
       prefix = s_prefix;
-      mask = s_mask;
+      mask |= 255u << shift;
       k = s_k;
-      __syncthreads();
     }
     kth = prefix;
     need_eq = k;
   }
 
+  // kept counts of the parts before this one
+  if (tid == 0) n_gt = n_eq = 0;
+  __syncthreads();
+  int before_gt = 0, before_eq = 0, all_gt = n_elig, all_eq = 0;
+  if (selecting) {
+    int cg_ = 0, ce = 0;
+    for (int u = lo + tid; u < hi; u += NT2) {
+      const uint32_t key = order_key(pr[u]);
+      const bool gt = u < s_eff || key > kth;
+      cg_ += gt;
+      ce += !gt && key == kth;
+    }
+    cg_ = __reduce_add_sync(0xffffffffu, cg_);
+    ce = __reduce_add_sync(0xffffffffu, ce);
+    if (lane == 0) {
+      if (cg_) atomicAdd(&n_gt, cg_);
+      if (ce) atomicAdd(&n_eq, ce);
+    }
+    cl.sync();
+    all_gt = 0;
+    for (int r = 0; r < C; ++r) {
+      const int g = *cl.map_shared_rank(&n_gt, r), q = *cl.map_shared_rank(&n_eq, r);
+      if (r < c) { before_gt += g; before_eq += q; }
+      all_gt += g;
+      all_eq += q;
+    }
+  } else {
+    before_gt = lo;
+  }
+  const int nkept = all_gt + min(all_eq, need_eq);
+
   float* sc = a.st.score + (size_t)pair * B;
   int32_t* ps = a.st.pos + (size_t)pair * B;
-  int run_keep = 0, run_eq = 0;
-  for (int base = 0; base < n_elig; base += NT2) {
-    const int u = base + threadIdx.x;
-    const bool in = u < n_elig;
-    float pv = 0.f;
-    uint32_t key = 0;
-    if (in) { pv = pr[u]; key = order_key(pv); }
-    const bool eq = in && selecting && u >= s_eff && key == kth;
-    int tot_eq;
-    const int eq_rank = run_eq + block_excl_scan_flag(eq, wsum, tot_eq);
-    const bool keep = in && (u < s_eff || !selecting || key > kth || (eq && eq_rank < need_eq));
-    int tot_keep;
-    const int slot = run_keep + block_excl_scan_flag(keep, wsum, tot_keep);
-    if (keep) { sc[slot] = pv; ps[slot] = u; }
-    run_eq += tot_eq;
-    run_keep += tot_keep;
+  const int slot_lo = before_gt + min(before_eq, need_eq);
+  int run_gt = before_gt, run_eq = before_eq;
+  for (int base = lo; base < hi; base += NT2 * EPT) {
+    float pv[EPT];
+    bool gt[EPT], eq[EPT];
+    int v = 0;
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) {
+      const int u = base + tid * EPT + e;
+      const bool in = u < hi;
+      pv[e] = in ? pr[u] : 0.f;
+      const uint32_t key = order_key(pv[e]);
+      gt[e] = in && (u < s_eff || !selecting || key > kth);
+      eq[e] = in && !gt[e] && key == kth;
+      v += (int)gt[e] + ((int)eq[e] << 16);
+    }
+    int tot;
+    const int ex = block_excl_scan2(v, wsum, tot);
+    int g = run_gt + (ex & 0xffff), q = run_eq + (ex >> 16);
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) {
+      if (gt[e] || (eq[e] && q < need_eq)) {
+        const int slot = g + min(q, need_eq);
+        if (dcheck(slot < B, a.st.err, DEVERR_INDEX)) {
+          sc[slot] = pv[e];
+          ps[slot] = base + tid * EPT + e;
+        }
+      }
+      g += gt[e];
+      q += eq[e];
+    }
+    run_gt += tot & 0xffff;
+    run_eq += tot >> 16;
   }
+  const int slot_hi = run_gt + min(run_eq, need_eq);
   __syncthreads();
-  const int nkept = run_keep;
 
-  // copy kept rows, one warp per row
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // copy this CTA's kept rows: a warp takes 4 rows at a time, K and V pieces of 16 bytes
   const int R = d * (int)sizeof(T);
   const int chunks = R / 16;
   const unsigned char* Kp = reinterpret_cast<const unsigned char*>(a.K) + ((size_t)bl * H + h) * Pm * R;
@@ -477,14 +566,26 @@ __global__ void __launch_bounds__(NT2) prefill_select_kernel(SelectArgs<T> a) {
   unsigned char* sK = static_cast<unsigned char*>(a.st.slotK) + (size_t)pair * B * R;
   unsigned char* sV = static_cast<unsigned char*>(a.st.slotV) + (size_t)pair * B * R;
   dcheck(nkept <= B, a.st.err, DEVERR_INDEX);
-  for (int slot = warp; slot < min(nkept, B); slot += NT2 / 32) {
-    const int u = ps[slot];
-    if (!dcheck(u >= 0 && u < P, a.st.err, DEVERR_INDEX)) continue;
-    for (int c = lane; c < chunks; c += 32) {
-      reinterpret_cast<uint4*>(sK + (size_t)slot * R)[c] =
-          reinterpret_cast<const uint4*>(Kp + (size_t)u * R)[c];
-      reinterpret_cast<uint4*>(sV + (size_t)slot * R)[c] =
-          reinterpret_cast<const uint4*>(Vp + (size_t)u * R)[c];
+  for (int slot0 = slot_lo + 4 * warp; slot0 < min(slot_hi, B); slot0 += 4 * NW) {
+    const int nr = min(4, min(slot_hi, B) - slot0);
+    for (int piece = lane; piece < 2 * chunks; piece += 32) {
+      const unsigned char* src = piece < chunks ? Kp : Vp;
+      unsigned char* dst = piece < chunks ? sK : sV;
+      const int off = (piece < chunks ? piece : piece - chunks) * 16;
+      uint4 x[4];
+      bool ok[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        ok[r] = false;
+        if (r < nr) {
+          const int u = ps[slot0 + r];
+          ok[r] = dcheck(u >= 0 && u < P, a.st.err, DEVERR_INDEX);
+          if (ok[r]) x[r] = *reinterpret_cast<const uint4*>(src + (size_t)u * R + off);
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        if (ok[r]) *reinterpret_cast<uint4*>(dst + (size_t)(slot0 + r) * R + off) = x[r];
     }
   }
   // window: positions max(0, P-D) .. P-1 at ring index t % D
@@ -492,11 +593,11 @@ __global__ void __launch_bounds__(NT2) prefill_select_kernel(SelectArgs<T> a) {
   unsigned char* rV = static_cast<unsigned char*>(a.st.ringV) + (size_t)pair * D * R;
   float* rQ = a.st.ringQm + (size_t)pair * D * d;
   const T* Qp = a.Q + ((size_t)bl * H * G + (size_t)h * G) * Pm * d;
-  for (int t = max(0, P - D) + warp; t < P; t += NT2 / 32) {
+  for (int t = max(0, P - D) + c * NW + warp; t < P; t += C * NW) {
     const int ri = t % D;
-    for (int c = lane; c < chunks; c += 32) {
-      reinterpret_cast<uint4*>(rK + (size_t)ri * R)[c] = reinterpret_cast<const uint4*>(Kp + (size_t)t * R)[c];
-      reinterpret_cast<uint4*>(rV + (size_t)ri * R)[c] = reinterpret_cast<const uint4*>(Vp + (size_t)t * R)[c];
+    for (int p = lane; p < chunks; p += 32) {
+      reinterpret_cast<uint4*>(rK + (size_t)ri * R)[p] = reinterpret_cast<const uint4*>(Kp + (size_t)t * R)[p];
+      reinterpret_cast<uint4*>(rV + (size_t)ri * R)[p] = reinterpret_cast<const uint4*>(Vp + (size_t)t * R)[p];
     }
     for (int i = lane; i < d; i += 32) {
       float acc = 0.f;
@@ -504,33 +605,61 @@ __global__ void __launch_bounds__(NT2) prefill_select_kernel(SelectArgs<T> a) {
       rQ[(size_t)ri * d + i] = acc * (1.0f / (float)G);
     }
   }
-  __syncthreads();
+  cl.sync();            // every kept priority of the pair is written; the counts are read
   if (nkept == B) {
-    // block minima over the long-range slots, then the head minimum
+    // block minima over the long-range slots, then the head minimum.  The priorities come
+    // from all CTAs of the cluster, so they are read from L2.
     const int NB = min_blocks(B);
     float* bsc = a.st.blk_score + (size_t)pair * NB;
     int32_t* bsl = a.st.blk_slot + (size_t)pair * NB;
-    for (int k = warp; k < NB; k += NT2 / 32) {
-      float m;
-      int mi;
-      block_min(sc, s, B, k, -1, 0.f, m, mi);
+    for (int k = c * NW + warp; k < NB; k += C * NW) {
+      float m = INFINITY;
+      int mi = 0x7fffffff;
+#pragma unroll
+      for (int r = 0; r < kMinBlock / 32; ++r) {
+        const int i = k * kMinBlock + r * 32 + lane;
+        if (i < B && i >= s) lex_min(m, mi, __ldcg(sc + i), i);
+      }
+      warp_lex_min(m, mi);
       if (lane == 0) { bsc[k] = m; bsl[k] = mi; }
     }
-    __syncthreads();
-    if (warp == 0) {
-      float m;
-      int mi;
-      blocks_min(bsc, bsl, NB, -1, 0.f, 0, m, mi);
+    cl.sync();
+    if (c == 0 && warp == 0) {
+      float m = INFINITY;
+      int mi = 0x7fffffff;
+      for (int k = lane; k < NB; k += 32) lex_min(m, mi, __ldcg(bsc + k), __ldcg(bsl + k));
+      warp_lex_min(m, mi);
       if (lane == 0) { a.st.min_score[pair] = m; a.st.min_slot[pair] = mi; }
     }
-  } else if (threadIdx.x == 0) {
+  } else if (c == 0 && tid == 0) {
     a.st.min_score[pair] = INFINITY;
     a.st.min_slot[pair] = -1;
   }
-  if (threadIdx.x == 0) {
+  if (c == 0 && tid == 0) {
     a.st.nvalid[pair] = nkept;
     a.st.len[pair] = P;
   }
+}
+
+// CTAs per pair: the largest power of two up to 8 that keeps the grid within two CTAs per SM
+// and gives every CTA at least 1024 tokens.
+template <typename T>
+cudaError_t launch_select(const SelectArgs<T>& sel, int pairs, cudaStream_t stream) {
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int C = 1;
+  while (C < 8 && (long long)pairs * (2 * C) <= 2 * sms && sel.Pmax >= 2048 * C) C *= 2;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(pairs * C));
+  cfg.blockDim = dim3(NT2);
+  cfg.stream = stream;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)C;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, prefill_select_kernel<T>, sel);
 }
 
 size_t score_smem(const Dims& dm) { return ((size_t)3 * dm.d * UT + 32 * dm.d + UT * NT1) * 4; }
@@ -591,24 +720,18 @@ static cudaError_t prefill_t(const State& st, const Dims& dm, const void* Q, con
     if (e != cudaSuccess) return e;
   }
   SelectArgs<T> sel{st, dm, (const T*)Q, (const T*)K, (const T*)V, plen, prio, first_seq, Pmax};
-  prefill_select_kernel<T><<<pairs, NT2, 0, stream>>>(sel);
-  return cudaGetLastError();
+  return launch_select(sel, pairs, stream);
 }
 
 cudaError_t launch_prefill_select(const State& st, const Dims& dm, const void* Q, const void* K,
                                   const void* V, const int32_t* plen, int first_seq, int n_seq,
                                   int Pmax, const float* prio, cudaStream_t stream) {
   const int pairs = n_seq * dm.H;
-  if (dm.dtype == KVPOP_F32) {
-    SelectArgs<float> sel{st, dm, (const float*)Q, (const float*)K, (const float*)V, plen, prio,
-                          first_seq, Pmax};
-    prefill_select_kernel<float><<<pairs, NT2, 0, stream>>>(sel);
-  } else {
-    SelectArgs<bf16> sel{st, dm, (const bf16*)Q, (const bf16*)K, (const bf16*)V, plen, prio,
-                         first_seq, Pmax};
-    prefill_select_kernel<bf16><<<pairs, NT2, 0, stream>>>(sel);
-  }
-  return cudaGetLastError();
+  if (dm.dtype == KVPOP_F32)
+    return launch_select(SelectArgs<float>{st, dm, (const float*)Q, (const float*)K, (const float*)V,
+                                           plen, prio, first_seq, Pmax}, pairs, stream);
+  return launch_select(SelectArgs<bf16>{st, dm, (const bf16*)Q, (const bf16*)K, (const bf16*)V, plen,
+                                        prio, first_seq, Pmax}, pairs, stream);
 }
 
 cudaError_t launch_prefill(const State& st, const Dims& dm, const void* Q, const void* K,
