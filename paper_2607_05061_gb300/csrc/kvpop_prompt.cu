@@ -21,8 +21,10 @@
 // bf16: m16n8k16 tensor-core MMAs (Q fragments in registers, K via ldmatrix,
 // V via ldmatrix.trans, probabilities packed to bf16 in registers), K/V rows
 // gathered by 16-byte cp.async into a 128-byte-swizzled double buffer.
-// fp32: CUDA-core kernel, one warp per (query, head) row, 32 keys per round.
+// fp32: CUDA-core kernel, 64 (query, head) rows against blocks of listed keys; one warp per
+// row where the key lists do not fit beside its tiles.
 #include <cstdlib>
+#include <type_traits>
 
 #include "kvpop_mma.cuh"
 #include "kvpop_prompt.cuh"
@@ -32,11 +34,11 @@ namespace {
 
 using namespace prompt;
 
-// ---------------------------------------------------------------- CUDA-core kernel
+// ---------------------------------------------------------------- fp32 kernel for long lists
 constexpr int SIMT_NT = 256;
 constexpr int SIMT_BM = 32;
 
-template <typename T, int HD, bool DENSE>
+template <int HD>
 __global__ void __launch_bounds__(SIMT_NT) prompt_simt_kernel(PromptArgs a) {
   extern __shared__ __align__(16) unsigned char smem_simt[];
   unsigned char* smem = smem_simt;
@@ -48,27 +50,22 @@ __global__ void __launch_bounds__(SIMT_NT) prompt_simt_kernel(PromptArgs a) {
   int32_t* posA = red + NW + 2;
   int32_t* posM = posA + a.capA;
   TileInfo ti;
-  if (DENSE) {
-    if (!dense_setup(a, SIMT_BM, ti)) return;
-  } else if (!tile_setup<SIMT_NT>(a, SIMT_BM, tauS, red, posA, posM, ti)) {
-    return;
-  }
-  const bool want_y = a.Y != nullptr;
+  if (!tile_setup<SIMT_NT>(a, SIMT_BM, tauS, red, posA, posM, ti)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int G = a.G, H = a.H, S = a.S;
   const int nA = ti.nA, nU = ti.nA + ti.nM;
-  const T* Kp = static_cast<const T*>(a.K) + (size_t)ti.pair * S * HD;
-  const T* Vp = static_cast<const T*>(a.V) + (size_t)ti.pair * S * HD;
-  const int32_t* rank = DENSE ? nullptr : a.rank + (size_t)ti.pair * S;
+  const float* Kp = static_cast<const float*>(a.K) + (size_t)ti.pair * S * HD;
+  const float* Vp = static_cast<const float*>(a.V) + (size_t)ti.pair * S * HD;
+  const int32_t* rank = a.rank + (size_t)ti.pair * S;
   float* q_s = qv + warp * HD;
   for (int r = warp; r < SIMT_BM * G; r += NW) {
     const int ql = r / G, g = r - ql * G, q = ti.q0 + ql;
     if (q > ti.q1) break;
     const size_t row = ((size_t)ti.seq * H * G + (size_t)ti.h * G + g) * S + q;
-    const T* qp = static_cast<const T*>(a.Q) + row * HD;
-    for (int i = lane; i < HD; i += 32) q_s[i] = to_f(qp[i]) * a.qscale;
+    const float* qp = static_cast<const float*>(a.Q) + row * HD;
+    for (int i = lane; i < HD; i += 32) q_s[i] = qp[i] * a.qscale;
     __syncwarp();
-    const int tq = DENSE ? 0 : tauS[ql];
+    const int tq = tauS[ql];
     float m = -INFINITY, l = 0.f, o[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) o[c] = 0.f;
@@ -77,20 +74,15 @@ __global__ void __launch_bounds__(SIMT_NT) prompt_simt_kernel(PromptArgs a) {
       int t = 0;
       bool keep = false;
       if (e < nU) {
-        if (DENSE) {
-          t = e;
-          keep = t <= q;
-        } else {
-          t = e < nA ? posA[e] : posM[e - nA];
-          keep = e < nA || keep_key(q, t, __ldg(rank + t), tq, a.s, a.w);
-        }
+        t = e < nA ? posA[e] : posM[e - nA];
+        keep = e < nA || keep_key(q, t, __ldg(rank + t), tq, a.s, a.w);
       }
       float logit = -INFINITY;
       if (keep) {
-        const T* kr = Kp + (size_t)t * HD;
+        const float* kr = Kp + (size_t)t * HD;
         float acc = 0.f;
 #pragma unroll 8
-        for (int i = 0; i < HD; ++i) acc = fmaf(q_s[i], to_f(kr[i]), acc);
+        for (int i = 0; i < HD; ++i) acc = fmaf(q_s[i], kr[i], acc);
         logit = acc;
       }
       float mx = logit;
@@ -105,7 +97,6 @@ __global__ void __launch_bounds__(SIMT_NT) prompt_simt_kernel(PromptArgs a) {
       for (int o2 = 16; o2; o2 >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, o2);
       l = l * alpha + ps;
       m = m_new;
-      if (!want_y) continue;
 #pragma unroll
       for (int c = 0; c < NC; ++c) o[c] *= alpha;
       const int nk = min(32, nU - e0);
@@ -113,20 +104,238 @@ __global__ void __launch_bounds__(SIMT_NT) prompt_simt_kernel(PromptArgs a) {
         const float pj = __shfl_sync(0xffffffffu, p, jj);
         const int tj = __shfl_sync(0xffffffffu, t, jj);
         if (pj != 0.f) {
-          const T* vr = Vp + (size_t)tj * HD;
+          const float* vr = Vp + (size_t)tj * HD;
 #pragma unroll
-          for (int c = 0; c < NC; ++c) o[c] = fmaf(pj, to_f(vr[lane + 32 * c]), o[c]);
+          for (int c = 0; c < NC; ++c) o[c] = fmaf(pj, vr[lane + 32 * c], o[c]);
         }
       }
     }
-    if (want_y) {
-      const float inv = 1.f / l;
-      float* yp = a.Y + row * HD;
+    const float inv = 1.f / l;
+    float* yp = a.Y + row * HD;
 #pragma unroll
-      for (int c = 0; c < NC; ++c) yp[lane + 32 * c] = o[c] * inv;
-    }
+    for (int c = 0; c < NC; ++c) yp[lane + 32 * c] = o[c] * inv;
     if (a.lse && lane == 0) a.lse[row] = (m + log2f(l)) * kLn2;
     __syncwarp();
+  }
+}
+
+// ---------------------------------------------------------------- fp32 kernel
+// One CTA: 64 (query, head) rows of one (sequence, KV head) against the tile's listed keys in
+// blocks of BN, K and V gathered by 16-byte cp.async into a double buffer (rows padded by 4
+// floats: conflict-free).  A thread holds 4 rows x BN / 16 keys of S (rows ty + 16 i, keys
+// tx + 16 j) and 4 rows x HD / 16 columns of O; the 16 threads of a row share its running
+// maximum by shuffles and pass P through shared memory, inside their own half-warp only.
+// Bound by FP32 FMA and the shared loads that feed it.  8 (pair) rows of 2039 tokens, G = 2,
+// d = 64, 324 keys a query: 123 us, against 3009 us with one warp per row, where
+// each lane walked a K row of its own.
+constexpr int PF_NT = 256;
+constexpr int PF_ROWS = 64;
+
+template <int HD>
+struct PfP {
+  static constexpr int BN = HD == 64 ? 64 : 32;
+  static constexpr int RS = HD + 4;
+  static constexpr int PS = BN + 4;
+  static constexpr int OFF_KV = PF_ROWS * RS;                 // floats: Q, then 2 x (K, V)
+  static constexpr int OFF_P = OFF_KV + 4 * BN * RS;
+  static constexpr int OFF_POS = OFF_P + PF_ROWS * PS;        // positions and ranks of 2 blocks
+  static constexpr int OFF_TAU = OFF_POS + 4 * BN;
+  static constexpr int OFF_RED = OFF_TAU + PF_ROWS;
+  static constexpr int OFF_LIST = OFF_RED + PF_NT / 32 + 4;
+  static_assert(OFF_LIST % 4 == 0, "");
+};
+
+template <int HD, int G, bool DENSE>
+__global__ void __launch_bounds__(PF_NT) prompt_f32_kernel(PromptArgs a) {
+  using P = PfP<HD>;
+  constexpr int BN = P::BN, NJ = BN / 16, NC = HD / 64, BM = PF_ROWS / G;
+  extern __shared__ __align__(16) float sm_pf[];
+  float* Qs = sm_pf;
+  float* Ps = sm_pf + P::OFF_P;
+  int32_t* posb = reinterpret_cast<int32_t*>(sm_pf + P::OFF_POS);
+  int32_t* rkb = posb + 2 * BN;
+  int* tauS = reinterpret_cast<int*>(sm_pf + P::OFF_TAU);
+  int* red = reinterpret_cast<int*>(sm_pf + P::OFF_RED);
+  int32_t* posA = reinterpret_cast<int32_t*>(sm_pf + P::OFF_LIST);
+  int32_t* posM = posA + a.capA;
+  TileInfo ti;
+  if (DENSE) {
+    if (!dense_setup(a, BM, ti)) return;
+  } else if (!tile_setup<PF_NT>(a, BM, tauS, red, posA, posM, ti)) {
+    return;
+  }
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int H = a.H, S = a.S;
+  const int nA = ti.nA, nU = ti.nA + ti.nM;
+  const float* Kp = static_cast<const float*>(a.K) + (size_t)ti.pair * S * HD;
+  const float* Vp = DENSE ? nullptr : static_cast<const float*>(a.V) + (size_t)ti.pair * S * HD;
+  const int32_t* rank = DENSE ? nullptr : a.rank + (size_t)ti.pair * S;
+  const size_t row0 = ((size_t)ti.seq * H * G + (size_t)ti.h * G) * S;
+  const float* Qbase = static_cast<const float*>(a.Q) + row0 * HD;
+  const int pad_t = DENSE ? 0 : (nA > 0 ? posA[0] : posM[0]);
+  auto entry = [&](int e) {
+    if (DENSE) return e < nU ? e : pad_t;
+    return e < nA ? posA[e] : (e < nU ? posM[e - nA] : pad_t);
+  };
+  auto issue = [&](int blk, int st) {
+    const uint32_t kd = (uint32_t)__cvta_generic_to_shared(sm_pf + P::OFF_KV + st * 2 * BN * P::RS);
+    const uint32_t vd = kd + BN * P::RS * 4;
+    for (int i = tid; i < BN * (HD / 4); i += PF_NT) {
+      const int key = i / (HD / 4), c = i - key * (HD / 4);
+      const size_t t = (size_t)entry(blk * BN + key) * HD + 4 * c;
+      const uint32_t off = (key * P::RS + 4 * c) * 4;
+      cp_async16(kd + off, Kp + t, 16);
+      if (!DENSE) cp_async16(vd + off, Vp + t, 16);
+    }
+    if (tid < BN) {
+      const int e = blk * BN + tid, t = entry(e);
+      posb[st * BN + tid] = e < nU ? t : INT_MAX;
+      if (!DENSE) rkb[st * BN + tid] = __ldg(rank + t);
+    }
+  };
+  issue(0, 0);
+  cp_commit();
+  for (int i = tid; i < PF_ROWS * (HD / 4); i += PF_NT) {
+    const int r = i / (HD / 4), c = i - r * (HD / 4);
+    const int q = ti.q0 + r / G, g = r % G;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (q <= ti.q1) v = *reinterpret_cast<const float4*>(Qbase + ((size_t)g * S + q) * HD + 4 * c);
+    v.x *= a.qscale; v.y *= a.qscale; v.z *= a.qscale; v.w *= a.qscale;
+    *reinterpret_cast<float4*>(Qs + r * P::RS + 4 * c) = v;
+  }
+  float m[4], l[4], o[4][NC][4];
+  int qi[4], tq[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = ty + 16 * i;
+    qi[i] = ti.q0 + r / G;
+    tq[i] = DENSE ? 0 : tauS[r / G];
+    m[i] = -INFINITY;
+    l[i] = 0.f;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) o[i][c][0] = o[i][c][1] = o[i][c][2] = o[i][c][3] = 0.f;
+  }
+  const int nblk = (nU + BN - 1) / BN;
+  for (int b = 0; b < nblk; ++b) {
+    const int st = b & 1;
+    if (b + 1 < nblk) issue(b + 1, st ^ 1);
+    cp_commit();
+    cp_wait<1>();
+    __syncthreads();
+    const float* Kb = sm_pf + P::OFF_KV + st * 2 * BN * P::RS;
+    const float* Vb = Kb + BN * P::RS;
+    float s[4][NJ];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) s[i][j] = 0.f;
+#pragma unroll 4
+    for (int c = 0; c < HD; c += 4) {
+      float4 qf[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) qf[i] = *reinterpret_cast<const float4*>(Qs + (ty + 16 * i) * P::RS + c);
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        const float4 k = *reinterpret_cast<const float4*>(Kb + (tx + 16 * j) * P::RS + c);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          s[i][j] = fmaf(qf[i].x, k.x, s[i][j]);
+          s[i][j] = fmaf(qf[i].y, k.y, s[i][j]);
+          s[i][j] = fmaf(qf[i].z, k.z, s[i][j]);
+          s[i][j] = fmaf(qf[i].w, k.w, s[i][j]);
+        }
+      }
+    }
+    const bool masked = (b + 1) * BN > nA;
+    bool zero = false;                             // some probability is exactly 0
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (masked) {
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+          const int e = b * BN + tx + 16 * j;
+          if (e < nA) continue;
+          const int t = posb[st * BN + tx + 16 * j];
+          const bool keep = e < nU && (DENSE ? t <= qi[i]
+                                             : keep_key(qi[i], t, rkb[st * BN + tx + 16 * j], tq[i], a.s, a.w));
+          if (!keep) s[i][j] = -INFINITY;
+        }
+      }
+      float mx = s[i][0];
+#pragma unroll
+      for (int j = 1; j < NJ; ++j) mx = fmaxf(mx, s[i][j]);
+#pragma unroll
+      for (int x = 1; x < 16; x <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, x));
+      const float mn = fmaxf(m[i], mx);
+      const float u = mn == -INFINITY ? 0.f : mn;
+      const float alpha = exp2f(m[i] - u);
+      float ps = 0.f;
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        const float p = exp2f(s[i][j] - u);
+        ps += p;
+        zero |= p == 0.f;
+        if (!DENSE) Ps[(ty + 16 * i) * P::PS + tx + 16 * j] = p;
+      }
+      l[i] = l[i] * alpha + ps;
+      m[i] = mn;
+      if (!DENSE) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+#pragma unroll
+          for (int x = 0; x < 4; ++x) o[i][c][x] *= alpha;
+      }
+    }
+    if (!DENSE) {
+      __syncwarp();                                // a row's P stays inside its half-warp
+      // a key whose probability is 0 for a row leaves it alone, whatever its value holds
+      auto pv = [&](auto skip) {
+#pragma unroll 2
+        for (int k0 = 0; k0 < BN; k0 += 4) {
+          float pr[4][4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float4 p4 = *reinterpret_cast<const float4*>(Ps + (ty + 16 * i) * P::PS + k0);
+            pr[i][0] = p4.x; pr[i][1] = p4.y; pr[i][2] = p4.z; pr[i][3] = p4.w;
+          }
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+              const float4 v = *reinterpret_cast<const float4*>(Vb + (k0 + x) * P::RS + 64 * c + 4 * tx);
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                if (decltype(skip)::value && pr[i][x] == 0.f) continue;
+                o[i][c][0] = fmaf(pr[i][x], v.x, o[i][c][0]);
+                o[i][c][1] = fmaf(pr[i][x], v.y, o[i][c][1]);
+                o[i][c][2] = fmaf(pr[i][x], v.z, o[i][c][2]);
+                o[i][c][3] = fmaf(pr[i][x], v.w, o[i][c][3]);
+              }
+            }
+          }
+        }
+      };
+      if (__any_sync(0xffffffffu, zero)) pv(std::true_type{});
+      else pv(std::false_type{});
+    }
+    __syncthreads();
+  }
+  cp_wait<0>();
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = ty + 16 * i;
+#pragma unroll
+    for (int x = 1; x < 16; x <<= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], x);
+    if (qi[i] > ti.q1) continue;
+    const size_t row = row0 + (size_t)(r % G) * S + qi[i];
+    if (!DENSE) {
+      const float inv = 1.f / l[i];
+#pragma unroll
+      for (int c = 0; c < NC; ++c)
+        *reinterpret_cast<float4*>(a.Y + row * HD + 64 * c + 4 * tx) =
+            make_float4(o[i][c][0] * inv, o[i][c][1] * inv, o[i][c][2] * inv, o[i][c][3] * inv);
+    }
+    if (a.lse && tx == 0) a.lse[row] = (m[i] + log2f(l[i])) * kLn2;
   }
 }
 
@@ -397,15 +606,28 @@ cudaError_t launch_tc(PromptArgs a, int n_pairs, cudaStream_t stream) {
   return launch_cfg(prompt_tc_kernel<HD, G, DENSE, WANT_Y>, grid, P::THREADS, smem, stream, a);
 }
 
-template <typename T, int HD, bool DENSE>
+template <int HD>
 cudaError_t launch_simt(PromptArgs a, int n_pairs, cudaStream_t stream) {
-  if (DENSE) a.capA = a.capM = 0;
-  else a.capM = a.s + 2 * SIMT_BM + a.w;
+  a.capM = a.s + 2 * SIMT_BM + a.w;
   const size_t smem = (size_t)(SIMT_NT / 32) * HD * 4 + (SIMT_BM + SIMT_NT / 32 + 2) * 4 +
                       (size_t)(a.capA + a.capM) * 4;
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   dim3 grid((a.S + SIMT_BM - 1) / SIMT_BM, n_pairs);
-  return launch_cfg(prompt_simt_kernel<T, HD, DENSE>, grid, SIMT_NT, smem, stream, a);
+  return launch_cfg(prompt_simt_kernel<HD>, grid, SIMT_NT, smem, stream, a);
+}
+
+// The tiled fp32 kernel where its lists fit beside the tiles (up to about 30000 entries), the
+// one-warp-per-row kernel beyond.
+template <int HD, int G, bool DENSE>
+cudaError_t launch_f32(PromptArgs a, int n_pairs, cudaStream_t stream) {
+  constexpr int BM = PF_ROWS / G;
+  PromptArgs b = a;
+  if (DENSE) b.capA = b.capM = 0;
+  else b.capM = b.s + 2 * BM + b.w;
+  const size_t smem = ((size_t)PfP<HD>::OFF_LIST + b.capA + b.capM) * 4;
+  if (!DENSE && smem > 227 * 1024) return launch_simt<HD>(a, n_pairs, stream);
+  return launch_cfg(prompt_f32_kernel<HD, G, DENSE>, dim3((a.S + BM - 1) / BM, n_pairs), PF_NT, smem,
+                    stream, b);
 }
 
 }  // namespace
@@ -439,8 +661,14 @@ cudaError_t dispatch(const PromptArgs& a, int n_pairs, int dtype, int d, int G, 
     if (G == 2) return launch_tc<64, 2, DENSE, WANT_Y>(a, n_pairs, stream);
     return launch_tc<64, 1, DENSE, WANT_Y>(a, n_pairs, stream);
   }
-  if (d == 128) return launch_simt<float, 128, DENSE>(a, n_pairs, stream);
-  return launch_simt<float, 64, DENSE>(a, n_pairs, stream);
+  if (d == 128) {
+    if (G == 4) return launch_f32<128, 4, DENSE>(a, n_pairs, stream);
+    if (G == 2) return launch_f32<128, 2, DENSE>(a, n_pairs, stream);
+    return launch_f32<128, 1, DENSE>(a, n_pairs, stream);
+  }
+  if (G == 4) return launch_f32<64, 4, DENSE>(a, n_pairs, stream);
+  if (G == 2) return launch_f32<64, 2, DENSE>(a, n_pairs, stream);
+  return launch_f32<64, 1, DENSE>(a, n_pairs, stream);
 }
 
 }  // namespace
