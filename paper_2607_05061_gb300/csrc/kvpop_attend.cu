@@ -23,7 +23,7 @@
 //    an error code and skips the remaining work without leaving a barrier.
 #include <type_traits>
 
-#include "kvpop_internal.cuh"
+#include "kvpop_sched.cuh"
 
 namespace kvpop {
 namespace {
@@ -148,18 +148,6 @@ __device__ __forceinline__ void unpack(const uint4& w, float (&f)[8]) {
   f[6] = __uint_as_float(w.w << 16); f[7] = __uint_as_float(w.w & 0xffff0000u);
 }
 
-__device__ __forceinline__ int tiles_of(int nv, int np, int tile) {
-  return (nv + tile - 1) / tile + (np + tile - 1) / tile;
-}
-
-// CTA whose tile range [c*T/N, (c+1)*T/N) contains tile t (N <= T).
-__device__ __forceinline__ int cta_of(long long t, long long T, long long N) {
-  return (int)(((t + 1) * N - 1) / T);
-}
-__device__ __forceinline__ long long cta_begin(long long c, long long T, long long N) {
-  return c * T / N;
-}
-
 template <typename T, int HD, int G>
 __global__ void __launch_bounds__(Traits<T, HD, G>::THREADS, 1) attend_kernel(AttendArgs a) {
   using Tr = Traits<T, HD, G>;
@@ -178,6 +166,11 @@ __global__ void __launch_bounds__(Traits<T, HD, G>::THREADS, 1) attend_kernel(At
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int npairs = a.pairs;
+
+  // a programmatic dependent of the ingest, as the kernel after it may be of this one: it is
+  // scheduled while its predecessor ends and waits here before it reads any state
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 
   // ---- prologue: tile counts of every pair, exclusive prefix over pairs ------------
   {
@@ -374,25 +367,9 @@ __global__ void __launch_bounds__(Traits<T, HD, G>::THREADS, 1) attend_kernel(At
       consumer_sync(NWC * 32);
       if (flag[1]) {
         __threadfence();
-        for (int idx = tid; idx < G * HD; idx += NWC * 32) {
-          const int g = idx / HD, i = idx - g * HD;
-          float ms = -INFINITY;
-          for (long long c = ca; c <= cb; ++c) {
-            const int slot = (prefix[p] < cta_begin(c, Ttot, NC)) ? 0 : 1;
-            const float* pc = a.part + ((size_t)c * 2 + slot) * Tr::PSTRIDE;
-            ms = fmaxf(ms, __ldcg(pc + G * HD + g));
-          }
-          float L = 0.f, O = 0.f;
-          for (long long c = ca; c <= cb; ++c) {
-            const int slot = (prefix[p] < cta_begin(c, Ttot, NC)) ? 0 : 1;
-            const float* pc = a.part + ((size_t)c * 2 + slot) * Tr::PSTRIDE;
-            const float mc = __ldcg(pc + G * HD + g);
-            const float f = (mc == -INFINITY) ? 0.f : fast_exp2(mc - ms);
-            L = fmaf(__ldcg(pc + G * HD + G + g), f, L);
-            O = fmaf(__ldcg(pc + g * HD + i), f, O);
-          }
-          a.out[((size_t)p * G + g) * HD + i] = O / L;
-        }
+        merge_partials<G, HD, NWC * 32>(ca, cb, a.part, a.out + (size_t)p * G * HD, mo,
+                                        [] { consumer_sync(NWC * 32); },
+                                        [](float x) { return fast_exp2(x); });
       }
     }
     consumer_sync(NWC * 32);
@@ -518,8 +495,17 @@ cudaError_t launch_t(const State& st, const Dims& dm, const void* q, float* out,
   a.D = dm.D;
   a.qscale = kLog2e / sqrtf((float)HD);
   const size_t smem = Tr::OFF_PREFIX + (size_t)(dm.pairs + 1) * 4;
-  attend_kernel<T, HD, G><<<grid, Tr::THREADS, smem, stream>>>(a);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3(grid < kMaxAttendGrid ? grid : kMaxAttendGrid, 1, 1);
+  cfg.blockDim = dim3(Tr::THREADS, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, attend_kernel<T, HD, G>, a);
 }
 
 }  // namespace

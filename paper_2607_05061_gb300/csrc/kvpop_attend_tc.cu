@@ -51,6 +51,13 @@ constexpr float kThr = 8.0f;
 #ifndef KVPOP_FUSED_SPLIT_K
 #define KVPOP_FUSED_SPLIT_K 5
 #endif
+// Two-kernel step: tiles that each CTA of the attention prefetches during the ingest.  More
+// helps a small batch a little (4-layer step at batch 8: 284 us with 8, 286 with 4), but beside
+// the mLSTM ingest it slows that one's state reads (batch 64: 186.5 us with 4, 187.5 with 8,
+// 192 with 16; 190.5 without).
+#ifndef KVPOP_TC_PREFETCH_TILES
+#define KVPOP_TC_PREFETCH_TILES 4
+#endif
 
 template <int HD, int G>
 struct TcTraits {
@@ -78,6 +85,8 @@ struct TcTraits {
 struct TcArgs {
   const int32_t* nvalid;
   const int32_t* len;
+  const bf16* slotK;           // for the prefetch; the copies go through the tensor maps
+  const bf16* slotV;
   const bf16* q;
   float* out;
   float* part;
@@ -189,11 +198,38 @@ __global__ void __launch_bounds__(FUSED ? TcTraits<HD, G>::THREADS_F : TcTraits<
     // the next step's kernel may be scheduled now: it waits for this grid before reading
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
+  if constexpr (!FUSED) {
+    // While the ingest runs, the schedule its state gives now sends this CTA's first tiles to
+    // L2: the ingest writes one slot and one window row per pair, so almost all of what the
+    // attention reads is already there, and the prefetch is only a hint.  The schedule itself
+    // stays valid once the caches are full (counts compared after the wait).
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    build_schedule<NT>(a.nvalid, a.len, npairs, a.B, a.D, TILE, prefix, scan, nullptr);
+    const long long T = prefix[npairs], N = min((long long)gridDim.x, T);
+    if (blockIdx.x < N && tid < KVPOP_TC_PREFETCH_TILES) {
+      const long long t = cta_begin(blockIdx.x, T, N) + tid;
+      if (t < cta_begin(blockIdx.x + 1, T, N)) {
+        int lo = 0, hi = npairs - 1;
+        while (lo < hi) {
+          const int mid = (lo + hi + 1) >> 1;
+          if (prefix[mid] <= t) lo = mid; else hi = mid - 1;
+        }
+        const int slot = (int)(t - prefix[lo]) * TILE;
+        if (slot < a.B) {
+          const size_t row = (size_t)lo * a.B + slot;
+          const uint32_t bytes = (uint32_t)(min(TILE, a.B - slot) * HD * 2);
+          prefetch_l2(a.slotK + row * HD, bytes);
+          prefetch_l2(a.slotV + row * HD, bytes);
+        }
+      }
+    }
+  }
   // Launched as a programmatic dependent of the kernel before it (the ingest, or the
   // previous fused step): everything below reads the state it writes, so wait here for
   // it to complete (a no-op without a predecessor).
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  build_schedule<NT>(a.nvalid, a.len, npairs, a.B, a.D, TILE, prefix, scan, a.err);
+  if (FUSED || schedule_changed<NT>(a.nvalid, a.len, npairs, a.B, a.D, TILE, prefix, a.err))
+    build_schedule<NT>(a.nvalid, a.len, npairs, a.B, a.D, TILE, prefix, scan, a.err);
   const long long Ttot = prefix[npairs];
   if constexpr (FUSED) {
     // lengths and used-slot counts read: their commits may start once every CTA of this
@@ -635,6 +671,8 @@ static TcArgs tc_args(const State& st, const Dims& dm, const void* q, float* out
   TcArgs a;
   a.nvalid = st.nvalid;
   a.len = st.len;
+  a.slotK = static_cast<const bf16*>(st.slotK);
+  a.slotV = static_cast<const bf16*>(st.slotV);
   a.q = static_cast<const bf16*>(q);
   a.out = out;
   a.part = st.part;
@@ -661,7 +699,7 @@ cudaError_t tc_launch(const State& st, const Dims& dm, const void* maps, const v
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.gridDim = dim3(grid, 1, 1);
+  cfg.gridDim = dim3(std::min(grid, kMaxAttendGrid), 1, 1);
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 1;

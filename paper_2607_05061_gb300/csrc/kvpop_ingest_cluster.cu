@@ -142,6 +142,12 @@ __global__ void __launch_bounds__(NT, 1) ingest_cluster_kernel(ClArgs<T> a) {
       bulk_g2s(smem_u32(smem + L.ws + off), wsrc + off, min(16384u, wbytes - off), bb);
     bulk_g2s(smem_u32(Ws + in_dim * FS), a.b1s + slice * FS, vbytes, bb);
     bulk_g2s(smem_u32(Ws + in_dim * FS + FS), a.w2s + slice * FS, vbytes, bb);
+  }
+  // A programmatic dependent of the kernel before it: the weights above never change, all
+  // that follows is state or input that kernel may still write.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (tid == 0) {
+    const uint32_t bb = smem_u32(&bar);
     // rows that do not depend on the sequence length first ...
     uint32_t rest = 0;
     for (int o = 0; o < OWN; ++o)
@@ -519,13 +525,15 @@ static cudaError_t launch_cl(const State& st, const Dims& dm, const float* W1s, 
   cfg.blockDim = dim3(NT, 1, 1);
   cfg.dynamicSmemBytes = cluster_ingest_smem(dm);
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = CS;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, ingest_cluster_kernel<T>, a);
 }
 

@@ -154,6 +154,10 @@ __global__ void __launch_bounds__(NTM, 1) ingest_mlstm_kernel(MIngestArgs<T> a) 
     for (uint32_t off = 0; off < bytes; off += 32768)
       bulk_g2s(smem_u32(smem + off), src + off, min(32768u, bytes - off), smem_u32(&bar));
   }
+  // the attention may be scheduled now; the weights above never change, all that follows is
+  // state or input that the kernel before this one may still write
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   T* ringK = static_cast<T*>(a.st.ringK);
   T* ringV = static_cast<T*>(a.st.ringV);
   {
@@ -678,17 +682,24 @@ cudaError_t launch_ingest_mlstm(const State& st, const Dims& dm, const MlstmDev&
                                 int32_t* evict_info, float* score_out, cudaStream_t stream) {
   dim3 grid((dm.batch + SBM - 1) / SBM, dm.H);
   const int esz = dm.dtype == KVPOP_F32 ? 4 : 2;
-  const size_t smem = mlstm_ingest_smem(dm.d, m.NC, esz);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(NTM);
+  cfg.dynamicSmemBytes = mlstm_ingest_smem(dm.d, m.NC, esz);
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
   if (dm.dtype == KVPOP_F32) {
     MIngestArgs<float> a{st, dm, to_mstate(m), (const float*)q, (const float*)k, (const float*)v,
                          override_, evict_info, score_out};
-    ingest_mlstm_kernel<float><<<grid, NTM, smem, stream>>>(a);
-  } else {
-    MIngestArgs<bf16> a{st, dm, to_mstate(m), (const bf16*)q, (const bf16*)k, (const bf16*)v,
-                        override_, evict_info, score_out};
-    ingest_mlstm_kernel<bf16><<<grid, NTM, smem, stream>>>(a);
+    return cudaLaunchKernelEx(&cfg, ingest_mlstm_kernel<float>, a);
   }
-  return cudaGetLastError();
+  MIngestArgs<bf16> a{st, dm, to_mstate(m), (const bf16*)q, (const bf16*)k, (const bf16*)v,
+                      override_, evict_info, score_out};
+  return cudaLaunchKernelEx(&cfg, ingest_mlstm_kernel<bf16>, a);
 }
 
 cudaError_t launch_prefill_mlstm_scores(const State& st, const Dims& dm, const MlstmDev& m,

@@ -28,6 +28,8 @@ __device__ __forceinline__ long long cta_begin(long long c, long long T, long lo
 // Block-wide exclusive prefix of per-pair tile counts into prefix[0..npairs]
 // (prefix[npairs] = total).  `scan` holds one int per warp.  Contains
 // __syncthreads; every thread of the block must call it.
+// The counts are read from L2: a kernel may call this before and after the wait for the
+// kernel that writes them, and no line of the first reading may serve the second.
 template <int NT>
 __device__ __forceinline__ void build_schedule(const int32_t* __restrict__ nvalid,
                                                const int32_t* __restrict__ len, int npairs, int B,
@@ -38,7 +40,7 @@ __device__ __forceinline__ void build_schedule(const int32_t* __restrict__ nvali
   const int beg = min(tid * per, npairs), end = min(beg + per, npairs);
   int local = 0;
   for (int i = beg; i < end; ++i)
-    local += tiles_of(used_slots(nvalid[i], B, err), window_rows(len[i], D, err), tile);
+    local += tiles_of(used_slots(__ldcg(nvalid + i), B, err), window_rows(__ldcg(len + i), D, err), tile);
   int incl = local;
 #pragma unroll
   for (int off = 1; off < 32; off <<= 1) {
@@ -56,9 +58,67 @@ __device__ __forceinline__ void build_schedule(const int32_t* __restrict__ nvali
   int run = scan[warp] + incl - local;
   for (int i = beg; i < end; ++i) {
     prefix[i] = run;
-    run += tiles_of(used_slots(nvalid[i], B, nullptr), window_rows(len[i], D, nullptr), tile);
+    run += tiles_of(used_slots(__ldcg(nvalid + i), B, nullptr), window_rows(__ldcg(len + i), D, nullptr), tile);
   }
   __syncthreads();
+}
+
+// Whether some pair's tile count is no longer the one in `prefix` (block-wide; every thread
+// calls it).  One round of reads where a rebuild takes two and the scan.
+template <int NT>
+__device__ __forceinline__ bool schedule_changed(const int32_t* __restrict__ nvalid,
+                                                 const int32_t* __restrict__ len, int npairs, int B,
+                                                 int D, int tile, const int* prefix, int32_t* err) {
+  bool differs = false;
+  for (int i = threadIdx.x; i < npairs; i += NT)
+    differs |= tiles_of(used_slots(__ldcg(nvalid + i), B, err), window_rows(__ldcg(len + i), D, err),
+                        tile) != prefix[i + 1] - prefix[i];
+  return __syncthreads_or(differs);
+}
+
+// Merges the partials that CTAs ca..cb left for one pair, in CTA order, and writes its output.
+// A partial's place is fixed by the split: the pair's first tile lies in CTA ca (second slot
+// of its two), every later CTA starts inside the pair (first slot).  The (max, sum) pairs are
+// fetched once for all threads into `fac` (2 G (cb - ca + 1) floats of shared memory), and the
+// rows are loaded 8 at a time, so a merge costs a few L2 latencies instead of one chain of
+// 2 (cb - ca + 1) per thread: a pair at batch 1 spreads over 19 CTAs, and a 4-layer step there
+// went from 316 to 235 us with this and the early launches below.
+constexpr int kMaxAttendGrid = 256;      // CTAs whose factors fit in the warps' partials (4 HD)
+
+template <int G, int HD, int NCT, typename SyncFn, typename ExpFn>
+__device__ __forceinline__ void merge_partials(long long ca, long long cb, const float* part, float* out,
+                                               float* fac, SyncFn sync, ExpFn ex) {
+  constexpr int PSTRIDE = G * HD + 2 * G;
+  const int tid = threadIdx.x;
+  const int n = (int)(cb - ca) + 1;
+  const float* first = part + ((size_t)ca * 2 + 1) * PSTRIDE;
+  auto at = [&](int c) { return c == 0 ? first : part + (size_t)(ca + c) * 2 * PSTRIDE; };
+  for (int i = tid; i < n * G; i += NCT) {
+    const float* pc = at(i / G) + G * HD + i % G;
+    fac[2 * i] = __ldcg(pc);
+    fac[2 * i + 1] = __ldcg(pc + G);
+  }
+  sync();
+  for (int idx = tid; idx < G * HD; idx += NCT) {
+    const int g = idx / HD, i = idx - g * HD;
+    float ms = -INFINITY;
+    for (int c = 0; c < n; ++c) ms = fmaxf(ms, fac[2 * (c * G + g)]);
+    float L = 0.f, O = 0.f;
+    for (int c0 = 0; c0 < n; c0 += 8) {
+      float row[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) row[k] = c0 + k < n ? __ldcg(at(c0 + k) + g * HD + i) : 0.f;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        if (c0 + k >= n) break;
+        const float mc = fac[2 * ((c0 + k) * G + g)];
+        const float f = (mc == -INFINITY) ? 0.f : ex(mc - ms);
+        L = fmaf(fac[2 * ((c0 + k) * G + g) + 1], f, L);
+        O = fmaf(row[k], f, O);
+      }
+    }
+    out[(size_t)g * HD + i] = O / L;
+  }
 }
 
 // Pair p's segment in this CTA is complete; mo/ml/mm hold NW warp partials
@@ -68,7 +128,7 @@ __device__ __forceinline__ void build_schedule(const int32_t* __restrict__ nvali
 // (tid < NCT) together; `sync` is their barrier; `flag` is one shared int.
 template <int G, int HD, int NW, int NCT, typename SyncFn>
 __device__ __forceinline__ void finish_pair(int p, const int* prefix, long long Ttot, long long NC,
-                                            long long t0, const float* mo, const float* ml,
+                                            long long t0, float* mo, const float* ml,
                                             const float* mm, float* out, float* part,
                                             int32_t* part_count, int* flag, SyncFn sync) {
   constexpr int PSTRIDE = G * HD + 2 * G;
@@ -113,25 +173,9 @@ __device__ __forceinline__ void finish_pair(int p, const int* prefix, long long 
     sync();
     if (*flag) {
       __threadfence();
-      for (int idx = tid; idx < G * HD; idx += NCT) {
-        const int g = idx / HD, i = idx - g * HD;
-        float ms = -INFINITY;
-        for (long long c = ca; c <= cb; ++c) {
-          const int slot = (prefix[p] < cta_begin(c, Ttot, NC)) ? 0 : 1;
-          const float* pc = part + ((size_t)c * 2 + slot) * PSTRIDE;
-          ms = fmaxf(ms, __ldcg(pc + G * HD + g));
-        }
-        float L = 0.f, O = 0.f;
-        for (long long c = ca; c <= cb; ++c) {
-          const int slot = (prefix[p] < cta_begin(c, Ttot, NC)) ? 0 : 1;
-          const float* pc = part + ((size_t)c * 2 + slot) * PSTRIDE;
-          const float mc = __ldcg(pc + G * HD + g);
-          const float f = (mc == -INFINITY) ? 0.f : exp2f(mc - ms);
-          L = fmaf(__ldcg(pc + G * HD + G + g), f, L);
-          O = fmaf(__ldcg(pc + g * HD + i), f, O);
-        }
-        out[((size_t)p * G + g) * HD + i] = O / L;
-      }
+      // the warps' own partials have been folded: their room holds the merge's factors
+      merge_partials<G, HD, NCT>(ca, cb, part, out + (size_t)p * G * HD, mo, sync,
+                                 [](float x) { return exp2f(x); });
     }
   }
   sync();
