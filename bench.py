@@ -680,7 +680,7 @@ def run_stack_bench(args, cfg, rank, local_rank, world, dev, dist):
                    "layers": cfg.n_layers, "hidden": cfg.hidden, "kv_heads": cfg.n_kv_heads,
                    "q_per_kv": cfg.q_per_kv, "head_dim": cfg.head_dim, "prompt_len": cfg.prompt_len,
                    "budget_B": cfg.budget_B, "delay_D": cfg.delay_D, "kv_dtype": cfg.kv_dtype,
-                   "projections": "cuBLAS bf16 GEMMs (torch.matmul), fp32 accumulate",
+                   "projections": "bf16, fp32 accumulate: q | k | v in one weight-streaming launch, output by cuBLAS (torch.matmul)",
                    "l2": f"inputs larger than L2: {cfg.n_layers * bytes_per_launch / 1e9:.2f} GB K/V "
                          f"+ {proj_bytes / 1e9:.2f} GB weights per step",
                    "graph": "one CUDA graph per step (all layers)",

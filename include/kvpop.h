@@ -352,6 +352,31 @@ kvpop_status kvpop_get_pair_state(kvpop_cache* cache, int32_t seq, int32_t head,
                                   int32_t* pos_host, float* score_host, int32_t* nvalid_host,
                                   cudaStream_t stream);
 
+/* Projections around the decode step of a layer stack (plain bf16 products with fp32
+ * sums, not part of the paper's method), for small batches.
+ * kvpop_project_supported: bit 0 set when kvpop_project_qkv takes these sizes (batch 1..32,
+ * hidden a multiple of 32, n_q and n_kv multiples of 8 and at least 48), bit 1 when
+ * kvpop_project_out does (batch 1..16, n_q a multiple of 32, hidden one of 8 and at least
+ * 48). */
+int32_t kvpop_project_supported(int32_t batch, int32_t hidden, int32_t n_q, int32_t n_kv);
+
+/* q = bf16(x Wq), k = bf16(x Wk), v = bf16(x Wv) in one launch.
+ *   x_dev [batch][hidden], Wq_dev [hidden][n_q], Wk_dev, Wv_dev [hidden][n_kv],
+ *   q_dev [batch][n_q], k_dev, v_dev [batch][n_kv], all bf16, 16-byte aligned.
+ * Asynchronous on `stream`; no allocation. */
+kvpop_status kvpop_project_qkv(const void* x_dev, const void* Wq_dev, const void* Wk_dev,
+                               const void* Wv_dev, int32_t batch, int32_t hidden, int32_t n_q,
+                               int32_t n_kv, void* q_dev, void* k_dev, void* v_dev,
+                               cudaStream_t stream);
+
+/* y = bf16(x + bf16(bf16(o) Wo)) in one launch: the attention's fp32 output through the
+ * output projection, added to the residual stream.
+ *   o_dev [batch][n_q] fp32, Wo_dev [n_q][hidden] bf16, x_dev and y_dev [batch][hidden]
+ *   bf16 (y_dev may be x_dev), all 16-byte aligned.  Asynchronous on `stream`. */
+kvpop_status kvpop_project_out(const float* o_dev, const void* Wo_dev, const void* x_dev,
+                               int32_t batch, int32_t n_q, int32_t hidden, void* y_dev,
+                               cudaStream_t stream);
+
 /* Allocation-free decode attention (no counterpart in the paper: it is an
  * interface convenience).  For callers that may not allocate device memory
  * when they decode -- a serving loop whose device memory is fixed up front and

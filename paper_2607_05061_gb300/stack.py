@@ -4,10 +4,12 @@ through the C ABI, the output projection and the residual add.
 This is the workload around the hot path for the Qwen3-8B-shaped stack
 (hidden 4096, 32 query / 8 KV heads, d = 128): it reproduces the decode loop
 of a dense-attention model whose attention layers are the KVpop caches, with no
-norms and no MLP blocks.  The projections are plain bf16 GEMMs run by cuBLAS
-(`torch.matmul`, fp32 accumulation); everything KVpop does per layer -- the
-delayed scorer, the keep-or-drop decision, the scatter and the attention over
-the compressed cache -- runs in `libkvpop.so`.
+norms and no MLP blocks.  The decode step's projections are plain bf16 products with
+fp32 sums: two launches of `libkvpop.so` per layer (q, k, v; output with the residual)
+for batches and sizes its weight-streaming kernel takes, cuBLAS (`torch.matmul`)
+otherwise and for the prompts.  Everything KVpop does per layer -- the delayed scorer,
+the keep-or-drop decision, the scatter and the attention over the compressed cache --
+runs in `libkvpop.so`.
 
 Rounding points (bf16): q, k, v after their projections; the attention output
 before the output projection; the projection result; the residual sum.
@@ -18,7 +20,7 @@ from typing import List, Optional, Sequence
 
 import torch
 
-from .kvpop import KVpopCache
+from .kvpop import KVpopCache, kvpop_project_supported, project_out, project_qkv
 
 
 class DecodeStack:
@@ -49,6 +51,17 @@ class DecodeStack:
         self.y = torch.empty((batch, hidden), dtype=dt, device=dev)
         self.x = [torch.empty((batch, hidden), dtype=dt, device=dev) for _ in range(2)]
         self.graph = None
+        # which projections the weight-streaming kernels take at these sizes (bit 0: q, k, v;
+        # bit 1: the output projection)
+        self._project = kvpop_project_supported(batch, hidden, self.Hq * head_dim,
+                                                n_kv_heads * head_dim)
+
+    def _plain(self, *want) -> bool:
+        """Whether the tensors are plain ones of the stack's own sizes, as the projection kernels
+        need (anything else takes, or is refused by, torch.matmul)."""
+        return all(t.dtype is torch.bfloat16 and t.shape == s and t.is_contiguous() and
+                   t.device == self.q.device and not t.requires_grad and t.data_ptr() % 16 == 0
+                   for t, s in want)
 
     # ------------------------------------------------------------------ prefill
     def prefill_layer(self, l: int, X: torch.Tensor, lengths: Sequence[int], first_seq: int = 0,
@@ -72,18 +85,27 @@ class DecodeStack:
                    evict_info=None, outputs=None):
         x = x_in
         for l, (L, cache) in enumerate(zip(self.layers, self.caches)):
-            torch.matmul(x, L["Wq"], out=self.q)
-            torch.matmul(x, L["Wk"], out=self.k)
-            torch.matmul(x, L["Wv"], out=self.v)
+            nxt = self.x[l % 2] if l + 1 < len(self.layers) else x_out
+            nq, nkv, hid = self.q.shape[1], self.k.shape[1], self.hidden
+            if self._project & 1 and self._plain((x, (self.b, hid)), (L["Wq"], (hid, nq)),
+                                                 (L["Wk"], (hid, nkv)), (L["Wv"], (hid, nkv))):
+                project_qkv(x, L["Wq"], L["Wk"], L["Wv"], self.q, self.k, self.v)
+            else:
+                torch.matmul(x, L["Wq"], out=self.q)
+                torch.matmul(x, L["Wk"], out=self.k)
+                torch.matmul(x, L["Wv"], out=self.v)
             ov = None if overrides is None else overrides[l]
             ei = None if evict_info is None else evict_info[l]
             cache.step(self.q, self.k, self.v, self.o, override=ov, evict_info=ei)
             if outputs is not None:
                 outputs[l].copy_(self.o)
-            self.o_bf.copy_(self.o)
-            torch.matmul(self.o_bf, L["Wo"], out=self.y)
-            nxt = self.x[l % 2] if l + 1 < len(self.layers) else x_out
-            torch.add(x, self.y, out=nxt)
+            if self._project & 2 and self._plain((x, (self.b, hid)), (nxt, (self.b, hid)),
+                                                 (L["Wo"], (nq, hid))):
+                project_out(self.o, L["Wo"], x, nxt)
+            else:
+                self.o_bf.copy_(self.o)
+                torch.matmul(self.o_bf, L["Wo"], out=self.y)
+                torch.add(x, self.y, out=nxt)
             x = nxt
         return x_out
 
