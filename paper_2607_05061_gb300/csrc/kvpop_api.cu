@@ -567,7 +567,7 @@ kvpop_status prefill_impl(kvpop_cache* c, const void* Q, const void* K, const vo
   // the mLSTM prefill also needs every prompt token's features (k~, v~, q~, gates)
   const size_t feat_bytes = c->mlstm ? pairs * (size_t)Pmax * mlstm_nf(c->dm.d) * 4 : 0;
   const size_t plen_off = prio_bytes;
-  const size_t feat_off = plen_off + 256;
+  const size_t feat_off = plen_off + al((size_t)n_seq * 4);
   const size_t rank_off = al(feat_off + feat_bytes);
   const size_t tau_off = rank_off + (outputs && !rank_out ? prio_bytes : 0);
   const size_t ws_off = tau_off + (outputs && !tau_out ? prio_bytes : 0);
