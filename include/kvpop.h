@@ -124,8 +124,8 @@ kvpop_status kvpop_init_cache(const kvpop_config* cfg, const kvpop_scorer* score
 /* As kvpop_init_cache with the mLSTM scorer; cfg->scorer_hidden is ignored.
  * The cache additionally holds the recurrent state (C, z, m) of every
  * (sequence, KV head), which prefill builds over the prompt and every decode
- * step advances by one token (in prefill, the chunkwise form of the recurrence:
- * 64-token chunks one after another per pair, the tokens of a chunk together). */
+ * step advances by one token (in prefill, the chunkwise form of the recurrence: the
+ * states between 64-token chunks first, then the tokens of all chunks together). */
 kvpop_status kvpop_init_cache_mlstm(const kvpop_config* cfg, const kvpop_mlstm_scorer* scorer,
                                     cudaStream_t stream, kvpop_cache** out);
 

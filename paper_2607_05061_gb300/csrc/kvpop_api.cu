@@ -377,6 +377,10 @@ static kvpop_status init_cache(const kvpop_config* cfg_in, const kvpop_scorer* s
     if (s == KVPOP_OK) { s = dev_alloc(c, &p, pairs * 4); md.m = (float*)p; }
     if (s == KVPOP_OK) { s = dev_alloc(c, &p, H * 2 * d * NCm * 4); md.Wcat = (float*)p; }
     if (s == KVPOP_OK) { s = dev_alloc(c, &p, (4 * H + H * hh) * 4); md.bi = (float*)p; }
+    if (s == KVPOP_OK && cfg->kv_dtype == KVPOP_BF16) {
+      s = dev_alloc(c, &p, mlstm_wt_bytes(dm.d, dm.H));
+      md.Wt = p;
+    }
     if (s == KVPOP_OK) {
       md.bf = md.bi + H; md.b = md.bf + H; md.a = md.b + H;
       s = from_cuda(NOTE(prepare_mlstm(dm)));
@@ -439,6 +443,7 @@ static kvpop_status init_cache(const kvpop_config* cfg_in, const kvpop_scorer* s
           e = NOTE(cudaMemcpy2DAsync(dst + 3 * hh + 1, NCm * 4, ms->wf + h * n2, 4, 4, n2,
                                      cudaMemcpyDefault, stream));
       }
+      if (e == cudaSuccess && md.Wt) e = NOTE(launch_mlstm_split(dm, md, stream));
       if (e == cudaSuccess) e = NOTE(cudaMemcpyAsync(md.bi, ms->bi, H * 4, cudaMemcpyDefault, stream));
       if (e == cudaSuccess) e = NOTE(cudaMemcpyAsync(md.bf, ms->bf, H * 4, cudaMemcpyDefault, stream));
       if (e == cudaSuccess) e = NOTE(cudaMemcpyAsync(md.b, ms->b, H * 4, cudaMemcpyDefault, stream));
@@ -565,7 +570,7 @@ kvpop_status prefill_impl(kvpop_cache* c, const void* Q, const void* K, const vo
   auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
   const size_t prio_bytes = al(pairs * (size_t)Pmax * 4);
   // the mLSTM prefill also needs every prompt token's features (k~, v~, q~, gates)
-  const size_t feat_bytes = c->mlstm ? pairs * (size_t)Pmax * mlstm_nf(c->dm.d) * 4 : 0;
+  const size_t feat_bytes = c->mlstm ? mlstm_prefill_bytes(c->dm.d, (int)pairs, Pmax) : 0;
   const size_t plen_off = prio_bytes;
   const size_t feat_off = plen_off + al((size_t)n_seq * 4);
   const size_t rank_off = al(feat_off + feat_bytes);

@@ -141,10 +141,15 @@ struct MlstmDev {
   float* bf;                   // [H]
   float* a;                    // [H][d/2]
   float* b;                    // [H]
+  void* Wt;                    // [H] W^T in three bf16 parts (bf16 caches, prompt scores)
   int NC;
 };
 int mlstm_nc(int d);
 int mlstm_nf(int d);
+size_t mlstm_wt_bytes(int d, int H);
+cudaError_t launch_mlstm_split(const Dims& dm, const MlstmDev& m, cudaStream_t stream);
+// Bytes behind `feat` of launch_prefill_mlstm_scores.
+size_t mlstm_prefill_bytes(int d, int pairs, int Pmax);
 bool mlstm_ok(const Dims& dm);
 cudaError_t prepare_mlstm(const Dims& dm);
 cudaError_t launch_ingest_mlstm(const State& st, const Dims& dm, const MlstmDev& m, const void* q,

@@ -15,7 +15,10 @@
 // [W_k | W_v | W_q | w_i | w_f | 0 pad], so one pass over x gives every
 // projection.  The decode kernel loads its head's Wcat whole into shared memory
 // with bulk copies (200 KB for d = 128) and serves 8 sequences per CTA.
+#include <algorithm>
+
 #include "kvpop_evict.cuh"
+#include "kvpop_mma.cuh"
 
 namespace kvpop {
 namespace {
@@ -278,19 +281,18 @@ __global__ void __launch_bounds__(NTM, 1) ingest_mlstm_kernel(MIngestArgs<T> a) 
 }
 
 // ------------------------------------------------------------------ prefill
-template <typename T>
 struct MProjArgs {
   Dims dm;
   MState ms;
-  const T* K;                      // [n_seq][H][Pmax][d]
-  const T* V;
+  const float* K;                  // [n_seq][H][Pmax][d]
+  const float* V;
   const int32_t* plen;
   float* feat;                     // [n_seq*H][Pmax][NF]: k~ (d) | v~ (d/2) | q~ (d) | a_i | a_f
   int Pmax, NF;
 };
 
-template <typename T>
-__global__ void __launch_bounds__(NTM) mlstm_proj_kernel(MProjArgs<T> a) {
+// fp32 K/V: column c of Wcat per thread, 32 tokens per CTA.
+__global__ void __launch_bounds__(NTM) mlstm_proj_kernel(MProjArgs a) {
   const Dims& dm = a.dm;
   const int d = dm.d, H = dm.H, NC = a.ms.NC, hh = d / 2, in2 = 2 * d, NF = a.NF;
   const int lp = blockIdx.y, bl = lp / H, h = lp - bl * H;
@@ -298,17 +300,17 @@ __global__ void __launch_bounds__(NTM) mlstm_proj_kernel(MProjArgs<T> a) {
   const int t0 = blockIdx.x * UTM;
   if (t0 >= P) return;
   const int nrow = min(UTM, P - t0);
-  extern __shared__ __align__(16) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem[];
   float* Xt = reinterpret_cast<float*>(smem);                  // [2d][UTM]
   float* pj = Xt + in2 * UTM;                                  // [UTM][NC]
   const size_t Pm = a.Pmax;
-  const T* Kp = a.K + ((size_t)bl * H + h) * Pm * d;
-  const T* Vp = a.V + ((size_t)bl * H + h) * Pm * d;
+  const float* Kp = a.K + ((size_t)bl * H + h) * Pm * d;
+  const float* Vp = a.V + ((size_t)bl * H + h) * Pm * d;
   for (int idx = threadIdx.x; idx < UTM * d; idx += NTM) {
     const int r = idx / d, i = idx - r * d;
     const bool in = r < nrow;
-    Xt[i * UTM + r] = in ? to_f(Kp[(size_t)(t0 + r) * d + i]) : 0.f;
-    Xt[(d + i) * UTM + r] = in ? to_f(Vp[(size_t)(t0 + r) * d + i]) : 0.f;
+    Xt[i * UTM + r] = in ? Kp[(size_t)(t0 + r) * d + i] : 0.f;
+    Xt[(d + i) * UTM + r] = in ? Vp[(size_t)(t0 + r) * d + i] : 0.f;
   }
   __syncthreads();
   const float* W = a.ms.Wcat + (size_t)h * in2 * NC;
@@ -348,6 +350,181 @@ __global__ void __launch_bounds__(NTM) mlstm_proj_kernel(MProjArgs<T> a) {
   }
 }
 
+// The same projections for bf16 K/V on the tensor cores with fp32 accuracy: x is exact in bf16
+// and every weight is split exactly into three bf16 parts (8 + 8 + 8 bits, W^T stored once per
+// cache), so W x is three products whose terms are exact.  The tensor unit rounds a running sum
+// toward zero; to keep that below the rounding of a chain of fp32 FMAs, each 64 inputs are
+// summed on their own, smallest parts first, and added to the total in fp32.  A CTA takes 128
+// tokens, a warp 16 of them with all columns, so the Hedgehog softmaxes run on the warp's
+// accumulators (a row lies in 4 lanes).  Bound by the mma.sync rate: 64 pairs of up to 4009
+// tokens, d = 128: 283 us, against 1125 us with fp32 FMAs.
+constexpr int PT_TOK = 128;
+constexpr int PT_KC = 64;                          // inputs per chunk: one 128-byte row of W^T
+
+template <int HD>
+struct PtP {
+  static constexpr int HH = HD / 2;
+  static constexpr int NT = (3 * HH + 2 + 7) / 8;  // 8-column tiles: W_k, W_v, W_q, gates
+  static constexpr int NCP = 8 * NT;
+  static constexpr int IN2 = 2 * HD;
+  static constexpr int NKC = IN2 / PT_KC;
+  static constexpr int XB = PT_TOK * IN2 * 2;      // tokens: NKC tiles of [128][64]
+  static constexpr int WB = 3 * NCP * PT_KC * 2;   // one chunk of the three parts
+  static constexpr int SMEM = XB + 2 * WB;
+};
+
+// W^T parts: wt [H][NKC][3][NCP][64] from Wcat [H][2d][NC]
+template <int HD>
+__global__ void mlstm_split_kernel(const float* __restrict__ Wcat, int NC, int H, bf16* __restrict__ wt) {
+  using P = PtP<HD>;
+  const int n = H * P::IN2 * P::NCP;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const int c = i % P::NCP, k = (i / P::NCP) % P::IN2, h = i / (P::NCP * P::IN2);
+    const float w = c < NC ? Wcat[((size_t)h * P::IN2 + k) * NC + c] : 0.f;
+    bf16 part[3] = {__float2bfloat16_rz(w), __float2bfloat16_rz(0.f), __float2bfloat16_rz(0.f)};
+    if (isfinite(w)) {
+      const float r1 = w - __bfloat162float(part[0]);
+      part[1] = __float2bfloat16_rz(r1);
+      part[2] = __float2bfloat16_rz(r1 - __bfloat162float(part[1]));
+    }
+    for (int q = 0; q < 3; ++q)
+      wt[((((size_t)h * P::NKC + k / PT_KC) * 3 + q) * P::NCP + c) * PT_KC + k % PT_KC] = part[q];
+  }
+}
+
+struct MProjTcArgs {
+  const bf16* K;                   // [n_seq][H][Pmax][d]
+  const bf16* V;
+  const bf16* wt;
+  const float* bi;
+  const float* bf;
+  const int32_t* plen;
+  float* feat;
+  int H, Pmax, NF;
+};
+
+template <int HD>
+__global__ void __launch_bounds__(NTM, 1) mlstm_proj_tc_kernel(MProjTcArgs a) {
+  using P = PtP<HD>;
+  constexpr int HH = P::HH, NT = P::NT, HT = HH / 8;   // HT: tiles of one projection
+  extern __shared__ __align__(128) unsigned char sm_pt[];
+  const int lp = blockIdx.y, bl = lp / a.H, h = lp - bl * a.H;
+  const int L = a.plen[bl], t0 = blockIdx.x * PT_TOK;
+  if (t0 >= L) return;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int g = lane >> 2, t4 = lane & 3;
+  const uint32_t xb = smem_u32(sm_pt), wb = xb + P::XB;
+  const bf16* Kp = a.K + (size_t)lp * a.Pmax * HD;
+  const bf16* Vp = a.V + (size_t)lp * a.Pmax * HD;
+  const bf16* wt = a.wt + (size_t)h * P::NKC * 3 * P::NCP * PT_KC;
+  auto load_w = [&](int kc) {
+    const bf16* src = wt + (size_t)kc * 3 * P::NCP * PT_KC;
+    for (int i = tid; i < 3 * P::NCP * 8; i += NTM)
+      cp_async16(wb + (kc & 1) * P::WB + swz(i >> 3, i & 7, 128), src + (size_t)i * 8, 16);
+  };
+  for (int i = tid; i < PT_TOK * (P::IN2 / 8); i += NTM) {
+    const int r = i / (P::IN2 / 8), c = i - r * (P::IN2 / 8);
+    const bool in = t0 + r < L;
+    const size_t row = (size_t)(in ? t0 + r : t0) * HD;
+    const bf16* src = c < HD / 8 ? Kp + row + 8 * c : Vp + row + 8 * c - HD;
+    cp_async16(xb + (c >> 3) * (PT_TOK * 128) + swz(r, c & 7, 128), src, in ? 16 : 0);
+  }
+  load_w(0);
+  cp_commit();
+  float acc[NT][4];
+#pragma unroll
+  for (int n = 0; n < NT; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
+  for (int kc = 0; kc < P::NKC; ++kc) {
+    if (kc + 1 < P::NKC) load_w(kc + 1);
+    cp_commit();
+    cp_wait<1>();
+    __syncthreads();
+    uint32_t x[4][4];                              // the warp's 16 tokens, 4 k-steps
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {
+      const int r = 16 * warp + ((lane >> 3) & 1) * 8 + (lane & 7);
+      ldsm_x4(xb + kc * (PT_TOK * 128) + swz(r, 2 * ks + (lane >> 4), 128), x[ks][0], x[ks][1], x[ks][2], x[ks][3]);
+    }
+    const uint32_t w0 = wb + (kc & 1) * P::WB;
+#pragma unroll
+    for (int n = 0; n < NT; ++n) {
+      float c[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int q = 2; q >= 0; --q) {               // smallest part first
+#pragma unroll
+        for (int k2 = 0; k2 < 2; ++k2) {
+          const int row = q * P::NCP + 8 * n + (lane & 7);
+          uint32_t b0, b1, b2, b3;
+          ldsm_x4(w0 + swz(row, 4 * k2 + (lane >> 3), 128), b0, b1, b2, b3);
+          mma_bf16(c, x[2 * k2][0], x[2 * k2][1], x[2 * k2][2], x[2 * k2][3], b0, b1);
+          mma_bf16(c, x[2 * k2 + 1][0], x[2 * k2 + 1][1], x[2 * k2 + 1][2], x[2 * k2 + 1][3], b2, b3);
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[n][e] += c[e];
+    }
+    __syncthreads();
+  }
+  cp_wait<0>();
+  // features of rows g and g + 8 of the warp: columns 8 n + 2 t4, + 1 are this lane's
+#pragma unroll
+  for (int rr = 0; rr < 2; ++rr) {
+    const int t = t0 + 16 * warp + g + 8 * rr;
+    float* o = a.feat + ((size_t)lp * a.Pmax + t) * a.NF;
+    const bool in = t < L;
+#pragma unroll
+    for (int part = 0; part < 2; ++part) {         // k~ from W_k's tiles, q~ from W_q's
+      const int n0 = part ? 2 * HT : 0;
+      float* dst = part ? o + HD + HH : o;
+      float mp = -INFINITY, mn = -INFINITY;
+#pragma unroll
+      for (int n = 0; n < HT; ++n)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const float v = acc[n0 + n][2 * rr + e];
+          mp = fmaxf(mp, v);
+          mn = fmaxf(mn, -v);
+        }
+#pragma unroll
+      for (int x = 1; x <= 2; x <<= 1) {
+        mp = fmaxf(mp, __shfl_xor_sync(0xffffffffu, mp, x));
+        mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, x));
+      }
+      float sp = 0.f, sn = 0.f;
+#pragma unroll
+      for (int n = 0; n < HT; ++n)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const float v = acc[n0 + n][2 * rr + e];
+          sp += expf(v - mp);
+          sn += expf(-v - mn);
+        }
+#pragma unroll
+      for (int x = 1; x <= 2; x <<= 1) {
+        sp += __shfl_xor_sync(0xffffffffu, sp, x);
+        sn += __shfl_xor_sync(0xffffffffu, sn, x);
+      }
+      if (in) {
+#pragma unroll
+        for (int n = 0; n < HT; ++n) {
+          const float v0 = acc[n0 + n][2 * rr], v1 = acc[n0 + n][2 * rr + 1];
+          *reinterpret_cast<float2*>(dst + 8 * n + 2 * t4) = make_float2(expf(v0 - mp) / sp, expf(v1 - mp) / sp);
+          *reinterpret_cast<float2*>(dst + HH + 8 * n + 2 * t4) = make_float2(expf(-v0 - mn) / sn, expf(-v1 - mn) / sn);
+        }
+      }
+    }
+    if (in) {
+#pragma unroll
+      for (int n = 0; n < HT; ++n)
+        *reinterpret_cast<float2*>(o + HD + 8 * n + 2 * t4) =
+            make_float2(acc[HT + n][2 * rr], acc[HT + n][2 * rr + 1]);
+      if (t4 == 0)
+        *reinterpret_cast<float2*>(o + 2 * HD + HH) =
+            make_float2(acc[3 * HT][2 * rr] + a.bi[h], acc[3 * HT][2 * rr + 1] + a.bf[h]);
+    }
+  }
+}
+
 struct MScanArgs {
   State st;
   Dims dm;
@@ -356,7 +533,11 @@ struct MScanArgs {
   const float* feat;
   const float* override_;          // [n_seq][H][Pmax] or nullptr
   float* prio;                     // [n_seq][H][Pmax]
+  float* seg;                      // [pairs][nseg - 1][d d/2 + d] states between segments
+  float* seg_scal;                 // [pairs][nseg][2] log-scale and log forget sum of a segment
+  float* seg_m;                    // [pairs][nseg] log-scale at a segment's start
   int first_seq, Pmax, NF;
+  int n, nseg;                     // chunks per segment, segments
 };
 
 // Chunkwise form of the same recurrence (App. A: the mLSTM as linear attention with
@@ -371,9 +552,39 @@ struct MScanArgs {
 //   h = (e^{m-R_t} q~_u^T C + sum_s W_ts v~_s) / (e^{m-R_t} q~_u^T z + sum_s W_ts),
 //   W_ts = e^{g_s - R_t} (q~_u . k~_s)  for s <= t,
 // so a chunk costs three small dense products (q~ K^T, q~ C, W V) plus the state
-// update C' = e^{m - R_{L-1}} C + K^T diag(e^{g - R_{L-1}}) V, all from shared memory
-// with register tiles; chunks follow one another, the tokens of a chunk do not.
+// update C' = e^{m - R_{L-1}} C + K^T diag(e^{g - R_{L-1}}) V.
+//
+// Chunks depend on each other only through (C, z, m), so a pair's chunks are cut into
+// segments: mlstm_seg_kernel takes every segment (but a pair's last) from an empty state,
+// mlstm_link_kernel chains those states, and mlstm_chunk_kernel reads out all segments at
+// once, each from its own start.  64 pairs of up to 4009 tokens, d = 128: 561 us
+// together, against 1557 us with the chunks of a pair one after another on 64 SMs.
 constexpr int CL = 64;             // tokens per chunk
+constexpr int NTC = 512;           // threads of the readout: two groups of 256
+
+template <int N>
+__device__ __forceinline__ void ld_vec(float (&x)[N], const float* p) {
+  if constexpr (N == 2) {
+    const float2 v = *reinterpret_cast<const float2*>(p);
+    x[0] = v.x; x[1] = v.y;
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; i += 4) {
+      const float4 v = *reinterpret_cast<const float4*>(p + i);
+      x[i] = v.x; x[i + 1] = v.y; x[i + 2] = v.z; x[i + 3] = v.w;
+    }
+  }
+}
+template <int N>
+__device__ __forceinline__ void st_vec(float* p, const float (&x)[N]) {
+  if constexpr (N == 2) {
+    *reinterpret_cast<float2*>(p) = make_float2(x[0], x[1]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; i += 4)
+      *reinterpret_cast<float4*>(p + i) = make_float4(x[i], x[i + 1], x[i + 2], x[i + 3]);
+  }
+}
 
 template <int HD>
 struct ChunkLayout {
@@ -381,107 +592,249 @@ struct ChunkLayout {
   static constexpr int QS = HD + 4;              // row strides (floats), multiples of 4
   static constexpr int VS = HH + 4;
   static constexpr int WS = CL + 4;
-  static constexpr int OFF_Q = 0;                // [CL][QS]  q~ of the read-out tokens
-  static constexpr int OFF_K = OFF_Q + CL * QS;  // [CL][QS]  k~ of the chunk's tokens
-  static constexpr int OFF_V = OFF_K + CL * QS;  // [CL][VS]  v~
-  static constexpr int OFF_C = OFF_V + CL * VS;  // [HD][VS]  state C
-  static constexpr int OFF_W = OFF_C + HD * VS;  // [CL][WS]  W_ts
-  static constexpr int OFF_Z = OFF_W + CL * WS;  // [HD]
-  static constexpr int OFF_G = OFF_Z + HD;       // [CL] g_s
-  static constexpr int OFF_R = OFF_G + CL;       // [CL] R_t
-  static constexpr int OFF_QZ = OFF_R + CL;      // [CL] q~ . z
-  static constexpr int OFF_SC = OFF_QZ + CL;     // [4] m, F_{L-1}
-  static constexpr int FLOATS = OFF_SC + 4;
+  // one buffer of a chunk's features (two of them, the next chunk's in flight)
+  static constexpr int B_K = 0;                  // [CL][QS]  k~ of the chunk's tokens
+  static constexpr int B_V = B_K + CL * QS;      // [CL][VS]  v~
+  static constexpr int B_G = B_V + CL * VS;      // [CL][4]   a_i, a_f
+  static constexpr int B_Q = B_G + CL * 4;       // [CL][QS]  q~ of the read-out tokens
+  static constexpr int BUF = B_Q + CL * QS;
+  static constexpr int BUF_S = B_Q;              // without q~ (segment states)
+  static constexpr int SEG = HD * HH + HD;       // floats of a state in global memory
 };
 
+// Gates of one chunk by one warp (two tokens per lane): g_s, R_t, e^{g_s - R_{L-1}}, and
+// F_{L-1} in sc[1].
+__device__ __forceinline__ void chunk_gates(const float* G, int t0, int P, float m, float* gs, float* Rs,
+                                            float* es, float* sc) {
+  const int lane = threadIdx.x & 31;
+  float lfv[2], aiv[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int r = 2 * lane + k;
+    const bool in = t0 + r < P;
+    aiv[k] = in ? G[4 * r] : -INFINITY;
+    lfv[k] = in ? -softplus(-G[4 * r + 1]) : 0.f;
+  }
+  const float f1 = lfv[0] + lfv[1];
+  float inc = f1;                                  // inclusive scan over lane pairs
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const float y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  const float Fa = inc - f1 + lfv[0], Fb = inc;    // F of tokens 2 lane, 2 lane + 1
+  const float ga = aiv[0] - Fa, gb = aiv[1] - Fb;
+  float run = fmaxf(ga, gb);                       // inclusive prefix max
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const float y = __shfl_up_sync(0xffffffffu, run, o);
+    if (lane >= o) run = fmaxf(run, y);
+  }
+  const float prev = __shfl_up_sync(0xffffffffu, run, 1);
+  const float before = lane == 0 ? -INFINITY : prev;
+  const float RL = fmaxf(m, __shfl_sync(0xffffffffu, run, 31));
+  gs[2 * lane] = ga;
+  gs[2 * lane + 1] = gb;
+  if (Rs) {
+    Rs[2 * lane] = fmaxf(m, fmaxf(before, ga));
+    Rs[2 * lane + 1] = fmaxf(m, run);
+  }
+  es[2 * lane] = __expf(ga - RL);
+  es[2 * lane + 1] = __expf(gb - RL);
+  if (lane == 31) {
+    sc[1] = Fb;                                    // F of the chunk's last token
+    sc[2] = RL;
+  }
+}
+
+// Copies one chunk's features into a buffer (rows past the prompt zero-filled).
+template <int HD, bool WITH_Q>
+__device__ __forceinline__ void load_chunk(const float* F, int NF, int t0, int P, int D, float* buf, int nt) {
+  using Ly = ChunkLayout<HD>;
+  const int tid = threadIdx.x;
+  const uint32_t b = smem_u32(buf);
+  for (int e = tid; e < CL * (HD / 4); e += nt) {
+    const int r = e / (HD / 4), c = e - r * (HD / 4), t = t0 + r, u = t - D;
+    const bool in = t < P;
+    cp_async16(b + (Ly::B_K + r * Ly::QS + 4 * c) * 4, F + (size_t)(in ? t : 0) * NF + 4 * c, in ? 16 : 0);
+    if (WITH_Q) {
+      const bool iq = in && u >= 0;
+      cp_async16(b + (Ly::B_Q + r * Ly::QS + 4 * c) * 4, F + (size_t)(iq ? u : 0) * NF + HD + Ly::HH + 4 * c,
+                 iq ? 16 : 0);
+    }
+  }
+  for (int e = tid; e < CL * (Ly::HH / 4); e += nt) {
+    const int r = e / (Ly::HH / 4), c = e - r * (Ly::HH / 4), t = t0 + r;
+    cp_async16(b + (Ly::B_V + r * Ly::VS + 4 * c) * 4, F + (size_t)(t < P ? t : 0) * NF + HD + 4 * c, t < P ? 16 : 0);
+  }
+  for (int r = tid; r < CL; r += nt)
+    cp_async16(b + (Ly::B_G + 4 * r) * 4, F + (size_t)(t0 + r < P ? t0 + r : 0) * NF + 2 * HD + Ly::HH,
+               t0 + r < P ? 16 : 0);
+}
+
+// acc += K^T diag(es) V on this thread's HD / 16 rows x HH / 16 columns of the state
 template <int HD>
-__global__ void __launch_bounds__(NTM) mlstm_chunk_kernel(MScanArgs a) {
+__device__ __forceinline__ void state_update(float (&acc)[HD / 16][HD / 32], const float* Ks, const float* Vs,
+                                             const float* es, int ty, int tx) {
+  using Ly = ChunkLayout<HD>;
+  constexpr int NR = HD / 16, NB = HD / 32;
+#pragma unroll 4
+  for (int s = 0; s < CL; ++s) {
+    float v[NB], k[NR];
+    ld_vec<NB>(v, Vs + s * Ly::VS + NB * tx);
+    ld_vec<NR>(k, Ks + s * Ly::QS + NR * ty);
+    const float w = es[s];
+#pragma unroll
+    for (int j = 0; j < NB; ++j) v[j] *= w;
+#pragma unroll
+    for (int i = 0; i < NR; ++i)
+#pragma unroll
+      for (int j = 0; j < NB; ++j) acc[i][j] = fmaf(k[i], v[j], acc[i][j]);
+  }
+}
+
+// State that a segment's tokens leave from an empty one (every segment but a pair's last).
+template <int HD>
+__global__ void __launch_bounds__(NTM) mlstm_seg_kernel(MScanArgs a) {
+  using Ly = ChunkLayout<HD>;
+  constexpr int HH = Ly::HH, NR = HD / 16, NB = HD / 32;
+  extern __shared__ __align__(16) float smf[];
+  __shared__ float gs[CL], es[CL], sc[4];
+  const int lp = blockIdx.y, seg = blockIdx.x;
+  const int P = a.plen[lp / a.dm.H];
+  const int c0 = seg * a.n, c1 = c0 + a.n;
+  if (c1 * CL >= P) return;                        // the pair's last segment, or past it
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  const float* F = a.feat + (size_t)lp * a.Pmax * a.NF;
+  float acc[NR][NB], zn = 0.f, m = -INFINITY, Ft = 0.f;
+#pragma unroll
+  for (int i = 0; i < NR; ++i)
+#pragma unroll
+    for (int j = 0; j < NB; ++j) acc[i][j] = 0.f;
+  load_chunk<HD, false>(F, a.NF, c0 * CL, P, 0, smf, NTM);
+  cp_commit();
+  for (int c = c0; c < c1; ++c) {
+    const float* buf = smf + ((c - c0) & 1) * Ly::BUF_S;
+    if (c + 1 < c1) load_chunk<HD, false>(F, a.NF, (c + 1) * CL, P, 0, smf + ((c + 1 - c0) & 1) * Ly::BUF_S, NTM);
+    cp_commit();
+    cp_wait<1>();
+    __syncthreads();
+    if (tid < 32) chunk_gates(buf + Ly::B_G, c * CL, P, m, gs, nullptr, es, sc);
+    __syncthreads();
+    const float RL = sc[2], wc = __expf(m - RL);
+#pragma unroll
+    for (int i = 0; i < NR; ++i)
+#pragma unroll
+      for (int j = 0; j < NB; ++j) acc[i][j] *= wc;
+    state_update<HD>(acc, buf + Ly::B_K, buf + Ly::B_V, es, ty, tx);
+    if (tid < HD) {
+      zn *= wc;
+      for (int s = 0; s < CL; ++s) zn = fmaf(es[s], buf[Ly::B_K + s * Ly::QS + tid], zn);
+    }
+    m = sc[1] + RL;
+    Ft += sc[1];
+    __syncthreads();
+  }
+  float* out = a.seg + ((size_t)lp * (a.nseg - 1) + seg) * Ly::SEG;
+#pragma unroll
+  for (int i = 0; i < NR; ++i) st_vec<NB>(out + (NR * ty + i) * HH + NB * tx, acc[i]);
+  if (tid < HD) out[HD * HH + tid] = zn;
+  if (tid == 0) {
+    a.seg_scal[((size_t)lp * a.nseg + seg) * 2] = m;
+    a.seg_scal[((size_t)lp * a.nseg + seg) * 2 + 1] = Ft;
+  }
+}
+
+// Chains the segments' states: slot j becomes the state at the start of segment j + 1.
+template <int HD>
+__global__ void __launch_bounds__(NTM) mlstm_link_kernel(MScanArgs a) {
+  using Ly = ChunkLayout<HD>;
+  const int lp = blockIdx.y, e = blockIdx.x * NTM + threadIdx.x;
+  const int P = a.plen[lp / a.dm.H];
+  const int last = P > 0 ? ((P + CL - 1) / CL - 1) / a.n : 0;
+  float* seg = a.seg + (size_t)lp * (a.nseg - 1) * Ly::SEG;
+  const float* sc = a.seg_scal + (size_t)lp * a.nseg * 2;
+  const bool in = e < Ly::SEG;
+  float c = 0.f, m = -INFINITY;
+  for (int j0 = 0; j0 < last; j0 += 8) {
+    float x[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) x[k] = in && j0 + k < last ? seg[(size_t)(j0 + k) * Ly::SEG + e] : 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (j0 + k >= last) break;
+      const float mc = sc[2 * (j0 + k)], m1 = m + sc[2 * (j0 + k) + 1];
+      const float mn = fmaxf(m1, mc);
+      c = expf(m1 - mn) * c + expf(mc - mn) * x[k];
+      m = mn;
+      if (in) seg[(size_t)(j0 + k) * Ly::SEG + e] = c;
+      if (e == 0) a.seg_m[(size_t)lp * a.nseg + j0 + k + 1] = m;
+    }
+  }
+}
+
+// Readout of one segment.  Threads 0-255 form S = q~ K^T, then the state update; threads
+// 256-511 the products with the state, then W V and the scores, so the two halves of a
+// chunk's FMAs run side by side.
+template <int HD>
+__global__ void __launch_bounds__(NTC, 1) mlstm_chunk_kernel(MScanArgs a) {
   using Ly = ChunkLayout<HD>;
   constexpr int HH = Ly::HH, QS = Ly::QS, VS = Ly::VS, WS = Ly::WS;
-  constexpr int NB = HH / 16;                    // column blocks of q~C / num per thread
+  constexpr int NB = HD / 32, NR = HD / 16;      // columns, rows of the state per thread
   const Dims& dm = a.dm;
   const int D = dm.D, H = dm.H, NF = a.NF;
-  const int lp = blockIdx.x, bl = lp / H, h = lp - bl * H;
-  const int pair = (a.first_seq + bl) * H + h;
+  const int lp = blockIdx.y, bl = lp / H, h = lp - bl * H;
   const int P = a.plen[bl];
+  const int seg = blockIdx.x, c0 = seg * a.n, nch = (P + CL - 1) / CL;
+  if (seg > 0 && c0 >= nch) return;
+  const int c1 = min(c0 + a.n, nch);
+  const bool last = c1 == nch;
   const size_t Pm = a.Pmax;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int ty = tid >> 4, tx = tid & 15;        // 16 x 16 thread grid
+  const int tid = threadIdx.x, lane = tid & 31;
+  const bool front = tid < 256;
+  const int gt = tid & 255, ty = gt >> 4, tx = gt & 15;
   extern __shared__ __align__(16) float smf[];
-  float* Qs = smf + Ly::OFF_Q;
-  float* Ks = smf + Ly::OFF_K;
-  float* Vs = smf + Ly::OFF_V;
-  float* Cs = smf + Ly::OFF_C;
-  float* Ws = smf + Ly::OFF_W;
-  float* zs = smf + Ly::OFF_Z;
-  float* gs = smf + Ly::OFF_G;
-  float* Rs = smf + Ly::OFF_R;
-  float* qz = smf + Ly::OFF_QZ;
-  float* sc = smf + Ly::OFF_SC;
-  for (int e = tid; e < HD * VS; e += NTM) Cs[e] = 0.f;
-  for (int e = tid; e < HD; e += NTM) zs[e] = 0.f;
-  if (tid == 0) sc[0] = -INFINITY;
+  float* Cs = smf + 2 * Ly::BUF;                 // [HD][VS]  state C
+  float* Ws = Cs + HD * VS;                      // [CL][WS]  W_ts
+  float* zs = Ws + CL * WS;                      // [HD]
+  float* gs = zs + HD;                           // [CL] g_s
+  float* Rs = gs + CL;                           // [CL] R_t
+  float* es = Rs + CL;                           // [CL] e^{g_s - R_{L-1}}
+  float* qz = es + CL;                           // [CL] q~ . z
+  float* sc = qz + CL;                           // [4] m, F_{L-1}, R_{L-1}
   const float* F = a.feat + (size_t)lp * Pm * NF;
   float* prio = a.prio + (size_t)lp * Pm;
-  const float* av = a.ms.a + (size_t)h * HH;
+  if (c0 < c1) load_chunk<HD, true>(F, NF, c0 * CL, P, D, smf, NTC);
+  cp_commit();
+  {
+    const float* s0 = seg > 0 ? a.seg + ((size_t)lp * (a.nseg - 1) + seg - 1) * Ly::SEG : nullptr;
+    for (int e = tid; e < HD * (HH / 4); e += NTC) {
+      const int r = e / (HH / 4), c = e - r * (HH / 4);
+      *reinterpret_cast<float4*>(Cs + r * VS + 4 * c) =
+          s0 ? *reinterpret_cast<const float4*>(s0 + r * HH + 4 * c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    for (int e = tid; e < HD; e += NTC) zs[e] = s0 ? s0[HD * HH + e] : 0.f;
+    if (tid == 0) sc[0] = seg > 0 ? a.seg_m[(size_t)lp * a.nseg + seg] : -INFINITY;
+  }
+  float av[NB];
+#pragma unroll
+  for (int j = 0; j < NB; ++j) av[j] = a.ms.a[(size_t)h * HH + NB * tx + j];
   const float bsc = a.ms.b[h];
-  __syncthreads();
 
-  for (int t0 = 0; t0 < P; t0 += CL) {
-    // ---- load the chunk: k~, v~ of tokens t0.., q~ of the tokens they read out ------
-    for (int e = tid; e < CL * (HD / 4); e += NTM) {
-      const int r = e / (HD / 4), c4 = e - r * (HD / 4);
-      const int t = t0 + r, u = t - D;
-      float4 kv = make_float4(0.f, 0.f, 0.f, 0.f), qv = kv;
-      if (t < P) kv = *reinterpret_cast<const float4*>(F + (size_t)t * NF + 4 * c4);
-      if (t < P && u >= 0) qv = *reinterpret_cast<const float4*>(F + (size_t)u * NF + HD + HH + 4 * c4);
-      *reinterpret_cast<float4*>(Ks + r * QS + 4 * c4) = kv;
-      *reinterpret_cast<float4*>(Qs + r * QS + 4 * c4) = qv;
-    }
-    for (int e = tid; e < CL * HH; e += NTM) {
-      const int r = e / HH, j = e - r * HH;
-      const int t = t0 + r;
-      Vs[r * VS + j] = t < P ? F[(size_t)t * NF + HD + j] : 0.f;
-    }
-    // gates: warp 0 scans the chunk's log forget gates (two tokens per lane)
-    if (warp == 0) {
-      const float m = sc[0];
-      float lfv[2], aiv[2];
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const int t = t0 + 2 * lane + k;
-        const bool in = t < P;
-        aiv[k] = in ? F[(size_t)t * NF + 2 * HD + HH] : -INFINITY;
-        lfv[k] = in ? -softplus(-F[(size_t)t * NF + 2 * HD + HH + 1]) : 0.f;
-      }
-      float f1 = lfv[0] + lfv[1], inc = f1;          // inclusive scan over lane pairs
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const float y = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += y;
-      }
-      const float Fa = inc - f1 + lfv[0], Fb = inc;  // F of tokens 2 lane, 2 lane + 1
-      const float ga = aiv[0] - Fa, gb = aiv[1] - Fb;
-      float gm = fmaxf(ga, gb), run = gm;            // inclusive prefix max
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const float y = __shfl_up_sync(0xffffffffu, run, o);
-        if (lane >= o) run = fmaxf(run, y);
-      }
-      const float prev = __shfl_up_sync(0xffffffffu, run, 1);
-      const float before = lane == 0 ? -INFINITY : prev;
-      gs[2 * lane] = ga;
-      gs[2 * lane + 1] = gb;
-      Rs[2 * lane] = fmaxf(m, fmaxf(before, ga));
-      Rs[2 * lane + 1] = fmaxf(m, run);
-      if (lane == 31) sc[1] = Fb;                    // F of the chunk's last token
-      (void)gm;
-    }
+  for (int ch = c0; ch < c1; ++ch) {
+    const int t0 = ch * CL;
+    const float* buf = smf + ((ch - c0) & 1) * Ly::BUF;
+    const float* Qs = buf + Ly::B_Q;
+    const float* Ks = buf + Ly::B_K;
+    const float* Vs = buf + Ly::B_V;
+    if (ch + 1 < c1) load_chunk<HD, true>(F, NF, t0 + CL, P, D, smf + ((ch + 1 - c0) & 1) * Ly::BUF, NTC);
+    cp_commit();
+    cp_wait<1>();
     __syncthreads();
-
-    // ---- S = q~ K^T -> W;  q~ C -> registers;  q~ . z ----------------------------------
-    {
-      float acc[4][4];
+    const float m = sc[0];
+    float acc[4][4], num[4][NB];
+    if (front) {
+      // ---- S = q~ K^T ------------------------------------------------------------------
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -500,6 +853,41 @@ __global__ void __launch_bounds__(NTM) mlstm_chunk_kernel(MScanArgs a) {
             acc[i][j] = fmaf(qa[i].x, kb[j].x, fmaf(qa[i].y, kb[j].y,
                         fmaf(qa[i].z, kb[j].z, fmaf(qa[i].w, kb[j].w, acc[i][j]))));
       }
+    } else {
+      if (tid >= NTC - 32) chunk_gates(buf + Ly::B_G, t0, P, m, gs, Rs, es, sc);
+      // ---- q~ C and q~ . z --------------------------------------------------------------
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < NB; ++j) num[i][j] = 0.f;
+#pragma unroll 2
+      for (int c = 0; c < HD; c += 4) {
+        float4 qa[4];
+        float cr[4][NB];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) qa[i] = *reinterpret_cast<const float4*>(Qs + (ty + 16 * i) * QS + c);
+#pragma unroll
+        for (int x = 0; x < 4; ++x) ld_vec<NB>(cr[x], Cs + (c + x) * VS + NB * tx);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < NB; ++j)
+            num[i][j] = fmaf(qa[i].x, cr[0][j], fmaf(qa[i].y, cr[1][j],
+                        fmaf(qa[i].z, cr[2][j], fmaf(qa[i].w, cr[3][j], num[i][j]))));
+      }
+      // warp w of the group takes rows 8w .. 8w + 7
+      const int w8 = gt >> 5;
+#pragma unroll
+      for (int rr = 0; rr < CL / 8; ++rr) {
+        const int t = w8 * (CL / 8) + rr;
+        float s = 0.f;
+        for (int c = lane; c < HD; c += 32) s = fmaf(Qs[t * QS + c], zs[c], s);
+        s = warp_sum(s);
+        if (lane == 0) qz[t] = s;
+      }
+    }
+    __syncthreads();                 // gates known; C and z read
+    if (front) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int t = ty + 16 * i;
@@ -511,45 +899,13 @@ __global__ void __launch_bounds__(NTM) mlstm_chunk_kernel(MScanArgs a) {
         }
       }
     }
-    float num[4][NB];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < NB; ++j) num[i][j] = 0.f;
-#pragma unroll 2
-    for (int c = 0; c < HD; c += 4) {
-      float4 qa[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) qa[i] = *reinterpret_cast<const float4*>(Qs + (ty + 16 * i) * QS + c);
-#pragma unroll
-      for (int j = 0; j < NB; ++j) {
-        const int col = tx + 16 * j;
-        const float c0 = Cs[(c + 0) * VS + col], c1 = Cs[(c + 1) * VS + col];
-        const float c2 = Cs[(c + 2) * VS + col], c3 = Cs[(c + 3) * VS + col];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          num[i][j] = fmaf(qa[i].x, c0, fmaf(qa[i].y, c1, fmaf(qa[i].z, c2, fmaf(qa[i].w, c3, num[i][j]))));
-      }
-    }
-    // q~ . z: warp w takes rows 8w .. 8w + 7
-#pragma unroll
-    for (int rr = 0; rr < CL / 8; ++rr) {
-      const int t = warp * (CL / 8) + rr;
-      float s = 0.f;
-      for (int c = lane; c < HD; c += 32) s = fmaf(Qs[t * QS + c], zs[c], s);
-      s = warp_sum(s);
-      if (lane == 0) qz[t] = s;
-    }
-    __syncthreads();
-
-    // ---- readout rows: num = e^{m-R} q~C + W V, den = e^{m-R} q~.z + sum_s W ----------
-    {
-      const float m = sc[0];
+    __syncthreads();                 // W written
+    if (!front) {
+      // ---- readout rows: num = e^{m-R} q~C + W V, den = e^{m-R} q~.z + sum_s W ----------
       float den[4], coef[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int t = ty + 16 * i;
-        coef[i] = __expf(m - Rs[t]);
+        coef[i] = __expf(m - Rs[ty + 16 * i]);
         den[i] = 0.f;
 #pragma unroll
         for (int j = 0; j < NB; ++j) num[i][j] *= coef[i];
@@ -557,20 +913,20 @@ __global__ void __launch_bounds__(NTM) mlstm_chunk_kernel(MScanArgs a) {
 #pragma unroll 4
       for (int s = 0; s < CL; s += 4) {
         float4 wa[4];
+        float v[4][NB];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           wa[i] = *reinterpret_cast<const float4*>(Ws + (ty + 16 * i) * WS + s);
           den[i] += (wa[i].x + wa[i].y) + (wa[i].z + wa[i].w);
         }
 #pragma unroll
-        for (int j = 0; j < NB; ++j) {
-          const int col = tx + 16 * j;
-          const float v0 = Vs[(s + 0) * VS + col], v1 = Vs[(s + 1) * VS + col];
-          const float v2 = Vs[(s + 2) * VS + col], v3 = Vs[(s + 3) * VS + col];
+        for (int x = 0; x < 4; ++x) ld_vec<NB>(v[x], Vs + (s + x) * VS + NB * tx);
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
-            num[i][j] = fmaf(wa[i].x, v0, fmaf(wa[i].y, v1, fmaf(wa[i].z, v2, fmaf(wa[i].w, v3, num[i][j]))));
-        }
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < NB; ++j)
+            num[i][j] = fmaf(wa[i].x, v[0][j], fmaf(wa[i].y, v[1][j],
+                        fmaf(wa[i].z, v[2][j], fmaf(wa[i].w, v[3][j], num[i][j]))));
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -580,7 +936,7 @@ __global__ void __launch_bounds__(NTM) mlstm_chunk_kernel(MScanArgs a) {
 #pragma unroll
         for (int j = 0; j < NB; ++j) {
           const float hv = num[i][j] / dn;
-          r = fmaf(av[tx + 16 * j], hv / (1.f + expf(-hv)), r);
+          r = fmaf(av[j], hv / (1.f + expf(-hv)), r);
         }
 #pragma unroll
         for (int o = 1; o < 16; o <<= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
@@ -591,58 +947,100 @@ __global__ void __launch_bounds__(NTM) mlstm_chunk_kernel(MScanArgs a) {
           prio[u] = static_priority(canon_score(rv), u, a.st.log_gamma, h);
         }
       }
-    }
-    // ---- state update C' = e^{m-R_L} C + K^T diag(e^{g-R_L}) V;  z likewise -------------
-    {
-      const float RL = Rs[CL - 1];
-      const float wc = __expf(sc[0] - RL);
-      constexpr int NR = HD / 16;
-      float acc[NR][NB];
+    } else if (last || ch + 1 < c1) {
+      // ---- state update C' = e^{m-R_L} C + K^T diag(e^{g-R_L}) V;  z likewise -------------
+      const float RL = sc[2], wc = __expf(m - RL);
+      float cn[NR][NB];
 #pragma unroll
-      for (int i = 0; i < NR; ++i)
+      for (int i = 0; i < NR; ++i) {
+        ld_vec<NB>(cn[i], Cs + (NR * ty + i) * VS + NB * tx);
 #pragma unroll
-        for (int j = 0; j < NB; ++j) acc[i][j] = wc * Cs[(ty + 16 * i) * VS + tx + 16 * j];
-#pragma unroll 4
-      for (int s = 0; s < CL; ++s) {
-        const float w = __expf(gs[s] - RL);
-        float vb[NB];
-#pragma unroll
-        for (int j = 0; j < NB; ++j) vb[j] = w * Vs[s * VS + tx + 16 * j];
-#pragma unroll
-        for (int i = 0; i < NR; ++i) {
-          const float kk = Ks[s * QS + ty + 16 * i];
-#pragma unroll
-          for (int j = 0; j < NB; ++j) acc[i][j] = fmaf(kk, vb[j], acc[i][j]);
-        }
+        for (int j = 0; j < NB; ++j) cn[i][j] *= wc;
       }
-      float zn = 0.f;
-      if (tid < HD) {
-        zn = wc * zs[tid];
-        for (int s = 0; s < CL; ++s) zn = fmaf(__expf(gs[s] - RL), Ks[s * QS + tid], zn);
+      state_update<HD>(cn, Ks, Vs, es, ty, tx);
+#pragma unroll
+      for (int i = 0; i < NR; ++i) st_vec<NB>(Cs + (NR * ty + i) * VS + NB * tx, cn[i]);
+      if (gt < HD) {
+        float zn = wc * zs[gt];
+        for (int s = 0; s < CL; ++s) zn = fmaf(es[s], Ks[s * QS + gt], zn);
+        zs[gt] = zn;
       }
-      __syncthreads();                 // every read of C, z and the scalars is done
-#pragma unroll
-      for (int i = 0; i < NR; ++i)
-#pragma unroll
-        for (int j = 0; j < NB; ++j) Cs[(ty + 16 * i) * VS + tx + 16 * j] = acc[i][j];
-      if (tid < HD) zs[tid] = zn;
-      if (tid == 0) sc[0] = sc[1] + RL;
+      if (gt == 0) sc[3] = sc[1] + RL;
     }
-    __syncthreads();
+    __syncthreads();                 // the chunk is done: its buffer, W and the gates are free
+    if (tid == 0) sc[0] = sc[3];
   }
+  cp_wait<0>();
+  __syncthreads();
+  if (!last) return;
+  const int pair = (a.first_seq + bl) * H + h;
   float* Cg = a.ms.C + (size_t)pair * HD * HH;
-  for (int e = tid; e < HD * HH; e += NTM) Cg[e] = Cs[(e / HH) * VS + (e % HH)];
-  for (int e = tid; e < HD; e += NTM) a.ms.z[(size_t)pair * HD + e] = zs[e];
+  for (int e = tid; e < HD * HH; e += NTC) Cg[e] = Cs[(e / HH) * VS + (e % HH)];
+  for (int e = tid; e < HD; e += NTC) a.ms.z[(size_t)pair * HD + e] = zs[e];
   if (tid == 0) a.ms.m[pair] = sc[0];
 }
 
 template <int HD>
-size_t chunk_smem() { return (size_t)ChunkLayout<HD>::FLOATS * 4; }
+size_t chunk_smem() {
+  using Ly = ChunkLayout<HD>;
+  return (size_t)(2 * Ly::BUF + HD * Ly::VS + CL * Ly::WS + HD + 4 * CL + 4) * 4;
+}
+template <int HD>
+size_t seg_smem() { return (size_t)2 * ChunkLayout<HD>::BUF_S * 4; }
+
+// Chunks per segment: one (no state is updated twice) while the states between segments stay
+// below 256 MB, else as many as that takes.
+int seg_chunks(int d, int pairs, int Pmax) {
+  const double bytes = (double)pairs * ((Pmax + CL - 1) / CL) * (d * (d / 2) + d) * 4.0;
+  return std::max(1, (int)(bytes / 256e6) + 1);
+}
+int seg_count(int d, int pairs, int Pmax) {
+  const int nch = (Pmax + CL - 1) / CL, n = seg_chunks(d, pairs, Pmax);
+  return std::max(1, (nch + n - 1) / n);
+}
+
+template <int HD>
+cudaError_t launch_scan(MScanArgs sa, int pairs, cudaStream_t stream) {
+  if (sa.nseg > 1) {
+    mlstm_seg_kernel<HD><<<dim3(sa.nseg - 1, pairs), NTM, seg_smem<HD>(), stream>>>(sa);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    mlstm_link_kernel<HD><<<dim3((ChunkLayout<HD>::SEG + NTM - 1) / NTM, pairs), NTM, 0, stream>>>(sa);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  mlstm_chunk_kernel<HD><<<dim3(sa.nseg, pairs), NTC, chunk_smem<HD>(), stream>>>(sa);
+  return cudaGetLastError();
+}
+
+template <int HD>
+cudaError_t launch_proj_tc(const MlstmDev& m, const void* K, const void* V, const int32_t* plen, int pairs,
+                           int H, int Pmax, int NF, float* feat, cudaStream_t stream) {
+  MProjTcArgs a{static_cast<const bf16*>(K), static_cast<const bf16*>(V), static_cast<const bf16*>(m.Wt),
+                m.bi, m.bf, plen, feat, H, Pmax, NF};
+  mlstm_proj_tc_kernel<HD><<<dim3((Pmax + PT_TOK - 1) / PT_TOK, pairs), NTM, PtP<HD>::SMEM, stream>>>(a);
+  return cudaGetLastError();
+}
 
 }  // namespace
 
 int mlstm_nc(int d) { return ((3 * (d / 2) + 2) + 3) & ~3; }
 int mlstm_nf(int d) { return ((2 * d + d / 2 + 2) + 3) & ~3; }
+size_t mlstm_wt_bytes(int d, int H) {
+  return d == 128 ? (size_t)H * PtP<128>::NKC * PtP<128>::WB : (size_t)H * PtP<64>::NKC * PtP<64>::WB;
+}
+cudaError_t launch_mlstm_split(const Dims& dm, const MlstmDev& m, cudaStream_t stream) {
+  bf16* wt = static_cast<bf16*>(m.Wt);
+  if (dm.d == 128) mlstm_split_kernel<128><<<512, 256, 0, stream>>>(m.Wcat, m.NC, dm.H, wt);
+  else mlstm_split_kernel<64><<<512, 256, 0, stream>>>(m.Wcat, m.NC, dm.H, wt);
+  return cudaGetLastError();
+}
+// Workspace of the prompt scores: every token's features, then the segments' states and scalars.
+size_t mlstm_prefill_bytes(int d, int pairs, int Pmax) {
+  const size_t nseg = seg_count(d, pairs, Pmax);
+  return ((size_t)pairs * Pmax * mlstm_nf(d) + (size_t)pairs * (nseg - 1) * (d * (d / 2) + d) +
+          3 * (size_t)pairs * nseg) * 4;
+}
 
 static MState to_mstate(const MlstmDev& m) {
   MState s;
@@ -659,16 +1057,21 @@ cudaError_t prepare_mlstm(const Dims& dm) {
   cudaError_t e;
   if (dm.dtype == KVPOP_F32) {
     e = raise_smem_limit(ingest_mlstm_kernel<float>, ism);
-    if (e == cudaSuccess)
-      e = raise_smem_limit(mlstm_proj_kernel<float>, psm);
+    if (e == cudaSuccess) e = raise_smem_limit(mlstm_proj_kernel, psm);
   } else {
     e = raise_smem_limit(ingest_mlstm_kernel<bf16>, ism);
-    if (e == cudaSuccess)
-      e = raise_smem_limit(mlstm_proj_kernel<bf16>, psm);
   }
-  if (e == cudaSuccess)
-    e = dm.d == 128 ? raise_smem_limit(mlstm_chunk_kernel<128>, chunk_smem<128>())
-                    : raise_smem_limit(mlstm_chunk_kernel<64>, chunk_smem<64>());
+  auto raise = [&](auto* chunk, size_t cs, auto* segk, size_t ss, auto* pk, size_t ps) {
+    if (e == cudaSuccess) e = raise_smem_limit(chunk, cs);
+    if (e == cudaSuccess) e = raise_smem_limit(segk, ss);
+    if (e == cudaSuccess) e = raise_smem_limit(pk, ps);
+  };
+  if (dm.d == 128)
+    raise(mlstm_chunk_kernel<128>, chunk_smem<128>(), mlstm_seg_kernel<128>, seg_smem<128>(),
+          mlstm_proj_tc_kernel<128>, PtP<128>::SMEM);
+  else
+    raise(mlstm_chunk_kernel<64>, chunk_smem<64>(), mlstm_seg_kernel<64>, seg_smem<64>(),
+          mlstm_proj_tc_kernel<64>, PtP<64>::SMEM);
   return e;
 }
 
@@ -708,25 +1111,25 @@ cudaError_t launch_prefill_mlstm_scores(const State& st, const Dims& dm, const M
                                         float* feat, float* prio, cudaStream_t stream) {
   const int NF = mlstm_nf(dm.d);
   const int pairs = n_seq * dm.H;
-  const size_t psm = (size_t)2 * dm.d * UTM * 4 + (size_t)UTM * m.NC * 4;
-  dim3 g1((Pmax + UTM - 1) / UTM, pairs);
   if (Pmax > 0) {
+    cudaError_t e;
     if (dm.dtype == KVPOP_F32) {
-      MProjArgs<float> a{dm, to_mstate(m), (const float*)K, (const float*)V, plen, feat, Pmax, NF};
-      mlstm_proj_kernel<float><<<g1, NTM, psm, stream>>>(a);
+      const size_t psm = (size_t)2 * dm.d * UTM * 4 + (size_t)UTM * m.NC * 4;
+      MProjArgs a{dm, to_mstate(m), (const float*)K, (const float*)V, plen, feat, Pmax, NF};
+      mlstm_proj_kernel<<<dim3((Pmax + UTM - 1) / UTM, pairs), NTM, psm, stream>>>(a);
+      e = cudaGetLastError();
     } else {
-      MProjArgs<bf16> a{dm, to_mstate(m), (const bf16*)K, (const bf16*)V, plen, feat, Pmax, NF};
-      mlstm_proj_kernel<bf16><<<g1, NTM, psm, stream>>>(a);
+      e = dm.d == 128 ? launch_proj_tc<128>(m, K, V, plen, pairs, dm.H, Pmax, NF, feat, stream)
+                      : launch_proj_tc<64>(m, K, V, plen, pairs, dm.H, Pmax, NF, feat, stream);
     }
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  MScanArgs sa{st, dm, to_mstate(m), plen, feat, override_, prio, first_seq, Pmax, NF};
-  if (dm.d == 128)
-    mlstm_chunk_kernel<128><<<pairs, NTM, chunk_smem<128>(), stream>>>(sa);
-  else
-    mlstm_chunk_kernel<64><<<pairs, NTM, chunk_smem<64>(), stream>>>(sa);
-  return cudaGetLastError();
+  MScanArgs sa{st, dm, to_mstate(m), plen, feat, override_, prio, nullptr, nullptr, nullptr, first_seq, Pmax, NF,
+               seg_chunks(dm.d, pairs, Pmax), seg_count(dm.d, pairs, Pmax)};
+  sa.seg = feat + (size_t)pairs * Pmax * NF;
+  sa.seg_scal = sa.seg + (size_t)pairs * (sa.nseg - 1) * (dm.d * (dm.d / 2) + dm.d);
+  sa.seg_m = sa.seg_scal + (size_t)2 * pairs * sa.nseg;
+  return dm.d == 128 ? launch_scan<128>(sa, pairs, stream) : launch_scan<64>(sa, pairs, stream);
 }
 
 }  // namespace kvpop
