@@ -633,8 +633,9 @@ cudaError_t launch_f32(PromptArgs a, int n_pairs, cudaStream_t stream) {
 }  // namespace
 
 bool prompt_t5_ok(int d, int G, int s, int w, int k);
-cudaError_t launch_prompt_t5(const prompt::PromptArgs& a, int n_pairs, int G, bool dense,
-                             bool want_y, cudaStream_t stream);
+cudaError_t launch_prompt_t5(const prompt::PromptArgs& a, int n_pairs, int G, cudaStream_t stream);
+cudaError_t launch_causal_lse_t5(const void* Q, const void* K, const int32_t* len, int n_seq, int H, int G,
+                                 int S, float* lse, int32_t* err, cudaStream_t stream);   // kvpop_target.cu
 
 namespace {
 
@@ -649,8 +650,7 @@ bool use_t5(int dtype, int d, int G, int s, int w, int k) {
 
 template <bool DENSE, bool WANT_Y>
 cudaError_t dispatch(const PromptArgs& a, int n_pairs, int dtype, int d, int G, cudaStream_t stream) {
-  if (use_t5(dtype, d, G, a.s, a.w, a.capA - a.s) && (DENSE || WANT_Y))
-    return launch_prompt_t5(a, n_pairs, G, DENSE, WANT_Y, stream);
+  if (!DENSE && use_t5(dtype, d, G, a.s, a.w, a.capA - a.s)) return launch_prompt_t5(a, n_pairs, G, stream);
   if (dtype == KVPOP_BF16) {
     if (d == 128) {
       if (G == 4) return launch_tc<128, 4, DENSE, WANT_Y>(a, n_pairs, stream);
@@ -695,6 +695,7 @@ cudaError_t launch_causal_lse(const void* Q, const void* K, const int32_t* len, 
                               int G, int d, int S, int dtype, float* lse, int32_t* err,
                               cudaStream_t stream) {
   if (n_seq <= 0 || S <= 0) return cudaSuccess;
+  if (use_t5(dtype, d, G, 0, 1, 0)) return launch_causal_lse_t5(Q, K, len, n_seq, H, G, S, lse, err, stream);
   PromptArgs a{Q, K, nullptr, nullptr, nullptr, nullptr, len, nullptr, lse, H, G, S, 0, 1, 0, 0,
                1.4426950408889634f / sqrtf((float)d), err};
   return dispatch<true, false>(a, n_seq * H, dtype, d, G, stream);

@@ -1,6 +1,5 @@
 // Masked prompt attention on the 5th-generation tensor cores (tcgen05), bf16
-// with head dimension 128 (App. C.1 mask, App. C.3; the dense causal form
-// gives the normalisers of App. D.1).
+// with head dimension 128 (App. C.1 mask, App. C.3).
 //
 // Same key lists as the m16n8k16 kernel (kvpop_prompt.cu), built for 256 / G
 // consecutive queries of one (sequence, KV head): the CTA's 256 (query, head)
@@ -70,7 +69,7 @@ constexpr int B_ODONE = 14;        // [2]  MMA -> softmax (one per half)
 constexpr int B_QFULL = 16;
 enum : int { T5ERR_WAIT = 21 };
 
-template <int G, bool DENSE, bool WANT_Y, int ST>
+template <int G, int ST>
 __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) {
   using L = Lay<ST>;
   constexpr int BM = T5_ROWS / G;
@@ -99,9 +98,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
   }
   if (warp == T5_MMA_WARP) tmem_alloc(sb + L::OFF_TMEM, T5_TMEM_COLS);
   TileInfo ti;
-  bool live;
-  if (DENSE) live = dense_setup(a, BM, ti);
-  else live = tile_setup<T5_THREADS>(a, BM, tauS, red, posA, posM, ti);
+  const bool live = tile_setup<T5_THREADS>(a, BM, tauS, red, posA, posM, ti);
   fence_before();
   __syncthreads();
   fence_after();
@@ -111,7 +108,6 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
     const int nblk = (nU + T5_BN - 1) / T5_BN;
     const size_t pair_off = (size_t)ti.pair * S;
     auto entry = [&](int e) -> int {
-      if (DENSE) return e < nU ? e : 0;
       if (e < nA) return posA[e];
       return e < nU ? posM[e - nA] : (nA > 0 ? posA[0] : posM[0]);
     };
@@ -120,7 +116,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
       const int pt = tid - 32 * (T5_MMA_WARP + 1);
       const bf16* Qb = static_cast<const bf16*>(a.Q) + ((size_t)ti.seq * H * G + (size_t)ti.h * G) * S * 128;
       const bf16* Kp = static_cast<const bf16*>(a.K) + pair_off * 128;
-      const bf16* Vp = WANT_Y ? static_cast<const bf16*>(a.V) + pair_off * 128 : nullptr;
+      const bf16* Vp = static_cast<const bf16*>(a.V) + pair_off * 128;
       for (int i = pt; i < T5_ROWS * 16; i += T5_PT) {
         const int r = i >> 4, c = i & 15;
         const int q = ti.q0 + r / G, g = r % G;
@@ -142,10 +138,8 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
           const uint32_t o0 = tile_off(key, c2, T5_BN), o1 = tile_off(key, c2 + 1, T5_BN);
           cp_async16(kd + o0, Kp + t, 16);
           cp_async16(kd + o1, Kp + t + 8, 16);
-          if (WANT_Y) {
-            cp_async16(vd + o0, Vp + t, 16);
-            cp_async16(vd + o1, Vp + t + 8, 16);
-          }
+          cp_async16(vd + o0, Vp + t, 16);
+          cp_async16(vd + o1, Vp + t + 8, 16);
         }
         cp_async_arrive_noinc(bar(B_FULL + st));
       }
@@ -172,7 +166,6 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
                        idS, ks > 0);
             commit(bar(B_SFULL + 2 * h + (j & 1)));
           }
-          if (!WANT_Y) commit(bar(B_EMPTY + st));
         };
         issue_s(0);
         if (nblk > 1) issue_s(1);
@@ -183,16 +176,14 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
           for (int h = 0; h < 2; ++h) {
             if (!(ok = mbar_wait(bar(B_PFULL + 2 * h + (j & 1)), (j >> 1) & 1, a.err, T5ERR_WAIT))) break;
             fence_after();
-            if (WANT_Y) {
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
-                mma_bf16(tmem + h * 128, kmajor_desc(sb + L::OFF_P + h * PB, T5_HALF, kk),
-                         mnmajor_desc(vb, T5_BN, kk), idO, (j > 0 || kk > 0));
-              commit(bar(B_ODONE + h));
-            }
+            for (int kk = 0; kk < 4; ++kk)
+              mma_bf16(tmem + h * 128, kmajor_desc(sb + L::OFF_P + h * PB, T5_HALF, kk),
+                       mnmajor_desc(vb, T5_BN, kk), idO, (j > 0 || kk > 0));
+            commit(bar(B_ODONE + h));
           }
           if (!ok) break;
-          if (WANT_Y) commit(bar(B_EMPTY + st));
+          commit(bar(B_EMPTY + st));
           if (j + 2 < nblk) issue_s(j + 2);
         }
       }
@@ -205,10 +196,10 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
       const int ql = rr / G, g = rr - ql * G;
       const int q = ti.q0 + ql;
       const bool valid = q <= ti.q1;
-      const int tq = DENSE ? 0 : tauS[ql];
+      const int tq = tauS[ql];
       const uint32_t trow = (uint32_t)((warp & 3) * 32) << 16;
       const uint32_t tO = tmem + trow + h * 128, tS = tmem + trow + 256 + h * 128;
-      const int32_t* rank = DENSE ? nullptr : a.rank + pair_off;
+      const int32_t* rank = a.rank + pair_off;
       const float c2 = a.qscale;
       float m = -INFINITY, l = 0.f;
       bool ok = true;
@@ -230,7 +221,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
               bool kp = false;
               if (e < nU) {
                 const int t = entry(e);
-                kp = DENSE ? t <= q : keep_key(q, t, __ldg(rank + t), tq, a.s, a.w);
+                kp = keep_key(q, t, __ldg(rank + t), tq, a.s, a.w);
               }
               if (!kp) s[i] = -INFINITY;
             }
@@ -276,7 +267,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
         const float sum = ((ps[0] + ps[1]) + (ps[2] + ps[3])) + ((ps[4] + ps[5]) + (ps[6] + ps[7]));
         l = l * alpha + sum;
         m = m_new;
-        if (WANT_Y && j >= 1) {
+        if (j >= 1) {
           // PV_{j-1} must have consumed the P tile (and landed in O) before either changes;
           // the exponentials above overlap with it
           if (!(ok = uniform(mbar_wait(bar(B_ODONE + h), (j - 1) & 1, a.err, T5ERR_WAIT)))) break;
@@ -295,24 +286,22 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
             tmem_wait_st();
           }
         }
-        if (WANT_Y) {
-          unsigned char* prow = sm5 + L::OFF_P + h * PB;
+        unsigned char* prow = sm5 + L::OFF_P + h * PB;
 #pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            uint4 v;
-            v.x = pack_bf16(s[8 * c + 0], s[8 * c + 1]);
-            v.y = pack_bf16(s[8 * c + 2], s[8 * c + 3]);
-            v.z = pack_bf16(s[8 * c + 4], s[8 * c + 5]);
-            v.w = pack_bf16(s[8 * c + 6], s[8 * c + 7]);
-            *reinterpret_cast<uint4*>(prow + tile_off(r, c, T5_HALF)) = v;
-          }
-          fence_async_smem();
+        for (int c = 0; c < 8; ++c) {
+          uint4 v;
+          v.x = pack_bf16(s[8 * c + 0], s[8 * c + 1]);
+          v.y = pack_bf16(s[8 * c + 2], s[8 * c + 3]);
+          v.z = pack_bf16(s[8 * c + 4], s[8 * c + 5]);
+          v.w = pack_bf16(s[8 * c + 6], s[8 * c + 7]);
+          *reinterpret_cast<uint4*>(prow + tile_off(r, c, T5_HALF)) = v;
         }
+        fence_async_smem();
         fence_before();
         mbar_arrive(bar(B_PFULL + 2 * h + b));
       }
       const size_t row = ((size_t)ti.seq * H * G + (size_t)ti.h * G + g) * S + q;
-      if (WANT_Y && ok && nblk > 0) {
+      if (ok && nblk > 0) {
         ok = uniform(mbar_wait(bar(B_ODONE + h), (nblk - 1) & 1, a.err, T5ERR_WAIT));
         fence_after();
         if (ok) {
@@ -345,10 +334,10 @@ size_t t5_smem(int capA, int capM) {
   return (size_t)Lay<ST>::OFF_LIST + (size_t)(capA + capM) * 4;
 }
 
-template <int G, bool DENSE, bool WANT_Y, int ST>
+template <int G, int ST>
 cudaError_t launch_t5_st(const PromptArgs& a, int n_pairs, size_t smem, cudaStream_t stream) {
   constexpr int BM = T5_ROWS / G;
-  auto k = prompt_t5_kernel<G, DENSE, WANT_Y, ST>;
+  auto k = prompt_t5_kernel<G, ST>;
   cudaError_t e = raise_smem_limit(k, smem);
   if (e != cudaSuccess) return e;
   dim3 grid((a.S + BM - 1) / BM, n_pairs);
@@ -356,14 +345,13 @@ cudaError_t launch_t5_st(const PromptArgs& a, int n_pairs, size_t smem, cudaStre
   return cudaGetLastError();
 }
 
-template <int G, bool DENSE, bool WANT_Y>
+template <int G>
 cudaError_t launch_t5_g(PromptArgs a, int n_pairs, cudaStream_t stream) {
   constexpr int BM = T5_ROWS / G;
-  if (DENSE) a.capA = a.capM = 0;
-  else a.capM = a.s + 2 * BM + a.w;
+  a.capM = a.s + 2 * BM + a.w;
   const size_t s3 = t5_smem<3>(a.capA, a.capM), s2 = t5_smem<2>(a.capA, a.capM);
-  if (s3 <= 227 * 1024) return launch_t5_st<G, DENSE, WANT_Y, 3>(a, n_pairs, s3, stream);
-  if (s2 <= 227 * 1024) return launch_t5_st<G, DENSE, WANT_Y, 2>(a, n_pairs, s2, stream);
+  if (s3 <= 227 * 1024) return launch_t5_st<G, 3>(a, n_pairs, s3, stream);
+  if (s2 <= 227 * 1024) return launch_t5_st<G, 2>(a, n_pairs, s2, stream);
   return cudaErrorInvalidValue;
 }
 
@@ -375,17 +363,10 @@ bool prompt_t5_ok(int d, int G, int s, int w, int k) {
   return Lay<2>::OFF_LIST + 4 * lists <= 227 * 1024;
 }
 
-cudaError_t launch_prompt_t5(const PromptArgs& a, int n_pairs, int G, bool dense, bool want_y,
-                             cudaStream_t stream) {
-  if (dense) {
-    if (G == 4) return launch_t5_g<4, true, false>(a, n_pairs, stream);
-    if (G == 2) return launch_t5_g<2, true, false>(a, n_pairs, stream);
-    return launch_t5_g<1, true, false>(a, n_pairs, stream);
-  }
-  (void)want_y;
-  if (G == 4) return launch_t5_g<4, false, true>(a, n_pairs, stream);
-  if (G == 2) return launch_t5_g<2, false, true>(a, n_pairs, stream);
-  return launch_t5_g<1, false, true>(a, n_pairs, stream);
+cudaError_t launch_prompt_t5(const PromptArgs& a, int n_pairs, int G, cudaStream_t stream) {
+  if (G == 4) return launch_t5_g<4>(a, n_pairs, stream);
+  if (G == 2) return launch_t5_g<2>(a, n_pairs, stream);
+  return launch_t5_g<1>(a, n_pairs, stream);
 }
 
 }  // namespace kvpop

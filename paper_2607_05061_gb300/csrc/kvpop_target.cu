@@ -13,20 +13,16 @@
 // value output of the pass is never formed.  bf16 on m16n8k16 tensor-core
 // MMAs, fp32 on CUDA cores (64 keys x 128 queries per block, target_f32_kernel).
 //
-// bf16 with d = 128 runs on the 5th-generation tensor cores (target_t5_kernel):
-// a CTA holds 256 keys as two 128-row A tiles in shared memory; producer warps
-// stream each head's query rows in blocks of 128 through a 4-stage cp.async ring
-// and store the block's -log2(e) LSE_d beside them; one thread issues S = K Q^T
-// per half into a tensor-memory double buffer; one softmax thread per (key,
-// half) reads its row with 32x32b loads.  s c - log2(e) LSE_d is the query's
-// log2 attention probability of the key, so the row's 2^x are summed with base 0
-// and a running maximum is taken only for a 64-column half whose sum leaves
-// [2^-60, 2^60].  The query rows are contiguous; the pass has no value half.
+// bf16 with d = 128 runs on the 5th-generation tensor cores (lse_t5_kernel), which also
+// serves the dense causal normalisers of App. D.1.
 //
 // Kernel 2 aggregates per KV head (Eq. 2, App. F.1-F.2):
 //   r_t = log(eps + Agg_g mbar_t^(g) / N_t),  N_t = max(1, S - (t + w)),
 // N_t clipped to L + 1 with a lookahead, Agg = max or mean; without count
 // normalisation N_t = 1.
+#include <cuda.h>
+
+#include <algorithm>
 #include <cstdlib>
 
 #include "kvpop_mma.cuh"
@@ -382,59 +378,100 @@ __global__ void __launch_bounds__(TgP<HD>::THREADS, 1) target_tc_kernel(TargetAr
 }
 
 // ---------------------------------------------------------------- tcgen05 kernel (d = 128)
+// Log-sum-exp of rows against streamed columns, S = A B^T, in two uses:
+//  * FUTURE (transposed pass): rows are 256 keys of one (sequence, KV head); for each query
+//    head its rows q >= t0 + w are streamed, with -log2(e) LSE_d added per column;
+//  * causal normalisers (App. D.1): rows are the 256 (head, query) pairs of 256 / G queries, the
+//    keys 0 .. q1 are streamed once for all of them.
+// Both operands come by TMA (128-byte swizzle; rows past the sequence read as zeros).  One
+// thread issues the copies and one the MMAs (M = 128, N = 128), per 128-row half into one of
+// two tensor-memory buffers; 16 softmax warps take 32 rows x 64 columns of every block apiece.
+// The tensor unit (64 clocks per MMA) and the exponentials (32 per clock) need about 1024
+// clocks of a 256 x 128 block each; what is paid is the issue slots of the softmax warps, so
+// barriers are arrived at once per warp and a warp holds its whole part in registers.
+// Blocks: longest tiles first over all pairs (tiles of one pair
+// after the other left the last pair's longest tile to the end: 1363 us for the future pass of
+// 8 heads x 16384 tokens, 4 query heads each, T6_SWAP_US us this way).
 constexpr int T6_HALF = 128;
-constexpr int T6_ROWS = 2 * T6_HALF;            // keys per CTA
-constexpr int T6_BN = 128;                      // queries per block (MMA N)
-constexpr int T6_ST = 4;                        // query-block stages
-constexpr int T6_MMA_WARP = 16;                 // warps 0-15 softmax, 16 MMA, 17-19 producers
-constexpr int T6_PT = 96;
-constexpr int T6_THREADS = 32 * 20;
-constexpr int T6_KB = T6_HALF * 256;            // key tile of one half
-constexpr int T6_QB = T6_BN * 256;              // query block
-constexpr int T6_OFF_Q = 2 * T6_KB;
+constexpr int T6_ROWS = 2 * T6_HALF;            // rows per CTA
+constexpr int T6_BN = 128;                      // columns per block (MMA N)
+constexpr int T6_ST = 4;                        // column-block stages
+constexpr int T6_SOFT = 16;                     // warps 0-15 softmax, 16 MMA, 17 copies
+constexpr int T6_MMA_WARP = T6_SOFT;
+constexpr int T6_THREADS = 32 * (T6_SOFT + 2);
+constexpr int T6_AB = T6_HALF * 256;            // row tile of one half, bytes
+constexpr int T6_QB = T6_BN * 256;              // column block, bytes
+constexpr int T6_OFF_Q = 2 * T6_AB;
 constexpr int T6_OFF_LSE = T6_OFF_Q + T6_ST * T6_QB;
 constexpr int T6_OFF_BAR = T6_OFF_LSE + T6_ST * T6_BN * 4;
 constexpr int T6_OFF_TMEM = T6_OFF_BAR + 8 * 32;
 constexpr int T6_OFF_PX = T6_OFF_TMEM + 16;      // [2 head parity][2 halves][128 rows][m, l, seq, -]
-constexpr int T6_SMEM = T6_OFF_PX + 2 * 2 * T6_HALF * 16;
+constexpr int T6_SMEM = T6_OFF_PX + 2 * 2 * T6_HALF * 16 + 1024;   // 1024: swizzle atom alignment
 constexpr int T6_FULL = 0, T6_EMPTY = T6_ST, T6_SFULL = 2 * T6_ST, T6_PFULL = 2 * T6_ST + 4,
-              T6_KFULL = 2 * T6_ST + 8;
+              T6_AFULL = 2 * T6_ST + 8;
 enum : int { T6ERR_WAIT = 22 };
 
-template <int G>
-__global__ void __launch_bounds__(T6_THREADS, 1) target_t5_kernel(TargetArgs a) {
+struct LseArgs {
+  const float* lse;          // FUTURE: [n][H*G][S] natural log
+  const int32_t* len;        // [n] or nullptr
+  float* out;                // [n][H*G][S]
+  int n_pairs, H, S, w, la;
+  float scale;               // log2(e) / sqrt(d)
+  int32_t* err;
+};
+
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z,
+                                            uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar)
+      : "memory");
+}
+
+// mapA: boxes of 64 columns x (FUTURE: 128, else min(128, 256 / G)) rows of the row operand;
+// mapB: 64 columns x 128 rows of the streamed one.  Both maps are [heads][S][128].
+template <int G, bool FUTURE>
+__global__ void __launch_bounds__(T6_THREADS, 1)
+    lse_t5_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, LseArgs a) {
   using namespace tc05;
-  extern __shared__ __align__(1024) unsigned char sm6[];
+  constexpr int NQ = FUTURE ? T6_ROWS : T6_ROWS / G;      // positions of a tile
+  constexpr int ABOX = FUTURE ? T6_HALF : (NQ < T6_HALF ? NQ : T6_HALF);
+  extern __shared__ unsigned char sm6_raw[];
+  unsigned char* sm6 = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(sm6_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t sb = smem_u32(sm6);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int pair = blockIdx.y, seq = pair / a.H, h0 = pair - seq * a.H;
-  const int S = a.S, L = row_len(a, seq), w = a.w, la = a.la;
-  const int t0 = blockIdx.x * T6_ROWS;
+  const int tile = blockIdx.x / a.n_pairs, pair = blockIdx.x - tile * a.n_pairs;
+  const int seq = pair / a.H, h0 = pair - seq * a.H;
+  const int S = a.S, L = a.len ? max(0, min(a.len[seq], S)) : S, w = a.w, la = a.la;
+  // longest first: the future of early keys, the past of late queries
+  const int t0 = (FUTURE ? tile : (S + NQ - 1) / NQ - 1 - tile) * NQ;
   if (t0 >= L) return;
-  const int t1 = min(t0 + T6_ROWS - 1, L - 1);
-  const size_t qrow0 = (size_t)seq * a.H * G + (size_t)h0 * G;
-  const int d_lo = t0 + w;
-  const int d_hi = la > 0 ? min(L - 1, t1 + w + la) : L - 1;
-  if (d_lo > d_hi) {                               // no key of the tile has a future query
+  const int t1 = min(t0 + NQ - 1, L - 1);
+  const int qrow0 = seq * a.H * G + h0 * G;
+  // streamed columns d_lo .. d_hi, once (causal) or per query head (FUTURE)
+  const int d_lo = FUTURE ? t0 + w : 0;
+  const int d_hi = !FUTURE ? t1 : la > 0 ? min(L - 1, t1 + w + la) : L - 1;
+  if (FUTURE && d_lo > d_hi) {                     // no key of the tile has a future query
     for (int i = tid; i < (t1 - t0 + 1) * G; i += T6_THREADS) {
       const int tl = i / G, g = i - tl * G;
-      a.logm[(qrow0 + g) * S + t0 + tl] = -INFINITY;
+      a.out[(size_t)(qrow0 + g) * S + t0 + tl] = -INFINITY;
     }
     return;
   }
   const int nblk = (d_hi - d_lo + T6_BN) / T6_BN;
-  const int total = G * nblk;
+  const int total = FUTURE ? G * nblk : nblk;
   auto bar = [&](int i) { return sb + T6_OFF_BAR + 8u * (uint32_t)i; };
   if (tid == 0) {
     for (int i = 0; i < T6_ST; ++i) {
-      mbar_init(bar(T6_FULL + i), 2 * T6_PT);            // cp.async arrivals + plain stores
-      mbar_init(bar(T6_EMPTY + i), 1 + 4 * T6_HALF);   // MMA commit + every softmax thread (LSE)
+      mbar_init(bar(T6_FULL + i), FUTURE ? 2 : 1);         // the copies, and the normalisers' warp
+      mbar_init(bar(T6_EMPTY + i), FUTURE ? 1 + T6_SOFT : 1);   // MMA commit, normalisers read
     }
     for (int i = 0; i < 4; ++i) {
       mbar_init(bar(T6_SFULL + i), 1);
-      mbar_init(bar(T6_PFULL + i), 2 * T6_HALF);
+      mbar_init(bar(T6_PFULL + i), T6_SOFT / 2);
     }
-    mbar_init(bar(T6_KFULL), T6_PT);
+    mbar_init(bar(T6_AFULL), 1);
     mbar_fence_init();
     // the softmax halves' exchange slots start with no head done
     int* px = reinterpret_cast<int*>(sm6 + T6_OFF_PX);
@@ -445,46 +482,58 @@ __global__ void __launch_bounds__(T6_THREADS, 1) target_t5_kernel(TargetArgs a) 
   __syncthreads();
   fence_after();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(sm6 + T6_OFF_TMEM);
-  const bf16* Kp = static_cast<const bf16*>(a.K) + (size_t)pair * S * 128;
-  if (warp > T6_MMA_WARP) {
-    // ---------------------------------------------------------------- producers
-    const int pt = tid - 32 * (T6_MMA_WARP + 1);
-    for (int i = pt; i < T6_ROWS * 16; i += T6_PT) {
-      const int r = i >> 4, c = i & 15;
-      const bool ok = t0 + r <= t1;
-      cp_async16(sb + (r >> 7) * T6_KB + tile_off(r & 127, c, T6_HALF),
-                 Kp + (size_t)(ok ? t0 + r : t0) * 128 + c * 8, ok ? 16 : 0);
-    }
-    cp_async_arrive_noinc(bar(T6_KFULL));
-    for (int j = 0; j < total; ++j) {
-      const int st = j % T6_ST;
-      if (j >= T6_ST && !mbar_wait(bar(T6_EMPTY + st), ((j / T6_ST) - 1) & 1, a.err, T6ERR_WAIT)) break;
-      const int g = j / nblk, b = j - g * nblk;
-      const int d0 = d_lo + b * T6_BN;
-      const bf16* Qg = static_cast<const bf16*>(a.Q) + (qrow0 + g) * S * 128;
-      const uint32_t qd = sb + T6_OFF_Q + st * T6_QB;
-      for (int i = pt; i < T6_BN * 16; i += T6_PT) {
-        const int r = i >> 4, c = i & 15;
-        const bool ok = d0 + r <= d_hi;
-        cp_async16(qd + tile_off(r, c, T6_BN), Qg + (size_t)(ok ? d0 + r : d0) * 128 + c * 8, ok ? 16 : 0);
+  if (warp == T6_MMA_WARP + 1) {
+    // ---------------------------------------------------------------- copies
+    if (lane == 0) {
+      mbar_arrive_expect_tx(bar(T6_AFULL), 2 * T6_AB);
+      for (int r0 = 0; r0 < T6_ROWS; r0 += ABOX) {
+        const int z = FUTURE ? pair : qrow0 + r0 / NQ, y = t0 + (FUTURE ? r0 : r0 % NQ);
+        const uint32_t dst = sb + (r0 >> 7) * T6_AB + (r0 & 127) * 128;
+        tma_load_3d(dst, &mapA, 0, y, z, bar(T6_AFULL));
+        tma_load_3d(dst + T6_HALF * 128, &mapA, 64, y, z, bar(T6_AFULL));
       }
-      // the block's queries' normalisers, stored once as -log2(e) LSE_d
-      float* nls = reinterpret_cast<float*>(sm6 + T6_OFF_LSE) + st * T6_BN;
-      const float* lse = a.lse + (qrow0 + g) * S;
-      for (int i = pt; i < T6_BN; i += T6_PT) nls[i] = -kLog2e * __ldg(lse + min(d0 + i, d_hi));
-      cp_async_arrive_noinc(bar(T6_FULL + st));
-      mbar_arrive(bar(T6_FULL + st));
     }
-    cp_wait<0>();
+    int j = 0;
+    for (; j < total; ++j) {
+      const int st = j % T6_ST;
+      const bool ok = j < T6_ST || mbar_wait(bar(T6_EMPTY + st), ((j / T6_ST) - 1) & 1, a.err, T6ERR_WAIT);
+      if (!__all_sync(0xffffffffu, ok)) break;
+      const int g = FUTURE ? j / nblk : 0, d0 = d_lo + (j - g * nblk) * T6_BN;
+      if (lane == 0) {
+        const uint32_t qd = sb + T6_OFF_Q + st * T6_QB;
+        const int z = FUTURE ? qrow0 + g : pair;
+        mbar_arrive_expect_tx(bar(T6_FULL + st), T6_QB);
+        tma_load_3d(qd, &mapB, 0, d0, z, bar(T6_FULL + st));
+        tma_load_3d(qd + T6_BN * 128, &mapB, 64, d0, z, bar(T6_FULL + st));
+      }
+      if (FUTURE) {
+        // the block's normalisers, stored once as -log2(e) LSE_d
+        float* nls = reinterpret_cast<float*>(sm6 + T6_OFF_LSE) + st * T6_BN;
+        const float* lse = a.lse + (size_t)(qrow0 + g) * S;
+        float v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = __ldg(lse + min(d0 + lane + 32 * i, d_hi));
+#pragma unroll
+        for (int i = 0; i < 4; ++i) nls[lane + 32 * i] = -kLog2e * v[i];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(T6_FULL + st));
+      }
+    }
+    // every copy has landed before the CTA ends (the waiting roles may have given up)
+    if (lane == 0) {
+      mbar_wait(bar(T6_AFULL), 0, a.err, T6ERR_WAIT);
+      for (int k = max(0, j - T6_ST); k < j; ++k)
+        mbar_wait(bar(T6_FULL + k % T6_ST), (k / T6_ST) & 1, a.err, T6ERR_WAIT);
+    }
+    __syncwarp();
   } else if (warp == T6_MMA_WARP) {
     // ---------------------------------------------------------------- MMA issue
     if (lane == 0) {
       const uint32_t idS = idesc_bf16(128, T6_BN, 0);
-      bool ok = mbar_wait(bar(T6_KFULL), 0, a.err, T6ERR_WAIT);
+      bool ok = mbar_wait(bar(T6_AFULL), 0, a.err, T6ERR_WAIT);
       for (int j = 0; j < total && ok; ++j) {
         const int st = j % T6_ST, b2 = j & 1;
         if (!(ok = mbar_wait(bar(T6_FULL + st), (j / T6_ST) & 1, a.err, T6ERR_WAIT))) break;
-        fence_async_smem();
         fence_after();
         const uint32_t qb = sb + T6_OFF_Q + st * T6_QB;
 #pragma unroll
@@ -496,7 +545,7 @@ __global__ void __launch_bounds__(T6_THREADS, 1) target_t5_kernel(TargetArgs a) 
           const uint32_t dS = tmem + hh * 256 + (uint32_t)b2 * T6_BN;
 #pragma unroll
           for (int ks = 0; ks < 8; ++ks)
-            mma_bf16(dS, kmajor_desc(sb + hh * T6_KB, T6_HALF, ks), kmajor_desc(qb, T6_BN, ks), idS, ks > 0);
+            mma_bf16(dS, kmajor_desc(sb + hh * T6_AB, T6_HALF, ks), kmajor_desc(qb, T6_BN, ks), idS, ks > 0);
           commit(bar(T6_SFULL + 2 * hh + b2));
         }
         if (!ok) break;
@@ -509,129 +558,124 @@ __global__ void __launch_bounds__(T6_THREADS, 1) target_t5_kernel(TargetArgs a) 
     __syncwarp();
   } else {
     // ---------------------------------------------------------------- softmax rows
-    // warp w: half hh = (w / 4) mod 2 of the CTA's keys, key row r = 32 (w mod 4) + lane (the
-    // warp's tensor-memory lane quarter), and columns [64 cs, 64 cs + 64) of every block with
-    // cs = w / 8: four warps per subpartition share the exponentials of a block.  The two
-    // column halves of a row keep their own (max, sum) over a head's blocks and meet at the
-    // head's end in shared memory.
+    // warp w: half hh = (w / 4) mod 2 of the CTA's rows, row r = 32 (w mod 4) + lane (the warp's
+    // tensor-memory lane quarter), and columns [64 cs, 64 cs + 64) of every block with cs = w / 8:
+    // four warps per subpartition share the exponentials of a block.  The two column halves of
+    // a row keep their own (max, sum) over a head's blocks and meet at its end in shared memory.
     const int hh = (warp >> 2) & 1, cs = warp >> 3;
-    const int r = (warp & 3) * 32 + lane;
-    const int t = t0 + hh * T6_HALF + r;
-    const int hi = t <= t1 ? future_hi(t, L, w, la) : -1;
-    const uint32_t tS = tmem + ((uint32_t)((warp & 3) * 32) << 16) + hh * 256;
-    const float* nlS = reinterpret_cast<const float*>(sm6 + T6_OFF_LSE);   // -log2(e) LSE_d per stage
+    const int r = (warp & 3) * 32 + lane, ra = hh * T6_HALF + r;
+    const int t = t0 + (FUTURE ? ra : ra % NQ);            // the row's position
+    const int lo = FUTURE ? t + w : 0;                     // columns the row takes: lo .. hi
+    const int hi = t > t1 ? -1 : FUTURE ? future_hi(t, L, w, la) : t;
+    const uint32_t tS = tmem + ((uint32_t)((warp & 3) * 32) << 16) + hh * 256 + 64 * cs;
+    const float* nlS = reinterpret_cast<const float*>(sm6 + T6_OFF_LSE) + 64 * cs;   // -log2(e) LSE_d
     float* pxs = reinterpret_cast<float*>(sm6 + T6_OFF_PX);
-    const float c2 = a.kscale;
+    const uint64_t cc = f2_pack(a.scale, a.scale);
     float m = -INFINITY, l = 0.f;
-    auto uniform = [](bool x) { return __all_sync(0xffffffffu, x); };
+    int g = 0, b = 0;
     for (int j = 0; j < total; ++j) {
       const int st = j % T6_ST, b2 = j & 1;
-      const int g = j / nblk, b = j - g * nblk;
-      const int d0 = d_lo + b * T6_BN;
-      if (!uniform(mbar_wait(bar(T6_SFULL + 2 * hh + b2), (j >> 1) & 1, a.err, T6ERR_WAIT))) break;
+      const int e0 = d_lo + b * T6_BN + 64 * cs;
+      bool ok = mbar_wait(bar(T6_SFULL + 2 * hh + b2), (j >> 1) & 1, a.err, T6ERR_WAIT);
       // the stage's normalisers (complete long before S; the wait orders their reads)
-      if (!uniform(mbar_wait(bar(T6_FULL + st), (j / T6_ST) & 1, a.err, T6ERR_WAIT))) break;
+      if (FUTURE) ok = ok && mbar_wait(bar(T6_FULL + st), (j / T6_ST) & 1, a.err, T6ERR_WAIT);
+      if (!__all_sync(0xffffffffu, ok)) break;
       fence_after();
-      // this thread's 64 columns as two 32-column parts, each folded into the running sum
-#pragma unroll 1
-      for (int c = 0; c < 2; ++c) {
-        const int col = 64 * cs + 32 * c;
-        const int e0 = d0 + col;
-        float s[32];
-        tmem_ld32(tS + b2 * T6_BN + col, s);
-        tmem_wait_ld();
-        if (c == 1) {
-          // the thread's part of the S buffer is in registers: the MMA may overwrite it
-          fence_before();
-          mbar_arrive(bar(T6_PFULL + 2 * hh + b2));
-        }
-        const bool masked = e0 < t1 + w || e0 + 31 > d_hi || (la > 0 && e0 + 31 > t0 + w + la);
-        if (masked) {                               // on the raw logits: -inf c2 + n = -inf
+      float s[2][32];
+      tmem_ld32(tS + b2 * T6_BN, s[0]);
+      tmem_ld32(tS + b2 * T6_BN + 32, s[1]);
+      tmem_wait_ld();
+      // the warp's part of the S buffer is in registers: the MMA may overwrite it
+      fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(T6_PFULL + 2 * hh + b2));
+      // some row of the tile ends (or begins) inside these columns
+      const bool masked = FUTURE ? (e0 < t1 + w || e0 + 63 > d_hi || (la > 0 && e0 + 63 > t0 + w + la))
+                                 : e0 + 63 > t0;
+      if (masked) {                                 // on the raw logits: -inf c2 + n = -inf
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
-            const int d = e0 + i;
-            if (d < t + w || d > hi) s[i] = -INFINITY;
+            const int d = e0 + 32 * c + i;
+            if (d < lo || d > hi) s[c][i] = -INFINITY;
           }
+      }
+      // FUTURE: x = s c2 - log2(e) LSE_d is the query's log2 attention probability of the key, so
+      // 2^x needs no running maximum unless the key lies outside the query's kept set with a much
+      // larger logit: sum with base 0.  Causal: x = s c2 - m with the first part's maximum as
+      // the base.  The maximum is taken only when a part's sum leaves [2^-60, 2^60] (overflow,
+      // NaN, or every term tiny or masked).
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const float nb1 = FUTURE || m == -INFINITY ? 0.f : -m;
+        const uint64_t nb = f2_pack(nb1, nb1);
+        uint64_t ps[4] = {0ull, 0ull, 0ull, 0ull};
+        float* sc = s[c];
+#pragma unroll
+        for (int i4 = 0; i4 < 8; ++i4) {
+          uint64_t n0 = nb, n1 = nb;
+          if (FUTURE) {
+            const float4 v = reinterpret_cast<const float4*>(nlS + st * T6_BN + 32 * c)[i4];
+            n0 = f2_pack(v.x, v.y);
+            n1 = f2_pack(v.z, v.w);
+          }
+          f2_unpack(f2_fma(f2_pack(sc[4 * i4], sc[4 * i4 + 1]), cc, n0), sc[4 * i4], sc[4 * i4 + 1]);
+          f2_unpack(f2_fma(f2_pack(sc[4 * i4 + 2], sc[4 * i4 + 3]), cc, n1), sc[4 * i4 + 2], sc[4 * i4 + 3]);
+          const int k = (2 * i4) & 3;
+          ps[k] = f2_add(ps[k], f2_pack(ex2(sc[4 * i4]), ex2(sc[4 * i4 + 1])));
+          ps[k + 1] = f2_add(ps[k + 1], f2_pack(ex2(sc[4 * i4 + 2]), ex2(sc[4 * i4 + 3])));
         }
-        // x = s c2 - log2(e) LSE_d is the query's log2 attention probability of the key, so
-        // 2^x needs no running maximum unless the key lies outside the query's kept set
-        // with a much larger logit: sum with base 0, and take the maximum only when the
-        // part's sum leaves [2^-60, 2^60] (overflow, NaN, or every term tiny or masked).
-        {
-          const float4* l4 = reinterpret_cast<const float4*>(nlS + st * T6_BN + col);
-          const uint64_t cc = f2_pack(c2, c2);
-          uint64_t ps[4] = {0ull, 0ull, 0ull, 0ull};
-#pragma unroll
-          for (int i4 = 0; i4 < 8; ++i4) {
-            const float4 v = l4[i4];
-            f2_unpack(f2_fma(f2_pack(s[4 * i4], s[4 * i4 + 1]), cc, f2_pack(v.x, v.y)), s[4 * i4],
-                      s[4 * i4 + 1]);
-            f2_unpack(f2_fma(f2_pack(s[4 * i4 + 2], s[4 * i4 + 3]), cc, f2_pack(v.z, v.w)), s[4 * i4 + 2],
-                      s[4 * i4 + 3]);
-            const int k = (2 * i4) & 3;
-            ps[k] = f2_add(ps[k], f2_pack(ex2(s[4 * i4]), ex2(s[4 * i4 + 1])));
-            ps[k + 1] = f2_add(ps[k + 1], f2_pack(ex2(s[4 * i4 + 2]), ex2(s[4 * i4 + 3])));
+        if (FUTURE && c == 1) {                    // the warp is done with the stage's normalisers
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar(T6_EMPTY + st));
+        }
+        const uint64_t p2 = f2_add(f2_add(ps[0], ps[1]), f2_add(ps[2], ps[3]));
+        float q0, q1;
+        f2_unpack(p2, q0, q1);
+        const float sum = q0 + q1;
+        if (sum >= 0x1p-60f && sum <= 0x1p60f && (FUTURE || m != -INFINITY)) {
+          if (!FUTURE) {
+            l += sum;
+          } else if (m <= 0.f) {                    // new base 0
+            l = (m == 0.f ? l : l * ex2(m)) + sum;
+            m = 0.f;
+          } else {
+            l = fmaf(sum, ex2(-m), l);
           }
-          // the stage's query rows and normalisers are no longer needed by this thread
-          if (c == 1) mbar_arrive(bar(T6_EMPTY + st));
-          float q[8];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) f2_unpack(ps[k], q[2 * k], q[2 * k + 1]);
-          const float sum = ((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7]));
-          if (sum >= 0x1p-60f && sum <= 0x1p60f) {
-            if (m <= 0.f) {                         // new base 0
-              l = (m == 0.f ? l : l * ex2(m)) + sum;
-              m = 0.f;
-            } else {
-              l = fmaf(sum, ex2(-m), l);
-            }
-            continue;
-          }
+          continue;
         }
         // part maximum: 8 chains of three-input maxima
         float pm[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) pm[k] = s[k];
+        for (int k = 0; k < 8; ++k) pm[k] = fmax3(sc[k], sc[8 + k], sc[16 + k]);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) pm[k] = fmax3(pm[k], s[8 + k], s[16 + k]);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) pm[k] = fmaxf(pm[k], s[24 + k]);
+        for (int k = 0; k < 8; ++k) pm[k] = fmaxf(pm[k], sc[24 + k]);
+        // the values in sc are relative to -nb1
         const float mx = fmax3(fmax3(pm[0], pm[1], pm[2]), fmax3(pm[3], pm[4], pm[5]), fmaxf(pm[6], pm[7]));
-        const float mn = fmaxf(m, mx);
-        const float base = mn == -INFINITY ? 0.f : mn;
-        // sum of 2^(x - base), differences and partial sums packed in pairs
-        const uint64_t nb = f2_pack(-base, -base);
-        uint64_t ps[4] = {0ull, 0ull, 0ull, 0ull};
+        const float mn = fmaxf(m, mx - nb1);
+        const float base = mn == -INFINITY ? 0.f : mn + nb1;
+        float part = 0.f;
 #pragma unroll
-        for (int i = 0; i < 32; i += 8) {
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            float x0, x1;
-            f2_unpack(f2_add(f2_pack(s[i + 2 * k], s[i + 2 * k + 1]), nb), x0, x1);
-            ps[k] = f2_add(ps[k], f2_pack(ex2(x0), ex2(x1)));
-          }
-        }
-        float q[8];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) f2_unpack(ps[k], q[2 * k], q[2 * k + 1]);
-        l = l * ex2(m - base) + (((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7])));
+        for (int i = 0; i < 32; ++i) part += ex2(sc[i] - base);
+        l = l * ex2(m - (mn == -INFINITY ? 0.f : mn)) + part;
         m = mn;
       }
-      if (b == nblk - 1) {
+      if (++b == nblk) {
         // head g done: the upper column half hands its (max, sum) to the lower, which merges
-        // and writes the key's log mass (slots alternate by head; a flag names the head)
+        // and writes the row's result (slots alternate by head; a flag names the head)
         float* px = pxs + (((size_t)(g & 1) * 2 + hh) * T6_HALF + r) * 4;
-        volatile int* seq = reinterpret_cast<volatile int*>(px) + 2;
+        volatile int* done = reinterpret_cast<volatile int*>(px) + 2;
         if (cs == 1) {
           px[0] = m;
           px[1] = l;
           __threadfence_block();
-          *seq = g + 1;
+          *done = g + 1;
         } else {
-          bool ready = *seq == g + 1;
+          bool ready = *done == g + 1;
           if (!ready) {
             const unsigned long long tw = globaltimer();
-            while (!(ready = *seq == g + 1))
+            while (!(ready = *done == g + 1))
               if (globaltimer() - tw > kWaitLimitNs) { atomicCAS(a.err, 0, T6ERR_WAIT); break; }
           }
           __threadfence_block();
@@ -640,16 +684,67 @@ __global__ void __launch_bounds__(T6_THREADS, 1) target_t5_kernel(TargetArgs a) 
           float Lr = 0.f;
           if (M != -INFINITY)
             Lr = (m == -INFINITY ? 0.f : l * ex2(m - M)) + (m1 == -INFINITY ? 0.f : l1 * ex2(m1 - M));
-          if (t <= t1) a.logm[(qrow0 + g) * S + t] = Lr > 0.f ? (M + __log2f(Lr)) * kLn2f : -INFINITY;
+          const int head = FUTURE ? g : ra / NQ;
+          if (t <= t1)
+            a.out[(size_t)(qrow0 + head) * S + t] = Lr > 0.f ? (M + __log2f(Lr)) * kLn2f : -INFINITY;
         }
         m = -INFINITY;
         l = 0.f;
+        ++g;
+        b = 0;
       }
     }
   }
   fence_before();
   __syncthreads();
   if (warp == T6_MMA_WARP) tmem_dealloc(tmem, 512);
+}
+
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
+                                  const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
+                                  const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+// [heads][S][128] bf16, boxes of 64 columns x `rows` rows of one head
+cudaError_t encode_heads(CUtensorMap* map, const void* base, long long heads, int S, int rows) {
+  static const EncodeTiledFn fn = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) !=
+            cudaSuccess || q != cudaDriverEntryPointSuccess)
+      p = nullptr;
+    return reinterpret_cast<EncodeTiledFn>(p);
+  }();
+  if (!fn) return cudaErrorNotSupported;
+  cuuint64_t dims[3] = {128, (cuuint64_t)S, (cuuint64_t)heads};
+  cuuint64_t strides[2] = {256, (cuuint64_t)S * 256};
+  cuuint32_t box[3] = {64, (cuuint32_t)rows, 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+template <int G, bool FUTURE>
+cudaError_t launch_lse_t5(const void* Q, const void* K, const LseArgs& a, int n_pairs, cudaStream_t stream) {
+  constexpr int NQ = FUTURE ? T6_ROWS : T6_ROWS / G;
+  CUtensorMap mq, mk;
+  // rows and columns: (keys, queries) of the future pass, (queries, keys) of the normalisers
+  cudaError_t e = encode_heads(&mq, Q, (long long)n_pairs * G, a.S, FUTURE ? T6_BN : std::min(T6_HALF, NQ));
+  if (e == cudaSuccess) e = encode_heads(&mk, K, n_pairs, a.S, T6_HALF);
+  if (e == cudaSuccess) e = raise_smem_limit(lse_t5_kernel<G, FUTURE>, T6_SMEM);
+  if (e != cudaSuccess) return e;
+  lse_t5_kernel<G, FUTURE><<<(unsigned)n_pairs * ((a.S + NQ - 1) / NQ), T6_THREADS, T6_SMEM, stream>>>(
+      FUTURE ? mk : mq, FUTURE ? mq : mk, a);
+  return cudaGetLastError();
+}
+
+template <bool FUTURE>
+cudaError_t dispatch_lse_t5(const void* Q, const void* K, const LseArgs& a, int G, int n_pairs, cudaStream_t stream) {
+  if (G == 4) return launch_lse_t5<4, FUTURE>(Q, K, a, n_pairs, stream);
+  if (G == 2) return launch_lse_t5<2, FUTURE>(Q, K, a, n_pairs, stream);
+  return launch_lse_t5<1, FUTURE>(Q, K, a, n_pairs, stream);
 }
 
 // ---------------------------------------------------------------- aggregation
@@ -695,6 +790,13 @@ __global__ void aggregate_kernel(AggArgs a) {
 
 }  // namespace
 
+// Causal normalisers of bf16 prompts with d = 128 (d and dtype checked by the caller).
+cudaError_t launch_causal_lse_t5(const void* Q, const void* K, const int32_t* len, int n_seq, int H, int G,
+                                 int S, float* lse, int32_t* err, cudaStream_t stream) {
+  const LseArgs a{nullptr, len, lse, n_seq * H, H, S, 0, 0, kLog2e / sqrtf(128.f), err};
+  return dispatch_lse_t5<false>(Q, K, a, G, n_seq * H, stream);
+}
+
 cudaError_t launch_future_target(const void* Q, const void* K, const float* lse, const int32_t* len,
                                  int n_seq, int H, int G, int d, int S, int w, int la, int dtype,
                                  float* logm, float* target, int agg, int count_norm, float eps,
@@ -707,18 +809,8 @@ cudaError_t launch_future_target(const void* Q, const void* K, const float* lse,
     return e && e[0] == '1';
   }();
   if (dtype == KVPOP_BF16 && d == 128 && !mma_sync) {
-    dim3 grid((S + T6_ROWS - 1) / T6_ROWS, n_pairs);
-    cudaError_t e = cudaSuccess;
-    if (G == 4) {
-      e = raise_smem_limit(target_t5_kernel<4>, T6_SMEM);
-      if (e == cudaSuccess) target_t5_kernel<4><<<grid, T6_THREADS, T6_SMEM, stream>>>(a);
-    } else if (G == 2) {
-      e = raise_smem_limit(target_t5_kernel<2>, T6_SMEM);
-      if (e == cudaSuccess) target_t5_kernel<2><<<grid, T6_THREADS, T6_SMEM, stream>>>(a);
-    } else {
-      e = raise_smem_limit(target_t5_kernel<1>, T6_SMEM);
-      if (e == cudaSuccess) target_t5_kernel<1><<<grid, T6_THREADS, T6_SMEM, stream>>>(a);
-    }
+    const LseArgs la_{lse, len, logm, n_pairs, H, S, w, la, a.kscale, err};
+    cudaError_t e = dispatch_lse_t5<true>(Q, K, la_, G, n_pairs, stream);
     if (e != cudaSuccess) return e;
   } else if (dtype == KVPOP_BF16) {
     const size_t smem = d == 128 ? TgP<128>::SMEM : TgP<64>::SMEM;
