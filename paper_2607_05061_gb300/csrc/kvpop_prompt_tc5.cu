@@ -146,46 +146,57 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
       cp_wait<0>();
     } else if (warp == T5_MMA_WARP) {
       // ---------------------------------------------------------------- MMA issue
-      if (lane == 0) {
-        const uint32_t idS = idesc_bf16(128, T5_BN, 0);
-        const uint32_t idO = idesc_bf16(128, 128, 1);
-        bool ok = mbar_wait(bar(B_QFULL), 0, a.err, T5ERR_WAIT);
-        if (ok) fence_async_smem();
-        auto issue_s = [&](int j) {
-          const int st = j % ST;
-          if (!ok || !(ok = mbar_wait(bar(B_FULL + st), (j / ST) & 1, a.err, T5ERR_WAIT))) return;
-          fence_async_smem();
-          fence_after();
-          const uint32_t kb = sb + OFF_KV + st * 2 * KVB;
+      // all lanes run the loop, one issues (see elect_one)
+      const uint32_t idS = idesc_bf16(128, T5_BN, 0);
+      const uint32_t idO = idesc_bf16(128, 128, 1);
+      const bool lead = elect_one();
+      const uint64_t qd0 = kmajor_desc(sb + OFF_Q, T5_HALF, 0), kd0 = kmajor_desc(sb + OFF_KV, T5_BN, 0);
+      const uint64_t pd0 = kmajor_desc(sb + L::OFF_P, T5_HALF, 0), vd0 = mnmajor_desc(sb + OFF_KV + KVB, T5_BN, 0);
+      bool ok = __all_sync(0xffffffffu, mbar_wait(bar(B_QFULL), 0, a.err, T5ERR_WAIT));
+      if (ok) fence_async_smem();
+      auto issue_s = [&](int j) {
+        const int st = j % ST;
+        ok = ok && mbar_wait(bar(B_FULL + st), (j / ST) & 1, a.err, T5ERR_WAIT);
+        if (!(ok = __all_sync(0xffffffffu, ok))) return;
+        fence_async_smem();
+        fence_after();
+        if (lead) {
+          const uint64_t kd = desc_at(kd0, st * 2 * KVB);
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
             const uint32_t dS = tmem + 256 + h * 128 + (uint32_t)(j & 1) * T5_BN;
+            const uint64_t qd = desc_at(qd0, h * QB);
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks)
-              mma_bf16(dS, kmajor_desc(sb + OFF_Q + h * QB, T5_HALF, ks), kmajor_desc(kb, T5_BN, ks),
-                       idS, ks > 0);
+              mma_bf16(dS, kmajor_step(qd, T5_HALF, ks), kmajor_step(kd, T5_BN, ks), idS, ks > 0);
             commit(bar(B_SFULL + 2 * h + (j & 1)));
           }
-        };
-        issue_s(0);
-        if (nblk > 1) issue_s(1);
-        for (int j = 0; j < nblk && ok; ++j) {
-          const int st = j % ST;
-          const uint32_t vb = sb + OFF_KV + st * 2 * KVB + KVB;
+        }
+        __syncwarp();
+      };
+      issue_s(0);
+      if (nblk > 1) issue_s(1);
+      for (int j = 0; j < nblk && ok; ++j) {
+        const int st = j % ST;
+        const uint64_t vd = desc_at(vd0, st * 2 * KVB);
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            if (!(ok = mbar_wait(bar(B_PFULL + 2 * h + (j & 1)), (j >> 1) & 1, a.err, T5ERR_WAIT))) break;
-            fence_after();
+        for (int h = 0; h < 2; ++h) {
+          ok = ok && mbar_wait(bar(B_PFULL + 2 * h + (j & 1)), (j >> 1) & 1, a.err, T5ERR_WAIT);
+          if (!(ok = __all_sync(0xffffffffu, ok))) break;
+          fence_after();
+          if (lead) {
+            const uint64_t pd = desc_at(pd0, h * PB);
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)
-              mma_bf16(tmem + h * 128, kmajor_desc(sb + L::OFF_P + h * PB, T5_HALF, kk),
-                       mnmajor_desc(vb, T5_BN, kk), idO, (j > 0 || kk > 0));
+              mma_bf16(tmem + h * 128, kmajor_step(pd, T5_HALF, kk), desc_at(vd, kk * 16 * 128), idO,
+                       (j > 0 || kk > 0));
             commit(bar(B_ODONE + h));
+            if (h == 1) commit(bar(B_EMPTY + st));
           }
-          if (!ok) break;
-          commit(bar(B_EMPTY + st));
-          if (j + 2 < nblk) issue_s(j + 2);
+          __syncwarp();
         }
+        if (!ok) break;
+        if (j + 2 < nblk) issue_s(j + 2);
       }
       __syncwarp();
     } else {

@@ -383,35 +383,42 @@ __global__ void __launch_bounds__(TgP<HD>::THREADS, 1) target_tc_kernel(TargetAr
 //    head its rows q >= t0 + w are streamed, with -log2(e) LSE_d added per column;
 //  * causal normalisers (App. D.1): rows are the 256 (head, query) pairs of 256 / G queries, the
 //    keys 0 .. q1 are streamed once for all of them.
-// Both operands come by TMA (128-byte swizzle; rows past the sequence read as zeros).  One
-// thread issues the copies and one the MMAs (M = 128, N = 128), per 128-row half into one of
-// two tensor-memory buffers; 16 softmax warps take 32 rows x 64 columns of every block apiece.
-// The tensor unit (64 clocks per MMA) and the exponentials (32 per clock) need about 1024
-// clocks of a 256 x 128 block each; what is paid is the issue slots of the softmax warps, so
-// barriers are arrived at once per warp and a warp holds its whole part in registers.
-// Blocks: longest tiles first over all pairs (tiles of one pair
-// after the other left the last pair's longest tile to the end: 1363 us for the future pass of
-// 8 heads x 16384 tokens, 4 query heads each, T6_SWAP_US us this way).
+// The rows sit in tensor memory as the MMA's A operand; the streamed operand comes by TMA
+// (128-byte swizzle; rows past the sequence read as zeros).  One warp issues the MMAs (M = 128,
+// N = 128), the tiles (block, 128-row half) taking three S buffers in turn; 16 softmax warps take
+// 32 rows x 64 columns of every block apiece.  A 256 x 128 block needs 1024 clocks of the tensor
+// unit (64 per MMA) and 1024 of the exponential unit (32 per clock); the softmax warps' code sets
+// the pace, about 1500 clocks (causal) and 2000 (future, which also reads a normaliser per
+// column).  What paid: barriers arrived at once per warp, a warp's whole part in registers
+// before its exponentials (the S buffer is free at once), and the MMA warp's operands kept
+// warp-uniform (see elect_one; 945 -> 815 us).  8 heads x 16384 tokens, 4 query heads each:
+// causal 794 us, against 1354 with 64-key blocks in the prompt kernel; future 980 us, against
+// 1363 with copies by cp.async, one arrival per thread and the rows in shared memory.  Measured
+// and not kept: a cluster of two CTAs sharing the streamed blocks by multicast (843 / 1075 us).
+// Blocks: longest tiles first over all pairs (tiles of one pair after the other left the last
+// pair's longest tile to the end).
 constexpr int T6_HALF = 128;
 constexpr int T6_ROWS = 2 * T6_HALF;            // rows per CTA
 constexpr int T6_BN = 128;                      // columns per block (MMA N)
-constexpr int T6_ST = 4;                        // column-block stages
+constexpr int T6_ST = 6;                        // column-block stages
 constexpr int T6_SOFT = 16;                     // warps 0-15 softmax, 16 MMA, 17 copies
 constexpr int T6_MMA_WARP = T6_SOFT;
 constexpr int T6_THREADS = 32 * (T6_SOFT + 2);
-constexpr int T6_AB = T6_HALF * 256;            // row tile of one half, bytes
 constexpr int T6_QB = T6_BN * 256;              // column block, bytes
-constexpr int T6_OFF_Q = 2 * T6_AB;
-constexpr int T6_OFF_LSE = T6_OFF_Q + T6_ST * T6_QB;
+constexpr int T6_OFF_LSE = T6_ST * T6_QB;
 constexpr int T6_OFF_BAR = T6_OFF_LSE + T6_ST * T6_BN * 4;
 constexpr int T6_OFF_TMEM = T6_OFF_BAR + 8 * 32;
 constexpr int T6_OFF_PX = T6_OFF_TMEM + 16;      // [2 head parity][2 halves][128 rows][m, l, seq, -]
 constexpr int T6_SMEM = T6_OFF_PX + 2 * 2 * T6_HALF * 16 + 1024;   // 1024: swizzle atom alignment
-constexpr int T6_FULL = 0, T6_EMPTY = T6_ST, T6_SFULL = 2 * T6_ST, T6_PFULL = 2 * T6_ST + 4,
-              T6_AFULL = 2 * T6_ST + 8;
+constexpr int T6_FULL = 0, T6_EMPTY = T6_ST, T6_SFULL = 2 * T6_ST, T6_PFULL = 2 * T6_ST + 3,
+              T6_AFULL = 2 * T6_ST + 6;
+// tensor memory: the row tiles of the two halves (64 columns each, two bf16 per word), then
+// three S buffers that the tiles (block, half) take in turn
+constexpr int T6_TM_S = 128;
 enum : int { T6ERR_WAIT = 22 };
 
 struct LseArgs {
+  const bf16* A;             // row operand: keys (FUTURE) or queries, [heads][S][128]
   const float* lse;          // FUTURE: [n][H*G][S] natural log
   const int32_t* len;        // [n] or nullptr
   float* out;                // [n][H*G][S]
@@ -429,14 +436,12 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
-// mapA: boxes of 64 columns x (FUTURE: 128, else min(128, 256 / G)) rows of the row operand;
-// mapB: 64 columns x 128 rows of the streamed one.  Both maps are [heads][S][128].
+// map: boxes of 64 columns x 128 rows of the streamed operand, [heads][S][128].
 template <int G, bool FUTURE>
 __global__ void __launch_bounds__(T6_THREADS, 1)
-    lse_t5_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, LseArgs a) {
+    lse_t5_kernel(const __grid_constant__ CUtensorMap map, LseArgs a) {
   using namespace tc05;
   constexpr int NQ = FUTURE ? T6_ROWS : T6_ROWS / G;      // positions of a tile
-  constexpr int ABOX = FUTURE ? T6_HALF : (NQ < T6_HALF ? NQ : T6_HALF);
   extern __shared__ unsigned char sm6_raw[];
   unsigned char* sm6 = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(sm6_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t sb = smem_u32(sm6);
@@ -467,16 +472,15 @@ __global__ void __launch_bounds__(T6_THREADS, 1)
       mbar_init(bar(T6_FULL + i), FUTURE ? 2 : 1);         // the copies, and the normalisers' warp
       mbar_init(bar(T6_EMPTY + i), FUTURE ? 1 + T6_SOFT : 1);   // MMA commit, normalisers read
     }
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < 3; ++i) {
       mbar_init(bar(T6_SFULL + i), 1);
       mbar_init(bar(T6_PFULL + i), T6_SOFT / 2);
     }
-    mbar_init(bar(T6_AFULL), 1);
+    mbar_init(bar(T6_AFULL), T6_SOFT / 2);
     mbar_fence_init();
-    // the softmax halves' exchange slots start with no head done
-    int* px = reinterpret_cast<int*>(sm6 + T6_OFF_PX);
-    for (int i = 0; i < 2 * 2 * T6_HALF; ++i) px[4 * i + 2] = 0;
   }
+  // the softmax halves' exchange slots start with no head done
+  for (int i = tid; i < 2 * 2 * T6_HALF; i += T6_THREADS) reinterpret_cast<int*>(sm6 + T6_OFF_PX)[4 * i + 2] = 0;
   if (warp == T6_MMA_WARP) tmem_alloc(sb + T6_OFF_TMEM, 512);
   fence_before();
   __syncthreads();
@@ -484,15 +488,6 @@ __global__ void __launch_bounds__(T6_THREADS, 1)
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(sm6 + T6_OFF_TMEM);
   if (warp == T6_MMA_WARP + 1) {
     // ---------------------------------------------------------------- copies
-    if (lane == 0) {
-      mbar_arrive_expect_tx(bar(T6_AFULL), 2 * T6_AB);
-      for (int r0 = 0; r0 < T6_ROWS; r0 += ABOX) {
-        const int z = FUTURE ? pair : qrow0 + r0 / NQ, y = t0 + (FUTURE ? r0 : r0 % NQ);
-        const uint32_t dst = sb + (r0 >> 7) * T6_AB + (r0 & 127) * 128;
-        tma_load_3d(dst, &mapA, 0, y, z, bar(T6_AFULL));
-        tma_load_3d(dst + T6_HALF * 128, &mapA, 64, y, z, bar(T6_AFULL));
-      }
-    }
     int j = 0;
     for (; j < total; ++j) {
       const int st = j % T6_ST;
@@ -500,11 +495,11 @@ __global__ void __launch_bounds__(T6_THREADS, 1)
       if (!__all_sync(0xffffffffu, ok)) break;
       const int g = FUTURE ? j / nblk : 0, d0 = d_lo + (j - g * nblk) * T6_BN;
       if (lane == 0) {
-        const uint32_t qd = sb + T6_OFF_Q + st * T6_QB;
+        const uint32_t qd = sb + st * T6_QB;
         const int z = FUTURE ? qrow0 + g : pair;
         mbar_arrive_expect_tx(bar(T6_FULL + st), T6_QB);
-        tma_load_3d(qd, &mapB, 0, d0, z, bar(T6_FULL + st));
-        tma_load_3d(qd + T6_BN * 128, &mapB, 64, d0, z, bar(T6_FULL + st));
+        tma_load_3d(qd, &map, 0, d0, z, bar(T6_FULL + st));
+        tma_load_3d(qd + T6_BN * 128, &map, 64, d0, z, bar(T6_FULL + st));
       }
       if (FUTURE) {
         // the block's normalisers, stored once as -log2(e) LSE_d
@@ -520,41 +515,48 @@ __global__ void __launch_bounds__(T6_THREADS, 1)
       }
     }
     // every copy has landed before the CTA ends (the waiting roles may have given up)
-    if (lane == 0) {
-      mbar_wait(bar(T6_AFULL), 0, a.err, T6ERR_WAIT);
+    if (lane == 0)
       for (int k = max(0, j - T6_ST); k < j; ++k)
         mbar_wait(bar(T6_FULL + k % T6_ST), (k / T6_ST) & 1, a.err, T6ERR_WAIT);
-    }
     __syncwarp();
   } else if (warp == T6_MMA_WARP) {
     // ---------------------------------------------------------------- MMA issue
-    if (lane == 0) {
-      const uint32_t idS = idesc_bf16(128, T6_BN, 0);
-      bool ok = mbar_wait(bar(T6_AFULL), 0, a.err, T6ERR_WAIT);
-      for (int j = 0; j < total && ok; ++j) {
-        const int st = j % T6_ST, b2 = j & 1;
-        if (!(ok = mbar_wait(bar(T6_FULL + st), (j / T6_ST) & 1, a.err, T6ERR_WAIT))) break;
-        fence_after();
-        const uint32_t qb = sb + T6_OFF_Q + st * T6_QB;
+    const uint32_t idS = idesc_bf16(128, T6_BN, 0);
+    const bool lead = elect_one();
+    const uint64_t bd0 = kmajor_desc(sb, T6_BN, 0);
+    bool ok = mbar_wait(bar(T6_AFULL), 0, a.err, T6ERR_WAIT);
+    int sbuf = 0;                                   // S buffer of the tile and its use so far
+    uint32_t use = 0;
+    for (int j = 0; j < total; ++j) {
+      const int st = j % T6_ST;
+      ok = ok && mbar_wait(bar(T6_FULL + st), (j / T6_ST) & 1, a.err, T6ERR_WAIT);
+      if (!__all_sync(0xffffffffu, ok)) break;
+      fence_after();
+      const uint64_t bd = desc_at(bd0, st * T6_QB);
 #pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-          // the softmax half must be done with S_{j-2} before its buffer is rewritten
-          if (j >= 2 && !(ok = mbar_wait(bar(T6_PFULL + 2 * hh + b2), ((j - 2) >> 1) & 1, a.err, T6ERR_WAIT)))
-            break;
-          fence_after();
-          const uint32_t dS = tmem + hh * 256 + (uint32_t)b2 * T6_BN;
+      for (int hh = 0; hh < 2; ++hh) {
+        // the warps of the buffer's last tile must have it in registers
+        if (use > 0) ok = ok && mbar_wait(bar(T6_PFULL + sbuf), (use - 1) & 1, a.err, T6ERR_WAIT);
+        if (!__all_sync(0xffffffffu, ok)) break;
+        fence_after();
+        if (lead) {
+          const uint32_t dS = tmem + T6_TM_S + (uint32_t)sbuf * T6_BN;
 #pragma unroll
           for (int ks = 0; ks < 8; ++ks)
-            mma_bf16(dS, kmajor_desc(sb + hh * T6_AB, T6_HALF, ks), kmajor_desc(qb, T6_BN, ks), idS, ks > 0);
-          commit(bar(T6_SFULL + 2 * hh + b2));
+            mma_bf16_ts(dS, tmem + hh * 64 + ks * 8, kmajor_step(bd, T6_BN, ks), idS, ks > 0);
+          commit(bar(T6_SFULL + sbuf));
+          if (hh == 1) commit(bar(T6_EMPTY + st));
         }
-        if (!ok) break;
-        commit(bar(T6_EMPTY + st));
+        __syncwarp();
+        if (++sbuf == 3) {
+          sbuf = 0;
+          ++use;
+        }
       }
-      // the last stage's release (the commit and the softmax) has landed before the CTA ends
-      if (ok && total > 0)
-        mbar_wait(bar(T6_EMPTY + (total - 1) % T6_ST), ((total - 1) / T6_ST) & 1, a.err, T6ERR_WAIT);
     }
+    // every MMA has completed (the last stage's release) before the CTA ends
+    if (__all_sync(0xffffffffu, ok) && total > 0)
+      mbar_wait(bar(T6_EMPTY + (total - 1) % T6_ST), ((total - 1) / T6_ST) & 1, a.err, T6ERR_WAIT);
     __syncwarp();
   } else {
     // ---------------------------------------------------------------- softmax rows
@@ -567,28 +569,55 @@ __global__ void __launch_bounds__(T6_THREADS, 1)
     const int t = t0 + (FUTURE ? ra : ra % NQ);            // the row's position
     const int lo = FUTURE ? t + w : 0;                     // columns the row takes: lo .. hi
     const int hi = t > t1 ? -1 : FUTURE ? future_hi(t, L, w, la) : t;
-    const uint32_t tS = tmem + ((uint32_t)((warp & 3) * 32) << 16) + hh * 256 + 64 * cs;
+    const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    const uint32_t tS = tl + T6_TM_S + 64 * cs;
     const float* nlS = reinterpret_cast<const float*>(sm6 + T6_OFF_LSE) + 64 * cs;   // -log2(e) LSE_d
     float* pxs = reinterpret_cast<float*>(sm6 + T6_OFF_PX);
     const uint64_t cc = f2_pack(a.scale, a.scale);
+    if (cs == 0) {
+      // the row into tensor memory as the MMA's A operand (zeros past the tile)
+      const bf16* src = a.A + ((size_t)(FUTURE ? pair : qrow0 + ra / NQ) * S + (t <= t1 ? t : t0)) * 128;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        float v[32];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float4 x = t <= t1 ? __ldg(reinterpret_cast<const float4*>(src + 64 * c) + i)
+                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+          v[4 * i] = x.x; v[4 * i + 1] = x.y; v[4 * i + 2] = x.z; v[4 * i + 3] = x.w;
+        }
+        tmem_st32(tl + hh * 64 + c * 32, v);
+      }
+      tmem_wait_st();
+      fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(T6_AFULL));
+    }
     float m = -INFINITY, l = 0.f;
     int g = 0, b = 0;
+    int sbuf = hh;                                   // S buffer of tile 2 j + hh, its phase
+    uint32_t ph = 0;
     for (int j = 0; j < total; ++j) {
-      const int st = j % T6_ST, b2 = j & 1;
+      const int st = j % T6_ST;
       const int e0 = d_lo + b * T6_BN + 64 * cs;
-      bool ok = mbar_wait(bar(T6_SFULL + 2 * hh + b2), (j >> 1) & 1, a.err, T6ERR_WAIT);
+      bool ok = mbar_wait(bar(T6_SFULL + sbuf), ph, a.err, T6ERR_WAIT);
       // the stage's normalisers (complete long before S; the wait orders their reads)
       if (FUTURE) ok = ok && mbar_wait(bar(T6_FULL + st), (j / T6_ST) & 1, a.err, T6ERR_WAIT);
       if (!__all_sync(0xffffffffu, ok)) break;
       fence_after();
       float s[2][32];
-      tmem_ld32(tS + b2 * T6_BN, s[0]);
-      tmem_ld32(tS + b2 * T6_BN + 32, s[1]);
+      tmem_ld32(tS + sbuf * T6_BN, s[0]);
+      tmem_ld32(tS + sbuf * T6_BN + 32, s[1]);
       tmem_wait_ld();
       // the warp's part of the S buffer is in registers: the MMA may overwrite it
       fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar(T6_PFULL + 2 * hh + b2));
+      if (lane == 0) mbar_arrive(bar(T6_PFULL + sbuf));
+      sbuf += 2;
+      if (sbuf >= 3) {
+        sbuf -= 3;
+        ph ^= 1;
+      }
       // some row of the tile ends (or begins) inside these columns
       const bool masked = FUTURE ? (e0 < t1 + w || e0 + 63 > d_hi || (la > 0 && e0 + 63 > t0 + w + la))
                                  : e0 + 63 > t0;
@@ -727,16 +756,16 @@ cudaError_t encode_heads(CUtensorMap* map, const void* base, long long heads, in
 }
 
 template <int G, bool FUTURE>
-cudaError_t launch_lse_t5(const void* Q, const void* K, const LseArgs& a, int n_pairs, cudaStream_t stream) {
+cudaError_t launch_lse_t5(const void* Q, const void* K, LseArgs a, int n_pairs, cudaStream_t stream) {
   constexpr int NQ = FUTURE ? T6_ROWS : T6_ROWS / G;
-  CUtensorMap mq, mk;
   // rows and columns: (keys, queries) of the future pass, (queries, keys) of the normalisers
-  cudaError_t e = encode_heads(&mq, Q, (long long)n_pairs * G, a.S, FUTURE ? T6_BN : std::min(T6_HALF, NQ));
-  if (e == cudaSuccess) e = encode_heads(&mk, K, n_pairs, a.S, T6_HALF);
+  a.A = static_cast<const bf16*>(FUTURE ? K : Q);
+  CUtensorMap map;
+  cudaError_t e = encode_heads(&map, FUTURE ? Q : K, (long long)n_pairs * (FUTURE ? G : 1), a.S, T6_BN);
   if (e == cudaSuccess) e = raise_smem_limit(lse_t5_kernel<G, FUTURE>, T6_SMEM);
   if (e != cudaSuccess) return e;
-  lse_t5_kernel<G, FUTURE><<<(unsigned)n_pairs * ((a.S + NQ - 1) / NQ), T6_THREADS, T6_SMEM, stream>>>(
-      FUTURE ? mk : mq, FUTURE ? mq : mk, a);
+  lse_t5_kernel<G, FUTURE><<<(unsigned)n_pairs * ((a.S + NQ - 1) / NQ), T6_THREADS, T6_SMEM, stream>>>(map,
+                                                                                                           a);
   return cudaGetLastError();
 }
 
@@ -793,7 +822,7 @@ __global__ void aggregate_kernel(AggArgs a) {
 // Causal normalisers of bf16 prompts with d = 128 (d and dtype checked by the caller).
 cudaError_t launch_causal_lse_t5(const void* Q, const void* K, const int32_t* len, int n_seq, int H, int G,
                                  int S, float* lse, int32_t* err, cudaStream_t stream) {
-  const LseArgs a{nullptr, len, lse, n_seq * H, H, S, 0, 0, kLog2e / sqrtf(128.f), err};
+  const LseArgs a{nullptr, nullptr, len, lse, n_seq * H, H, S, 0, 0, kLog2e / sqrtf(128.f), err};
   return dispatch_lse_t5<false>(Q, K, a, G, n_seq * H, stream);
 }
 
@@ -809,7 +838,7 @@ cudaError_t launch_future_target(const void* Q, const void* K, const float* lse,
     return e && e[0] == '1';
   }();
   if (dtype == KVPOP_BF16 && d == 128 && !mma_sync) {
-    const LseArgs la_{lse, len, logm, n_pairs, H, S, w, la, a.kscale, err};
+    const LseArgs la_{nullptr, lse, len, logm, n_pairs, H, S, w, la, a.kscale, err};
     cudaError_t e = dispatch_lse_t5<true>(Q, K, la_, G, n_pairs, stream);
     if (e != cudaSuccess) return e;
   } else if (dtype == KVPOP_BF16) {

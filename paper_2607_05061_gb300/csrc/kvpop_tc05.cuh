@@ -54,6 +54,31 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b
       "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// the same with A in tensor memory (lane = row, a 32-bit column = two consecutive k)
+__device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc,
+                                            uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// One lane of the (converged) warp.  An MMA warp runs its loop in all lanes and lets this one
+// issue: addresses and descriptors then stay warp-uniform, where a loop inside one lane's branch
+// spends its own issue slots, shared with the other warps, on every operand of every MMA.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+// descriptor of an address `bytes` further (the address field does not carry out of the low word)
+__device__ __forceinline__ uint64_t desc_at(uint64_t d, uint32_t bytes) { return d + (bytes >> 4); }
+// k-step ks of a K-major tile whose first k-step has descriptor d
+__device__ __forceinline__ uint64_t kmajor_step(uint64_t d, int rows, int ks) {
+  return desc_at(d, (uint32_t)((ks >> 2) * rows * 128 + (ks & 3) * 32));
+}
 // arrive once on `bar` when every MMA this thread issued so far has completed
 __device__ __forceinline__ void commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
