@@ -596,44 +596,41 @@ size_t tc_smem(int capA, int capM) {
 }
 
 template <int HD, int G, bool DENSE, bool WANT_Y>
-cudaError_t launch_tc(PromptArgs a, int n_pairs, cudaStream_t stream) {
+cudaError_t launch_tc(PromptArgs a, cudaStream_t stream) {
   using P = TcP<HD, G>;
   if (DENSE) a.capA = a.capM = 0;
   else a.capM = a.s + 2 * P::BM + a.w;
   const size_t smem = tc_smem<HD, G>(a.capA, a.capM);
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  dim3 grid((a.S + P::BM - 1) / P::BM, n_pairs);
-  return launch_cfg(prompt_tc_kernel<HD, G, DENSE, WANT_Y>, grid, P::THREADS, smem, stream, a);
+  return launch_cfg(prompt_tc_kernel<HD, G, DENSE, WANT_Y>, tile_grid(a, P::BM), P::THREADS, smem, stream, a);
 }
 
 template <int HD>
-cudaError_t launch_simt(PromptArgs a, int n_pairs, cudaStream_t stream) {
+cudaError_t launch_simt(PromptArgs a, cudaStream_t stream) {
   a.capM = a.s + 2 * SIMT_BM + a.w;
   const size_t smem = (size_t)(SIMT_NT / 32) * HD * 4 + (SIMT_BM + SIMT_NT / 32 + 2) * 4 +
                       (size_t)(a.capA + a.capM) * 4;
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  dim3 grid((a.S + SIMT_BM - 1) / SIMT_BM, n_pairs);
-  return launch_cfg(prompt_simt_kernel<HD>, grid, SIMT_NT, smem, stream, a);
+  return launch_cfg(prompt_simt_kernel<HD>, tile_grid(a, SIMT_BM), SIMT_NT, smem, stream, a);
 }
 
 // The tiled fp32 kernel where its lists fit beside the tiles (up to about 30000 entries), the
 // one-warp-per-row kernel beyond.
 template <int HD, int G, bool DENSE>
-cudaError_t launch_f32(PromptArgs a, int n_pairs, cudaStream_t stream) {
+cudaError_t launch_f32(PromptArgs a, cudaStream_t stream) {
   constexpr int BM = PF_ROWS / G;
   PromptArgs b = a;
   if (DENSE) b.capA = b.capM = 0;
   else b.capM = b.s + 2 * BM + b.w;
   const size_t smem = ((size_t)PfP<HD>::OFF_LIST + b.capA + b.capM) * 4;
-  if (!DENSE && smem > 227 * 1024) return launch_simt<HD>(a, n_pairs, stream);
-  return launch_cfg(prompt_f32_kernel<HD, G, DENSE>, dim3((a.S + BM - 1) / BM, n_pairs), PF_NT, smem,
-                    stream, b);
+  if (!DENSE && smem > 227 * 1024) return launch_simt<HD>(a, stream);
+  return launch_cfg(prompt_f32_kernel<HD, G, DENSE>, tile_grid(a, BM), PF_NT, smem, stream, b);
 }
 
 }  // namespace
 
 bool prompt_t5_ok(int d, int G, int s, int w, int k);
-cudaError_t launch_prompt_t5(const prompt::PromptArgs& a, int n_pairs, int G, cudaStream_t stream);
+cudaError_t launch_prompt_t5(const prompt::PromptArgs& a, int G, cudaStream_t stream);
 cudaError_t launch_causal_lse_t5(const void* Q, const void* K, const int32_t* len, int n_seq, int H, int G,
                                  int S, float* lse, int32_t* err, cudaStream_t stream);   // kvpop_target.cu
 
@@ -649,26 +646,26 @@ bool use_t5(int dtype, int d, int G, int s, int w, int k) {
 }
 
 template <bool DENSE, bool WANT_Y>
-cudaError_t dispatch(const PromptArgs& a, int n_pairs, int dtype, int d, int G, cudaStream_t stream) {
-  if (!DENSE && use_t5(dtype, d, G, a.s, a.w, a.capA - a.s)) return launch_prompt_t5(a, n_pairs, G, stream);
+cudaError_t dispatch(const PromptArgs& a, int dtype, int d, int G, cudaStream_t stream) {
+  if (!DENSE && use_t5(dtype, d, G, a.s, a.w, a.capA - a.s)) return launch_prompt_t5(a, G, stream);
   if (dtype == KVPOP_BF16) {
     if (d == 128) {
-      if (G == 4) return launch_tc<128, 4, DENSE, WANT_Y>(a, n_pairs, stream);
-      if (G == 2) return launch_tc<128, 2, DENSE, WANT_Y>(a, n_pairs, stream);
-      return launch_tc<128, 1, DENSE, WANT_Y>(a, n_pairs, stream);
+      if (G == 4) return launch_tc<128, 4, DENSE, WANT_Y>(a, stream);
+      if (G == 2) return launch_tc<128, 2, DENSE, WANT_Y>(a, stream);
+      return launch_tc<128, 1, DENSE, WANT_Y>(a, stream);
     }
-    if (G == 4) return launch_tc<64, 4, DENSE, WANT_Y>(a, n_pairs, stream);
-    if (G == 2) return launch_tc<64, 2, DENSE, WANT_Y>(a, n_pairs, stream);
-    return launch_tc<64, 1, DENSE, WANT_Y>(a, n_pairs, stream);
+    if (G == 4) return launch_tc<64, 4, DENSE, WANT_Y>(a, stream);
+    if (G == 2) return launch_tc<64, 2, DENSE, WANT_Y>(a, stream);
+    return launch_tc<64, 1, DENSE, WANT_Y>(a, stream);
   }
   if (d == 128) {
-    if (G == 4) return launch_f32<128, 4, DENSE>(a, n_pairs, stream);
-    if (G == 2) return launch_f32<128, 2, DENSE>(a, n_pairs, stream);
-    return launch_f32<128, 1, DENSE>(a, n_pairs, stream);
+    if (G == 4) return launch_f32<128, 4, DENSE>(a, stream);
+    if (G == 2) return launch_f32<128, 2, DENSE>(a, stream);
+    return launch_f32<128, 1, DENSE>(a, stream);
   }
-  if (G == 4) return launch_f32<64, 4, DENSE>(a, n_pairs, stream);
-  if (G == 2) return launch_f32<64, 2, DENSE>(a, n_pairs, stream);
-  return launch_f32<64, 1, DENSE>(a, n_pairs, stream);
+  if (G == 4) return launch_f32<64, 4, DENSE>(a, stream);
+  if (G == 2) return launch_f32<64, 2, DENSE>(a, stream);
+  return launch_f32<64, 1, DENSE>(a, stream);
 }
 
 }  // namespace
@@ -686,9 +683,9 @@ cudaError_t launch_prompt_attend(const void* Q, const void* K, const void* V, co
                                  int n_seq, int H, int G, int d, int S, int s, int w, int k,
                                  int dtype, float* Y, float* lse, int32_t* err, cudaStream_t stream) {
   if (n_seq <= 0 || S <= 0) return cudaSuccess;
-  PromptArgs a{Q, K, V, rank, tau, order, len, Y, lse, H, G, S, s, w, s + k, 0,
+  PromptArgs a{Q, K, V, rank, tau, order, len, Y, lse, n_seq * H, H, G, S, s, w, s + k, 0,
                1.4426950408889634f / sqrtf((float)d), err};
-  return dispatch<false, true>(a, n_seq * H, dtype, d, G, stream);
+  return dispatch<false, true>(a, dtype, d, G, stream);
 }
 
 cudaError_t launch_causal_lse(const void* Q, const void* K, const int32_t* len, int n_seq, int H,
@@ -696,9 +693,9 @@ cudaError_t launch_causal_lse(const void* Q, const void* K, const int32_t* len, 
                               cudaStream_t stream) {
   if (n_seq <= 0 || S <= 0) return cudaSuccess;
   if (use_t5(dtype, d, G, 0, 1, 0)) return launch_causal_lse_t5(Q, K, len, n_seq, H, G, S, lse, err, stream);
-  PromptArgs a{Q, K, nullptr, nullptr, nullptr, nullptr, len, nullptr, lse, H, G, S, 0, 1, 0, 0,
+  PromptArgs a{Q, K, nullptr, nullptr, nullptr, nullptr, len, nullptr, lse, n_seq * H, H, G, S, 0, 1, 0, 0,
                1.4426950408889634f / sqrtf((float)d), err};
-  return dispatch<true, false>(a, n_seq * H, dtype, d, G, stream);
+  return dispatch<true, false>(a, dtype, d, G, stream);
 }
 
 }  // namespace kvpop

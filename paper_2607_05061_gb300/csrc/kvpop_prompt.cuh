@@ -21,7 +21,7 @@ struct PromptArgs {
   const int32_t* len;        // [n_seq] or nullptr (= S)
   float* Y;                  // [n_seq][H*G][S][d]
   float* lse;                // [n_seq][H*G][S] or nullptr
-  int H, G, S, s, w;
+  int n_pairs, H, G, S, s, w;
   int capA, capM;
   float qscale;              // log2(e) / sqrt(d)
   int32_t* err;              // first-error word or nullptr
@@ -43,18 +43,27 @@ struct TileInfo {
   int nA, nM;
 };
 
+// Pair and queries of a CTA; blocks run over the pairs first, from the last tile down, so the
+// longest tiles of all pairs come first and the launch ends on short ones.
+__device__ __forceinline__ bool tile_bounds(const PromptArgs& a, int BM, TileInfo& ti) {
+  const int tile = blockIdx.x / a.n_pairs;
+  ti.pair = blockIdx.x - tile * a.n_pairs;
+  ti.seq = ti.pair / a.H;
+  ti.h = ti.pair - ti.seq * a.H;
+  ti.L = a.len ? max(0, min(a.len[ti.seq], a.S)) : a.S;
+  ti.q0 = ((int)(gridDim.x / a.n_pairs) - 1 - tile) * BM;
+  if (ti.q0 >= ti.L) return false;
+  ti.q1 = min(ti.q0 + BM - 1, ti.L - 1);
+  return true;
+}
+inline unsigned tile_grid(const PromptArgs& a, int BM) { return (unsigned)a.n_pairs * ((a.S + BM - 1) / BM); }
+
 template <int NT>
 __device__ bool tile_setup(const PromptArgs& a, int BM, int* tauS, int* red, int32_t* posA,
                            int32_t* posM, TileInfo& ti) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int NW = NT / 32;
-  ti.pair = blockIdx.y;
-  ti.seq = ti.pair / a.H;
-  ti.h = ti.pair - ti.seq * a.H;
-  ti.L = a.len ? max(0, min(a.len[ti.seq], a.S)) : a.S;
-  ti.q0 = (gridDim.x - 1 - blockIdx.x) * BM;        // longest tiles first
-  if (ti.q0 >= ti.L) return false;
-  ti.q1 = min(ti.q0 + BM - 1, ti.L - 1);
+  if (!tile_bounds(a, BM, ti)) return false;
   const int nq = ti.q1 - ti.q0 + 1;
   const int32_t* tau = a.tau + (size_t)ti.pair * a.S;
   const int32_t* rank = a.rank + (size_t)ti.pair * a.S;
@@ -173,13 +182,7 @@ __device__ bool tile_setup(const PromptArgs& a, int BM, int* tauS, int* red, int
 // of the tile (list A), q0 + 1 .. q1 only the later ones (list M); a key's
 // list index is its position.
 __device__ __forceinline__ bool dense_setup(const PromptArgs& a, int BM, TileInfo& ti) {
-  ti.pair = blockIdx.y;
-  ti.seq = ti.pair / a.H;
-  ti.h = ti.pair - ti.seq * a.H;
-  ti.L = a.len ? max(0, min(a.len[ti.seq], a.S)) : a.S;
-  ti.q0 = (gridDim.x - 1 - blockIdx.x) * BM;
-  if (ti.q0 >= ti.L) return false;
-  ti.q1 = min(ti.q0 + BM - 1, ti.L - 1);
+  if (!tile_bounds(a, BM, ti)) return false;
   ti.nA = ti.q0 + 1;
   ti.nM = ti.q1 - ti.q0;
   return true;

@@ -20,6 +20,11 @@
 //    running maximum that is only raised when a logit exceeds it by 2^8 (the
 //    row of the accumulator is then rescaled in place), write the bf16
 //    probabilities into the half's swizzled P tile and hand it over.
+// What bounds it is the chain of hand-offs per 64-key block, about 2200 clocks against 1280 of
+// the tensor unit.  One 32768-token prompt of 8 heads (4096 keys a query): 2053 us; 2768 us
+// before the MMA warp's operands were kept warp-uniform (2368), the mask of the blocks that
+// need one was reduced to a run of queries per key and the tiles of all pairs ran longest
+// first; 2 x 8192 tokens with a window of 256: 1034 -> 521 us.
 // Outputs as the other kernels: y in fp32 and the natural-log normaliser.
 // Every wait is bounded; on expiry the kernel records an error code, stops
 // issuing work, lets its copies drain and frees its tensor memory.  Every
@@ -81,6 +86,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
   int* red = reinterpret_cast<int*>(sm5 + L::OFF_RED);
   int32_t* posA = reinterpret_cast<int32_t*>(sm5 + L::OFF_LIST);
   int32_t* posM = posA + a.capA;
+  uint32_t* keepM = reinterpret_cast<uint32_t*>(posM + a.capM);   // [capM + T5_BN]
 
   if (tid == 0) {
     for (int i = 0; i < ST; ++i) {
@@ -89,7 +95,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
     }
     for (int i = 0; i < 4; ++i) {
       mbar_init(bar(B_SFULL + i), 1);
-      mbar_init(bar(B_PFULL + i), 128);
+      mbar_init(bar(B_PFULL + i), T5_HALF / 32);
     }
     mbar_init(bar(B_ODONE + 0), 1);
     mbar_init(bar(B_ODONE + 1), 1);
@@ -99,6 +105,27 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
   if (warp == T5_MMA_WARP) tmem_alloc(sb + L::OFF_TMEM, T5_TMEM_COLS);
   TileInfo ti;
   const bool live = tile_setup<T5_THREADS>(a, BM, tauS, red, posA, posM, ti);
+  if (live) {
+    // Which queries of the tile keep an M entry: a run that starts at the key's own position and
+    // ends where the cutoff falls below its rank (once dropped a key stays dropped), found once
+    // per entry as (first query, number) instead of testing the mask for every row.
+    const int32_t* rank = a.rank + (size_t)ti.pair * a.S;
+    const int nq = ti.q1 - ti.q0 + 1;
+    for (int i = tid; i < ti.nM + T5_BN; i += T5_THREADS) {
+      uint32_t word = 0;                            // past the list: no query
+      if (i < ti.nM) {
+        const int t = posM[i], r = __ldg(rank + t);
+        const int first = max(0, t - ti.q0);
+        int lo = first, hi = nq;                    // the run's end lies in [lo, hi]
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (keep_key(ti.q0 + mid, t, r, tauS[mid], a.s, a.w)) lo = mid + 1; else hi = mid;
+        }
+        word = (uint32_t)first | (uint32_t)(lo - first) << 16;
+      }
+      keepM[i] = word;
+    }
+  }
   fence_before();
   __syncthreads();
   fence_after();
@@ -207,10 +234,8 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
       const int ql = rr / G, g = rr - ql * G;
       const int q = ti.q0 + ql;
       const bool valid = q <= ti.q1;
-      const int tq = tauS[ql];
       const uint32_t trow = (uint32_t)((warp & 3) * 32) << 16;
       const uint32_t tO = tmem + trow + h * 128, tS = tmem + trow + 256 + h * 128;
-      const int32_t* rank = a.rank + pair_off;
       const float c2 = a.qscale;
       float m = -INFINITY, l = 0.f;
       bool ok = true;
@@ -225,16 +250,12 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
         tmem_ld32(tS + b * T5_BN + 32, *reinterpret_cast<float(*)[32]>(s + 32));
         tmem_wait_ld();
         if ((j + 1) * T5_BN > nA) {                 // block holds keys that need the mask
+          const int nf = nA - j * T5_BN;            // entries before it need none
 #pragma unroll
           for (int i = 0; i < 64; ++i) {
-            const int e = j * T5_BN + i;
-            if (e >= nA) {
-              bool kp = false;
-              if (e < nU) {
-                const int t = entry(e);
-                kp = keep_key(q, t, __ldg(rank + t), tq, a.s, a.w);
-              }
-              if (!kp) s[i] = -INFINITY;
+            if (i >= nf) {
+              const uint32_t kw = keepM[i - nf];
+              if ((uint32_t)(ql - (int)(kw & 0xffffu)) >= (kw >> 16)) s[i] = -INFINITY;
             }
           }
         }
@@ -309,7 +330,8 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
         }
         fence_async_smem();
         fence_before();
-        mbar_arrive(bar(B_PFULL + 2 * h + b));
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(B_PFULL + 2 * h + b));
       }
       const size_t row = ((size_t)ti.seq * H * G + (size_t)ti.h * G + g) * S + q;
       if (ok && nblk > 0) {
@@ -342,27 +364,26 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
 
 template <int ST>
 size_t t5_smem(int capA, int capM) {
-  return (size_t)Lay<ST>::OFF_LIST + (size_t)(capA + capM) * 4;
+  return (size_t)Lay<ST>::OFF_LIST + (size_t)(capA + 2 * capM + T5_BN) * 4;
 }
 
 template <int G, int ST>
-cudaError_t launch_t5_st(const PromptArgs& a, int n_pairs, size_t smem, cudaStream_t stream) {
+cudaError_t launch_t5_st(const PromptArgs& a, size_t smem, cudaStream_t stream) {
   constexpr int BM = T5_ROWS / G;
   auto k = prompt_t5_kernel<G, ST>;
   cudaError_t e = raise_smem_limit(k, smem);
   if (e != cudaSuccess) return e;
-  dim3 grid((a.S + BM - 1) / BM, n_pairs);
-  k<<<grid, T5_THREADS, smem, stream>>>(a);
+  k<<<tile_grid(a, BM), T5_THREADS, smem, stream>>>(a);
   return cudaGetLastError();
 }
 
 template <int G>
-cudaError_t launch_t5_g(PromptArgs a, int n_pairs, cudaStream_t stream) {
+cudaError_t launch_t5_g(PromptArgs a, cudaStream_t stream) {
   constexpr int BM = T5_ROWS / G;
   a.capM = a.s + 2 * BM + a.w;
   const size_t s3 = t5_smem<3>(a.capA, a.capM), s2 = t5_smem<2>(a.capA, a.capM);
-  if (s3 <= 227 * 1024) return launch_t5_st<G, 3>(a, n_pairs, s3, stream);
-  if (s2 <= 227 * 1024) return launch_t5_st<G, 2>(a, n_pairs, s2, stream);
+  if (s3 <= 227 * 1024) return launch_t5_st<G, 3>(a, s3, stream);
+  if (s2 <= 227 * 1024) return launch_t5_st<G, 2>(a, s2, stream);
   return cudaErrorInvalidValue;
 }
 
@@ -370,14 +391,14 @@ cudaError_t launch_t5_g(PromptArgs a, int n_pairs, cudaStream_t stream) {
 
 bool prompt_t5_ok(int d, int G, int s, int w, int k) {
   if (d != 128 || !(G == 1 || G == 2 || G == 4)) return false;
-  const long long lists = (long long)s + k + s + 2 * T5_ROWS + w;
+  const long long lists = (long long)s + k + 2 * ((long long)s + 2 * T5_ROWS + w) + T5_BN;
   return Lay<2>::OFF_LIST + 4 * lists <= 227 * 1024;
 }
 
-cudaError_t launch_prompt_t5(const PromptArgs& a, int n_pairs, int G, cudaStream_t stream) {
-  if (G == 4) return launch_t5_g<4>(a, n_pairs, stream);
-  if (G == 2) return launch_t5_g<2>(a, n_pairs, stream);
-  return launch_t5_g<1>(a, n_pairs, stream);
+cudaError_t launch_prompt_t5(const PromptArgs& a, int G, cudaStream_t stream) {
+  if (G == 4) return launch_t5_g<4>(a, stream);
+  if (G == 2) return launch_t5_g<2>(a, stream);
+  return launch_t5_g<1>(a, stream);
 }
 
 }  // namespace kvpop
