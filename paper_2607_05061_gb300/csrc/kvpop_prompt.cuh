@@ -104,37 +104,34 @@ __device__ bool tile_setup(const PromptArgs& a, int BM, int* tauS, int* red, int
     const bool by_rank = order != nullptr && tmax < hi - s;
     const int n_walk = by_rank ? tmax + 1 : hi - s + 1;
     for (int c0 = 0; c0 < n_walk; c0 += NT * EPT) {
-      const int i0 = c0 + tid * EPT;
+      // a warp reads 32 EPT consecutive entries, 32 at a time, and keeps their order
+      const int i0 = c0 + warp * (32 * EPT) + lane;
       int r[EPT], t[EPT];
+      // unconditional loads first (past the end: the last entry again), so all are in flight
+      // together; behind a branch each would wait for the one before
+      const int32_t* list = by_rank ? order : rank + s;
+#pragma unroll
+      for (int e = 0; e < EPT; ++e) t[e] = __ldg(list + min(i0 + 32 * e, n_walk - 1));
 #pragma unroll
       for (int e = 0; e < EPT; ++e) {
-        const int i = i0 + e;
-        if (i >= n_walk) {
-          r[e] = INT_MAX;
-          t[e] = 0;
-        } else if (by_rank) {
-          t[e] = __ldg(order + i);
-          r[e] = (t[e] >= s && t[e] <= hi) ? i : INT_MAX;
+        const int i = i0 + 32 * e;
+        if (by_rank) {
+          r[e] = (i < n_walk && t[e] >= s && t[e] <= hi) ? i : INT_MAX;
         } else {
+          r[e] = i < n_walk ? t[e] : INT_MAX;
           t[e] = s + i;
-          r[e] = __ldg(rank + s + i);
         }
       }
-      int ca = 0, cm = 0;
+      static_assert(NT * EPT < 65536, "two 16-bit counts per word");
+      uint32_t inA[EPT], inM[EPT];
+      int v = 0;                              // the warp's A entries, M entries << 16
 #pragma unroll
       for (int e = 0; e < EPT; ++e) {
-        ca += r[e] <= tmin;
-        cm += (r[e] > tmin) & (r[e] <= tmax);
+        inA[e] = __ballot_sync(0xffffffffu, r[e] <= tmin);
+        inM[e] = __ballot_sync(0xffffffffu, r[e] > tmin && r[e] <= tmax);
+        v += __popc(inA[e]) + (__popc(inM[e]) << 16);
       }
-      static_assert(NT * EPT < 65536, "two 16-bit counts per word");
-      const int v = ca | (cm << 16);        // at most NT * EPT per field
-      int x = v;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-      }
-      if (lane == 31) red[warp] = x;
+      if (lane == 0) red[warp] = v;
       __syncthreads();
       int off = 0, tot = 0;
 #pragma unroll
@@ -143,17 +140,18 @@ __device__ bool tile_setup(const PromptArgs& a, int BM, int* tauS, int* red, int
         if (i < warp) off += y;
         tot += y;
       }
-      const int ex = off + x - v;
-      int ia = nA + (ex & 0xffff), im = nM + (ex >> 16);
+      int ia = nA + (off & 0xffff), im = nM + (off >> 16);
+      const uint32_t lt = (1u << lane) - 1u;
 #pragma unroll
       for (int e = 0; e < EPT; ++e) {
+        const int ja = ia + __popc(inA[e] & lt), jm = im + __popc(inM[e] & lt);
         if (r[e] <= tmin) {
-          if (ia < a.capA) posA[ia] = t[e];
-          ++ia;
+          if (ja < a.capA) posA[ja] = t[e];
         } else if (r[e] <= tmax) {
-          if (im < a.capM) posM[im] = t[e];
-          ++im;
+          if (jm < a.capM) posM[jm] = t[e];
         }
+        ia += __popc(inA[e]);
+        im += __popc(inM[e]);
       }
       nA += tot & 0xffff;
       nM += tot >> 16;

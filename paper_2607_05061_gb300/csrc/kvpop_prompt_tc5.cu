@@ -99,13 +99,25 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
     }
     mbar_init(bar(B_ODONE + 0), 1);
     mbar_init(bar(B_ODONE + 1), 1);
-    mbar_init(bar(B_QFULL), T5_PT);
+    mbar_init(bar(B_QFULL), T5_THREADS);
     mbar_fence_init();
   }
   if (warp == T5_MMA_WARP) tmem_alloc(sb + L::OFF_TMEM, T5_TMEM_COLS);
   TileInfo ti;
+  // the query rows travel while the key lists are built; their arrival is counted below
+  if (tile_bounds(a, BM, ti)) {
+    const bf16* Qb = static_cast<const bf16*>(a.Q) + ((size_t)ti.seq * a.H * G + (size_t)ti.h * G) * a.S * 128;
+    for (int i = tid; i < T5_ROWS * 16; i += T5_THREADS) {
+      const int r = i >> 4, c = i & 15;
+      const int q = ti.q0 + r / G, g = r % G;
+      const bool ok = q <= ti.q1;
+      cp_async16(sb + OFF_Q + (r >> 7) * QB + tile_off(r & 127, c, T5_HALF),
+                 Qb + ((size_t)g * a.S + (ok ? q : ti.q0)) * 128 + c * 8, ok ? 16 : 0);
+    }
+  }
   const bool live = tile_setup<T5_THREADS>(a, BM, tauS, red, posA, posM, ti);
   if (live) {
+    cp_async_arrive_noinc(bar(B_QFULL));            // the barriers are set up: a block sync lies between
     // Which queries of the tile keep an M entry: a run that starts at the key's own position and
     // ends where the cutoff falls below its rank (once dropped a key stays dropped), found once
     // per entry as (first query, number) instead of testing the mask for every row.
@@ -141,17 +153,8 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
     if (warp > T5_MMA_WARP) {
       // ---------------------------------------------------------------- producers
       const int pt = tid - 32 * (T5_MMA_WARP + 1);
-      const bf16* Qb = static_cast<const bf16*>(a.Q) + ((size_t)ti.seq * H * G + (size_t)ti.h * G) * S * 128;
       const bf16* Kp = static_cast<const bf16*>(a.K) + pair_off * 128;
       const bf16* Vp = static_cast<const bf16*>(a.V) + pair_off * 128;
-      for (int i = pt; i < T5_ROWS * 16; i += T5_PT) {
-        const int r = i >> 4, c = i & 15;
-        const int q = ti.q0 + r / G, g = r % G;
-        const bool ok = q <= ti.q1;
-        cp_async16(sb + OFF_Q + (r >> 7) * QB + tile_off(r & 127, c, T5_HALF),
-                   Qb + ((size_t)g * S + (ok ? q : ti.q0)) * 128 + c * 8, ok ? 16 : 0);
-      }
-      cp_async_arrive_noinc(bar(B_QFULL));
       for (int j = 0; j < nblk; ++j) {
         const int st = j % ST;
         if (j >= ST && !mbar_wait(bar(B_EMPTY + st), ((j / ST) - 1) & 1, a.err, T5ERR_WAIT)) break;
@@ -338,25 +341,37 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
         ok = uniform(mbar_wait(bar(B_ODONE + h), (nblk - 1) & 1, a.err, T5ERR_WAIT));
         fence_after();
         if (ok) {
+          // a warp's 32 rows pass through shared memory, so that a store writes one whole row:
+          // half 0 in the query tile (every S is done), half 1, whose last product is the last
+          // of all, in the first K/V stages
           const float inv = 1.f / l;
-          float4* y = reinterpret_cast<float4*>(a.Y + row * 128);
+          const uint32_t tile = sb + (h ? OFF_KV : OFF_Q) + (warp & 3) * (32 * 512);
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             float o[32];
             tmem_ld32(tO + c * 32, o);
             tmem_wait_ld();
-            if (valid) {
 #pragma unroll
-              for (int i = 0; i < 8; ++i)
-                y[c * 8 + i] = make_float4(o[4 * i] * inv, o[4 * i + 1] * inv, o[4 * i + 2] * inv,
-                                           o[4 * i + 3] * inv);
-            }
+            for (int i = 0; i < 8; ++i)
+              *reinterpret_cast<float4*>(sm5 + (tile - sb) + lane * 512 + (((c * 8 + i) ^ lane) << 4)) =
+                  make_float4(o[4 * i] * inv, o[4 * i + 1] * inv, o[4 * i + 2] * inv, o[4 * i + 3] * inv);
+          }
+          __syncwarp();
+          const int r0 = h * T5_HALF + (warp & 3) * 32;
+          float* Yp = a.Y + ((size_t)ti.seq * H * G + (size_t)ti.h * G) * S * 128;
+#pragma unroll 8
+          for (int i = 0; i < 32; ++i) {
+            const int qi = ti.q0 + (r0 + i) / G;
+            if (qi > ti.q1) break;
+            const float4 v = *reinterpret_cast<const float4*>(sm5 + (tile - sb) + i * 512 + ((lane ^ i) << 4));
+            *reinterpret_cast<float4*>(Yp + ((size_t)((r0 + i) % G) * S + qi) * 128 + 4 * lane) = v;
           }
         }
       }
       if (ok && valid && a.lse) a.lse[row] = l > 0.f ? (m + __log2f(l)) * kLn2 : -INFINITY;
     }
   }
+  cp_wait<0>();
   fence_before();
   __syncthreads();
   if (warp == T5_MMA_WARP) tmem_dealloc(tmem, T5_TMEM_COLS);
