@@ -9,9 +9,9 @@
 //    cp.async into 128B-swizzled tiles (2 or 3 stages, as shared memory
 //    allows); completion arrives on the stage's mbarrier asynchronously
 //    (cp.async.mbarrier.arrive.noinc).
-//  * 1 MMA warp: one thread issues, per half, S = Q K^T (M 128, N 64, K 128;
+//  * 1 MMA warp: one lane issues, per half, S = Q K^T (M 128, N 64, K 128;
 //    Q and K K-major) into one of two tensor-memory S buffers, and O += P V
-//    (M 128, N 128, K 64; P K-major from shared memory, V read MN-major straight
+//    (M 128, N 128, K 64; P from tensor memory, V read MN-major straight
 //    from its gathered rows) into the half's tensor-memory accumulator;
 //    tcgen05.commit signals S ready, P consumed and the stage free.  Tensor
 //    memory: O of both halves (256 columns) and their S double buffers (256).
@@ -19,12 +19,17 @@
 //    (32x32b loads), apply the mask on the few blocks that need it, keep a
 //    running maximum that is only raised when a logit exceeds it by 2^8 (the
 //    row of the accumulator is then rescaled in place), write the bf16
-//    probabilities into the half's swizzled P tile and hand it over.
-// What bounds it is the chain of hand-offs per 64-key block, about 2200 clocks against 1280 of
-// the tensor unit.  One 32768-token prompt of 8 heads (4096 keys a query): 2053 us; 2768 us
-// before the MMA warp's operands were kept warp-uniform (2368), the mask of the blocks that
-// need one was reduced to a run of queries per key and the tiles of all pairs ran longest
-// first; 2 x 8192 tokens with a window of 256: 1034 -> 521 us.
+//    probabilities over the row's logits and hand them over.  (S_{j+2} follows
+//    PV_j into the buffer, in the order the MMAs are issued.)
+// What bounds it: the shared-memory bytes of a 64-key block (query tile and keys of S 96 KB,
+// values 32, the gathered rows written 32: 1250 clocks at 128 bytes each) and the tensor unit
+// (1280) are both close to the 1700 clocks it takes; a tile's prologue and epilogue add about
+// 20000.  One 32768-token prompt of 8 heads (4096 keys a query), us: 2768 at first; 2368 with
+// the MMA warp's operands kept warp-uniform; 2053 with the mask reduced to a run of queries per
+// key and the longest tiles of all pairs first; 1967 with the prologue's loads in flight
+// together and the outputs stored as whole rows; 1833 with P in tensor memory instead of a
+// shared tile (64 KB less per block, and a fourth stage).  2 x 8192 tokens with a window of
+// 256: 1034 -> 458.
 // Outputs as the other kernels: y in fp32 and the natural-log normaliser.
 // Every wait is bounded; on expiry the kernel records an error code, stops
 // issuing work, lets its copies drain and frees its tensor memory.  Every
@@ -53,25 +58,23 @@ constexpr float T5_THR = 8.0f;
 
 constexpr int QB = T5_HALF * 256;                // Q tile of one half, bytes
 constexpr int KVB = T5_BN * 256;                 // K (or V) block, bytes
-constexpr int PB = T5_HALF * T5_BN * 2;          // P tile of one half, bytes
 constexpr int OFF_Q = 0;
 constexpr int OFF_KV = OFF_Q + 2 * QB;           // stages of [K | V]
 template <int ST>
 struct Lay {
-  static constexpr int OFF_P = OFF_KV + ST * 2 * KVB;
-  static constexpr int OFF_BAR = OFF_P + 2 * PB;
+  static constexpr int OFF_BAR = OFF_KV + ST * 2 * KVB;
   static constexpr int OFF_TMEM = OFF_BAR + 256;
   static constexpr int OFF_TAU = OFF_TMEM + 16;
   static constexpr int OFF_RED = OFF_TAU + T5_ROWS * 4;
   static constexpr int OFF_LIST = OFF_RED + 16 * 4;
 };
 // barrier indices
-constexpr int B_FULL = 0;          // [3]  producers -> MMA
-constexpr int B_EMPTY = 3;         // [3]  MMA -> producers
-constexpr int B_SFULL = 6;         // [2 halves][2 buffers]  MMA -> softmax
-constexpr int B_PFULL = 10;        // [2][2]  softmax -> MMA
-constexpr int B_ODONE = 14;        // [2]  MMA -> softmax (one per half)
-constexpr int B_QFULL = 16;
+constexpr int B_FULL = 0;          // [4]  producers -> MMA
+constexpr int B_EMPTY = 4;         // [4]  MMA -> producers
+constexpr int B_SFULL = 8;         // [2 halves][2 buffers]  MMA -> softmax
+constexpr int B_PFULL = 12;        // [2][2]  softmax -> MMA
+constexpr int B_ODONE = 16;        // [2]  MMA -> softmax (one per half)
+constexpr int B_QFULL = 18;
 enum : int { T5ERR_WAIT = 21 };
 
 template <int G, int ST>
@@ -181,7 +184,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
       const uint32_t idO = idesc_bf16(128, 128, 1);
       const bool lead = elect_one();
       const uint64_t qd0 = kmajor_desc(sb + OFF_Q, T5_HALF, 0), kd0 = kmajor_desc(sb + OFF_KV, T5_BN, 0);
-      const uint64_t pd0 = kmajor_desc(sb + L::OFF_P, T5_HALF, 0), vd0 = mnmajor_desc(sb + OFF_KV + KVB, T5_BN, 0);
+      const uint64_t vd0 = mnmajor_desc(sb + OFF_KV + KVB, T5_BN, 0);
       bool ok = __all_sync(0xffffffffu, mbar_wait(bar(B_QFULL), 0, a.err, T5ERR_WAIT));
       if (ok) fence_async_smem();
       auto issue_s = [&](int j) {
@@ -215,11 +218,10 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
           if (!(ok = __all_sync(0xffffffffu, ok))) break;
           fence_after();
           if (lead) {
-            const uint64_t pd = desc_at(pd0, h * PB);
+            const uint32_t tP = tmem + 256 + h * 128 + (uint32_t)(j & 1) * T5_BN;
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)
-              mma_bf16(tmem + h * 128, kmajor_step(pd, T5_HALF, kk), desc_at(vd, kk * 16 * 128), idO,
-                       (j > 0 || kk > 0));
+              mma_bf16_ts(tmem + h * 128, tP + 8 * kk, desc_at(vd, kk * 16 * 128), idO, (j > 0 || kk > 0));
             commit(bar(B_ODONE + h));
             if (h == 1) commit(bar(B_EMPTY + st));
           }
@@ -302,36 +304,27 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
         const float sum = ((ps[0] + ps[1]) + (ps[2] + ps[3])) + ((ps[4] + ps[5]) + (ps[6] + ps[7]));
         l = l * alpha + sum;
         m = m_new;
-        if (j >= 1) {
-          // PV_{j-1} must have consumed the P tile (and landed in O) before either changes;
-          // the exponentials above overlap with it
+        if (j >= 1 && __any_sync(0xffffffffu, resc)) {
+          // PV_{j-1} must have landed in O before O changes (PV_{j-2} has: S_j came after it)
           if (!(ok = uniform(mbar_wait(bar(B_ODONE + h), (j - 1) & 1, a.err, T5ERR_WAIT)))) break;
-          if (__any_sync(0xffffffffu, resc)) {
-            fence_after();
-            const float f = resc ? alpha : 1.f;
+          fence_after();
+          const float f = resc ? alpha : 1.f;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              float o[32];
-              tmem_ld32(tO + c * 32, o);
-              tmem_wait_ld();
+          for (int c = 0; c < 4; ++c) {
+            float o[32];
+            tmem_ld32(tO + c * 32, o);
+            tmem_wait_ld();
 #pragma unroll
-              for (int i = 0; i < 32; ++i) o[i] *= f;
-              tmem_st32(tO + c * 32, o);
-            }
-            tmem_wait_st();
+            for (int i = 0; i < 32; ++i) o[i] *= f;
+            tmem_st32(tO + c * 32, o);
           }
         }
-        unsigned char* prow = sm5 + L::OFF_P + h * PB;
+        // the probabilities take the place of their logits, two to a word: the A operand of PV_j
+        float pw[32];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          uint4 v;
-          v.x = pack_bf16(s[8 * c + 0], s[8 * c + 1]);
-          v.y = pack_bf16(s[8 * c + 2], s[8 * c + 3]);
-          v.z = pack_bf16(s[8 * c + 4], s[8 * c + 5]);
-          v.w = pack_bf16(s[8 * c + 6], s[8 * c + 7]);
-          *reinterpret_cast<uint4*>(prow + tile_off(r, c, T5_HALF)) = v;
-        }
-        fence_async_smem();
+        for (int i = 0; i < 32; ++i) pw[i] = __uint_as_float(pack_bf16(s[2 * i], s[2 * i + 1]));
+        tmem_st32(tS + b * T5_BN, pw);
+        tmem_wait_st();
         fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(B_PFULL + 2 * h + b));
@@ -396,7 +389,8 @@ template <int G>
 cudaError_t launch_t5_g(PromptArgs a, cudaStream_t stream) {
   constexpr int BM = T5_ROWS / G;
   a.capM = a.s + 2 * BM + a.w;
-  const size_t s3 = t5_smem<3>(a.capA, a.capM), s2 = t5_smem<2>(a.capA, a.capM);
+  const size_t s4 = t5_smem<4>(a.capA, a.capM), s3 = t5_smem<3>(a.capA, a.capM), s2 = t5_smem<2>(a.capA, a.capM);
+  if (s4 <= 227 * 1024) return launch_t5_st<G, 4>(a, s4, stream);
   if (s3 <= 227 * 1024) return launch_t5_st<G, 3>(a, s3, stream);
   if (s2 <= 227 * 1024) return launch_t5_st<G, 2>(a, s2, stream);
   return cudaErrorInvalidValue;
