@@ -118,15 +118,18 @@ def _ck(status: int, what: str):
 
 
 def _ptr(t) -> Optional[int]:
-    if t is None:
-        return None
-    if isinstance(t, int):
-        return t
-    return t.data_ptr()
+    return t if t is None or isinstance(t, int) else t.data_ptr()
+
+
+# The current stream's handle without a torch.cuda.Stream object around it (a decode step of a
+# small cache takes less time on the GPU than its call takes on the host).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream=None) -> int:
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         stream = torch.cuda.current_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
@@ -196,8 +199,10 @@ class KVpopCache:
         _ck(kvpop_decode_attend(self.handle, _ptr(q), _ptr(out), _stream(stream)), "kvpop_decode_attend")
 
     def step(self, q, k, v, out, override=None, evict_info=None, score_out=None, stream=None):
-        _ck(kvpop_decode_step(self.handle, _ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(override),
-                              _ptr(evict_info), _ptr(score_out), _stream(stream)), "kvpop_decode_step")
+        status = kvpop_decode_step(self.handle, _ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(override),
+                                   _ptr(evict_info), _ptr(score_out), _stream(stream))
+        if status != 0:
+            _ck(status, "kvpop_decode_step")
 
     @property
     def fused_step(self) -> bool:
