@@ -19,6 +19,7 @@
 
 #include "kvpop_evict.cuh"
 #include "kvpop_mma.cuh"
+#include "kvpop_tc05.cuh"
 
 namespace kvpop {
 namespace {
@@ -350,30 +351,43 @@ __global__ void __launch_bounds__(NTM) mlstm_proj_kernel(MProjArgs a) {
   }
 }
 
-// The same projections for bf16 K/V on the tensor cores with fp32 accuracy: x is exact in bf16
-// and every weight is split exactly into three bf16 parts (8 + 8 + 8 bits, W^T stored once per
-// cache), so W x is three products whose terms are exact.  The tensor unit rounds a running sum
-// toward zero; to keep that below the rounding of a chain of fp32 FMAs, each 64 inputs are
-// summed on their own, smallest parts first, and added to the total in fp32.  A CTA takes 128
-// tokens, a warp 16 of them with all columns, so the Hedgehog softmaxes run on the warp's
-// accumulators (a row lies in 4 lanes).  Bound by the mma.sync rate: 64 pairs of up to 4009
-// tokens, d = 128: 283 us, against 1125 us with fp32 FMAs.
+// The same projections for bf16 K/V on tcgen05 with fp32 accuracy: x is exact in bf16 and every
+// weight is split exactly into three bf16 parts (8 + 8 + 8 bits, W^T stored once per cache as
+// the shared-memory image of its tiles), so W x is three products whose terms are exact.  The
+// tensor unit rounds a running sum toward zero; to keep that below the rounding of a chain of
+// fp32 FMAs, each 64 inputs are summed on their own, smallest parts first, and added in fp32
+// (two accumulators of 128 inputs each: out.score 1.1e-6 from 64 bits, 6.8e-7 this way).  A CTA
+// takes 128 tokens: one warp copies the weights (80 KB per 64 inputs, two buffers) and issues
+// the MMAs (M = 128, N = 208); 8 warps load the tokens and, one thread per token and feature
+// map, add up the token's accumulator rows and run the Hedgehog softmaxes on them, then hand
+// whole rows of features to a bulk store.  Bound by the
+// weights' way from L2 (320 KB per CTA) and the exponentials.  64 pairs of up to 4009 tokens,
+// d = 128: 205 us, against 283 us on mma.sync and 1125 us with fp32 FMAs.
 constexpr int PT_TOK = 128;
-constexpr int PT_KC = 64;                          // inputs per chunk: one 128-byte row of W^T
+constexpr int PT_KC = 64;                          // inputs per chunk: one 128-byte row
+constexpr int PT_THREADS = NTM + 32;
+enum : int { PTERR_WAIT = 31 };
 
 template <int HD>
 struct PtP {
   static constexpr int HH = HD / 2;
-  static constexpr int NT = (3 * HH + 2 + 7) / 8;  // 8-column tiles: W_k, W_v, W_q, gates
-  static constexpr int NCP = 8 * NT;
+  static constexpr int NCP = (3 * HH + 2 + 15) / 16 * 16;   // columns: W_k, W_v, W_q, gates, zeros
   static constexpr int IN2 = 2 * HD;
   static constexpr int NKC = IN2 / PT_KC;
+  static constexpr int NF = ((2 * HD + HH + 2) + 3) & ~3;
   static constexpr int XB = PT_TOK * IN2 * 2;      // tokens: NKC tiles of [128][64]
-  static constexpr int WB = 3 * NCP * PT_KC * 2;   // one chunk of the three parts
-  static constexpr int SMEM = XB + 2 * WB;
+  static constexpr int WT = NCP * PT_KC * 2;       // one part of one chunk
+  static constexpr int WB = 3 * WT;
+  static constexpr int ROUNDS = NKC / 2;           // two chunks, one per accumulator, a round
+  static constexpr int OFF_BAR = XB + 2 * WB;
+  static constexpr int SMEM = OFF_BAR + 64 + 1024;
+  static constexpr int TM_COLS = 2 * NCP <= 256 ? 256 : 512;
+  static_assert(PT_TOK * NF * 4 <= OFF_BAR, "the features are staged over the operands");
+  static_assert(NF * 4 % 16 == 0, "rows of features leave by bulk copies");
 };
 
-// W^T parts: wt [H][NKC][3][NCP][64] from Wcat [H][2d][NC]
+// W^T parts: wt [H][NKC][3][NCP][64] in the 128-byte-swizzled order of a K-major tile, from
+// Wcat [H][2d][NC]
 template <int HD>
 __global__ void mlstm_split_kernel(const float* __restrict__ Wcat, int NC, int H, bf16* __restrict__ wt) {
   using P = PtP<HD>;
@@ -387,8 +401,9 @@ __global__ void mlstm_split_kernel(const float* __restrict__ Wcat, int NC, int H
       part[1] = __float2bfloat16_rz(r1);
       part[2] = __float2bfloat16_rz(r1 - __bfloat162float(part[1]));
     }
+    const int kk = k % PT_KC;
     for (int q = 0; q < 3; ++q)
-      wt[((((size_t)h * P::NKC + k / PT_KC) * 3 + q) * P::NCP + c) * PT_KC + k % PT_KC] = part[q];
+      wt[(((size_t)h * P::NKC + k / PT_KC) * 3 + q) * P::NCP * PT_KC + swz(c, kk / 8, 128) / 2 + kk % 8] = part[q];
   }
 }
 
@@ -400,129 +415,193 @@ struct MProjTcArgs {
   const float* bf;
   const int32_t* plen;
   float* feat;
-  int H, Pmax, NF;
+  int32_t* err;
+  int H, Pmax;
 };
 
 template <int HD>
-__global__ void __launch_bounds__(NTM, 1) mlstm_proj_tc_kernel(MProjTcArgs a) {
+__global__ void __launch_bounds__(PT_THREADS, 1) mlstm_proj_tc_kernel(MProjTcArgs a) {
+  using namespace tc05;
   using P = PtP<HD>;
-  constexpr int HH = P::HH, NT = P::NT, HT = HH / 8;   // HT: tiles of one projection
-  extern __shared__ __align__(128) unsigned char sm_pt[];
+  constexpr int HH = P::HH, NF = P::NF;
+  extern __shared__ unsigned char sm_pt_raw[];
+  unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(sm_pt_raw) + 1023) & ~(uintptr_t)1023);
   const int lp = blockIdx.y, bl = lp / a.H, h = lp - bl * a.H;
   const int L = a.plen[bl], t0 = blockIdx.x * PT_TOK;
   if (t0 >= L) return;
+  const int nrow = min(PT_TOK, L - t0);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int g = lane >> 2, t4 = lane & 3;
-  const uint32_t xb = smem_u32(sm_pt), wb = xb + P::XB;
-  const bf16* Kp = a.K + (size_t)lp * a.Pmax * HD;
-  const bf16* Vp = a.V + (size_t)lp * a.Pmax * HD;
-  const bf16* wt = a.wt + (size_t)h * P::NKC * 3 * P::NCP * PT_KC;
-  auto load_w = [&](int kc) {
-    const bf16* src = wt + (size_t)kc * 3 * P::NCP * PT_KC;
-    for (int i = tid; i < 3 * P::NCP * 8; i += NTM)
-      cp_async16(wb + (kc & 1) * P::WB + swz(i >> 3, i & 7, 128), src + (size_t)i * 8, 16);
-  };
-  for (int i = tid; i < PT_TOK * (P::IN2 / 8); i += NTM) {
-    const int r = i / (P::IN2 / 8), c = i - r * (P::IN2 / 8);
-    const bool in = t0 + r < L;
-    const size_t row = (size_t)(in ? t0 + r : t0) * HD;
-    const bf16* src = c < HD / 8 ? Kp + row + 8 * c : Vp + row + 8 * c - HD;
-    cp_async16(xb + (c >> 3) * (PT_TOK * 128) + swz(r, c & 7, 128), src, in ? 16 : 0);
+  const uint32_t sb = smem_u32(sm);
+  auto bar = [&](int i) { return sb + P::OFF_BAR + 8u * (uint32_t)i; };
+  if (tid == 0) {                                  // 0, 1 W; 2 x; 3, 4 MMAs done; 5 sums read
+    for (int i = 0; i < 6; ++i) mbar_init(bar(i), i == 2 || i == 5 ? NTM : 1);
+    mbar_fence_init();
   }
-  load_w(0);
-  cp_commit();
-  float acc[NT][4];
-#pragma unroll
-  for (int n = 0; n < NT; ++n) acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
-  for (int kc = 0; kc < P::NKC; ++kc) {
-    if (kc + 1 < P::NKC) load_w(kc + 1);
-    cp_commit();
-    cp_wait<1>();
-    __syncthreads();
-    uint32_t x[4][4];                              // the warp's 16 tokens, 4 k-steps
-#pragma unroll
-    for (int ks = 0; ks < 4; ++ks) {
-      const int r = 16 * warp + ((lane >> 3) & 1) * 8 + (lane & 7);
-      ldsm_x4(xb + kc * (PT_TOK * 128) + swz(r, 2 * ks + (lane >> 4), 128), x[ks][0], x[ks][1], x[ks][2], x[ks][3]);
-    }
-    const uint32_t w0 = wb + (kc & 1) * P::WB;
-#pragma unroll
-    for (int n = 0; n < NT; ++n) {
-      float c[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-      for (int q = 2; q >= 0; --q) {               // smallest part first
-#pragma unroll
-        for (int k2 = 0; k2 < 2; ++k2) {
-          const int row = q * P::NCP + 8 * n + (lane & 7);
-          uint32_t b0, b1, b2, b3;
-          ldsm_x4(w0 + swz(row, 4 * k2 + (lane >> 3), 128), b0, b1, b2, b3);
-          mma_bf16(c, x[2 * k2][0], x[2 * k2][1], x[2 * k2][2], x[2 * k2][3], b0, b1);
-          mma_bf16(c, x[2 * k2 + 1][0], x[2 * k2 + 1][1], x[2 * k2 + 1][2], x[2 * k2 + 1][3], b2, b3);
-        }
+  if (warp == NTM / 32) tmem_alloc(sb + P::OFF_BAR + 48, P::TM_COLS);
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(sm + P::OFF_BAR + 48);
+  if (warp == NTM / 32) {
+    // ---------------------------------------------------------------- weights, MMA issue
+    const bf16* wt = a.wt + (size_t)h * P::NKC * 3 * P::NCP * PT_KC;
+    const bool lead = elect_one();
+    auto load_w = [&](int kc) {
+      if (lead) {
+        mbar_arrive_expect_tx(bar(kc & 1), P::WB);
+        for (int q = 0; q < 3; ++q)
+          bulk_g2s(sb + P::XB + (kc & 1) * P::WB + q * P::WT, wt + (size_t)(3 * kc + q) * P::NCP * PT_KC, P::WT,
+                   bar(kc & 1));
       }
+      __syncwarp();
+    };
+    auto all = [](bool x) { return __all_sync(0xffffffffu, x); };
+    const uint32_t id = idesc_bf16(128, P::NCP, 0);
+    const uint64_t xd0 = kmajor_desc(sb, PT_TOK, 0), wd0 = kmajor_desc(sb + P::XB, P::NCP, 0);
+    int asked = 0, waited = 0;                     // chunks requested, chunks seen to land
+    for (; asked < 2 && asked < P::NKC; ++asked) load_w(asked);
+    bool ok = all(mbar_wait(bar(2), 0, a.err, PTERR_WAIT));
+    if (ok) fence_async_smem();
+    for (int kc = 0; kc < P::NKC && ok; ++kc) {
+      if (!(ok = all(mbar_wait(bar(kc & 1), (kc >> 1) & 1, a.err, PTERR_WAIT)))) break;
+      waited = kc + 1;
+      if (kc >= 2 && kc % 2 == 0 && !(ok = all(mbar_wait(bar(5), (kc / 2 - 1) & 1, a.err, PTERR_WAIT)))) break;
+      fence_after();
+      if (lead) {
+        const uint64_t xd = desc_at(xd0, kc * PT_TOK * 128), wd = desc_at(wd0, (kc & 1) * P::WB);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) acc[n][e] += c[e];
+        for (int q = 2; q >= 0; --q)               // smallest part first
+#pragma unroll
+          for (int ks = 0; ks < 4; ++ks)
+            mma_bf16(tmem + (kc & 1) * P::NCP, kmajor_step(xd, PT_TOK, ks),
+                     kmajor_step(desc_at(wd, q * P::WT), P::NCP, ks), id, !(q == 2 && ks == 0));
+        commit(bar(3 + (kc & 1)));
+      }
+      __syncwarp();
+      if (asked < P::NKC) {                        // the buffer's next chunk, once its MMAs are done
+        if (!(ok = all(mbar_wait(bar(3 + (kc & 1)), (kc >> 1) & 1, a.err, PTERR_WAIT)))) break;
+        load_w(asked++);
+      }
     }
-    __syncthreads();
-  }
-  cp_wait<0>();
-  // features of rows g and g + 8 of the warp: columns 8 n + 2 t4, + 1 are this lane's
+    if (!ok)                                       // copies in flight land before the CTA ends
+      for (int kc = waited; kc < asked; ++kc) mbar_wait(bar(kc & 1), (kc >> 1) & 1, nullptr, 0);
+    __syncwarp();
+  } else {
+    // ---------------------------------------------------------------- tokens, features
+    const bf16* Kp = a.K + (size_t)lp * a.Pmax * HD;
+    const bf16* Vp = a.V + (size_t)lp * a.Pmax * HD;
+    for (int i = tid; i < PT_TOK * (P::IN2 / 8); i += NTM) {
+      const int r = i / (P::IN2 / 8), c = i - r * (P::IN2 / 8);
+      const bool in = r < nrow;
+      const size_t row = (size_t)(in ? t0 + r : t0) * HD;
+      const bf16* src = c < HD / 8 ? Kp + row + 8 * c : Vp + row + 8 * c - HD;
+      cp_async16(sb + (c >> 3) * (PT_TOK * 128) + swz(r, c & 7, 128), src, in ? 16 : 0);
+    }
+    cp_async_arrive_noinc(bar(2));
+    // thread: token r = 32 (warp mod 4) + lane; warps 0-3 take k~ and half of v~, 4-7 q~, the
+    // other half of v~ and the gates
+    const int quarter = warp & 3, sel = warp >> 2, r = quarter * 32 + lane;
+    const uint32_t tr = tmem + ((uint32_t)(quarter * 32) << 16);
+    float* row = reinterpret_cast<float*>(sm) + (size_t)r * NF;
+    constexpr int NV = HH / 32;                    // 32-column groups of one projection
+    constexpr int G0 = 3 * HH - (P::NCP - 16);     // gate a_i in the last 16 columns, a_f next to it
+    static_assert(G0 >= 0 && G0 + 1 < 16, "");
+    const bool with_v = NV == 2 || sel == 0;       // v~: one group each, or the only one
+    float y[NV][32], x[32], gi = 0.f, gf = 0.f;
+    bool ok = true;
 #pragma unroll
-  for (int rr = 0; rr < 2; ++rr) {
-    const int t = t0 + 16 * warp + g + 8 * rr;
-    float* o = a.feat + ((size_t)lp * a.Pmax + t) * a.NF;
-    const bool in = t < L;
+    for (int rd = 0; rd < P::ROUNDS; ++rd) {
+      ok = ok && mbar_wait(bar(3), rd & 1, a.err, PTERR_WAIT) && mbar_wait(bar(4), rd & 1, a.err, PTERR_WAIT);
+      ok = __all_sync(0xffffffffu, ok);
+      fence_after();
+      if (!ok) break;
+      auto columns = [&](int c0, float (&v)[32]) {   // 32 columns of the token's projections
+        float u[32], w[32];
+        tmem_ld32(tr + c0, u);
+        tmem_ld32(tr + P::NCP + c0, w);
+        tmem_wait_ld();
 #pragma unroll
-    for (int part = 0; part < 2; ++part) {         // k~ from W_k's tiles, q~ from W_q's
-      const int n0 = part ? 2 * HT : 0;
-      float* dst = part ? o + HD + HH : o;
+        for (int i = 0; i < 32; ++i) v[i] = rd ? v[i] + (u[i] + w[i]) : u[i] + w[i];
+      };
+#pragma unroll
+      for (int g = 0; g < NV; ++g) columns((sel ? 2 * HH : 0) + 32 * g, y[g]);
+      if (with_v) columns(HH + (NV == 2 ? 32 * sel : 0), x);
+      if (sel == 1) {
+        // the gates' tile (the columns past them hold zeros or belong to the other accumulator)
+        float u[32], w[32];
+        tmem_ld32(tr + P::NCP - 16, u);
+        tmem_ld32(tr + 2 * P::NCP - 32, w);
+        tmem_wait_ld();
+        gi += u[G0] + w[G0 + 16];
+        gf += u[G0 + 1] + w[G0 + 17];
+      }
+      if (rd + 1 < P::ROUNDS) {
+        fence_before();
+        mbar_arrive(bar(5));
+      }
+    }
+    cp_wait<0>();
+    if (ok) {
+      auto put = [&](int at, const float (&v)[32]) {
+#pragma unroll
+        for (int i = 0; i < 32; i += 4)
+          *reinterpret_cast<float4*>(row + at + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+      };
+      // the operands are read: features take their place, rows of NF floats
+      if (with_v) put(HD + (NV == 2 ? 32 * sel : 0), x);
+      if (sel == 1)
+        *reinterpret_cast<float4*>(row + 2 * HD + HH) = make_float4(gi + a.bi[h], gf + a.bf[h], 0.f, 0.f);
+      float ep[NV][32], en[NV][32];
       float mp = -INFINITY, mn = -INFINITY;
 #pragma unroll
-      for (int n = 0; n < HT; ++n)
+      for (int g = 0; g < NV; ++g)
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const float v = acc[n0 + n][2 * rr + e];
-          mp = fmaxf(mp, v);
-          mn = fmaxf(mn, -v);
+        for (int i = 0; i < 32; ++i) {
+          mp = fmaxf(mp, y[g][i]);
+          mn = fmaxf(mn, -y[g][i]);
         }
+      float ps[4] = {}, ns[4] = {};
 #pragma unroll
-      for (int x = 1; x <= 2; x <<= 1) {
-        mp = fmaxf(mp, __shfl_xor_sync(0xffffffffu, mp, x));
-        mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, x));
-      }
-      float sp = 0.f, sn = 0.f;
+      for (int g = 0; g < NV; ++g)
 #pragma unroll
-      for (int n = 0; n < HT; ++n)
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const float v = acc[n0 + n][2 * rr + e];
-          sp += expf(v - mp);
-          sn += expf(-v - mn);
+        for (int i = 0; i < 32; ++i) {
+          ep[g][i] = expf(y[g][i] - mp);
+          en[g][i] = expf(-y[g][i] - mn);
+          ps[i & 3] += ep[g][i];
+          ns[i & 3] += en[g][i];
         }
+      const float sp = (ps[0] + ps[1]) + (ps[2] + ps[3]), sn = (ns[0] + ns[1]) + (ns[2] + ns[3]);
 #pragma unroll
-      for (int x = 1; x <= 2; x <<= 1) {
-        sp += __shfl_xor_sync(0xffffffffu, sp, x);
-        sn += __shfl_xor_sync(0xffffffffu, sn, x);
-      }
-      if (in) {
+      for (int g = 0; g < NV; ++g)
 #pragma unroll
-        for (int n = 0; n < HT; ++n) {
-          const float v0 = acc[n0 + n][2 * rr], v1 = acc[n0 + n][2 * rr + 1];
-          *reinterpret_cast<float2*>(dst + 8 * n + 2 * t4) = make_float2(expf(v0 - mp) / sp, expf(v1 - mp) / sp);
-          *reinterpret_cast<float2*>(dst + HH + 8 * n + 2 * t4) = make_float2(expf(-v0 - mn) / sn, expf(-v1 - mn) / sn);
+        for (int i = 0; i < 32; ++i) {
+          ep[g][i] /= sp;
+          en[g][i] /= sn;
         }
+      const int at = sel ? HD + HH : 0;
+#pragma unroll
+      for (int g = 0; g < NV; ++g) {
+        put(at + 32 * g, ep[g]);
+        put(at + HH + 32 * g, en[g]);
       }
     }
-    if (in) {
-#pragma unroll
-      for (int n = 0; n < HT; ++n)
-        *reinterpret_cast<float2*>(o + HD + 8 * n + 2 * t4) =
-            make_float2(acc[HT + n][2 * rr], acc[HT + n][2 * rr + 1]);
-      if (t4 == 0)
-        *reinterpret_cast<float2*>(o + 2 * HD + HH) =
-            make_float2(acc[3 * HT][2 * rr] + a.bi[h], acc[3 * HT][2 * rr + 1] + a.bf[h]);
+    // the quarter's rows leave together: both warps' parts are there
+    fence_async_smem();
+    asm volatile("bar.sync %0, 64;" ::"r"(1 + quarter) : "memory");
+    if (sel == 0 && lane == 0 && ok && quarter * 32 < nrow) {
+      const uint32_t bytes = (uint32_t)(min(32, nrow - quarter * 32) * NF * 4);
+      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
+                       a.feat + ((size_t)lp * a.Pmax + t0 + quarter * 32) * NF),
+                   "r"(sb + (uint32_t)(quarter * 32 * NF * 4)), "r"(bytes)
+                   : "memory");
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+      asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
     }
+    __syncwarp();
   }
+  fence_before();
+  __syncthreads();
+  if (warp == NTM / 32) tmem_dealloc(tmem, P::TM_COLS);
 }
 
 struct MScanArgs {
@@ -1015,10 +1094,10 @@ cudaError_t launch_scan(MScanArgs sa, int pairs, cudaStream_t stream) {
 
 template <int HD>
 cudaError_t launch_proj_tc(const MlstmDev& m, const void* K, const void* V, const int32_t* plen, int pairs,
-                           int H, int Pmax, int NF, float* feat, cudaStream_t stream) {
+                           int H, int Pmax, float* feat, int32_t* err, cudaStream_t stream) {
   MProjTcArgs a{static_cast<const bf16*>(K), static_cast<const bf16*>(V), static_cast<const bf16*>(m.Wt),
-                m.bi, m.bf, plen, feat, H, Pmax, NF};
-  mlstm_proj_tc_kernel<HD><<<dim3((Pmax + PT_TOK - 1) / PT_TOK, pairs), NTM, PtP<HD>::SMEM, stream>>>(a);
+                m.bi, m.bf, plen, feat, err, H, Pmax};
+  mlstm_proj_tc_kernel<HD><<<dim3((Pmax + PT_TOK - 1) / PT_TOK, pairs), PT_THREADS, PtP<HD>::SMEM, stream>>>(a);
   return cudaGetLastError();
 }
 
@@ -1119,8 +1198,8 @@ cudaError_t launch_prefill_mlstm_scores(const State& st, const Dims& dm, const M
       mlstm_proj_kernel<<<dim3((Pmax + UTM - 1) / UTM, pairs), NTM, psm, stream>>>(a);
       e = cudaGetLastError();
     } else {
-      e = dm.d == 128 ? launch_proj_tc<128>(m, K, V, plen, pairs, dm.H, Pmax, NF, feat, stream)
-                      : launch_proj_tc<64>(m, K, V, plen, pairs, dm.H, Pmax, NF, feat, stream);
+      e = dm.d == 128 ? launch_proj_tc<128>(m, K, V, plen, pairs, dm.H, Pmax, feat, st.err, stream)
+                      : launch_proj_tc<64>(m, K, V, plen, pairs, dm.H, Pmax, feat, st.err, stream);
     }
     if (e != cudaSuccess) return e;
   }
