@@ -488,6 +488,18 @@ __global__ void __launch_bounds__(FUSED ? TcTraits<HD, G>::THREADS_F : TcTraits<
     if (ok && key0 < cnt) {
       const uint32_t kbase = smem_u32(smem + (size_t)s * Tr::STAGE_BYTES);
       const uint32_t vbase = kbase + NH * Tr::HALF_BYTES;
+      if (key0 + 16 > cnt) {
+        // Rows past the last key hold whatever was in shared memory (a window box is narrower
+        // than its tile) or in the store: their weight is 0, and so has their V to be, for
+        // 0 times an infinity or NaN would reach the sums.
+        for (int i = lane; i < (key0 + 16 - cnt) * NH * 8; i += 32) {
+          const int row = cnt + i / (NH * 8), c = i % (NH * 8);
+          *reinterpret_cast<uint4*>(smem + (size_t)s * Tr::STAGE_BYTES + (NH + (c >> 3)) * Tr::HALF_BYTES +
+                                    row * 128 + (c & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // before the stage's next copies
+        __syncwarp();
+      }
       // ---- S^T = K Q^T over d, two accumulator chains
       float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
       {
