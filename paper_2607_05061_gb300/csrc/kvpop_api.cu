@@ -304,6 +304,7 @@ static kvpop_status init_cache(const kvpop_config* cfg_in, const kvpop_scorer* s
   ALLOC(len, int32_t*, pairs * 4)
   ALLOC(min_score, float*, pairs * 4)
   ALLOC(min_slot, int32_t*, pairs * 4)
+  ALLOC(step_slots, int2*, pairs * sizeof(int2))
   ALLOC(blk_score, float*, pairs * NB * 4)
   ALLOC(blk_slot, int32_t*, pairs * NB * 4)
   float* w = nullptr;
@@ -488,6 +489,7 @@ static kvpop_status init_cache(const kvpop_config* cfg_in, const kvpop_scorer* s
     }
     if (e == cudaSuccess) e = NOTE(cudaMemsetAsync(c->st.nvalid, 0, pairs * 4, stream));
     if (e == cudaSuccess) e = NOTE(cudaMemsetAsync(c->st.len, 0, pairs * 4, stream));
+    if (e == cudaSuccess) e = NOTE(cudaMemsetAsync(c->st.step_slots, 0xff, pairs * sizeof(int2), stream));
     if (e == cudaSuccess) e = NOTE(cudaMemsetAsync(c->st.part_count, 0, pairs * 4, stream));
     if (e == cudaSuccess) e = NOTE(cudaMemsetAsync(c->st.err, 0, 16 * 4, stream));
     if (e == cudaSuccess) e = NOTE(cudaMemsetAsync(c->st.pos, 0xff, pairs * B * 4, stream));
@@ -772,14 +774,19 @@ kvpop_status kvpop_decode_ingest(kvpop_cache* c, const void* q, const void* k, c
   return poison_on(c, NOTE(launch_ingest(c->st, c->dm, q, k, v, override_, evict_info, score_out, stream)));
 }
 
-kvpop_status kvpop_decode_attend(kvpop_cache* c, const void* q, float* out, cudaStream_t stream) {
+static kvpop_status attend_from(kvpop_cache* c, const void* q, float* out, bool after_ingest,
+                                cudaStream_t stream) {
   kvpop_status s = usable(c);
   if (s != KVPOP_OK) return s;
   if (!q || !out) return KVPOP_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(out)) return KVPOP_ERR_ALIGN;
   if (c->use_tc)
-    return poison_on(c, NOTE(tc_launch(c->st, c->dm, tc_map_ptr(c), q, out, c->attend_grid, stream)));
+    return poison_on(c, NOTE(tc_launch(c->st, c->dm, tc_map_ptr(c), q, out, c->attend_grid, after_ingest, stream)));
   return poison_on(c, NOTE(launch_attend(c->st, c->dm, q, out, c->attend_grid, stream)));
+}
+
+kvpop_status kvpop_decode_attend(kvpop_cache* c, const void* q, float* out, cudaStream_t stream) {
+  return attend_from(c, q, out, false, stream);
 }
 
 kvpop_status kvpop_decode_step(kvpop_cache* c, const void* q, const void* k, const void* v,
@@ -800,7 +807,7 @@ kvpop_status kvpop_decode_step(kvpop_cache* c, const void* q, const void* k, con
   }
   s = kvpop_decode_ingest(c, q, k, v, override_, evict_info, score_out, stream);
   if (s != KVPOP_OK) return s;
-  return kvpop_decode_attend(c, q, out, stream);
+  return attend_from(c, q, out, true, stream);
 }
 
 int32_t kvpop_step_is_fused(const kvpop_cache* c) {
@@ -909,6 +916,8 @@ kvpop_status kvpop_import_state(kvpop_cache* c, const void* host_buf, size_t byt
     off += b.bytes;
   }
   if (e == cudaSuccess) e = NOTE(cudaMemsetAsync(c->st.part_count, 0, (size_t)c->dm.pairs * 4, stream));
+  if (e == cudaSuccess)
+    e = NOTE(cudaMemsetAsync(c->st.step_slots, 0xff, (size_t)c->dm.pairs * sizeof(int2), stream));
   if (e == cudaSuccess) e = NOTE(cudaStreamSynchronize(stream));
   return poison_on(c, e);
 }

@@ -49,8 +49,8 @@ __device__ __forceinline__ void blocks_min(const float* __restrict__ bs, const i
   mi = bi;
 }
 
-// Warp-collective rebuild of every block minimum and of the head minimum.
-__device__ __forceinline__ void rebuild_min(float* __restrict__ sc, int s, int B, int j_new,
+// Warp-collective rebuild of every block minimum and of the head minimum, whose slot it returns.
+__device__ __forceinline__ int rebuild_min(float* __restrict__ sc, int s, int B, int j_new,
                                             float v_new, float* __restrict__ bs,
                                             int32_t* __restrict__ bsl, float* min_score,
                                             int32_t* min_slot) {
@@ -67,10 +67,11 @@ __device__ __forceinline__ void rebuild_min(float* __restrict__ sc, int s, int B
   int mi;
   blocks_min(bs, bsl, NB, -1, 0.f, 0, m, mi);
   if (lane == 0) { *min_score = m; *min_slot = mi; }
+  return mi;
 }
 
 // Warp-collective update after slot j took priority v (the head was full).
-__device__ __forceinline__ void update_min(const float* __restrict__ sc, int s, int B, int j, float v,
+__device__ __forceinline__ int update_min(const float* __restrict__ sc, int s, int B, int j, float v,
                                            float* __restrict__ bs, int32_t* __restrict__ bsl,
                                            float* min_score, int32_t* min_slot) {
   const int lane = threadIdx.x & 31;
@@ -87,6 +88,7 @@ __device__ __forceinline__ void update_min(const float* __restrict__ sc, int s, 
     *min_score = m;
     *min_slot = mi;
   }
+  return mi;
 }
 
 }  // namespace kvpop

@@ -43,11 +43,13 @@ __device__ __forceinline__ void evict_and_scatter(const State& st, const Dims& d
       dk[i] = k_u[i];
       dv[i] = v_u[i];
     }
+    int min_now = -1;
     if (nv == B)
-      update_min(sc, dm.s, B, slot, prio, bsc, bsl, st.min_score + pair, st.min_slot + pair);
+      min_now = update_min(sc, dm.s, B, slot, prio, bsc, bsl, st.min_score + pair, st.min_slot + pair);
     else if (nv + 1 == B)
-      rebuild_min(sc, dm.s, B, slot, prio, bsc, bsl, st.min_score + pair, st.min_slot + pair);
+      min_now = rebuild_min(sc, dm.s, B, slot, prio, bsc, bsl, st.min_score + pair, st.min_slot + pair);
     if (lane == 0) {
+      st.step_slots[pair] = make_int2(min_now, slot);
       sc[slot] = prio;
       ps[slot] = u;
       st.nvalid[pair] = nv < B ? nv + 1 : nv;

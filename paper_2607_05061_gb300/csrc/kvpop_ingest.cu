@@ -260,11 +260,13 @@ __global__ void __launch_bounds__(NT) ingest_kernel(IngestArgs<T> a) {
       dk[i] = rawk[warp * d + i];
       dv[i] = rawv[warp * d + i];
     }
+    int min_now = -1;
     if (nv == B)
-      update_min(sc, dm.s, B, slot, prio, bsc, bsl, a.st.min_score + pair, a.st.min_slot + pair);
+      min_now = update_min(sc, dm.s, B, slot, prio, bsc, bsl, a.st.min_score + pair, a.st.min_slot + pair);
     else if (nv + 1 == B)
-      rebuild_min(sc, dm.s, B, slot, prio, bsc, bsl, a.st.min_score + pair, a.st.min_slot + pair);
+      min_now = rebuild_min(sc, dm.s, B, slot, prio, bsc, bsl, a.st.min_score + pair, a.st.min_slot + pair);
     if (lane == 0) {
+      a.st.step_slots[pair] = make_int2(min_now, slot);
       sc[slot] = prio;
       ps[slot] = u;
       a.st.nvalid[pair] = nv < B ? nv + 1 : nv;

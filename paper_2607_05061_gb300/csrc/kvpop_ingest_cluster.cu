@@ -3,9 +3,9 @@
 //
 // The 8 CTAs of a cluster split the scorer's hidden units: CTA r holds the
 // slice [r*FS, (r+1)*FS) of W1 (3d x FS fp32, 48 KB for d = 128, F = 256),
-// loaded in one go by bulk copies together with everything its two "owned"
-// sequences need (window query means, the leaving token's K/V row, the new
-// q/k/v).  Each owner builds its sequences' scorer inputs
+// loaded in one go by bulk copies together with what its two "owned"
+// sequences need (the leaving token's K/V row, the new q/k/v); the window's
+// query means are added up straight from the ring, a row per warp at a time.  Each owner builds its sequences' scorer inputs
 // x = [k_u; v_u; qbar_u] (Sec. 3.3 delayed scoring, App. E.4) and writes them
 // into every CTA of the cluster through distributed shared memory; after a
 // cluster barrier each CTA evaluates its hidden slice for all 16 sequences and
@@ -14,6 +14,12 @@
 // App. C.1 (static priority, App. B.3) and scatter the token into its slot.
 // The state the eviction reads (used slots, the cached minimum, its block) is
 // loaded at kernel start so its latency hides behind the scorer.
+//
+// Bound by latency: five dependent passes over L2 and two cluster barriers.  Without the
+// window in shared memory (131 KB of the 184 it took) two CTAs share an SM, which leaves 120 of
+// 152 SMs to the attention meanwhile; stores that a barrier's release would wait for come after
+// the barriers.  Batch 1, d = 128, F = 256, window 128, from its wait to the end: 14.2 -> 11.7 us
+// beside the attention, 14.2 -> 12.5 us alone.
 #include "kvpop_argmin.cuh"
 
 namespace kvpop {
@@ -68,27 +74,18 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
                : "memory");
 }
 
-// D (16x8, fp32) += A (16x8, tf32, row) B (8x8, tf32, col), legacy tensor-core MMA
-__device__ __forceinline__ void mma_tf32_16x8x8(float (&c)[4], const uint32_t (&a)[4],
-                                                const uint32_t (&b)[2]) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7},"
-      " {%8, %9}, {%0, %1, %2, %3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
 struct ClLayout {              // byte offsets into dynamic shared memory
   int ws, x, qm, qrow, ring, newkv, part, total;
 };
-__host__ __device__ inline ClLayout cl_layout(int d, int D, int G, int FS, int esz) {
+__host__ __device__ inline ClLayout cl_layout(int d, int G, int FS, int esz) {
   ClLayout L;
   const int R = d * esz;
   int o = 0;
   L.ws = o;    o += 3 * d * FS * 4;                 // W1 slice, then b1, w2 slices
   o += 2 * FS * 4;
   L.x = o;     o += SBC * (3 * d + 4) * 4;          // scorer inputs of the 16 sequences (row stride 3d + 4)
-  L.qm = o;    o += OWN * D * d * 4;                // window query means of the owned sequences
+  L.qm = o;                                         // the warps' sums of the window query means, then the
+  o += max(NT / 32 * OWN * d, NT * SBC) * 4;        // scorer's [NT / FS][16][FS]
   L.qrow = o;  o += OWN * G * R;                    // new queries
   L.ring = o;  o += OWN * 2 * R;                    // K, V row of the leaving token
   L.newkv = o; o += OWN * 2 * R;                    // new K, V row
@@ -98,7 +95,7 @@ __host__ __device__ inline ClLayout cl_layout(int d, int D, int G, int FS, int e
 }
 
 template <typename T>
-__global__ void __launch_bounds__(NT, 1) ingest_cluster_kernel(ClArgs<T> a) {
+__global__ void __launch_bounds__(NT, 3) ingest_cluster_kernel(ClArgs<T> a) {
   const Dims& dm = a.dm;
   const int d = dm.d, D = dm.D, G = dm.G, F = dm.F, B = dm.B, H = dm.H, FS = a.FS;
   const int in_dim = 3 * d;
@@ -107,7 +104,7 @@ __global__ void __launch_bounds__(NT, 1) ingest_cluster_kernel(ClArgs<T> a) {
   const uint32_t rank = cluster_rank();
   const int group = blockIdx.x / CS;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const ClLayout L = cl_layout(d, D, G, FS, (int)sizeof(T));
+  const ClLayout L = cl_layout(d, G, FS, (int)sizeof(T));
 
   extern __shared__ __align__(128) unsigned char smem[];
   float* Ws = reinterpret_cast<float*>(smem + L.ws);
@@ -115,7 +112,7 @@ __global__ void __launch_bounds__(NT, 1) ingest_cluster_kernel(ClArgs<T> a) {
   const float* w2s = b1s + FS;
   float* X = reinterpret_cast<float*>(smem + L.x);           // [SBC][3d + 4]
   const int XS = in_dim + 4;
-  float* rqm = reinterpret_cast<float*>(smem + L.qm);        // [OWN][D][d]
+  float* qsum = reinterpret_cast<float*>(smem + L.qm);       // [warp][OWN][d] sums of window query means
   T* qrow = reinterpret_cast<T*>(smem + L.qrow);             // [OWN][G][d]
   T* ring = reinterpret_cast<T*>(smem + L.ring);             // [OWN][2][d]
   T* newkv = reinterpret_cast<T*>(smem + L.newkv);           // [OWN][2][d]
@@ -125,9 +122,6 @@ __global__ void __launch_bounds__(NT, 1) ingest_cluster_kernel(ClArgs<T> a) {
 
   // sequences of this cluster: group*SBC + j; CTA `rank` owns j = OWN*rank + o
   const int own_b0 = group * SBC + OWN * (int)rank;
-
-  // the attention that follows may be scheduled now; it waits for this grid to complete
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   // ---- issue every load this CTA needs ------------------------------------------------
   if (tid == 0) {
@@ -143,21 +137,31 @@ __global__ void __launch_bounds__(NT, 1) ingest_cluster_kernel(ClArgs<T> a) {
     bulk_g2s(smem_u32(Ws + in_dim * FS), a.b1s + slice * FS, vbytes, bb);
     bulk_g2s(smem_u32(Ws + in_dim * FS + FS), a.w2s + slice * FS, vbytes, bb);
   }
+  // the owned sequences' window query means and block minima on their way to L2 (a hint: the
+  // step before may still write a row of them)
+  if (tid < OWN && own_b0 + tid < dm.batch) {
+    const size_t pair = (size_t)(own_b0 + tid) * H + h;
+    const size_t qb = (size_t)D * d * 4;
+    for (size_t off = 0; off < qb; off += 16384)
+      prefetch_l2(a.st.ringQm + pair * D * d + off / 4, (uint32_t)min((size_t)16384, qb - off));
+  }
   // A programmatic dependent of the kernel before it: the weights above never change, all
   // that follows is state or input that kernel may still write.
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  // The attention that follows may be scheduled now, and not earlier: it starts on keys that
+  // this step does not change, so all that came before has to be complete.
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid == 0) {
     const uint32_t bb = smem_u32(&bar);
     // rows that do not depend on the sequence length first ...
     uint32_t rest = 0;
     for (int o = 0; o < OWN; ++o)
-      if (own_b0 + o < dm.batch) rest += (uint32_t)(D * d * 4 + G * R + 2 * R);
+      if (own_b0 + o < dm.batch) rest += (uint32_t)(G * R + 2 * R);
     mbar_expect_tx(bb, rest);
     for (int o = 0; o < OWN; ++o) {
       const int b = own_b0 + o;
       if (b >= dm.batch) continue;
       const int pair = b * H + h;
-      bulk_g2s(smem_u32(rqm + (size_t)o * D * d), a.st.ringQm + (size_t)pair * D * d, D * d * 4, bb);
       bulk_g2s(smem_u32(qrow + (size_t)o * G * d), a.q + (size_t)pair * G * d, G * R, bb);
       bulk_g2s(smem_u32(newkv + (size_t)(2 * o) * d), a.k + (size_t)pair * d, R, bb);
       bulk_g2s(smem_u32(newkv + (size_t)(2 * o + 1) * d), a.v + (size_t)pair * d, R, bb);
@@ -196,10 +200,14 @@ __global__ void __launch_bounds__(NT, 1) ingest_cluster_kernel(ClArgs<T> a) {
   int nbs[kMaxBlkLanes];
 #pragma unroll
   for (int t = 0; t < kMaxBlkLanes; ++t) { nbv[t] = INFINITY; nbs[t] = 0x7fffffff; }
+  float ev_b2 = 0.f, ev_override = 0.f, ev_lg = 0.f;
   if (warp < OWN) {
     const int b = own_b0 + warp;
     if (b < dm.batch) {
       const int pair = b * H + h;
+      ev_b2 = a.st.b2[h];
+      if (a.override_) ev_override = a.override_[pair];
+      if (a.st.log_gamma) ev_lg = a.st.log_gamma[h];
       ev_nv = a.st.nvalid[pair];
       ev_mscore = a.st.min_score[pair];
       ev_mslot = a.st.min_slot[pair];
@@ -216,6 +224,32 @@ __global__ void __launch_bounds__(NT, 1) ingest_cluster_kernel(ClArgs<T> a) {
           nbs[t] = (t < nbl && k < NB) ? a.st.blk_slot[(size_t)pair * NB + k] : 0x7fffffff;
         }
       }
+    }
+  }
+  // window query means of the owned sequences, all but the leaving token's: warp w adds rows
+  // w, w + 8, ... straight from the ring
+  for (int o = 0; o < OWN; ++o) {
+    const int b = own_b0 + o;
+    if (b >= dm.batch) break;
+    const int pair = b * H + h;
+    const int len = a.st.len[pair], leaving = len >= 0 ? len % D : 0;
+    const float4* src = reinterpret_cast<const float4*>(a.st.ringQm + (size_t)pair * D * d);
+    for (int c = lane; c < d / 4; c += 32) {
+      float4 s4 = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int w0 = warp; w0 < D; w0 += 8 * (NT / 32)) {
+        float4 row[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int w = w0 + j * (NT / 32);
+          row[j] = w < D ? __ldcg(src + (size_t)w * (d / 4) + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if (w0 + j * (NT / 32) != leaving) {
+            s4.x += row[j].x; s4.y += row[j].y; s4.z += row[j].z; s4.w += row[j].w;
+          }
+      }
+      *reinterpret_cast<float4*>(qsum + ((size_t)warp * OWN + o) * d + 4 * c) = s4;
     }
   }
   __syncthreads();
@@ -248,129 +282,63 @@ __global__ void __launch_bounds__(NT, 1) ingest_cluster_kernel(ClArgs<T> a) {
             e[t] = to_f(vu[i - d]);
           } else {
             const int c = i - 2 * d;
-            float qsum = 0.f;
-            for (int g = 0; g < G; ++g) qsum += to_f(qrow[(o * G + g) * d + c]);
-            const float qm_p = qsum * (1.0f / (float)G);
-            // qbar_u: queries u+1 .. p in position order, averaged over D
+            float qnew = 0.f;
+            for (int g = 0; g < G; ++g) qnew += to_f(qrow[(o * G + g) * d + c]);
+            // qbar_u: queries u+1 .. p, averaged over D
             float acc = 0.f;
-            for (int jj = 1; jj < D; ++jj) {
-              int w = ri + jj;
-              w = w >= D ? w - D : w;
-              acc += rqm[((size_t)o * D + w) * d + c];
-            }
-            acc += qm_p;
+#pragma unroll
+            for (int w = 0; w < NT / 32; ++w) acc += qsum[((size_t)w * OWN + o) * d + c];
+            acc += qnew * (1.0f / (float)G);
             e[t] = acc / (float)D;
           }
         }
         val = make_float4(e[0], e[1], e[2], e[3]);
       }
 #pragma unroll
-      for (int dst = 0; dst < CS; ++dst) st_cluster_v4(map_rank(xrow + i4 * 16, dst), val);
-    }
-    if (ok && b < dm.batch) {
-      // push the new token into the window slot of u (u's copy stays in smem)
-      const int pair = b * H + h;
-      T* dk = static_cast<T*>(a.st.ringK) + ((size_t)pair * D + ri) * d;
-      T* dv = static_cast<T*>(a.st.ringV) + ((size_t)pair * D + ri) * d;
-      float* dq = a.st.ringQm + ((size_t)pair * D + ri) * d;
-      for (int i = qq * 32 + lane; i < d; i += 128) {
-        dk[i] = newkv[(2 * o) * d + i];
-        dv[i] = newkv[(2 * o + 1) * d + i];
-        float qsum = 0.f;
-        for (int g = 0; g < G; ++g) qsum += to_f(qrow[(o * G + g) * d + i]);
-        dq[i] = qsum * (1.0f / (float)G);
-      }
+      for (int dst = 0; dst < CS && b < dm.batch; ++dst) st_cluster_v4(map_rank(xrow + i4 * 16, dst), val);
     }
   }
   cluster_sync();   // every X row is in every CTA
 
-  // ---- this CTA's hidden slice for all 16 sequences --------------------------------------
-  // H[16 sequences][FS] = X W, fp32-accurate.  With FS a multiple of 8 it runs on the tensor
-  // pipe: m16n8k8 tf32 MMAs, each operand split into a tf32 head and its residual and
-  // X W = X_hi W_hi + X_hi W_lo + X_lo W_hi (the dropped X_lo W_lo is below fp32 rounding);
-  // warp w takes k-steps [w K8 / 8, (w + 1) K8 / 8) of the 3d inputs.  Otherwise thread
-  // (f, ks) accumulates unit f over input slice ks for every sequence.  Either way the
-  // partial sums meet in shared memory (over the input rows, no longer needed), then warp w
-  // adds b1, applies the activation and contracts with w2 for sequences 2w, 2w+1.
+  // ---- this CTA's hidden slice for the cluster's sequences -------------------------------
+  // H[n sequences][FS] = X W in fp32: thread (f, ks) takes unit f over input slice ks, four
+  // sequences at a time, with the weights conflict-free and the inputs broadcast from shared
+  // memory.  The partial sums meet in shared memory, then warp w adds b1, applies the
+  // activation and contracts with w2 for sequences 2w, 2w+1.  The work is the batch's, and at
+  // most 0.8 us of FMAs for 16 sequences, where 3xTF32 on mma.sync took 1.7 us of them for one
+  // sequence as for 16 (16 rows either way).
+  const int nact = min(SBC, dm.batch - group * SBC);
   {
-    // (the 8 warp partials of [16][FS] must fit in the input rows: 8 FS <= 3d + 4)
-    const bool tc = (FS % 8) == 0 && (in_dim % 64) == 0 && 8 * FS <= XS && FS <= 64;
-    int NKS;                                          // partial sums per (sequence, unit)
-    float* red = X;                                   // [NKS][SBC][FS]
-    if (tc) {
-      NKS = NT / 32;
-      const int g = lane >> 2, tig = lane & 3;
-      const int k8 = in_dim / 8, kper = k8 / NKS, kb = warp * kper;
-      float acc[8][4];                                // up to FS = 64: 8 n-tiles
-#pragma unroll
-      for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) acc[nt][e] = 0.f;
-      auto split = [](float x, uint32_t& hi, uint32_t& lo) {
-        asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(hi) : "f"(x));
-        lo = __float_as_uint(x - __uint_as_float(hi));
-      };
-      for (int kk = 0; kk < kper; ++kk) {
-        const int k0 = (kb + kk) * 8;
-        uint32_t ah[4], al[4];
-        split(X[(size_t)g * XS + k0 + tig], ah[0], al[0]);
-        split(X[(size_t)(g + 8) * XS + k0 + tig], ah[1], al[1]);
-        split(X[(size_t)g * XS + k0 + tig + 4], ah[2], al[2]);
-        split(X[(size_t)(g + 8) * XS + k0 + tig + 4], ah[3], al[3]);
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-          if (nt * 8 >= FS) break;
-          uint32_t bh[2], bl[2];
-          split(Ws[(size_t)(k0 + tig) * FS + nt * 8 + g], bh[0], bl[0]);
-          split(Ws[(size_t)(k0 + tig + 4) * FS + nt * 8 + g], bh[1], bl[1]);
-          mma_tf32_16x8x8(acc[nt], ah, bh);
-          mma_tf32_16x8x8(acc[nt], ah, bl);
-          mma_tf32_16x8x8(acc[nt], al, bh);
-        }
-      }
-      __syncthreads();                                // every warp is done with X
-#pragma unroll
-      for (int nt = 0; nt < 8; ++nt) {
-        if (nt * 8 >= FS) break;
-        const int col = nt * 8 + 2 * tig;
-        float* r0 = red + ((size_t)warp * SBC + g) * FS + col;
-        float* r8 = red + ((size_t)warp * SBC + g + 8) * FS + col;
-        r0[0] = acc[nt][0];
-        r0[1] = acc[nt][1];
-        r8[0] = acc[nt][2];
-        r8[1] = acc[nt][3];
-      }
-    } else {
-      // NKS * FS <= 3d keeps the partial sums inside the input rows
-      NKS = min(NT / FS, in_dim / FS);
-      const int SL = ((in_dim + NKS - 1) / NKS + 3) & ~3;   // inputs per slice, multiple of 4
-      const int f = tid % FS, ks = tid / FS;
-      float acc[SBC];
-#pragma unroll
-      for (int j = 0; j < SBC; ++j) acc[j] = 0.f;
-      if (ks < NKS) {
-        const int i_end = min(in_dim, (ks + 1) * SL);
-        for (int i = ks * SL; i < i_end; i += 4) {
+    const int NKS = min(NT / FS, in_dim / FS);        // partial sums per (sequence, unit)
+    const int SL = ((in_dim + NKS - 1) / NKS + 3) & ~3;   // inputs per slice, multiple of 4
+    float* red = qsum;                                // [NKS][SBC][FS]
+    const int f = tid % FS, ks = tid / FS;
+    const int i0 = ks * SL, i1 = min(in_dim, (ks + 1) * SL);
+    if (ks < NKS) {
+#pragma unroll 1
+      for (int j0 = 0; j0 < nact; j0 += 4) {
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        const float* xr = X + (size_t)j0 * XS;
+#pragma unroll 3
+        for (int i = i0; i < i1; i += 4) {
           const float w0 = Ws[(i + 0) * FS + f], w1 = Ws[(i + 1) * FS + f];
           const float w2 = Ws[(i + 2) * FS + f], w3 = Ws[(i + 3) * FS + f];
 #pragma unroll
-          for (int j = 0; j < SBC; ++j) {
-            const float4 u = *reinterpret_cast<const float4*>(X + (size_t)j * XS + i);
+          for (int j = 0; j < 4; ++j) {
+            const float4 u = *reinterpret_cast<const float4*>(xr + (size_t)j * XS + i);
             acc[j] = fmaf(u.x, w0, fmaf(u.y, w1, fmaf(u.z, w2, fmaf(u.w, w3, acc[j]))));
           }
         }
-      }
-      __syncthreads();                                // every thread is done with X
-      if (ks < NKS) {
 #pragma unroll
-        for (int j = 0; j < SBC; ++j) red[((size_t)ks * SBC + j) * FS + f] = acc[j];
+        for (int j = 0; j < 4; ++j) red[((size_t)ks * SBC + j0 + j) * FS + f] = acc[j];
       }
     }
     __syncthreads();
     float c0 = 0.f, c1 = 0.f;
     const int j0 = 2 * warp, j1 = 2 * warp + 1;
-    for (int ff = lane; ff < FS; ff += 32) {
+    for (int ff = lane; ff < FS && j0 < nact; ff += 32) {
       float a0 = b1s[ff], a1 = a0;
+#pragma unroll 4
       for (int kk = 0; kk < NKS; ++kk) {
         a0 += red[((size_t)kk * SBC + j0) * FS + ff];
         a1 += red[((size_t)kk * SBC + j1) * FS + ff];
@@ -385,7 +353,7 @@ __global__ void __launch_bounds__(NT, 1) ingest_cluster_kernel(ClArgs<T> a) {
       c1 += __shfl_xor_sync(0xffffffffu, c1, off);
     }
     // sequences 2w, 2w+1 are owned by CTA w (OWN = 2): part[rank][o] there
-    if (lane == 0) {
+    if (lane == 0 && j0 < nact) {
       const uint32_t dst = (uint32_t)warp;
       st_cluster_f32(map_rank(smem_u32(part + rank * OWN + 0), dst), c0);
       st_cluster_f32(map_rank(smem_u32(part + rank * OWN + 1), dst), c1);
@@ -397,8 +365,27 @@ __global__ void __launch_bounds__(NT, 1) ingest_cluster_kernel(ClArgs<T> a) {
     mbar_wait(smem_u32(&bar), 0, a.st.err, DEVERR_TIMEOUT_DRAIN);
   }
 
+  // ---- the window: the new token takes the slot of u (u's copy stays in shared memory) -------
+  // (after the cluster's barriers, which would wait for these stores)
+  if (warp >= OWN) {
+    for (int o = 0; o < OWN && ok; ++o) {
+      const int b = own_b0 + o;
+      if (b >= dm.batch) break;
+      const size_t at = ((size_t)(b * H + h) * D + (s_p[o] >= 0 ? s_p[o] % D : 0)) * d;
+      T* dk = static_cast<T*>(a.st.ringK) + at;
+      T* dv = static_cast<T*>(a.st.ringV) + at;
+      for (int i = tid - OWN * 32; i < d; i += NT - OWN * 32) {
+        dk[i] = newkv[(2 * o) * d + i];
+        dv[i] = newkv[(2 * o + 1) * d + i];
+        float qnew = 0.f;
+        for (int g = 0; g < G; ++g) qnew += to_f(qrow[(o * G + g) * d + i]);
+        a.st.ringQm[at + i] = qnew * (1.0f / (float)G);
+      }
+    }
+    return;
+  }
+
   // ---- owners: score, keep-or-drop, scatter ------------------------------------------------
-  if (warp >= OWN) return;
   const int o = warp;
   const int b = own_b0 + o;
   if (b >= dm.batch || !ok) return;
@@ -414,11 +401,11 @@ __global__ void __launch_bounds__(NT, 1) ingest_cluster_kernel(ClArgs<T> a) {
   }
   float r = 0.f;
   for (int src = 0; src < CS; ++src) r += part[src * OWN + o];
-  r += a.st.b2[h];
-  if (a.override_) r = a.override_[pair];
+  r += ev_b2;
+  if (a.override_) r = ev_override;
   r = canon_score(r);
   const int u = p - D;
-  const float prio = static_priority(r, u, a.st.log_gamma, h);
+  const float prio = decayed(r, u, ev_lg);
 
   float* sc = a.st.score + (size_t)pair * B;
   int32_t* ps = a.st.pos + (size_t)pair * B;
@@ -443,6 +430,7 @@ __global__ void __launch_bounds__(NT, 1) ingest_cluster_kernel(ClArgs<T> a) {
       dk[i] = ku[i];
       dv[i] = vu[i];
     }
+    int min_now = -1;
     if (ev_nv == B) {
       if (reg_min) {
         // block of the replaced slot from the prefetched priorities, then the head minimum
@@ -472,13 +460,15 @@ __global__ void __launch_bounds__(NT, 1) ingest_cluster_kernel(ClArgs<T> a) {
           a.st.min_score[pair] = m;
           a.st.min_slot[pair] = mi;
         }
+        min_now = mi;
       } else {
-        update_min(sc, dm.s, B, slot, prio, bsc, bsl, a.st.min_score + pair, a.st.min_slot + pair);
+        min_now = update_min(sc, dm.s, B, slot, prio, bsc, bsl, a.st.min_score + pair, a.st.min_slot + pair);
       }
     } else if (ev_nv + 1 == B) {
-      rebuild_min(sc, dm.s, B, slot, prio, bsc, bsl, a.st.min_score + pair, a.st.min_slot + pair);
+      min_now = rebuild_min(sc, dm.s, B, slot, prio, bsc, bsl, a.st.min_score + pair, a.st.min_slot + pair);
     }
     if (lane == 0) {
+      a.st.step_slots[pair] = make_int2(min_now, slot);
       sc[slot] = prio;
       ps[slot] = u;
       a.st.nvalid[pair] = ev_nv < B ? ev_nv + 1 : ev_nv;
@@ -498,12 +488,13 @@ int cluster_ingest_fs(const Dims& dm) { return ((dm.F + 31) / 32 * 32) / CS; }
 
 bool cluster_ingest_ok(const Dims& dm) {
   const int FS = cluster_ingest_fs(dm);
-  const ClLayout L = cl_layout(dm.d, dm.D, dm.G, FS, dm.dtype == KVPOP_F32 ? 4 : 2);
-  return FS <= 64 && L.total <= 200 * 1024;
+  const ClLayout L = cl_layout(dm.d, dm.G, FS, dm.dtype == KVPOP_F32 ? 4 : 2);
+  // a CTA reads its two sequences' windows by itself: up to 190 tokens of d = 128
+  return FS <= 64 && L.total - NT * SBC * 4 + OWN * dm.D * dm.d * 4 <= 200 * 1024;
 }
 
 size_t cluster_ingest_smem(const Dims& dm) {
-  return cl_layout(dm.d, dm.D, dm.G, cluster_ingest_fs(dm), dm.dtype == KVPOP_F32 ? 4 : 2).total;
+  return cl_layout(dm.d, dm.G, cluster_ingest_fs(dm), dm.dtype == KVPOP_F32 ? 4 : 2).total;
 }
 
 cudaError_t prepare_ingest_cluster(const Dims& dm) {

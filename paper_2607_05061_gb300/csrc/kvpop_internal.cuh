@@ -84,6 +84,8 @@ struct State {                 // device pointers of one cache
   int32_t* len;                // [pairs]         tokens seen (same for all heads of a sequence)
   float* min_score;            // [pairs]         argmin over slots [s, B) when full
   int32_t* min_slot;           // [pairs]
+  int2* step_slots;            // [pairs]         (min_slot, slot last written), written as one word;
+                               //                 the first is -1 until the pair is full
   float* blk_score;            // [pairs][NB]     per-block minima (blocks of 64 slots)
   int32_t* blk_slot;           // [pairs][NB]
   // scorer (hidden width padded to Fp = F rounded up to 4, zero weights)
@@ -168,8 +170,9 @@ cudaError_t launch_prefill_select(const State& st, const Dims& dm, const void* Q
 size_t tc_maps_size();
 cudaError_t tc_make_maps(const State& st, const Dims& dm, void* maps_out);
 cudaError_t tc_config(const Dims& dm, AttendConfig* out);
+// after_ingest: the launch before it on the stream is this cache's ingest.
 cudaError_t tc_launch(const State& st, const Dims& dm, const void* maps, const void* q, float* out,
-                      int grid, cudaStream_t stream);
+                      int grid, bool after_ingest, cudaStream_t stream);
 // The whole decode step in one tensor-core kernel (bf16, d = 128, F <= 256): attention over
 // the keys that cannot change this step while extra warps run the delayed scorer,
 // keep-or-drop and scatter; each pair's last arrival merges.
@@ -255,11 +258,11 @@ __device__ __forceinline__ float canon_score(float r) {
 }
 
 // Static priority (App. B.3, decay step n = 1) in explicit fp32 ops.
+__device__ __forceinline__ float decayed(float r, int u, float lg) {
+  return lg == 0.0f ? r : canon_score(__fsub_rn(r, __fmul_rn((float)u, lg)));
+}
 __device__ __forceinline__ float static_priority(float r, int u, const float* log_gamma, int h) {
-  if (log_gamma == nullptr) return r;
-  float lg = log_gamma[h];
-  if (lg == 0.0f) return r;
-  return canon_score(__fsub_rn(r, __fmul_rn((float)u, lg)));
+  return decayed(r, u, log_gamma == nullptr ? 0.0f : log_gamma[h]);
 }
 
 // Exact-erf GELU.

@@ -158,10 +158,11 @@ __global__ void __launch_bounds__(NTM, 1) ingest_mlstm_kernel(MIngestArgs<T> a) 
     for (uint32_t off = 0; off < bytes; off += 32768)
       bulk_g2s(smem_u32(smem + off), src + off, min(32768u, bytes - off), smem_u32(&bar));
   }
-  // the attention may be scheduled now; the weights above never change, all that follows is
-  // state or input that the kernel before this one may still write
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // The weights above never change, all that follows is state or input that the kernel before
+  // this one may still write.  The attention may be scheduled after that, and not earlier: it
+  // starts on keys that this step does not change.
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   T* ringK = static_cast<T*>(a.st.ringK);
   T* ringV = static_cast<T*>(a.st.ringV);
   {

@@ -629,11 +629,16 @@ __global__ void __launch_bounds__(NT2) prefill_select_kernel(SelectArgs<T> a) {
       int mi = 0x7fffffff;
       for (int k = lane; k < NB; k += 32) lex_min(m, mi, __ldcg(bsc + k), __ldcg(bsl + k));
       warp_lex_min(m, mi);
-      if (lane == 0) { a.st.min_score[pair] = m; a.st.min_slot[pair] = mi; }
+      if (lane == 0) {
+        a.st.min_score[pair] = m;
+        a.st.min_slot[pair] = mi;
+        a.st.step_slots[pair] = make_int2(mi, mi);
+      }
     }
   } else if (c == 0 && tid == 0) {
     a.st.min_score[pair] = INFINITY;
     a.st.min_slot[pair] = -1;
+    a.st.step_slots[pair] = make_int2(-1, -1);
   }
   if (c == 0 && tid == 0) {
     a.st.nvalid[pair] = nkept;

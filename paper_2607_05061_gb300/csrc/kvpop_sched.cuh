@@ -9,6 +9,8 @@
 // order, which keeps the result independent of arrival order.
 #pragma once
 
+#include <type_traits>
+
 #include "kvpop_internal.cuh"
 
 namespace kvpop {
@@ -80,9 +82,11 @@ __device__ __forceinline__ bool schedule_changed(const int32_t* __restrict__ nva
 // A partial's place is fixed by the split: the pair's first tile lies in CTA ca (second slot
 // of its two), every later CTA starts inside the pair (first slot).  The (max, sum) pairs are
 // fetched once for all threads into `fac` (2 G (cb - ca + 1) floats of shared memory), and the
-// rows are loaded 8 at a time, so a merge costs a few L2 latencies instead of one chain of
-// 2 (cb - ca + 1) per thread: a pair at batch 1 spreads over 19 CTAs, and a 4-layer step there
-// went from 316 to 235 us with this and the early launches below.
+// rows are loaded 20 at a time with them, so a merge costs an L2 latency or two instead of one
+// chain of 2 (cb - ca + 1) per thread: a pair at batch 1 spreads over 19 CTAs,
+// and from its last arrival to the end of the launch went 8 us with 8 single rows in flight, 6
+// with 20 double ones (a 4-layer step at batch 1: 316 us with the chain, 235 with this and the
+// early launches below).
 constexpr int kMaxAttendGrid = 256;      // CTAs whose factors fit in the warps' partials (4 HD)
 
 template <int G, int HD, int NCT, typename SyncFn, typename ExpFn>
@@ -98,26 +102,40 @@ __device__ __forceinline__ void merge_partials(long long ca, long long cb, const
     fac[2 * i] = __ldcg(pc);
     fac[2 * i + 1] = __ldcg(pc + G);
   }
+  // V neighbouring outputs per thread, RB rows in flight; the first ones travel with the factors
+  constexpr int V = (G * HD) % (2 * NCT) == 0 ? 2 : 1, RB = 20;
+  using Vec = std::conditional_t<V == 2, float2, float>;
+  auto load = [&](Vec (&row)[RB], int c0, int idx) {
+#pragma unroll
+    for (int k = 0; k < RB; ++k)
+      if (c0 + k < n) row[k] = __ldcg(reinterpret_cast<const Vec*>(at(c0 + k) + idx));
+  };
+  Vec row[RB];
+  if (V * tid < G * HD) load(row, 0, V * tid);
   sync();
-  for (int idx = tid; idx < G * HD; idx += NCT) {
-    const int g = idx / HD, i = idx - g * HD;
+  for (int idx = V * tid; idx < G * HD; idx += V * NCT) {
+    const int g = idx / HD;
     float ms = -INFINITY;
     for (int c = 0; c < n; ++c) ms = fmaxf(ms, fac[2 * (c * G + g)]);
-    float L = 0.f, O = 0.f;
-    for (int c0 = 0; c0 < n; c0 += 8) {
-      float row[8];
+    float L = 0.f, O[V] = {};
+    for (int c0 = 0; c0 < n; c0 += RB) {
+      if (c0 > 0 || idx >= V * NCT) load(row, c0, idx);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) row[k] = c0 + k < n ? __ldcg(at(c0 + k) + g * HD + i) : 0.f;
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
+      for (int k = 0; k < RB; ++k) {
         if (c0 + k >= n) break;
         const float mc = fac[2 * ((c0 + k) * G + g)];
         const float f = (mc == -INFINITY) ? 0.f : ex(mc - ms);
         L = fmaf(fac[2 * ((c0 + k) * G + g) + 1], f, L);
-        O = fmaf(row[k], f, O);
+        if constexpr (V == 2) {
+          O[0] = fmaf(row[k].x, f, O[0]);
+          O[1] = fmaf(row[k].y, f, O[1]);
+        } else {
+          O[0] = fmaf(row[k], f, O[0]);
+        }
       }
     }
-    out[(size_t)g * HD + i] = O / L;
+#pragma unroll
+    for (int v = 0; v < V; ++v) out[idx + v] = O[v] / L;
   }
 }
 

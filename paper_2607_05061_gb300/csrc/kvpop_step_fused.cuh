@@ -138,10 +138,6 @@ __device__ __forceinline__ const float* pair_partial(const float* part, const fl
   return part + ((size_t)c * 2 + slot) * PSTRIDE;
 }
 
-__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
 // Online merge of one more (max, sum, output) part into a running (M, L, O), log2 domain.
 __device__ __forceinline__ void merge_part(float& M, float& L, float& O, float m, float l, float o) {
   if (m == -INFINITY) return;
