@@ -149,7 +149,10 @@ __device__ __forceinline__ void consumer_sync() {
 // FUSED: the whole decode step (kvpop_step_fused.cuh): the consumers stream only the keys
 // that cannot change this step, the scorer warps ingest the new token meanwhile, and each
 // pair's last arrival merges.  Otherwise the attention alone, over the state the ingest left.
-template <int HD, int G, bool FUSED>
+// TAIL: V rows past a tile's last key are zeroed.  The one-kernel step goes without where whole
+// 16-key groups of the window exist (at its register limit the code costs 0.5% even where it
+// does not run: cr8x 164.3 -> 164.8 us); its slots past the used ones hold zeros.
+template <int HD, int G, bool FUSED, bool TAIL>
 __global__ void __launch_bounds__(FUSED ? TcTraits<HD, G>::THREADS_F : TcTraits<HD, G>::THREADS,
                                   KVPOP_TC_MINBLOCKS)
     attend_tc_kernel(const __grid_constant__ CUtensorMap mapSK, const __grid_constant__ CUtensorMap mapSV,
@@ -214,8 +217,8 @@ __global__ void __launch_bounds__(FUSED ? TcTraits<HD, G>::THREADS_F : TcTraits<
     // of the two slots in step_slots.  An ingest that writes slot s turns (s, .) into
     // (next minimum, s) in one word, so s is named whichever it meets.  Tiles are taken in the
     // order and by the warps they always are: the result is the same bit for bit.  Every pair's
-    // window tile waits, so this grid never completes before the ingest has.  With this, the
-    // ingest on two CTAs an SM (see there) and the merge's wider loads, an ingest and attention
+    // window tile waits, so this grid never completes before the ingest has.  With this, a
+    // shorter ingest (see there) and the merge's wider loads, an ingest and attention
     // of 3072 slots take 18.3 us at batch 1 (24.7 with the wait first) and 34.3 at batch 8 (38.8);
     // with the mLSTM ingest at batch 64 a step takes 182 us (184).
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -540,7 +543,7 @@ __global__ void __launch_bounds__(FUSED ? TcTraits<HD, G>::THREADS_F : TcTraits<
     if (ok && key0 < cnt) {
       const uint32_t kbase = smem_u32(smem + (size_t)s * Tr::STAGE_BYTES);
       const uint32_t vbase = kbase + NH * Tr::HALF_BYTES;
-      if (key0 + 16 > cnt) {
+      if (TAIL && key0 + 16 > cnt) {
         // Rows past the last key hold whatever was in shared memory (a window box is narrower
         // than its tile) or in the store: their weight is 0, and so has their V to be, for
         // 0 times an infinity or NaN would reach the sums.
@@ -697,7 +700,7 @@ cudaError_t tc_config(const Dims& dm, AttendConfig* out) {
     out->threads = TcTraits<HD_, G_>::THREADS;                         \
     out->smem_fixed = tc_smem<HD_, G_>(0) - 4;                         \
     out->tile = TcTraits<HD_, G_>::TILE;                               \
-    out->func = (const void*)attend_tc_kernel<HD_, G_, false>;         \
+    out->func = (const void*)attend_tc_kernel<HD_, G_, false, true>;   \
     return cudaSuccess;                                                \
   }
   TC_CASES(CFG)
@@ -723,7 +726,8 @@ cudaError_t tc_fused_config(const Dims& dm, AttendConfig* out) {
     out->threads = TcTraits<HD_, G_>::THREADS_F;                               \
     out->smem_fixed = tc_fused_smem_of(tc_smem<HD_, G_>(0) - 4, dm.Fp) + 16;   \
     out->tile = TcTraits<HD_, G_>::TILE;                                       \
-    out->func = (const void*)attend_tc_kernel<HD_, G_, true>;                  \
+    out->func = dm.D % 16 ? (const void*)attend_tc_kernel<HD_, G_, true, true> \
+                          : (const void*)attend_tc_kernel<HD_, G_, true, false>; \
     return cudaSuccess;                                                        \
   }
   if (tc_fused_ok(dm)) { TC_FUSED_CASES(CFG) }
@@ -774,7 +778,7 @@ cudaError_t tc_launch(const State& st, const Dims& dm, const void* maps, const v
   if (dm.d == HD_ && dm.G == G_) {                                                        \
     cfg.blockDim = dim3(TcTraits<HD_, G_>::THREADS, 1, 1);                                \
     cfg.dynamicSmemBytes = tc_smem<HD_, G_>(dm.pairs);                                    \
-    return cudaLaunchKernelEx(&cfg, attend_tc_kernel<HD_, G_, false>, m->sk, m->sv, m->rk, \
+    return cudaLaunchKernelEx(&cfg, attend_tc_kernel<HD_, G_, false, true>, m->sk, m->sv, m->rk, \
                               m->rv, a, f);                                               \
   }
   TC_CASES(LAUNCH)
@@ -822,8 +826,9 @@ cudaError_t tc_launch_fused(const State& st, const Dims& dm, const void* maps, c
   if (dm.d == HD_ && dm.G == G_) {                                                         \
     cfg.blockDim = dim3(TcTraits<HD_, G_>::THREADS_F, 1, 1);                               \
     cfg.dynamicSmemBytes = tc_fused_smem_of(tc_smem<HD_, G_>(dm.pairs), dm.Fp);            \
-    return cudaLaunchKernelEx(&cfg, attend_tc_kernel<HD_, G_, true>, m->sk, m->sv, m->rk,  \
-                              m->rv, a, f);                                                \
+    return cudaLaunchKernelEx(&cfg, dm.D % 16 ? attend_tc_kernel<HD_, G_, true, true>      \
+                                              : attend_tc_kernel<HD_, G_, true, false>,    \
+                              m->sk, m->sv, m->rk, m->rv, a, f);                           \
   }
   TC_FUSED_CASES(LAUNCH)
 #undef LAUNCH

@@ -15,11 +15,11 @@
 // The state the eviction reads (used slots, the cached minimum, its block) is
 // loaded at kernel start so its latency hides behind the scorer.
 //
-// Bound by latency: five dependent passes over L2 and two cluster barriers.  Without the
-// window in shared memory (131 KB of the 184 it took) two CTAs share an SM, which leaves 120 of
-// 152 SMs to the attention meanwhile; stores that a barrier's release would wait for come after
-// the barriers.  Batch 1, d = 128, F = 256, window 128, from its wait to the end: 14.2 -> 11.7 us
-// beside the attention, 14.2 -> 12.5 us alone.
+// Bound by latency: dependent passes over L2 and two cluster barriers.  95 KB of shared memory
+// whatever the window (209 with a window of 128 held there): two CTAs share an SM, which leaves
+// 120 of 152 SMs to the attention meanwhile.  Stores that a barrier's release would wait for come
+// after the barriers.  Batch 1, d = 128, F = 256, window 16, beside the attention, from its wait
+// to the end: 14.2 -> 11.7 us (of the scorer: 4.9 -> 2.8).
 #include "kvpop_argmin.cuh"
 
 namespace kvpop {

@@ -40,3 +40,30 @@ def test_nothing_past_the_last_key(cuda_device, dtype, tol, B, D, n, d):
                 assert (out[s, h * G + g].double() - w @ v).abs().max() <= tol
     assert torch.isfinite(out).all()
     cache.free()
+
+
+@pytest.mark.parametrize("D,B,n", [(5, 40, 60), (17, 129, 200), (16, 40, 60), (16, 40, 50)])
+def test_one_kernel_step_past_the_last_key(cuda_device, monkeypatch, D, B, n):
+    """The one-kernel step over the same: finite, and equal to the two kernels within the
+    rounding of the probabilities."""
+    from paper_2607_05061_gb300 import kvpop
+    b, H, G, d = 9, 2, 4, 128
+    z = torch.zeros
+    K, V, Q = (randn((b, h, n, d), 3 + i, cuda_device, torch.bfloat16) for i, h in enumerate((H, H, H * G)))
+    q, k, v = (randn((b, h * d), 9 + i, cuda_device, torch.bfloat16) for i, h in enumerate((H * G, H, H)))
+    nan = torch.full((2048, 2048), float("nan"), dtype=torch.bfloat16, device=cuda_device)
+    outs = []
+    for name, other in (("KVPOP_FUSED_STEP", "KVPOP_SPLIT_STEP"), ("KVPOP_SPLIT_STEP", "KVPOP_FUSED_STEP")):
+        monkeypatch.delenv(other, raising=False)
+        monkeypatch.setenv(name, "1")
+        cache = kvpop.KVpopCache(b, H, G, d, B, D, 4, torch.bfloat16, z(H, 3 * d, 4), z(H, 4), z(H, 4), z(H))
+        assert kvpop.kvpop_step_is_fused(cache.handle) == (name == "KVPOP_FUSED_STEP")
+        cache.prefill(Q, K, V, [n] * b)
+        out = torch.empty((b, H * G, d), device=cuda_device)
+        torch.matmul(nan, nan)
+        cache.step(q, k, v, out)
+        cache.check()
+        outs.append(out)
+        cache.free()
+    assert torch.isfinite(outs[0]).all()
+    assert (outs[0] - outs[1]).abs().max() <= 1e-2
