@@ -1070,10 +1070,10 @@ def run_prompt_bench(args):
     metric, what = prompt_metric(args.workload)
     if args.workload == "prompt":
         kname = (("prompt_t5_kernel" if d == 128 and not os.environ.get("KVPOP_PROMPT_MMA_SYNC")
-                  else "prompt_tc_kernel") if cfg.kv_dtype == "bf16" else "prompt_simt_kernel")
+                  else "prompt_tc_kernel") if cfg.kv_dtype == "bf16" else "prompt_f32_kernel")
     else:
-        kname = (("target_t5_kernel" if d == 128 and not os.environ.get("KVPOP_TARGET_MMA_SYNC")
-                  else "target_tc_kernel") if cfg.kv_dtype == "bf16" else "target_simt_kernel")
+        kname = (("lse_t5_kernel" if d == 128 and not os.environ.get("KVPOP_TARGET_MMA_SYNC")
+                  else "target_tc_kernel") if cfg.kv_dtype == "bf16" else "target_f32_kernel")
     rec = {
         "metric": metric, "value": tokens / (step_ms / 1e3), "unit": "tokens/s", "n_gpus": world,
         "steps": Kn, "warmup": W, "ms_per_step": step_ms, "higher_is_better": True,
