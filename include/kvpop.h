@@ -377,6 +377,19 @@ kvpop_status kvpop_project_out(const float* o_dev, const void* Wo_dev, const voi
                                int32_t batch, int32_t n_q, int32_t hidden, void* y_dev,
                                cudaStream_t stream);
 
+/* The same for settled weights: every kernel and copy that writes them has completed before
+ * the work queued last on `stream` starts.  Their weights are read while that work still runs;
+ * the two calls above read them after it, as any kernel does.  In a layer stack's step on one
+ * stream the first projection takes the plain form and the ones behind it these: no projection
+ * lets anything behind it start before all that precedes it is complete. */
+kvpop_status kvpop_project_qkv_settled(const void* x_dev, const void* Wq_dev, const void* Wk_dev,
+                                       const void* Wv_dev, int32_t batch, int32_t hidden,
+                                       int32_t n_q, int32_t n_kv, void* q_dev, void* k_dev,
+                                       void* v_dev, cudaStream_t stream);
+kvpop_status kvpop_project_out_settled(const float* o_dev, const void* Wo_dev, const void* x_dev,
+                                       int32_t batch, int32_t n_q, int32_t hidden, void* y_dev,
+                                       cudaStream_t stream);
+
 /* Allocation-free decode attention (no counterpart in the paper: it is an
  * interface convenience).  For callers that may not allocate device memory
  * when they decode -- a serving loop whose device memory is fixed up front and

@@ -721,23 +721,45 @@ int32_t kvpop_project_supported(int32_t batch, int32_t hidden, int32_t n_q, int3
          (proj_ok(batch, n_q, hidden, true) ? 2 : 0);
 }
 
-kvpop_status kvpop_project_qkv(const void* x, const void* Wq, const void* Wk, const void* Wv,
-                               int32_t batch, int32_t hidden, int32_t n_q, int32_t n_kv, void* q,
-                               void* k, void* v, cudaStream_t stream) {
+static kvpop_status project_qkv(const void* x, const void* Wq, const void* Wk, const void* Wv,
+                                int32_t batch, int32_t hidden, int32_t n_q, int32_t n_kv, void* q,
+                                void* k, void* v, bool settled, cudaStream_t stream) {
   if (!proj_ok(batch, hidden, n_q, false) || !proj_ok(batch, hidden, n_kv, false) || !x || !Wq || !Wk || !Wv ||
       !q || !k || !v)
     return KVPOP_ERR_INVALID_ARG;
   if (!aligned16(x) || !aligned16(Wq) || !aligned16(Wk) || !aligned16(Wv) || !aligned16(q) ||
       !aligned16(k) || !aligned16(v))
     return KVPOP_ERR_ALIGN;
-  return from_cuda(NOTE(launch_proj_qkv(x, Wq, Wk, Wv, batch, hidden, n_q, n_kv, q, k, v, stream)));
+  return from_cuda(NOTE(launch_proj_qkv(x, Wq, Wk, Wv, batch, hidden, n_q, n_kv, q, k, v, settled, stream)));
+}
+
+static kvpop_status project_out(const float* o, const void* Wo, const void* x, int32_t batch,
+                                int32_t n_q, int32_t hidden, void* y, bool settled, cudaStream_t stream) {
+  if (!proj_ok(batch, n_q, hidden, true) || !o || !Wo || !x || !y) return KVPOP_ERR_INVALID_ARG;
+  if (!aligned16(o) || !aligned16(Wo) || !aligned16(x) || !aligned16(y)) return KVPOP_ERR_ALIGN;
+  return from_cuda(NOTE(launch_proj_out(o, Wo, x, batch, n_q, hidden, y, settled, stream)));
+}
+
+kvpop_status kvpop_project_qkv(const void* x, const void* Wq, const void* Wk, const void* Wv,
+                               int32_t batch, int32_t hidden, int32_t n_q, int32_t n_kv, void* q,
+                               void* k, void* v, cudaStream_t stream) {
+  return project_qkv(x, Wq, Wk, Wv, batch, hidden, n_q, n_kv, q, k, v, false, stream);
+}
+
+kvpop_status kvpop_project_qkv_settled(const void* x, const void* Wq, const void* Wk, const void* Wv,
+                                       int32_t batch, int32_t hidden, int32_t n_q, int32_t n_kv,
+                                       void* q, void* k, void* v, cudaStream_t stream) {
+  return project_qkv(x, Wq, Wk, Wv, batch, hidden, n_q, n_kv, q, k, v, true, stream);
 }
 
 kvpop_status kvpop_project_out(const float* o, const void* Wo, const void* x, int32_t batch,
                                int32_t n_q, int32_t hidden, void* y, cudaStream_t stream) {
-  if (!proj_ok(batch, n_q, hidden, true) || !o || !Wo || !x || !y) return KVPOP_ERR_INVALID_ARG;
-  if (!aligned16(o) || !aligned16(Wo) || !aligned16(x) || !aligned16(y)) return KVPOP_ERR_ALIGN;
-  return from_cuda(NOTE(launch_proj_out(o, Wo, x, batch, n_q, hidden, y, stream)));
+  return project_out(o, Wo, x, batch, n_q, hidden, y, false, stream);
+}
+
+kvpop_status kvpop_project_out_settled(const float* o, const void* Wo, const void* x, int32_t batch,
+                                       int32_t n_q, int32_t hidden, void* y, cudaStream_t stream) {
+  return project_out(o, Wo, x, batch, n_q, hidden, y, true, stream);
 }
 
 kvpop_status kvpop_standalone_status(cudaStream_t stream) {

@@ -240,12 +240,13 @@ cudaError_t launch_future_target(const void* Q, const void* K, const float* lse,
                                  float* logm, float* target, int agg, int count_norm, float eps,
                                  int32_t* err, cudaStream_t stream);
 
-// Projections of the decode stack (M rows of K, N columns).
+// Projections of the decode stack (M rows of K, N columns).  settled: no kernel that may still
+// run at the launch writes the weights.
 bool proj_ok(int M, int K, int N, bool x_f32);
 cudaError_t launch_proj_qkv(const void* x, const void* Wq, const void* Wk, const void* Wv, int M, int K,
-                            int nq, int nkv, void* q, void* k, void* v, cudaStream_t stream);
+                            int nq, int nkv, void* q, void* k, void* v, bool settled, cudaStream_t stream);
 cudaError_t launch_proj_out(const float* o, const void* Wo, const void* res, int M, int K, int N,
-                            void* y, cudaStream_t stream);
+                            void* y, bool settled, cudaStream_t stream);
 
 // ------------------------------------------------------------------ device helpers
 __device__ __forceinline__ float to_f(float x) { return x; }

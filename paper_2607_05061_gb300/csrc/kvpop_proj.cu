@@ -6,9 +6,11 @@
 // over the whole contraction, so nothing is exchanged between CTAs.  Each of its 8 warps takes
 // its own part of the contraction through a private ring of cp.async stages (32 weight rows of
 // up to 96 bytes, and the same 32 columns of x), with no barrier until the warps' fp32 sums
-// meet in shared memory at the end, in warp order.  The weights depend on no earlier kernel:
-// the ring is filled with them before griddepcontrol.wait, while the kernel before this one
-// still runs.  The products run on mma.sync with the weights as the 16-row operand and the
+// meet in shared memory at the end, in warp order.  While the kernel before this one still runs,
+// the first stages' weights go to L2, which is only a hint and so needs no order with a kernel
+// that may write them, and into the ring after griddepcontrol.wait; weights that the caller
+// states to be settled go into the ring at once.  The next kernel may start after that wait, and
+// so after all that came before this one.  The products run on mma.sync with the weights as the 16-row operand and the
 // sequences as the 8-column one: at so few rows the tensor work is far below the stream.
 // Device time at hidden 4096, 32 query and 8 KV heads, alone and cold: q, k, v at 1 to 8 rows
 // 14 us (7.5 us at the copy rate) against 32 us of cuBLAS's six launches, the output 13 us
@@ -36,6 +38,7 @@ struct ProjArgs {
   int groups[3];                       // column groups up to and including matrix i
   int N[3];
   int M, K;
+  int settled;                         // nothing that may still run writes the weights
 };
 
 template <int MT, bool XF32>
@@ -67,8 +70,6 @@ __global__ void __launch_bounds__(PJ_NT, 1) proj_kernel(ProjArgs a) {
     m = c < a.groups[0] ? 0 : c < a.groups[1] ? 1 : 2;
     return (c - (m ? a.groups[m - 1] : 0)) * 8;
   };
-  // the next kernel may be scheduled now; it waits for this grid before it reads anything
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   // the warp's stages of the contraction
   const int nst = K / PJ_KS;
@@ -110,11 +111,26 @@ __global__ void __launch_bounds__(PJ_NT, 1) proj_kernel(ProjArgs a) {
                  m < a.M ? 16 : 0);
     }
   };
+  if (a.settled) {
 #pragma unroll
-  for (int s = 0; s < ST; ++s)
-    if (s < ns) load_w(s);
+    for (int s = 0; s < ST; ++s)
+      if (s < ns) load_w(s);
+  } else {
+#pragma unroll
+    for (int s = 0; s < ST; ++s)
+#pragma unroll
+      for (int j = 0; j < PJ_NG; ++j)
+        if (s < ns && j < ng) prefetch_l2_line(src[j] + s * step[j]);
+  }
   cp_commit();
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  // a kernel that starts from here on starts after all that precedes this one
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (!a.settled) {
+#pragma unroll
+    for (int s = 0; s < ST; ++s)
+      if (s < ns) load_w(s);
+  }
 #pragma unroll
   for (int s = 0; s < ST; ++s) {
     if (s < ns) load_x(s);
@@ -232,8 +248,9 @@ bool proj_ok(int M, int K, int N, bool x_f32) {
 }
 
 cudaError_t launch_proj_qkv(const void* x, const void* Wq, const void* Wk, const void* Wv, int M, int K,
-                            int nq, int nkv, void* q, void* k, void* v, cudaStream_t stream) {
+                            int nq, int nkv, void* q, void* k, void* v, bool settled, cudaStream_t stream) {
   ProjArgs a{};
+  a.settled = settled;
   a.x = x;
   const void* W[3] = {Wq, Wk, Wv};
   void* y[3] = {q, k, v};
@@ -250,8 +267,9 @@ cudaError_t launch_proj_qkv(const void* x, const void* Wq, const void* Wk, const
 }
 
 cudaError_t launch_proj_out(const float* o, const void* Wo, const void* res, int M, int K, int N,
-                            void* y, cudaStream_t stream) {
+                            void* y, bool settled, cudaStream_t stream) {
   ProjArgs a{};
+  a.settled = settled;
   a.x = o;
   a.W[0] = static_cast<const bf16*>(Wo);
   a.y[0] = static_cast<bf16*>(y);

@@ -90,6 +90,9 @@ _SIGS = {
     "kvpop_project_qkv": (ctypes.c_int, [_P, _P, _P, _P, c_int32, c_int32, c_int32, c_int32, _P, _P, _P,
                                          _P]),
     "kvpop_project_out": (ctypes.c_int, [_P, _P, _P, c_int32, c_int32, c_int32, _P, _P]),
+    "kvpop_project_qkv_settled": (ctypes.c_int, [_P, _P, _P, _P, c_int32, c_int32, c_int32, c_int32, _P,
+                                                 _P, _P, _P]),
+    "kvpop_project_out_settled": (ctypes.c_int, [_P, _P, _P, c_int32, c_int32, c_int32, _P, _P]),
     "kvpop_standalone_status": (ctypes.c_int, [_P]),
     "kvpop_last_error": (ctypes.c_char_p, []),
     "kvpop_debug_fail_alloc_after": (None, [c_int32]),
@@ -314,17 +317,21 @@ def future_target(Q, K, lse, window: int, lookahead: int = 0, agg: str = "max",
     return logm, target
 
 
-def project_qkv(x, Wq, Wk, Wv, q, k, v, stream=None):
+def project_qkv(x, Wq, Wk, Wv, q, k, v, stream=None, settled=False):
     """``q, k, v = bf16(x Wq), bf16(x Wk), bf16(x Wv)`` (contiguous bf16, up to 64 rows) in one
-    launch."""
-    _ck(kvpop_project_qkv(_ptr(x), _ptr(Wq), _ptr(Wk), _ptr(Wv), x.shape[0], x.shape[1], Wq.shape[1],
-                          Wk.shape[1], _ptr(q), _ptr(k), _ptr(v), _stream(stream)), "kvpop_project_qkv")
+    launch.  ``settled``: whatever writes the weights has completed before the work queued last
+    on the stream starts; they are then read while that work runs."""
+    f = kvpop_project_qkv_settled if settled else kvpop_project_qkv
+    _ck(f(_ptr(x), _ptr(Wq), _ptr(Wk), _ptr(Wv), x.shape[0], x.shape[1], Wq.shape[1], Wk.shape[1],
+          _ptr(q), _ptr(k), _ptr(v), _stream(stream)), "kvpop_project_qkv")
 
 
-def project_out(o, Wo, x, y, stream=None):
-    """``y = bf16(x + bf16(bf16(o) Wo))`` (``o`` fp32, the others contiguous bf16) in one launch."""
-    _ck(kvpop_project_out(_ptr(o), _ptr(Wo), _ptr(x), x.shape[0], Wo.shape[0], x.shape[1], _ptr(y),
-                          _stream(stream)), "kvpop_project_out")
+def project_out(o, Wo, x, y, stream=None, settled=False):
+    """``y = bf16(x + bf16(bf16(o) Wo))`` (``o`` fp32, the others contiguous bf16) in one launch;
+    ``settled`` as in ``project_qkv``."""
+    f = kvpop_project_out_settled if settled else kvpop_project_out
+    _ck(f(_ptr(o), _ptr(Wo), _ptr(x), x.shape[0], Wo.shape[0], x.shape[1], _ptr(y), _stream(stream)),
+        "kvpop_project_out")
 
 
 def parse_state(blob: bytes, cfg: kvpop_config) -> dict:

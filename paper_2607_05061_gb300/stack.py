@@ -82,14 +82,19 @@ class DecodeStack:
 
     # ------------------------------------------------------------------ decode
     def _step_into(self, x_in: torch.Tensor, x_out: torch.Tensor, overrides=None,
-                   evict_info=None, outputs=None):
+                   evict_info=None, outputs=None, settled=False):
+        # ``settled``: no kernel that may write weights can still run beside the projections.  It
+        # holds behind the first of them, which lets nothing start before all that precedes it is
+        # complete; before that only where the caller knows it.
         x = x_in
         for l, (L, cache) in enumerate(zip(self.layers, self.caches)):
             nxt = self.x[l % 2] if l + 1 < len(self.layers) else x_out
             nq, nkv, hid = self.q.shape[1], self.k.shape[1], self.hidden
             if self._project & 1 and self._plain((x, (self.b, hid)), (L["Wq"], (hid, nq)),
                                                  (L["Wk"], (hid, nkv)), (L["Wv"], (hid, nkv))):
-                project_qkv(x, L["Wq"], L["Wk"], L["Wv"], self.q, self.k, self.v)
+                project_qkv(x, L["Wq"], L["Wk"], L["Wv"], self.q, self.k, self.v,
+                            settled=settled)
+                settled = True
             else:
                 torch.matmul(x, L["Wq"], out=self.q)
                 torch.matmul(x, L["Wk"], out=self.k)
@@ -101,7 +106,8 @@ class DecodeStack:
                 outputs[l].copy_(self.o)
             if self._project & 2 and self._plain((x, (self.b, hid)), (nxt, (self.b, hid)),
                                                  (L["Wo"], (nq, hid))):
-                project_out(self.o, L["Wo"], x, nxt)
+                project_out(self.o, L["Wo"], x, nxt, settled=settled)
+                settled = True
             else:
                 self.o_bf.copy_(self.o)
                 torch.matmul(self.o_bf, L["Wo"], out=self.y)
@@ -123,7 +129,8 @@ class DecodeStack:
         g = torch.cuda.CUDAGraph()
         with torch.cuda.stream(s):
             with torch.cuda.graph(g, stream=s):
-                self._step_into(x_in, x_out)
+                # a replay starts after all that is queued before it is complete
+                self._step_into(x_in, x_out, settled=True)
         torch.cuda.current_stream().wait_stream(s)
         self.graph = g
         return g
