@@ -408,8 +408,9 @@ constexpr int T6_QB = T6_BN * 256;              // column block, bytes
 constexpr int T6_OFF_LSE = T6_ST * T6_QB;
 constexpr int T6_OFF_BAR = T6_OFF_LSE + T6_ST * T6_BN * 4;
 constexpr int T6_OFF_TMEM = T6_OFF_BAR + 8 * 32;
-constexpr int T6_OFF_PX = T6_OFF_TMEM + 16;      // [2 head parity][2 halves][128 rows][m, l, seq, -]
-constexpr int T6_SMEM = T6_OFF_PX + 2 * 2 * T6_HALF * 16 + 1024;   // 1024: swizzle atom alignment
+constexpr int T6_OFF_PX = T6_OFF_TMEM + 16;      // [query head][2 halves][128 rows][m, l, done, -]
+constexpr int T6_MAX_G = 4;                      // query heads per KV head
+constexpr int T6_SMEM = T6_OFF_PX + T6_MAX_G * 2 * T6_HALF * 16 + 1024;   // 1024: swizzle atom alignment
 constexpr int T6_FULL = 0, T6_EMPTY = T6_ST, T6_SFULL = 2 * T6_ST, T6_PFULL = 2 * T6_ST + 3,
               T6_AFULL = 2 * T6_ST + 6;
 // tensor memory: the row tiles of the two halves (64 columns each, two bf16 per word), then
@@ -480,7 +481,8 @@ __global__ void __launch_bounds__(T6_THREADS, 1)
     mbar_fence_init();
   }
   // the softmax halves' exchange slots start with no head done
-  for (int i = tid; i < 2 * 2 * T6_HALF; i += T6_THREADS) reinterpret_cast<int*>(sm6 + T6_OFF_PX)[4 * i + 2] = 0;
+  static_assert(G <= T6_MAX_G, "one slot per head");
+  for (int i = tid; i < G * 2 * T6_HALF; i += T6_THREADS) reinterpret_cast<int*>(sm6 + T6_OFF_PX)[4 * i + 2] = 0;
   if (warp == T6_MMA_WARP) tmem_alloc(sb + T6_OFF_TMEM, 512);
   fence_before();
   __syncthreads();
@@ -692,19 +694,20 @@ __global__ void __launch_bounds__(T6_THREADS, 1)
       }
       if (++b == nblk) {
         // head g done: the upper column half hands its (max, sum) to the lower, which merges
-        // and writes the row's result (slots alternate by head; a flag names the head)
-        float* px = pxs + (((size_t)(g & 1) * 2 + hh) * T6_HALF + r) * 4;
+        // and writes the row's result.  Every head has a slot of its own: the upper half may be
+        // heads ahead (it needs the lower one only to have loaded its logits).
+        volatile float* px = pxs + (((size_t)g * 2 + hh) * T6_HALF + r) * 4;
         volatile int* done = reinterpret_cast<volatile int*>(px) + 2;
         if (cs == 1) {
           px[0] = m;
           px[1] = l;
           __threadfence_block();
-          *done = g + 1;
+          *done = 1;
         } else {
-          bool ready = *done == g + 1;
+          bool ready = *done != 0;
           if (!ready) {
             const unsigned long long tw = globaltimer();
-            while (!(ready = *done == g + 1))
+            while (!(ready = *done != 0))
               if (globaltimer() - tw > kWaitLimitNs) { atomicCAS(a.err, 0, T6ERR_WAIT); break; }
           }
           __threadfence_block();
