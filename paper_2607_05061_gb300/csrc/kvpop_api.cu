@@ -304,7 +304,7 @@ static kvpop_status init_cache(const kvpop_config* cfg_in, const kvpop_scorer* s
   ALLOC(len, int32_t*, pairs * 4)
   ALLOC(min_score, float*, pairs * 4)
   ALLOC(min_slot, int32_t*, pairs * 4)
-  ALLOC(step_slots, int2*, pairs * sizeof(int2))
+  ALLOC(step_slots, unsigned long long*, pairs * 8)
   ALLOC(blk_score, float*, pairs * NB * 4)
   ALLOC(blk_slot, int32_t*, pairs * NB * 4)
   float* w = nullptr;
@@ -489,7 +489,7 @@ static kvpop_status init_cache(const kvpop_config* cfg_in, const kvpop_scorer* s
     }
     if (e == cudaSuccess) e = NOTE(cudaMemsetAsync(c->st.nvalid, 0, pairs * 4, stream));
     if (e == cudaSuccess) e = NOTE(cudaMemsetAsync(c->st.len, 0, pairs * 4, stream));
-    if (e == cudaSuccess) e = NOTE(cudaMemsetAsync(c->st.step_slots, 0xff, pairs * sizeof(int2), stream));
+    if (e == cudaSuccess) e = NOTE(cudaMemsetAsync(c->st.step_slots, 0xff, pairs * 8, stream));
     if (e == cudaSuccess) e = NOTE(cudaMemsetAsync(c->st.part_count, 0, pairs * 4, stream));
     if (e == cudaSuccess) e = NOTE(cudaMemsetAsync(c->st.err, 0, 16 * 4, stream));
     if (e == cudaSuccess) e = NOTE(cudaMemsetAsync(c->st.pos, 0xff, pairs * B * 4, stream));
@@ -939,7 +939,7 @@ kvpop_status kvpop_import_state(kvpop_cache* c, const void* host_buf, size_t byt
   }
   if (e == cudaSuccess) e = NOTE(cudaMemsetAsync(c->st.part_count, 0, (size_t)c->dm.pairs * 4, stream));
   if (e == cudaSuccess)
-    e = NOTE(cudaMemsetAsync(c->st.step_slots, 0xff, (size_t)c->dm.pairs * sizeof(int2), stream));
+    e = NOTE(cudaMemsetAsync(c->st.step_slots, 0xff, (size_t)c->dm.pairs * 8, stream));
   if (e == cudaSuccess) e = NOTE(cudaStreamSynchronize(stream));
   return poison_on(c, e);
 }

@@ -85,7 +85,7 @@ struct TcTraits {
 struct TcArgs {
   const int32_t* nvalid;
   const int32_t* len;
-  const int2* step_slots;      // the two slots that an ingest still running may write
+  const unsigned long long* step_slots;   // the two slots that an ingest still running may write
   int after_ingest;            // launched right behind this cache's ingest
   const bf16* slotK;           // for the prefetch; the copies go through the tensor maps
   const bf16* slotV;
@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(FUSED ? TcTraits<HD, G>::THREADS_F : TcTraits<
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (a.after_ingest) {
       bool full = true;
-      for (int i = tid; i < npairs; i += NT) full &= __ldcg(a.step_slots + i).x >= 0 && __ldcg(a.len + i) > a.D;
+      for (int i = tid; i < npairs; i += NT) full &= get_step_slots(a.step_slots + i).x >= 0 && __ldcg(a.len + i) > a.D;
       early = __syncthreads_and(full);
     }
     if (early) {
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(FUSED ? TcTraits<HD, G>::THREADS_F : TcTraits<
         if constexpr (!FUSED) {
           if (running) {                           // does this step change the tile?
             if (p != named) {
-              const int2 w = __ldcg(a.step_slots + p);
+              const int2 w = get_step_slots(a.step_slots + p);
               named = p;
               slot_a = w.x / TILE;
               slot_b = w.y / TILE;

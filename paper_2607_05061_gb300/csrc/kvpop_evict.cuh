@@ -49,7 +49,7 @@ __device__ __forceinline__ void evict_and_scatter(const State& st, const Dims& d
     else if (nv + 1 == B)
       min_now = rebuild_min(sc, dm.s, B, slot, prio, bsc, bsl, st.min_score + pair, st.min_slot + pair);
     if (lane == 0) {
-      st.step_slots[pair] = make_int2(min_now, slot);
+      put_step_slots(st.step_slots + pair, min_now, slot);
       sc[slot] = prio;
       ps[slot] = u;
       st.nvalid[pair] = nv < B ? nv + 1 : nv;

@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(NT) ingest_kernel(IngestArgs<T> a) {
     else if (nv + 1 == B)
       min_now = rebuild_min(sc, dm.s, B, slot, prio, bsc, bsl, a.st.min_score + pair, a.st.min_slot + pair);
     if (lane == 0) {
-      a.st.step_slots[pair] = make_int2(min_now, slot);
+      put_step_slots(a.st.step_slots + pair, min_now, slot);
       sc[slot] = prio;
       ps[slot] = u;
       a.st.nvalid[pair] = nv < B ? nv + 1 : nv;

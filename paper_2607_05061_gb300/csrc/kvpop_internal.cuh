@@ -84,8 +84,8 @@ struct State {                 // device pointers of one cache
   int32_t* len;                // [pairs]         tokens seen (same for all heads of a sequence)
   float* min_score;            // [pairs]         argmin over slots [s, B) when full
   int32_t* min_slot;           // [pairs]
-  int2* step_slots;            // [pairs]         (min_slot, slot last written), written as one word;
-                               //                 the first is -1 until the pair is full
+  unsigned long long* step_slots;   // [pairs]    (min_slot, slot last written) in one word (see
+                               //                 put_step_slots); min_slot is -1 until the pair is full
   float* blk_score;            // [pairs][NB]     per-block minima (blocks of 64 slots)
   int32_t* blk_slot;           // [pairs][NB]
   // scorer (hidden width padded to Fp = F rounded up to 4, zero weights)
@@ -249,6 +249,18 @@ cudaError_t launch_proj_out(const float* o, const void* Wo, const void* res, int
                             void* y, bool settled, cudaStream_t stream);
 
 // ------------------------------------------------------------------ device helpers
+// step_slots is written by an ingest while the attention behind it reads it: one 64-bit access on
+// either side, so that a reader never meets the new minimum with the old slot (the two halves of a
+// vector access have no such order).
+__device__ __forceinline__ void put_step_slots(unsigned long long* p, int min_slot, int slot) {
+  const unsigned long long w = (unsigned)min_slot | (unsigned long long)(unsigned)slot << 32;
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+}
+__device__ __forceinline__ int2 get_step_slots(const unsigned long long* p) {
+  unsigned long long w;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+  return make_int2((int)(unsigned)w, (int)(unsigned)(w >> 32));
+}
 __device__ __forceinline__ float to_f(float x) { return x; }
 __device__ __forceinline__ float to_f(bf16 x) { return __bfloat162float(x); }
 

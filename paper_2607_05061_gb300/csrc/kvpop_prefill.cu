@@ -632,13 +632,13 @@ __global__ void __launch_bounds__(NT2) prefill_select_kernel(SelectArgs<T> a) {
       if (lane == 0) {
         a.st.min_score[pair] = m;
         a.st.min_slot[pair] = mi;
-        a.st.step_slots[pair] = make_int2(mi, mi);
+        put_step_slots(a.st.step_slots + pair, mi, mi);
       }
     }
   } else if (c == 0 && tid == 0) {
     a.st.min_score[pair] = INFINITY;
     a.st.min_slot[pair] = -1;
-    a.st.step_slots[pair] = make_int2(-1, -1);
+    put_step_slots(a.st.step_slots + pair, -1, -1);
   }
   if (c == 0 && tid == 0) {
     a.st.nvalid[pair] = nkept;
