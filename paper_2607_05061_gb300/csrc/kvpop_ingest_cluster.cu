@@ -65,6 +65,14 @@ __device__ __forceinline__ void st_cluster_v4(uint32_t addr, float4 v) {
 __device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
+// Two halves of a barrier that orders nothing: every CTA of the cluster has started, so that its
+// shared memory may be written.
+__device__ __forceinline__ void cluster_started_arrive() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_started_wait() {
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
                    : "memory");
@@ -123,6 +131,7 @@ __global__ void __launch_bounds__(NT, 3) ingest_cluster_kernel(ClArgs<T> a) {
   // sequences of this cluster: group*SBC + j; CTA `rank` owns j = OWN*rank + o
   const int own_b0 = group * SBC + OWN * (int)rank;
 
+  cluster_started_arrive();
   // ---- issue every load this CTA needs ------------------------------------------------
   if (tid == 0) {
     mbar_init(smem_u32(&bar), 1);
@@ -254,6 +263,8 @@ __global__ void __launch_bounds__(NT, 3) ingest_cluster_kernel(ClArgs<T> a) {
   }
   __syncthreads();
   const bool ok = mbar_wait(smem_u32(&bar), 0, a.st.err, DEVERR_TIMEOUT_FULL);
+  __syncwarp();
+  cluster_started_wait();
 
   // ---- scorer inputs of the owned sequences, broadcast to the cluster; window update --
   // warp w builds a quarter of the input row of owned sequence w / 4

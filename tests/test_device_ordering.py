@@ -25,3 +25,14 @@ def test_step_slots_is_read_and_written_as_one_word(name):
         return
     assert not re.search(r"step_slots\s*\[", text)
     assert not re.search(r"ld\w*\(\s*(a\.|st\.|a\.st\.)?step_slots", text)
+
+
+def test_cluster_ingest_writes_no_peer_before_all_have_started():
+    """A CTA's shared memory may be written by its cluster only once it runs: each CTA arrives at a
+    cluster barrier at its start and waits for it before the first remote store."""
+    text = source("kvpop_ingest_cluster.cu")
+    body = text[text.index("ingest_cluster_kernel(ClArgs"):]
+    at = [body.index(x) for x in ("cluster_started_arrive();", "griddepcontrol.wait", "cluster_started_wait();",
+                                  "st_cluster_v4(")]
+    assert at == sorted(at)
+    assert "cluster_sync();" not in body[:at[2]]
