@@ -636,7 +636,12 @@ __global__ void __launch_bounds__(T6_THREADS, 1)
       // 2^x needs no running maximum unless the key lies outside the query's kept set with a much
       // larger logit: sum with base 0.  Causal: x = s c2 - m with the first part's maximum as
       // the base.  The maximum is taken only when a part's sum leaves [2^-60, 2^60] (overflow,
-      // NaN, or every term tiny or masked).
+      // NaN, or every term tiny or masked); causal, [2^-60, 2^8]: an exponent is formed in fp32 and
+      // so is off by up to its size times 2^-24.  Mean error from 64 bits of 8 heads x 16384
+      // tokens with outlier channels 7.7e-7 (2^60: 7.9e-7; a base moved at 2^8 of one logit, as in
+      // the prompt kernel: 7.7e-7), where the first keys' logits lie 32 below the others' 8.0e-7
+      // (1.8e-6; 8.0e-7), at 802 us (798; 1352).
+      constexpr float kMaxSum = FUTURE ? 0x1p60f : 0x1p8f;
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
         const float nb1 = FUTURE || m == -INFINITY ? 0.f : -m;
@@ -665,7 +670,7 @@ __global__ void __launch_bounds__(T6_THREADS, 1)
         float q0, q1;
         f2_unpack(p2, q0, q1);
         const float sum = q0 + q1;
-        if (sum >= 0x1p-60f && sum <= 0x1p60f && (FUTURE || m != -INFINITY)) {
+        if (sum >= 0x1p-60f && sum <= kMaxSum && (FUTURE || m != -INFINITY)) {
           if (!FUTURE) {
             l += sum;
           } else if (m <= 0.f) {                    // new base 0
