@@ -601,6 +601,8 @@ kvpop_status prefill_impl(kvpop_cache* c, const void* Q, const void* K, const vo
     e = NOTE(launch_prefill(c->st, c->dm, Q, K, V, plen_dev, first_seq, n_seq, Pmax, override_, prio,
                             sc_map_ptr(c), stream));
   }
+  if (e == cudaSuccess && c->use_fused)
+    e = NOTE(tc_zero_unused_v(c->st, c->dm, first_seq * c->dm.H, (int)pairs, stream));
   if (e == cudaSuccess && outputs && Pmax > 0) {
     int32_t* rank = rank_out ? rank_out : reinterpret_cast<int32_t*>(base + rank_off);
     int32_t* tau = tau_out ? tau_out : reinterpret_cast<int32_t*>(base + tau_off);
@@ -940,6 +942,7 @@ kvpop_status kvpop_import_state(kvpop_cache* c, const void* host_buf, size_t byt
   if (e == cudaSuccess) e = NOTE(cudaMemsetAsync(c->st.part_count, 0, (size_t)c->dm.pairs * 4, stream));
   if (e == cudaSuccess)
     e = NOTE(cudaMemsetAsync(c->st.step_slots, 0xff, (size_t)c->dm.pairs * 8, stream));
+  if (e == cudaSuccess && c->use_fused) e = NOTE(tc_zero_unused_v(c->st, c->dm, 0, c->dm.pairs, stream));
   if (e == cudaSuccess) e = NOTE(cudaStreamSynchronize(stream));
   return poison_on(c, e);
 }

@@ -149,9 +149,10 @@ __device__ __forceinline__ void consumer_sync() {
 // FUSED: the whole decode step (kvpop_step_fused.cuh): the consumers stream only the keys
 // that cannot change this step, the scorer warps ingest the new token meanwhile, and each
 // pair's last arrival merges.  Otherwise the attention alone, over the state the ingest left.
-// TAIL: V rows past a tile's last key are zeroed.  The one-kernel step goes without where whole
-// 16-key groups of the window exist (at its register limit the code costs 0.5% even where it
-// does not run: cr8x 164.3 -> 164.8 us); its slots past the used ones hold zeros.
+// TAIL: V rows past a tile's last key are zeroed.  The one-kernel step goes without where the
+// budget and the window are whole 16-key groups, so that no group reaches into another pair's rows
+// (at its register limit the code costs 0.5% even where it does not run: cr8x 164.3 -> 164.8 us);
+// such a cache keeps the V rows past its used ones zero (zero_unused_v_kernel).
 template <int HD, int G, bool FUSED, bool TAIL>
 __global__ void __launch_bounds__(FUSED ? TcTraits<HD, G>::THREADS_F : TcTraits<HD, G>::THREADS,
                                   KVPOP_TC_MINBLOCKS)
@@ -691,6 +692,27 @@ cudaError_t tc_make_maps(const State& st, const Dims& dm, void* maps_out) {
 
 size_t tc_maps_size() { return sizeof(TcMaps); }
 
+// Whether the one-kernel step has to zero V rows past a tile's last key by itself.
+static bool fused_tail(const Dims& dm) { return dm.D % 16 != 0 || dm.B % 16 != 0; }
+
+// V rows of the unused slots and window entries of pairs first_pair + blockIdx.x.
+__global__ void __launch_bounds__(256) zero_unused_v_kernel(State st, Dims dm, int first_pair) {
+  const size_t pair = (size_t)first_pair + blockIdx.x;
+  const int nv = used_slots(st.nvalid[pair], dm.B, nullptr), np = window_rows(st.len[pair], dm.D, nullptr);
+  const int R = dm.d * (int)sizeof(bf16) / 16;
+  uint4* slots = static_cast<uint4*>(st.slotV) + (pair * dm.B + nv) * R;
+  uint4* ring = static_cast<uint4*>(st.ringV) + (pair * dm.D + np) * R;
+  for (size_t i = threadIdx.x; i < (size_t)(dm.B - nv) * R; i += blockDim.x) slots[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (size_t i = threadIdx.x; i < (size_t)(dm.D - np) * R; i += blockDim.x) ring[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+cudaError_t tc_zero_unused_v(const State& st, const Dims& dm, int first_pair, int n_pairs,
+                             cudaStream_t stream) {
+  if (fused_tail(dm) || n_pairs <= 0) return cudaSuccess;
+  zero_unused_v_kernel<<<n_pairs, 256, 0, stream>>>(st, dm, first_pair);
+  return cudaGetLastError();
+}
+
 #define TC_CASES(X) X(64, 1) X(64, 2) X(64, 4) X(128, 1) X(128, 2) X(128, 4)
 #define TC_FUSED_CASES(X) X(128, 1) X(128, 2) X(128, 4)
 
@@ -726,8 +748,8 @@ cudaError_t tc_fused_config(const Dims& dm, AttendConfig* out) {
     out->threads = TcTraits<HD_, G_>::THREADS_F;                               \
     out->smem_fixed = tc_fused_smem_of(tc_smem<HD_, G_>(0) - 4, dm.Fp) + 16;   \
     out->tile = TcTraits<HD_, G_>::TILE;                                       \
-    out->func = dm.D % 16 ? (const void*)attend_tc_kernel<HD_, G_, true, true> \
-                          : (const void*)attend_tc_kernel<HD_, G_, true, false>; \
+    out->func = fused_tail(dm) ? (const void*)attend_tc_kernel<HD_, G_, true, true> \
+                               : (const void*)attend_tc_kernel<HD_, G_, true, false>; \
     return cudaSuccess;                                                        \
   }
   if (tc_fused_ok(dm)) { TC_FUSED_CASES(CFG) }
@@ -826,8 +848,8 @@ cudaError_t tc_launch_fused(const State& st, const Dims& dm, const void* maps, c
   if (dm.d == HD_ && dm.G == G_) {                                                         \
     cfg.blockDim = dim3(TcTraits<HD_, G_>::THREADS_F, 1, 1);                               \
     cfg.dynamicSmemBytes = tc_fused_smem_of(tc_smem<HD_, G_>(dm.pairs), dm.Fp);            \
-    return cudaLaunchKernelEx(&cfg, dm.D % 16 ? attend_tc_kernel<HD_, G_, true, true>      \
-                                              : attend_tc_kernel<HD_, G_, true, false>,    \
+    return cudaLaunchKernelEx(&cfg, fused_tail(dm) ? attend_tc_kernel<HD_, G_, true, true> \
+                                                   : attend_tc_kernel<HD_, G_, true, false>, \
                               m->sk, m->sv, m->rk, m->rv, a, f);                           \
   }
   TC_FUSED_CASES(LAUNCH)

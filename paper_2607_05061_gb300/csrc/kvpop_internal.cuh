@@ -184,6 +184,10 @@ struct FusedBufs {
   int2* start_prev;            // [grid] where each CTA's range began last launch (zero at init)
 };
 bool tc_fused_ok(const Dims& dm);
+// After a prompt or an import: V rows past the used ones to zero, where the one-kernel step relies
+// on it (its launch).
+cudaError_t tc_zero_unused_v(const State& st, const Dims& dm, int first_pair, int n_pairs,
+                             cudaStream_t stream);
 int tc_fused_max_grid();         // largest grid the fused kernel's split table holds
 cudaError_t tc_fused_config(const Dims& dm, AttendConfig* out);
 cudaError_t tc_launch_fused(const State& st, const Dims& dm, const void* maps, const FusedBufs& fb,
