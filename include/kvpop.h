@@ -144,8 +144,10 @@ kvpop_status kvpop_free(kvpop_cache* cache);
  *   Q_dev  [n_seq][H*G][Pmax][d]    K_dev, V_dev [n_seq][H][Pmax][d]
  *   score_override_dev  [n_seq][H][Pmax] fp32 raw scores used instead of the
  *                        scorer (entry u), or NULL
- * Uses a stream-ordered temporary of n_seq*H*Pmax*4 bytes and synchronises
- * `stream` before returning (the host length array may be reused at once).
+ * Uses a stream-ordered temporary of n_seq*H*Pmax*4 bytes -- with the mLSTM scorer
+ * (2.5*d + 5)*4 at most per (sequence, head, token) and up to 256 MB of states between
+ * segments of the prompts, without which it does, more slowly, where they do not fit -- and
+ * synchronises `stream` before returning (the host length array may be reused at once).
  * The lengths are host values and the batch may come in chunks of sequences
  * because a whole batch's prompts need not fit in device memory at once (128
  * ragged prompts of up to 65536 tokens are about 35 GB of bf16 Q/K/V); the

@@ -571,21 +571,34 @@ kvpop_status prefill_impl(kvpop_cache* c, const void* Q, const void* K, const vo
   const size_t pairs = (size_t)n_seq * c->dm.H;
   auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
   const size_t prio_bytes = al(pairs * (size_t)Pmax * 4);
-  // the mLSTM prefill also needs every prompt token's features (k~, v~, q~, gates)
-  const size_t feat_bytes = c->mlstm ? mlstm_prefill_bytes(c->dm.d, (int)pairs, Pmax) : 0;
+  // the mLSTM prefill also needs every prompt token's features (k~, v~, q~, gates), and states
+  // between the segments of a prompt, which it does without where they do not fit
+  bool one_segment = false;
+  size_t feat_off = 0, rank_off = 0, tau_off = 0, ws_off = 0, bytes = 0;
   const size_t plen_off = prio_bytes;
-  const size_t feat_off = plen_off + al((size_t)n_seq * 4);
-  const size_t rank_off = al(feat_off + feat_bytes);
-  const size_t tau_off = rank_off + (outputs && !rank_out ? prio_bytes : 0);
-  const size_t ws_off = tau_off + (outputs && !tau_out ? prio_bytes : 0);
-  const size_t ws_bytes = outputs ? topk_workspace_bytes((int)pairs, Pmax) : 0;
+  auto lay_out = [&] {
+    const size_t feat_bytes = c->mlstm ? mlstm_prefill_bytes(c->dm.d, (int)pairs, Pmax, one_segment) : 0;
+    feat_off = plen_off + al((size_t)n_seq * 4);
+    rank_off = al(feat_off + feat_bytes);
+    tau_off = rank_off + (outputs && !rank_out ? prio_bytes : 0);
+    ws_off = tau_off + (outputs && !tau_out ? prio_bytes : 0);
+    bytes = ws_off + (outputs ? topk_workspace_bytes((int)pairs, Pmax) : 0) + 256;
+  };
   void* tmp = nullptr;
-  if (g_fail_after > 0 && --g_fail_after == 0) return KVPOP_ERR_OOM;
-  cudaError_t e = NOTE(cudaMallocAsync(&tmp, ws_off + ws_bytes + 256, stream));
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return from_cuda(e);
+  auto allocate = [&] {
+    if (g_fail_after > 0 && --g_fail_after == 0) return cudaErrorMemoryAllocation;
+    const cudaError_t r = NOTE(cudaMallocAsync(&tmp, bytes, stream));
+    if (r != cudaSuccess) cudaGetLastError();
+    return r;
+  };
+  lay_out();
+  cudaError_t e = allocate();
+  if (e == cudaErrorMemoryAllocation && c->mlstm) {
+    one_segment = true;
+    lay_out();
+    e = allocate();
   }
+  if (e != cudaSuccess) return from_cuda(e);
   char* base = static_cast<char*>(tmp);
   float* prio = reinterpret_cast<float*>(base);
   int32_t* plen_dev = reinterpret_cast<int32_t*>(base + plen_off);
@@ -593,7 +606,7 @@ kvpop_status prefill_impl(kvpop_cache* c, const void* Q, const void* K, const vo
   if (e == cudaSuccess && c->mlstm) {
     float* feat = reinterpret_cast<float*>(base + feat_off);
     e = NOTE(launch_prefill_mlstm_scores(c->st, c->dm, c->md, K, V, plen_dev, first_seq, n_seq, Pmax,
-                                         override_, feat, prio, stream));
+                                         override_, feat, one_segment, prio, stream));
     if (e == cudaSuccess)
       e = NOTE(launch_prefill_select(c->st, c->dm, Q, K, V, plen_dev, first_seq, n_seq, Pmax, prio,
                                      stream));

@@ -150,8 +150,9 @@ int mlstm_nc(int d);
 int mlstm_nf(int d);
 size_t mlstm_wt_bytes(int d, int H);
 cudaError_t launch_mlstm_split(const Dims& dm, const MlstmDev& m, cudaStream_t stream);
-// Bytes behind `feat` of launch_prefill_mlstm_scores.
-size_t mlstm_prefill_bytes(int d, int pairs, int Pmax);
+// Bytes behind `feat` of launch_prefill_mlstm_scores.  one_segment: the chunks of a prompt one
+// after another, with no states kept between them.
+size_t mlstm_prefill_bytes(int d, int pairs, int Pmax, bool one_segment);
 bool mlstm_ok(const Dims& dm);
 cudaError_t prepare_mlstm(const Dims& dm);
 cudaError_t launch_ingest_mlstm(const State& st, const Dims& dm, const MlstmDev& m, const void* q,
@@ -160,7 +161,8 @@ cudaError_t launch_ingest_mlstm(const State& st, const Dims& dm, const MlstmDev&
 cudaError_t launch_prefill_mlstm_scores(const State& st, const Dims& dm, const MlstmDev& m,
                                         const void* K, const void* V, const int32_t* plen,
                                         int first_seq, int n_seq, int Pmax, const float* override_,
-                                        float* feat, float* prio, cudaStream_t stream);
+                                        float* feat, bool one_segment, float* prio,
+                                        cudaStream_t stream);
 // Selection + compaction + window fill of the prefill, from precomputed priorities.
 cudaError_t launch_prefill_select(const State& st, const Dims& dm, const void* Q, const void* K,
                                   const void* V, const int32_t* plen, int first_seq, int n_seq,

@@ -1069,13 +1069,15 @@ template <int HD>
 size_t seg_smem() { return (size_t)2 * ChunkLayout<HD>::BUF_S * 4; }
 
 // Chunks per segment: one (no state is updated twice) while the states between segments stay
-// below 256 MB, else as many as that takes.
-int seg_chunks(int d, int pairs, int Pmax) {
+// below 256 MB, else as many as that takes; all of a prompt's (no states between) where the caller
+// has no room for them.
+int seg_chunks(int d, int pairs, int Pmax, bool one_segment) {
+  if (one_segment) return std::max(1, (Pmax + CL - 1) / CL);
   const double bytes = (double)pairs * ((Pmax + CL - 1) / CL) * (d * (d / 2) + d) * 4.0;
   return std::max(1, (int)(bytes / 256e6) + 1);
 }
-int seg_count(int d, int pairs, int Pmax) {
-  const int nch = (Pmax + CL - 1) / CL, n = seg_chunks(d, pairs, Pmax);
+int seg_count(int d, int pairs, int Pmax, bool one_segment) {
+  const int nch = (Pmax + CL - 1) / CL, n = seg_chunks(d, pairs, Pmax, one_segment);
   return std::max(1, (nch + n - 1) / n);
 }
 
@@ -1116,8 +1118,8 @@ cudaError_t launch_mlstm_split(const Dims& dm, const MlstmDev& m, cudaStream_t s
   return cudaGetLastError();
 }
 // Workspace of the prompt scores: every token's features, then the segments' states and scalars.
-size_t mlstm_prefill_bytes(int d, int pairs, int Pmax) {
-  const size_t nseg = seg_count(d, pairs, Pmax);
+size_t mlstm_prefill_bytes(int d, int pairs, int Pmax, bool one_segment) {
+  const size_t nseg = seg_count(d, pairs, Pmax, one_segment);
   return ((size_t)pairs * Pmax * mlstm_nf(d) + (size_t)pairs * (nseg - 1) * (d * (d / 2) + d) +
           3 * (size_t)pairs * nseg) * 4;
 }
@@ -1188,7 +1190,8 @@ cudaError_t launch_ingest_mlstm(const State& st, const Dims& dm, const MlstmDev&
 cudaError_t launch_prefill_mlstm_scores(const State& st, const Dims& dm, const MlstmDev& m,
                                         const void* K, const void* V, const int32_t* plen,
                                         int first_seq, int n_seq, int Pmax, const float* override_,
-                                        float* feat, float* prio, cudaStream_t stream) {
+                                        float* feat, bool one_segment, float* prio,
+                                        cudaStream_t stream) {
   const int NF = mlstm_nf(dm.d);
   const int pairs = n_seq * dm.H;
   if (Pmax > 0) {
@@ -1205,7 +1208,7 @@ cudaError_t launch_prefill_mlstm_scores(const State& st, const Dims& dm, const M
     if (e != cudaSuccess) return e;
   }
   MScanArgs sa{st, dm, to_mstate(m), plen, feat, override_, prio, nullptr, nullptr, nullptr, first_seq, Pmax, NF,
-               seg_chunks(dm.d, pairs, Pmax), seg_count(dm.d, pairs, Pmax)};
+               seg_chunks(dm.d, pairs, Pmax, one_segment), seg_count(dm.d, pairs, Pmax, one_segment)};
   sa.seg = feat + (size_t)pairs * Pmax * NF;
   sa.seg_scal = sa.seg + (size_t)pairs * (sa.nseg - 1) * (dm.d * (dm.d / 2) + dm.d);
   sa.seg_m = sa.seg_scal + (size_t)2 * pairs * sa.nseg;
