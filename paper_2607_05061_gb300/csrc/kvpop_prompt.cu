@@ -629,7 +629,7 @@ cudaError_t launch_f32(PromptArgs a, cudaStream_t stream) {
 
 }  // namespace
 
-bool prompt_t5_ok(int d, int G, int s, int w, int k);
+bool prompt_t5_ok(int d, int G, int S, int s, int w, int k);
 cudaError_t launch_prompt_t5(const prompt::PromptArgs& a, int G, cudaStream_t stream);
 cudaError_t launch_causal_lse_t5(const void* Q, const void* K, const int32_t* len, int n_seq, int H, int G,
                                  int S, float* lse, int32_t* err, cudaStream_t stream);   // kvpop_target.cu
@@ -637,17 +637,17 @@ cudaError_t launch_causal_lse_t5(const void* Q, const void* K, const int32_t* le
 namespace {
 
 // tcgen05 kernel for bf16 with d = 128 (KVPOP_PROMPT_MMA_SYNC=1 selects the m16n8k16 kernel)
-bool use_t5(int dtype, int d, int G, int s, int w, int k) {
+bool use_t5(int dtype, int d, int G, int S, int s, int w, int k) {
   static const bool off = [] {
     const char* e = getenv("KVPOP_PROMPT_MMA_SYNC");
     return e && e[0] == '1';
   }();
-  return !off && dtype == KVPOP_BF16 && prompt_t5_ok(d, G, s, w, k);
+  return !off && dtype == KVPOP_BF16 && prompt_t5_ok(d, G, S, s, w, k);
 }
 
 template <bool DENSE, bool WANT_Y>
 cudaError_t dispatch(const PromptArgs& a, int dtype, int d, int G, cudaStream_t stream) {
-  if (!DENSE && use_t5(dtype, d, G, a.s, a.w, a.capA - a.s)) return launch_prompt_t5(a, G, stream);
+  if (!DENSE && use_t5(dtype, d, G, a.S, a.s, a.w, a.capA - a.s)) return launch_prompt_t5(a, G, stream);
   if (dtype == KVPOP_BF16) {
     if (d == 128) {
       if (G == 4) return launch_tc<128, 4, DENSE, WANT_Y>(a, stream);
@@ -692,7 +692,7 @@ cudaError_t launch_causal_lse(const void* Q, const void* K, const int32_t* len, 
                               int G, int d, int S, int dtype, float* lse, int32_t* err,
                               cudaStream_t stream) {
   if (n_seq <= 0 || S <= 0) return cudaSuccess;
-  if (use_t5(dtype, d, G, 0, 1, 0)) return launch_causal_lse_t5(Q, K, len, n_seq, H, G, S, lse, err, stream);
+  if (use_t5(dtype, d, G, S, 0, 1, 0)) return launch_causal_lse_t5(Q, K, len, n_seq, H, G, S, lse, err, stream);
   PromptArgs a{Q, K, nullptr, nullptr, nullptr, nullptr, len, nullptr, lse, n_seq * H, H, G, S, 0, 1, 0, 0,
                1.4426950408889634f / sqrtf((float)d), err};
   return dispatch<true, false>(a, dtype, d, G, stream);

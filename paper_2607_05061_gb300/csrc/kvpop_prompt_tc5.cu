@@ -6,7 +6,7 @@
 // rows form two 128-row halves that share every gathered K/V block, so each
 // gathered byte feeds two M = 128 MMAs.  Roles:
 //  * 3 producer warps gather the block's K and V rows by position with 16-byte
-//    cp.async into 128B-swizzled tiles (2 or 3 stages, as shared memory
+//    cp.async into 128B-swizzled tiles (2 to 4 stages, as shared memory
 //    allows); completion arrives on the stage's mbarrier asynchronously
 //    (cp.async.mbarrier.arrive.noinc).
 //  * 1 MMA warp: one lane issues, per half, S = Q K^T (M 128, N 64, K 128;
@@ -55,6 +55,7 @@ constexpr int T5_THREADS = 32 * (T5_MMA_WARP + 1 + T5_NPROD);   // 12 warps: 168
 static_assert(T5_THREADS / 32 + 2 <= 16, "the prologue's per-warp reduction slots");
 constexpr int T5_TMEM_COLS = 512;                // O_h: 128 h .. ; S_{h,b}: 256 + 128 h + 64 b
 constexpr float T5_THR = 8.0f;
+constexpr int T5_POS_BITS = 18;                  // of a packed position
 
 constexpr int QB = T5_HALF * 256;                // Q tile of one half, bytes
 constexpr int KVB = T5_BN * 256;                 // K (or V) block, bytes
@@ -77,7 +78,9 @@ constexpr int B_ODONE = 16;        // [2]  MMA -> softmax (one per half)
 constexpr int B_QFULL = 18;
 enum : int { T5ERR_WAIT = 21 };
 
-template <int G, int ST>
+// PACK: an M entry's position and the length of its run of queries share a word (below), so that
+// long windows keep their lists in shared memory once.
+template <int G, int ST, bool PACK>
 __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) {
   using L = Lay<ST>;
   constexpr int BM = T5_ROWS / G;
@@ -89,7 +92,7 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
   int* red = reinterpret_cast<int*>(sm5 + L::OFF_RED);
   int32_t* posA = reinterpret_cast<int32_t*>(sm5 + L::OFF_LIST);
   int32_t* posM = posA + a.capA;
-  uint32_t* keepM = reinterpret_cast<uint32_t*>(posM + a.capM);   // [capM + T5_BN]
+  uint32_t* keepM = reinterpret_cast<uint32_t*>(PACK ? posM : posM + a.capM);   // [capM + T5_BN]
 
   if (tid == 0) {
     for (int i = 0; i < ST; ++i) {
@@ -136,7 +139,8 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
           const int mid = (lo + hi) >> 1;
           if (keep_key(ti.q0 + mid, t, r, tauS[mid], a.s, a.w)) lo = mid + 1; else hi = mid;
         }
-        word = (uint32_t)first | (uint32_t)(lo - first) << 16;
+        word = PACK ? (uint32_t)t | (uint32_t)(lo - first) << T5_POS_BITS
+                    : (uint32_t)first | (uint32_t)(lo - first) << 16;
       }
       keepM[i] = word;
     }
@@ -150,8 +154,9 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
     const int nblk = (nU + T5_BN - 1) / T5_BN;
     const size_t pair_off = (size_t)ti.pair * S;
     auto entry = [&](int e) -> int {
+      constexpr int mask = PACK ? (1 << T5_POS_BITS) - 1 : -1;
       if (e < nA) return posA[e];
-      return e < nU ? posM[e - nA] : (nA > 0 ? posA[0] : posM[0]);
+      return e < nU ? posM[e - nA] & mask : (nA > 0 ? posA[0] : posM[0] & mask);
     };
     if (warp > T5_MMA_WARP) {
       // ---------------------------------------------------------------- producers
@@ -260,7 +265,8 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
           for (int i = 0; i < 64; ++i) {
             if (i >= nf) {
               const uint32_t kw = keepM[i - nf];
-              if ((uint32_t)(ql - (int)(kw & 0xffffu)) >= (kw >> 16)) s[i] = -INFINITY;
+              const int first = PACK ? max(0, (int)(kw & ((1u << T5_POS_BITS) - 1)) - ti.q0) : (int)(kw & 0xffffu);
+              if ((uint32_t)(ql - first) >= (kw >> (PACK ? T5_POS_BITS : 16))) s[i] = -INFINITY;
             }
           }
         }
@@ -370,38 +376,43 @@ __global__ void __launch_bounds__(T5_THREADS, 1) prompt_t5_kernel(PromptArgs a) 
   if (warp == T5_MMA_WARP) tmem_dealloc(tmem, T5_TMEM_COLS);
 }
 
-template <int ST>
-size_t t5_smem(int capA, int capM) {
-  return (size_t)Lay<ST>::OFF_LIST + (size_t)(capA + 2 * capM + T5_BN) * 4;
+template <int ST, bool PACK>
+size_t t5_smem(long long capA, long long capM) {
+  return (size_t)Lay<ST>::OFF_LIST + (size_t)(capA + (PACK ? 1 : 2) * capM + T5_BN) * 4;
 }
 
-template <int G, int ST>
+template <int G, int ST, bool PACK>
 cudaError_t launch_t5_st(const PromptArgs& a, size_t smem, cudaStream_t stream) {
   constexpr int BM = T5_ROWS / G;
-  auto k = prompt_t5_kernel<G, ST>;
+  auto k = prompt_t5_kernel<G, ST, PACK>;
   cudaError_t e = raise_smem_limit(k, smem);
   if (e != cudaSuccess) return e;
   k<<<tile_grid(a, BM), T5_THREADS, smem, stream>>>(a);
   return cudaGetLastError();
 }
 
+// As many stages as the lists leave room for; packed lists where not even two are left otherwise
+// (windows beyond about 12000 tokens).
 template <int G>
 cudaError_t launch_t5_g(PromptArgs a, cudaStream_t stream) {
   constexpr int BM = T5_ROWS / G;
   a.capM = a.s + 2 * BM + a.w;
-  const size_t s4 = t5_smem<4>(a.capA, a.capM), s3 = t5_smem<3>(a.capA, a.capM), s2 = t5_smem<2>(a.capA, a.capM);
-  if (s4 <= 227 * 1024) return launch_t5_st<G, 4>(a, s4, stream);
-  if (s3 <= 227 * 1024) return launch_t5_st<G, 3>(a, s3, stream);
-  if (s2 <= 227 * 1024) return launch_t5_st<G, 2>(a, s2, stream);
+  const size_t s4 = t5_smem<4, false>(a.capA, a.capM), s3 = t5_smem<3, false>(a.capA, a.capM);
+  const size_t s2 = t5_smem<2, false>(a.capA, a.capM), sp = t5_smem<2, true>(a.capA, a.capM);
+  if (s4 <= 227 * 1024) return launch_t5_st<G, 4, false>(a, s4, stream);
+  if (s3 <= 227 * 1024) return launch_t5_st<G, 3, false>(a, s3, stream);
+  if (s2 <= 227 * 1024) return launch_t5_st<G, 2, false>(a, s2, stream);
+  if (sp <= 227 * 1024) return launch_t5_st<G, 2, true>(a, sp, stream);
   return cudaErrorInvalidValue;
 }
 
 }  // namespace
 
-bool prompt_t5_ok(int d, int G, int s, int w, int k) {
+bool prompt_t5_ok(int d, int G, int S, int s, int w, int k) {
   if (d != 128 || !(G == 1 || G == 2 || G == 4)) return false;
-  const long long lists = (long long)s + k + 2 * ((long long)s + 2 * T5_ROWS + w) + T5_BN;
-  return Lay<2>::OFF_LIST + 4 * lists <= 227 * 1024;
+  const long long capM = (long long)s + 2 * T5_ROWS + w;
+  return (S <= 1 << T5_POS_BITS ? t5_smem<2, true>((long long)s + k, capM)
+                                : t5_smem<2, false>((long long)s + k, capM)) <= 227 * 1024;
 }
 
 cudaError_t launch_prompt_t5(const PromptArgs& a, int G, cudaStream_t stream) {
