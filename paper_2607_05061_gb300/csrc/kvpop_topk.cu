@@ -474,6 +474,9 @@ cudaError_t launch_topk(const float* prio, const int32_t* len, int rows_per_len,
                         int n_rows, int S, int s, int w, int k, int32_t* rank, int32_t* tau,
                         int32_t* order, void* workspace, cudaStream_t stream) {
   if (n_rows <= 0 || S <= 0) return cudaSuccess;
+  // no token is eligible either way, and no position is computed past 2 S
+  s = std::min(s, S);
+  w = std::min(w, S);
   const size_t n = (size_t)n_rows * S;
   char* ws = static_cast<char*>(workspace);
   auto al = [](size_t x) { return (x + 255) & ~size_t(255); };
