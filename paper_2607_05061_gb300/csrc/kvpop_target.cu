@@ -839,6 +839,9 @@ cudaError_t launch_future_target(const void* Q, const void* K, const float* lse,
                                  float* logm, float* target, int agg, int count_norm, float eps,
                                  int32_t* err, cudaStream_t stream) {
   if (n_seq <= 0 || S <= 0) return cudaSuccess;
+  // beyond S both say the same as S, and no position is computed past 3 S
+  w = std::min(w, S);
+  la = std::min(la, S);
   TargetArgs a{Q, K, lse, len, logm, H, G, S, w, la, 1.4426950408889634f / sqrtf((float)d), err};
   const int n_pairs = n_seq * H;
   static const bool mma_sync = [] {
