@@ -317,18 +317,43 @@ def future_target(Q, K, lse, window: int, lookahead: int = 0, agg: str = "max",
     return logm, target
 
 
+def _shape(what, name, t, dtype, rows, cols, more_rows=False):
+    """Refuses a tensor that a call would read or write past its end or as another type."""
+    ok = t.dtype == dtype and t.dim() == 2 and t.shape[1] == cols and t.is_contiguous()
+    if not ok or (t.shape[0] < rows if more_rows else t.shape[0] != rows):
+        raise ValueError(f"{what}: {name} is {t.dtype} {tuple(t.shape)}, not contiguous {dtype} ({rows}, {cols})")
+
+
 def project_qkv(x, Wq, Wk, Wv, q, k, v, stream=None, settled=False):
-    """``q, k, v = bf16(x Wq), bf16(x Wk), bf16(x Wv)`` (contiguous bf16, up to 64 rows) in one
-    launch.  ``settled``: whatever writes the weights has completed before the work queued last
-    on the stream starts; they are then read while that work runs."""
+    """``q, k, v = bf16(x Wq), bf16(x Wk), bf16(x Wv)`` (contiguous bf16, up to 32 rows, ``Wk`` and
+    ``Wv`` of one width) in one launch.  ``settled``: whatever writes the weights has completed
+    before the work queued last on the stream starts; they are then read while that work runs."""
+    bf, (M, K) = torch.bfloat16, x.shape
+    _shape("project_qkv", "x", x, bf, M, K)
+    for name, W, y, n in (("q", Wq, q, Wq.shape[1]), ("k", Wk, k, Wk.shape[1]), ("v", Wv, v, Wk.shape[1])):
+        _shape("project_qkv", "W" + name, W, bf, K, n)
+        _shape("project_qkv", name, y, bf, M, n, more_rows=True)
+    _project_qkv(x, Wq, Wk, Wv, q, k, v, stream, settled)
+
+
+def _project_qkv(x, Wq, Wk, Wv, q, k, v, stream=None, settled=False):
     f = kvpop_project_qkv_settled if settled else kvpop_project_qkv
     _ck(f(_ptr(x), _ptr(Wq), _ptr(Wk), _ptr(Wv), x.shape[0], x.shape[1], Wq.shape[1], Wk.shape[1],
           _ptr(q), _ptr(k), _ptr(v), _stream(stream)), "kvpop_project_qkv")
 
 
 def project_out(o, Wo, x, y, stream=None, settled=False):
-    """``y = bf16(x + bf16(bf16(o) Wo))`` (``o`` fp32, the others contiguous bf16) in one launch;
-    ``settled`` as in ``project_qkv``."""
+    """``y = bf16(x + bf16(bf16(o) Wo))`` (``o`` fp32, the others contiguous bf16, up to 16 rows) in
+    one launch; ``settled`` as in ``project_qkv``."""
+    bf, (M, N), K = torch.bfloat16, x.shape, Wo.shape[0]
+    _shape("project_out", "o", o, torch.float32, M, K, more_rows=True)
+    _shape("project_out", "Wo", Wo, bf, K, N)
+    _shape("project_out", "x", x, bf, M, N)
+    _shape("project_out", "y", y, bf, M, N, more_rows=True)
+    _project_out(o, Wo, x, y, stream, settled)
+
+
+def _project_out(o, Wo, x, y, stream=None, settled=False):
     f = kvpop_project_out_settled if settled else kvpop_project_out
     _ck(f(_ptr(o), _ptr(Wo), _ptr(x), x.shape[0], Wo.shape[0], x.shape[1], _ptr(y), _stream(stream)),
         "kvpop_project_out")

@@ -20,7 +20,7 @@ from typing import List, Optional, Sequence
 
 import torch
 
-from .kvpop import KVpopCache, kvpop_project_supported, project_out, project_qkv
+from .kvpop import KVpopCache, _project_out, _project_qkv, kvpop_project_supported
 
 
 class DecodeStack:
@@ -92,8 +92,8 @@ class DecodeStack:
             nq, nkv, hid = self.q.shape[1], self.k.shape[1], self.hidden
             if self._project & 1 and self._plain((x, (self.b, hid)), (L["Wq"], (hid, nq)),
                                                  (L["Wk"], (hid, nkv)), (L["Wv"], (hid, nkv))):
-                project_qkv(x, L["Wq"], L["Wk"], L["Wv"], self.q, self.k, self.v,
-                            settled=settled)
+                _project_qkv(x, L["Wq"], L["Wk"], L["Wv"], self.q, self.k, self.v,
+                             settled=settled)
                 settled = True
             else:
                 torch.matmul(x, L["Wq"], out=self.q)
@@ -106,7 +106,7 @@ class DecodeStack:
                 outputs[l].copy_(self.o)
             if self._project & 2 and self._plain((x, (self.b, hid)), (nxt, (self.b, hid)),
                                                  (L["Wo"], (nq, hid))):
-                project_out(self.o, L["Wo"], x, nxt, settled=settled)
+                _project_out(self.o, L["Wo"], x, nxt, settled=settled)
                 settled = True
             else:
                 self.o_bf.copy_(self.o)
