@@ -362,6 +362,11 @@ kvpop_status kvpop_get_pair_state(kvpop_cache* cache, int32_t seq, int32_t head,
  * 48). */
 int32_t kvpop_project_supported(int32_t batch, int32_t hidden, int32_t n_q, int32_t n_kv);
 
+/* The same bits where the calls are also faster than library products on the current device:
+ * columns that fit its SMs at once (n_q + 2 n_kv, or hidden, up to 7296 on GB300), and for
+ * kvpop_project_out batch * n_q up to 65536. */
+int32_t kvpop_project_preferred(int32_t batch, int32_t hidden, int32_t n_q, int32_t n_kv);
+
 /* q = bf16(x Wq), k = bf16(x Wk), v = bf16(x Wv) in one launch.
  *   x_dev [batch][hidden], Wq_dev [hidden][n_q], Wk_dev, Wv_dev [hidden][n_kv],
  *   q_dev [batch][n_q], k_dev, v_dev [batch][n_kv], all bf16, 16-byte aligned.

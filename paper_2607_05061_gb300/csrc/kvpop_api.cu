@@ -736,6 +736,13 @@ int32_t kvpop_project_supported(int32_t batch, int32_t hidden, int32_t n_q, int3
          (proj_ok(batch, n_q, hidden, true) ? 2 : 0);
 }
 
+int32_t kvpop_project_preferred(int32_t batch, int32_t hidden, int32_t n_q, int32_t n_kv) {
+  const int32_t can = kvpop_project_supported(batch, hidden, n_q, n_kv);
+  const bool qkv = (can & 1) && (long long)n_q + 2ll * n_kv <= INT32_MAX &&
+                   proj_faster(batch, hidden, n_q + 2 * n_kv, false);
+  return (qkv ? 1 : 0) | ((can & 2) && proj_faster(batch, n_q, hidden, true) ? 2 : 0);
+}
+
 static kvpop_status project_qkv(const void* x, const void* Wq, const void* Wk, const void* Wv,
                                 int32_t batch, int32_t hidden, int32_t n_q, int32_t n_kv, void* q,
                                 void* k, void* v, bool settled, cudaStream_t stream) {

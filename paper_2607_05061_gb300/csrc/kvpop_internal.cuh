@@ -249,6 +249,7 @@ cudaError_t launch_future_target(const void* Q, const void* K, const float* lse,
 // Projections of the decode stack (M rows of K, N columns).  settled: no kernel that may still
 // run at the launch writes the weights.
 bool proj_ok(int M, int K, int N, bool x_f32);
+bool proj_faster(int M, int K, int columns, bool x_f32);
 cudaError_t launch_proj_qkv(const void* x, const void* Wq, const void* Wk, const void* Wv, int M, int K,
                             int nq, int nkv, void* q, void* k, void* v, bool settled, cudaStream_t stream);
 cudaError_t launch_proj_out(const float* o, const void* Wo, const void* res, int M, int K, int N,

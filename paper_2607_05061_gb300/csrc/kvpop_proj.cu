@@ -247,6 +247,21 @@ bool proj_ok(int M, int K, int N, bool x_f32) {
   return M >= 1 && M <= (x_f32 ? 16 : 32) && K >= PJ_KS && K % PJ_KS == 0 && N >= 8 * PJ_NG && N % 8 == 0;
 }
 
+// Where the kernel is the faster way, of the sizes it takes.  Its columns have to fit the SMs at
+// once: a CTA holds an SM for its part of the columns, so a second wave leaves most of the SMs idle
+// (a layer of hidden 8192 with 64 query and 16 KV heads at batch 1 and 16, cuBLAS / q, k, v here /
+// the output here: 82 / 84 / 95 us and 108 / 116 / 128; with 7168 and 56 heads, 1344 and 896 column
+// groups for 912 places, 76 / 77 / 75 at batch 1).  Within that q, k, v are faster throughout (hidden
+// 8192, 32 heads, batch 16: 79.5 / 79.6; batch 1: 65.7 / 59.5).  For the output every CTA reads all
+// rows of fp32 x through L2, and more of them than 2^16 values cost what the launches save (8192
+// wide, batch 8: 79.9 / 77.7 us a layer, batch 16: 99.0 / 101.3).
+bool proj_faster(int M, int K, int columns, bool x_f32) {
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaGetLastError();                  // no device: the rule for GB300
+  return columns / 8 <= PJ_NG * sms && (!x_f32 || (long long)M * K <= 1 << 16);
+}
+
 cudaError_t launch_proj_qkv(const void* x, const void* Wq, const void* Wk, const void* Wv, int M, int K,
                             int nq, int nkv, void* q, void* k, void* v, bool settled, cudaStream_t stream) {
   ProjArgs a{};

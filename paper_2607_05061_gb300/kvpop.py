@@ -87,6 +87,7 @@ _SIGS = {
                                            c_int32, c_int32, ctypes.c_int, _P, _P, c_int32, c_int32,
                                            c_float, _P]),
     "kvpop_project_supported": (c_int32, [c_int32, c_int32, c_int32, c_int32]),
+    "kvpop_project_preferred": (c_int32, [c_int32, c_int32, c_int32, c_int32]),
     "kvpop_project_qkv": (ctypes.c_int, [_P, _P, _P, _P, c_int32, c_int32, c_int32, c_int32, _P, _P, _P,
                                          _P]),
     "kvpop_project_out": (ctypes.c_int, [_P, _P, _P, c_int32, c_int32, c_int32, _P, _P]),

@@ -20,7 +20,7 @@ from typing import List, Optional, Sequence
 
 import torch
 
-from .kvpop import KVpopCache, _project_out, _project_qkv, kvpop_project_supported
+from .kvpop import KVpopCache, _project_out, _project_qkv, kvpop_project_preferred
 
 
 class DecodeStack:
@@ -51,9 +51,9 @@ class DecodeStack:
         self.y = torch.empty((batch, hidden), dtype=dt, device=dev)
         self.x = [torch.empty((batch, hidden), dtype=dt, device=dev) for _ in range(2)]
         self.graph = None
-        # which projections the weight-streaming kernels take at these sizes (bit 0: q, k, v;
-        # bit 1: the output projection)
-        self._project = kvpop_project_supported(batch, hidden, self.Hq * head_dim,
+        # which projections the weight-streaming kernels take at these sizes, and faster (bit 0:
+        # q, k, v; bit 1: the output projection)
+        self._project = kvpop_project_preferred(batch, hidden, self.Hq * head_dim,
                                                 n_kv_heads * head_dim)
 
     def _plain(self, *want) -> bool:
