@@ -3,8 +3,8 @@
 // Kernel 1 ranks a row's tokens by static priority, higher first, equal priorities by
 // position: a stable least-significant-digit radix sort of the order-reversed fp32 bit
 // pattern, 4 passes of 8 bits.  A cluster of up to 8 CTAs holds the row in registers and
-// shared memory (rank_cluster_kernel); rows too long for that take one CTA that sorts
-// through global memory (rank_kernel).  The last pass writes rank[position] directly.
+// shared memory (rank_cluster_kernel); rows too long for that, and short ones, take one CTA that
+// sorts through global memory (rank_kernel).  The last pass writes rank[position] directly.
 //
 // Kernel 2 computes tau_q for every query position, a row's queries split over CTAs and
 // their warps.  The paper inserts each newly eligible rank into a Fenwick tree and reads
@@ -174,7 +174,8 @@ __global__ void __launch_bounds__(RK_NT) rank_cluster_kernel(RankArgs a) {
   for (int i = L + c * RK_NT + tid; i < S; i += C * RK_NT) a.rank[ro + i] = -1;
 }
 
-// Rows longer than 8 * 512 * 32 tokens: one CTA per row, keys and positions in global memory.
+// Short rows (kShortRow), and rows longer than 8 * 512 * 32 tokens: one CTA per row, keys and
+// positions in global memory.
 // Within a round of RK_NT tokens the stable offset of each token inside its digit bucket
 // comes from a warp match on the digit plus per-warp bucket counts; one histogram pass up
 // front gives every pass its bucket bases.
@@ -439,6 +440,13 @@ cudaError_t launch_rank_cluster(const RankArgs& ra, int C, cudaStream_t stream) 
   return cudaLaunchKernelEx(&cfg, rank_cluster_kernel<I>, ra);
 }
 
+// Rows up to here take the one-CTA rank kernel, whose passes over so few tokens cost less than the
+// cluster kernel's set-up (ranks and cutoffs, us: 1 row of 256 tokens 14.4 against 16.5, 20000 of 64
+// 318 against 422, 4000 of 256 123 against 130; from 512 on the cluster kernel, 1000 rows 61 against
+// 67), and their queries are spread over all warps of one CTA: 16, or 8 where there are rows for
+// more than two CTAs an SM (20000 of 64: 363 with 16, 318 with 8; 300 of 128: 14.5 and 16.5).
+constexpr int kShortRow = 384;
+
 // CTAs per row C (a power of two up to 8) and items per thread: the largest C that keeps the
 // grid within two CTAs per SM and gives every CTA at least 1024 elements, more where the row
 // does not fit otherwise.
@@ -447,7 +455,7 @@ cudaError_t launch_rank(const RankArgs& ra, int sms, cudaStream_t stream) {
   while (C < 8 && (long long)ra.n_rows * (2 * C) <= 2 * sms && ra.S > 2 * RK_NT * C) C *= 2;
   while (C < 8 && ra.S > 32 * RK_NT * C) C *= 2;
   const int per = (ra.S + C - 1) / C;
-  if (per > 32 * RK_NT || (long long)ra.n_rows * C > INT_MAX) {
+  if (ra.S <= kShortRow || per > 32 * RK_NT || (long long)ra.n_rows * C > INT_MAX) {
     rank_kernel<<<ra.n_rows, RK_NT, 0, stream>>>(ra);
     return cudaGetLastError();
   }
@@ -491,12 +499,16 @@ cudaError_t launch_topk(const float* prio, const int32_t* len, int rows_per_len,
   if (e != cudaSuccess) return e;
   // warps per CTA: up to 16, each with its own bitset of S bits beside the CTA's
   const size_t words_bytes = (size_t)((S + 31) / 32) * 4;
-  const int nch = (int)std::max<size_t>(1, std::min<size_t>(CUT_MAX_WARPS, (200 * 1024) / words_bytes - 1));
+  int nch = (int)std::max<size_t>(1, std::min<size_t>(CUT_MAX_WARPS, (200 * 1024) / words_bytes - 1));
   // queries per warp: enough CTAs for about two per SM, at least 32 (a warp's reads of the
   // newcomers' ranks) and at most 512 (the serial chain of one warp)
   const int want = std::max(1, (2 * sms + n_rows - 1) / n_rows);
   const int per = (S + nch * want - 1) / (nch * want);
-  const int chunk = std::min(512, std::max(32, (per + 31) / 32 * 32));
+  int chunk = std::min(512, std::max(32, (per + 31) / 32 * 32));
+  if (S <= kShortRow) {
+    nch = n_rows > 2 * sms ? CUT_MAX_WARPS / 2 : CUT_MAX_WARPS;
+    chunk = (S + nch - 1) / nch;
+  }
   const int split = (S + nch * chunk - 1) / (nch * chunk);
   const size_t smem = (size_t)(nch + 1) * words_bytes;
   e = raise_smem_limit(cutoff_kernel, smem);
