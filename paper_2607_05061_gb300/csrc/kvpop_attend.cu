@@ -367,9 +367,12 @@ __global__ void __launch_bounds__(Traits<T, HD, G>::THREADS, 1) attend_kernel(At
       consumer_sync(NWC * 32);
       if (flag[1]) {
         __threadfence();
-        merge_partials<G, HD, NWC * 32>(ca, cb, a.part, a.out + (size_t)p * G * HD, mo,
-                                        [] { consumer_sync(NWC * 32); },
-                                        [](float x) { return fast_exp2(x); });
+        // two rows at a time: at the kernel's register limit (168) more of them spill what the
+        // loop over the keys holds (bf16, G = 4, d = 128: 64 x 8 pairs of 4112 keys 364 us with
+        // 20, 300 with 2; batch 1 18.5 with either)
+        merge_partials<G, HD, NWC * 32, 2>(ca, cb, a.part, a.out + (size_t)p * G * HD, mo,
+                                           [] { consumer_sync(NWC * 32); },
+                                           [](float x) { return fast_exp2(x); });
       }
     }
     consumer_sync(NWC * 32);

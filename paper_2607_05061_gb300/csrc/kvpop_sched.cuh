@@ -82,14 +82,14 @@ __device__ __forceinline__ bool schedule_changed(const int32_t* __restrict__ nva
 // A partial's place is fixed by the split: the pair's first tile lies in CTA ca (second slot
 // of its two), every later CTA starts inside the pair (first slot).  The (max, sum) pairs are
 // fetched once for all threads into `fac` (2 G (cb - ca + 1) floats of shared memory), and the
-// rows are loaded 20 at a time with them, so a merge costs an L2 latency or two instead of one
+// rows are loaded RB at a time with them, so a merge costs an L2 latency or two instead of one
 // chain of 2 (cb - ca + 1) per thread: a pair at batch 1 spreads over 19 CTAs,
 // and from its last arrival to the end of the launch went 8 us with 8 single rows in flight, 6
 // with 20 double ones (a 4-layer step at batch 1: 316 us with the chain, 235 with this and the
 // early launches below).
 constexpr int kMaxAttendGrid = 256;      // CTAs whose factors fit in the warps' partials (4 HD)
 
-template <int G, int HD, int NCT, typename SyncFn, typename ExpFn>
+template <int G, int HD, int NCT, int RB = 20, typename SyncFn, typename ExpFn>
 __device__ __forceinline__ void merge_partials(long long ca, long long cb, const float* part, float* out,
                                                float* fac, SyncFn sync, ExpFn ex) {
   constexpr int PSTRIDE = G * HD + 2 * G;
@@ -103,7 +103,7 @@ __device__ __forceinline__ void merge_partials(long long ca, long long cb, const
     fac[2 * i + 1] = __ldcg(pc + G);
   }
   // V neighbouring outputs per thread, RB rows in flight; the first ones travel with the factors
-  constexpr int V = (G * HD) % (2 * NCT) == 0 ? 2 : 1, RB = 20;
+  constexpr int V = (G * HD) % (2 * NCT) == 0 ? 2 : 1;
   using Vec = std::conditional_t<V == 2, float2, float>;
   auto load = [&](Vec (&row)[RB], int c0, int idx) {
 #pragma unroll
