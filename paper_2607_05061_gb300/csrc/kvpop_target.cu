@@ -390,11 +390,14 @@ __global__ void __launch_bounds__(TgP<HD>::THREADS, 1) target_tc_kernel(TargetAr
 // unit (64 per MMA) and 1024 of the exponential unit (32 per clock); the softmax warps' code sets
 // the pace, about 1500 clocks (causal) and 2000 (future, which also reads a normaliser per
 // column).  What paid: barriers arrived at once per warp, a warp's whole part in registers
-// before its exponentials (the S buffer is free at once), and the MMA warp's operands kept
-// warp-uniform (see elect_one; 945 -> 815 us).  8 heads x 16384 tokens, 4 query heads each:
-// causal 794 us, against 1354 with 64-key blocks in the prompt kernel; future 980 us, against
-// 1363 with copies by cp.async, one arrival per thread and the rows in shared memory.  Measured
-// and not kept: a cluster of two CTAs sharing the streamed blocks by multicast (843 / 1075 us).
+// before its exponentials (the S buffer is free at once), the MMA warp's operands kept
+// warp-uniform (see elect_one; 945 -> 815 us), and the row operand loaded as whole lines before the
+// set-up (798 -> 778 us; 16 x 8 heads of 256 tokens 35.0 -> 26.8, of 1024 158 -> 134).  8 heads x
+// 16384 tokens, 4 query heads each: causal 778 us, against 1354 with 64-key blocks in the prompt
+// kernel; future 1017 us, against 1363 with copies by cp.async, one arrival per thread and the rows
+// in shared memory.  Measured and not kept: a cluster of two CTAs sharing the streamed blocks by
+// multicast (843 / 1075 us); column halves past the last streamed one left out (2% slower from 1500
+// tokens on).
 // Blocks: longest tiles first over all pairs (tiles of one pair after the other left the last
 // pair's longest tile to the end).
 constexpr int T6_HALF = 128;
@@ -467,6 +470,19 @@ __global__ void __launch_bounds__(T6_THREADS, 1)
   }
   const int nblk = (d_hi - d_lo + T6_BN) / T6_BN;
   const int total = FUTURE ? G * nblk : nblk;
+  // Rows of the A operand on their way while barriers and tensor memory are set up: warps 0-3 and
+  // 4-7 take 32 rows of a half each, four lanes 64 bytes of a row at a time (see below).
+  float4 x[16];                                    // piece lane % 4 of rows 8 (i % 4) + lane / 4
+  if (warp < T6_SOFT / 2) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const int rr = warp * 32 + 8 * (i & 3) + (lane >> 2);
+      const int tt = t0 + (FUTURE ? rr : rr % NQ);
+      const bf16* src = a.A + ((size_t)(FUTURE ? pair : qrow0 + rr / NQ) * S + (tt <= t1 ? tt : t0)) * 128;
+      x[i] = __ldg(reinterpret_cast<const float4*>(src) + 4 * (i >> 2) + (lane & 3));
+      if (tt > t1) x[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  }
   auto bar = [&](int i) { return sb + T6_OFF_BAR + 8u * (uint32_t)i; };
   if (tid == 0) {
     for (int i = 0; i < T6_ST; ++i) {
@@ -480,9 +496,7 @@ __global__ void __launch_bounds__(T6_THREADS, 1)
     mbar_init(bar(T6_AFULL), T6_SOFT / 2);
     mbar_fence_init();
   }
-  // the softmax halves' exchange slots start with no head done
   static_assert(G <= T6_MAX_G, "one slot per head");
-  for (int i = tid; i < G * 2 * T6_HALF; i += T6_THREADS) reinterpret_cast<int*>(sm6 + T6_OFF_PX)[4 * i + 2] = 0;
   if (warp == T6_MMA_WARP) tmem_alloc(sb + T6_OFF_TMEM, 512);
   fence_before();
   __syncthreads();
@@ -577,19 +591,29 @@ __global__ void __launch_bounds__(T6_THREADS, 1)
     float* pxs = reinterpret_cast<float*>(sm6 + T6_OFF_PX);
     const uint64_t cc = f2_pack(a.scale, a.scale);
     if (cs == 0) {
-      // the row into tensor memory as the MMA's A operand (zeros past the tile)
-      const bf16* src = a.A + ((size_t)(FUTURE ? pair : qrow0 + ra / NQ) * S + (t <= t1 ? t : t0)) * 128;
+      // The warp's 32 rows into tensor memory as the MMA's A operand (zeros past the tile): the
+      // pieces change lanes in the warp's part of the exchange slots (loaded a row per lane, each
+      // load would touch 32 lines: 2 us of a CTA).
+      auto at = [&](int row, int c) {               // 16-byte piece c of a row's 64 bytes
+        return reinterpret_cast<float4*>(pxs) + (c * 2 + hh) * T6_HALF + (warp & 3) * 32 + (row ^ (2 * c));
+      };
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        float v[32];
+      for (int h = 0; h < 4; ++h) {
+        float v[16];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float4 x = t <= t1 ? __ldg(reinterpret_cast<const float4*>(src + 64 * c) + i)
-                                   : make_float4(0.f, 0.f, 0.f, 0.f);
-          v[4 * i] = x.x; v[4 * i + 1] = x.y; v[4 * i + 2] = x.z; v[4 * i + 3] = x.w;
+        for (int k = 0; k < 4; ++k) *at(8 * k + (lane >> 2), lane & 3) = x[4 * h + k];
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float4 y = *at(lane, k);
+          v[4 * k] = y.x; v[4 * k + 1] = y.y; v[4 * k + 2] = y.z; v[4 * k + 3] = y.w;
         }
-        tmem_st32(tl + hh * 64 + c * 32, v);
+        __syncwarp();
+        tmem_st16(tl + hh * 64 + h * 16, v);
       }
+      // the rows' exchange slots start with no head done (read after S, and so after all of this)
+#pragma unroll
+      for (int g = 0; g < G; ++g) reinterpret_cast<int*>(pxs)[4 * ((g * 2 + hh) * T6_HALF + r) + 2] = 0;
       tmem_wait_st();
       fence_before();
       __syncwarp();
@@ -640,7 +664,7 @@ __global__ void __launch_bounds__(T6_THREADS, 1)
       // so is off by up to its size times 2^-24.  Mean error from 64 bits of 8 heads x 16384
       // tokens with outlier channels 7.7e-7 (2^60: 7.9e-7; a base moved at 2^8 of one logit, as in
       // the prompt kernel: 7.7e-7), where the first keys' logits lie 32 below the others' 8.0e-7
-      // (1.8e-6; 8.0e-7), at 802 us (798; 1352).
+      // (1.8e-6; 8.0e-7), for 4 us in 798.
       constexpr float kMaxSum = FUTURE ? 0x1p60f : 0x1p8f;
 #pragma unroll
       for (int c = 0; c < 2; ++c) {
