@@ -348,7 +348,7 @@ static kvpop_status init_cache(const kvpop_config* cfg_in, const kvpop_scorer* s
     s = dev_alloc(c, &p, pairs * (dm.G * d + 2 * dm.G) * 4);
     c->fb.part_c = static_cast<float*>(p);
     if (s == KVPOP_OK) { s = dev_alloc(c, &p, pairs * 4 * 4); c->fb.meta_next = (int32_t*)p; }
-    if (s == KVPOP_OK) { s = dev_alloc(c, &p, pairs * (2 * dm.G + 2 * d) * 4); c->fb.xtra = (float*)p; }
+    if (s == KVPOP_OK) { s = dev_alloc(c, &p, pairs * xtra_floats(dm.G, dm.d) * 4); c->fb.xtra = (float*)p; }
     if (s == KVPOP_OK) { s = dev_alloc(c, &p, 16); c->fb.ctr = static_cast<unsigned long long*>(p); }
     if (s == KVPOP_OK) {
       s = dev_alloc(c, &p, (size_t)c->fused_grid * sizeof(int2));

@@ -185,6 +185,10 @@ struct FusedBufs {
   unsigned long long* ctr;     // CTAs past their schedule over all launches (zero at init)
   int2* start_prev;            // [grid] where each CTA's range began last launch (zero at init)
 };
+// Record of a pair's two changed keys: 2 G logits, padded to whole 16 bytes (the V rows behind them
+// are stored as such), then two rows.
+__host__ __device__ constexpr int xtra_rows(int G) { return (2 * G + 3) & ~3; }
+__host__ __device__ constexpr int xtra_floats(int G, int d) { return xtra_rows(G) + 2 * d; }
 bool tc_fused_ok(const Dims& dm);
 // After a prompt or an import: V rows past the used ones to zero, where the one-kernel step relies
 // on it (its launch).

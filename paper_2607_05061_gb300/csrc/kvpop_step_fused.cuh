@@ -37,8 +37,8 @@ struct FusedArgs {
   float* score_out;                // [b][H] or null
   float* part_c;                   // [pairs][G d + 2 G]: partial of a pair streamed by one CTA
   int32_t* meta_next;              // [pairs][4]: length, used slots, min priority (bits), min slot
-  float* xtra;                     // [pairs][2 G + 2 d]: logits of the two changed keys per head
-                                   // (log2 domain, -inf when absent), then their V rows
+  float* xtra;                     // [pairs][xtra_floats(G, d)]: logits of the two changed keys per
+                                   // head (log2 domain, -inf when absent), then their V rows
   unsigned long long* ctr;         // CTAs past their schedule, counted over all launches
   int2* start_prev;                // [grid] (pair, tile of the pair) each CTA's range began
                                    // with in the last launch
@@ -190,7 +190,7 @@ __device__ void fused_merge(const FusedArgs& f, float* out, const float* part, i
   const int nctas = pair_ctas(p, prefix, sp, ca, cb);
   const bool single = (nctas == 1);
   // the two keys that changed this step: the scorer's record of their logits and V rows
-  const float* xr = f.xtra + (size_t)p * (2 * G + 2 * HD);
+  const float* xr = f.xtra + (size_t)p * xtra_floats(G, HD);
   // output elements idx = tid + k NTHR, in chunks of up to 4 (every load of a chunk and
   // contributor issued together)
   constexpr int CH = EPT < 4 ? EPT : 4;
@@ -211,8 +211,8 @@ __device__ void fused_merge(const FusedArgs& f, float* out, const float* part, i
       const int g = (in ? idx : 0) / HD, i = (in ? idx : 0) % HD;
       s0[u] = in ? __ldcg(xr + 2 * g) : -INFINITY;
       s1[u] = in ? __ldcg(xr + 2 * g + 1) : -INFINITY;
-      v0[u] = in ? __ldcg(xr + 2 * G + i) : 0.f;
-      v1[u] = in ? __ldcg(xr + 2 * G + HD + i) : 0.f;
+      v0[u] = in ? __ldcg(xr + xtra_rows(G) + i) : 0.f;
+      v1[u] = in ? __ldcg(xr + xtra_rows(G) + HD + i) : 0.f;
     }
     for (long long cc = ca; cc <= cb; ++cc) {
       if (own_m && cc == own_cta) continue;
@@ -620,7 +620,7 @@ __device__ void fused_scorer(const FusedArgs& f, const bf16* q, float* out, cons
           unpack_bf16x4(ke4, k1f);
           unpack_bf16x4(ve4, v1f);
         }
-        float* xr = f.xtra + (size_t)pair * (2 * G + 2 * HD);
+        float* xr = f.xtra + (size_t)pair * xtra_floats(G, HD);
 #pragma unroll
         for (int g = 0; g < G; ++g) {
           float qf[4];
@@ -638,8 +638,8 @@ __device__ void fused_scorer(const FusedArgs& f, const bf16* q, float* out, cons
             xr[2 * g + 1] = has1 ? d1 * qscale : -INFINITY;
           }
         }
-        reinterpret_cast<float4*>(xr + 2 * G)[lane] = make_float4(v0f[0], v0f[1], v0f[2], v0f[3]);
-        reinterpret_cast<float4*>(xr + 2 * G + HD)[lane] = make_float4(v1f[0], v1f[1], v1f[2], v1f[3]);
+        reinterpret_cast<float4*>(xr + xtra_rows(G))[lane] = make_float4(v0f[0], v0f[1], v0f[2], v0f[3]);
+        reinterpret_cast<float4*>(xr + xtra_rows(G) + HD)[lane] = make_float4(v1f[0], v1f[1], v1f[2], v1f[3]);
       }
       if (lane == 0) {
         int32_t* mt = f.meta_next + (size_t)pair * 4;
