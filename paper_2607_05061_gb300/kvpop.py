@@ -351,6 +351,8 @@ def project_out(o, Wo, x, y, stream=None, settled=False):
     _shape("project_out", "Wo", Wo, bf, K, N)
     _shape("project_out", "x", x, bf, M, N)
     _shape("project_out", "y", y, bf, M, N, more_rows=True)
+    if 0 < abs(x.data_ptr() - y.data_ptr()) < 2 * M * N:
+        raise ValueError("project_out: y overlaps x (it may only be x)")
     _project_out(o, Wo, x, y, stream, settled)
 
 

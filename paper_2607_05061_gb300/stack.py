@@ -63,6 +63,12 @@ class DecodeStack:
                    t.device == self.q.device and not t.requires_grad and t.data_ptr() % 16 == 0
                    for t, s in want)
 
+    @staticmethod
+    def _overlap(a, b) -> bool:
+        """Whether two tensors of one size share some of their memory, but not all of it in place
+        (the output kernel would read what it has written; torch.add refuses such a pair)."""
+        return 0 < abs(a.data_ptr() - b.data_ptr()) < a.numel() * a.element_size()
+
     # ------------------------------------------------------------------ prefill
     def prefill_layer(self, l: int, X: torch.Tensor, lengths: Sequence[int], first_seq: int = 0,
                       override=None):
@@ -105,7 +111,7 @@ class DecodeStack:
             if outputs is not None:
                 outputs[l].copy_(self.o)
             if self._project & 2 and self._plain((x, (self.b, hid)), (nxt, (self.b, hid)),
-                                                 (L["Wo"], (nq, hid))):
+                                                 (L["Wo"], (nq, hid))) and not self._overlap(x, nxt):
                 _project_out(self.o, L["Wo"], x, nxt, settled=settled)
                 settled = True
             else:

@@ -8,6 +8,9 @@ def bf(*shape):
     return torch.zeros(shape, dtype=torch.bfloat16)
 
 
+BUF = bf(5, 64)
+
+
 def call(name, **other):
     from paper_2607_05061_gb300 import kvpop
     M, K, nq, nkv = 4, 64, 96, 48
@@ -25,7 +28,7 @@ def call(name, **other):
     ("project_qkv", dict(k=torch.zeros(4, 48))),
     ("project_out", dict(o=torch.zeros(4, 64))), ("project_out", dict(o=bf(4, 96))), ("project_out", dict(o=torch.zeros(3, 96))),
     ("project_out", dict(Wo=bf(96, 56))), ("project_out", dict(y=bf(4, 56))), ("project_out", dict(y=bf(2, 64))),
-    ("project_out", dict(x=bf(64, 4).T))])
+    ("project_out", dict(x=bf(64, 4).T)), ("project_out", dict(x=BUF[:4], y=BUF[1:]))])
 def test_wrong_tensors_are_refused(name, other):
     from paper_2607_05061_gb300 import build
     build.build()
