@@ -357,7 +357,9 @@ __global__ void __launch_bounds__(NTM) mlstm_proj_kernel(MProjArgs a) {
 // the shared-memory image of its tiles), so W x is three products whose terms are exact.  The
 // tensor unit rounds a running sum toward zero; to keep that below the rounding of a chain of
 // fp32 FMAs, each 64 inputs are summed on their own, smallest parts first, and added in fp32
-// (two accumulators of 128 inputs each: out.score 1.1e-6 from 64 bits, 6.8e-7 this way).  A CTA
+// (two accumulators of 128 inputs each: out.score 1.1e-6 from 64 bits, 6.8e-7 this way; the scores
+// of prompts of 250 to 4009 tokens, with the readout below, 2.1e-7 to 2.9e-7 in the mean and 4.2e-6
+// at most, against 5.4e-7 to 6.4e-7 and 1.8e-5 with chains of fp32 FMAs).  A CTA
 // takes 128 tokens: one warp copies the weights (80 KB per 64 inputs, two buffers) and issues
 // the MMAs (M = 128, N = 208); 8 warps load the tokens and, one thread per token and feature
 // map, add up the token's accumulator rows and run the Hedgehog softmaxes on them, then hand
