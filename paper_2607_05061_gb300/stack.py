@@ -134,6 +134,8 @@ class DecodeStack:
         s.wait_stream(torch.cuda.current_stream())
         g = torch.cuda.CUDAGraph()
         with torch.cuda.stream(s):
+            # cuBLAS, which some projections may need, sets itself up outside a capture only
+            torch.matmul(self.x[0], self.x[0].T)
             with torch.cuda.graph(g, stream=s):
                 # a replay starts after all that is queued before it is complete
                 self._step_into(x_in, x_out, settled=True)
