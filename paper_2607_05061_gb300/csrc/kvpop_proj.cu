@@ -9,9 +9,10 @@
 // meet in shared memory at the end, in warp order.  While the kernel before this one still runs,
 // the first stages' weights go to L2, which is only a hint and so needs no order with a kernel
 // that may write them, and into the ring after griddepcontrol.wait; weights that the caller
-// states to be settled go into the ring at once.  The next kernel may start after that wait, and
-// so after all that came before this one.  The products run on mma.sync with the weights as the 16-row operand and the
-// sequences as the 8-column one: at so few rows the tensor work is far below the stream.
+// states to be settled go into the ring at once (hidden 4096, batch 1: 11.6 us, 12.7 otherwise).
+// The next kernel may start after that wait, and so after all that came before this one.  The
+// products run on mma.sync with the weights as the 16-row operand and the sequences as the
+// 8-column one: at so few rows the tensor work is far below the stream.
 // Device time at hidden 4096, 32 query and 8 KV heads, alone and cold: q, k, v at 1 to 8 rows
 // 14 us (7.5 us at the copy rate) against 32 us of cuBLAS's six launches, the output 13 us
 // (5 us) against 18 us of four; a 4-layer step at batch 1 230 -> 198 us, at batch 8 284 -> 245.

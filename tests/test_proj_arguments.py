@@ -26,7 +26,8 @@ def call(name, **other):
     ("project_qkv", dict(Wk=bf(32, 48))), ("project_qkv", dict(Wq=bf(63, 96))), ("project_qkv", dict(q=bf(4, 88))),
     ("project_qkv", dict(Wq=bf(96, 64).T)), ("project_qkv", dict(x=torch.zeros(4, 64))),
     ("project_qkv", dict(k=torch.zeros(4, 48))),
-    ("project_out", dict(o=torch.zeros(4, 64))), ("project_out", dict(o=bf(4, 96))), ("project_out", dict(o=torch.zeros(3, 96))),
+    ("project_out", dict(o=torch.zeros(4, 64))), ("project_out", dict(o=bf(4, 96))),
+    ("project_out", dict(o=torch.zeros(3, 96))),
     ("project_out", dict(Wo=bf(96, 56))), ("project_out", dict(y=bf(4, 56))), ("project_out", dict(y=bf(2, 64))),
     ("project_out", dict(x=bf(64, 4).T)), ("project_out", dict(x=BUF[:4], y=BUF[1:]))])
 def test_wrong_tensors_are_refused(name, other):
